@@ -99,7 +99,6 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     // 4 and 5 tokens at G / k = 3.9).
     p->mma_min_tokens = max(2, min(kMmaMinTokens, (int)ceilf(1.15f * (float)p->G / (float)cfg->k)));
     alloc((void **)&p->mask, nt * 4 * sizeof(uint32_t));
-    alloc((void **)&p->gmask, (size_t)kMaxG * 4 * sizeof(uint32_t));
     alloc((void **)&p->counts, (size_t)kMaxG * sizeof(int32_t));
     alloc((void **)&p->offsets, (size_t)(kMaxG + 1) * sizeof(int32_t));
     alloc((void **)&p->token_ids, nt * cfg->k * sizeof(int32_t));
@@ -112,22 +111,24 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
         alloc((void **)&p->act, 2 * max(nt, (size_t)128) * cfg->d_ff * 2);
         // slices * padded tokens never exceeds 128 * (SMs / column tiles): see launch_ffn_mma
         const size_t slice_rows = (size_t)128 * (p->sm_count / max(1, cfg->d / 256) + 1);
-        alloc((void **)&p->mma_partial, max(slice_rows, m_pad) * cfg->d * sizeof(float));
+        const size_t decode_rows = (size_t)decode_slices(p) * min(nt, (size_t)kDecodeMaxTokens);
+        alloc((void **)&p->mma_partial, max(max(slice_rows, max(decode_rows, 2 * min(nt, (size_t)kDecodeMaxTokens))), m_pad) * cfg->d * sizeof(float));
+        alloc((void **)&p->rscale, nt * sizeof(float));
     }
     alloc((void **)&p->x_host_in, nt * cfg->d * sizeof(float));
     alloc((void **)&p->x_host_out, nt * cfg->d * sizeof(float));
     for (int i = 0; i < 2 * CS_STAGE_COUNT; ++i)
         if (e == cudaSuccess) e = cudaEventCreate(&p->ev[i]);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemset(p->status, 0, sizeof(DeviceStatus));
     if (e == cudaSuccess) e = cudaMemset(p->ticket, 0, nt * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(p->slot_table, 0, nt * kSlotTablePitch * sizeof(int32_t));
     if (e == cudaSuccess && prepare_sketch(p) != CS_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess && prepare_recover(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && prepare_solvers(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && prepare_ffn_gather(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && p->mma_ok && prepare_ffn_mma(p) != CS_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess && p->mma_ok && prepare_decode(p) != CS_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess) e = cudaMemset(p->mask, 0, nt * 4 * sizeof(uint32_t));
     if (e != cudaSuccess) {
         cs_plan_destroy(p);
         return CS_ERR_CUDA;
@@ -142,13 +143,10 @@ cs_status cs_plan_destroy(cs_plan *p) {
     cudaFree(p->partial); cudaFree(p->gram); cudaFree(p->slot_table); cudaFree(p->ticket);
     cudaFree(p->resid_buf); cudaFree(p->fb_flags); cudaFree(p->fb_list); cudaFree(p->fb_count); cudaFree(p->hbar); cudaFree(p->colsum);
     cudaFree(p->status); cudaFree(p->x_host_in); cudaFree(p->x_host_out);
-    cudaFree(p->mask); cudaFree(p->gmask); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
-    cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial);
+    cudaFree(p->mask); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
+    cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial); cudaFree(p->rscale);
     for (int i = 0; i < 2 * CS_STAGE_COUNT; ++i)
         if (p->ev[i] != nullptr) cudaEventDestroy(p->ev[i]);
-    if (p->ev_fork != nullptr) cudaEventDestroy(p->ev_fork);
-    if (p->ev_join != nullptr) cudaEventDestroy(p->ev_join);
-    if (p->side != nullptr) cudaStreamDestroy(p->side);
     delete p;
     return CS_OK;
 }
@@ -176,9 +174,9 @@ cs_status cs_recover_warm(cs_plan *plan, const float *Phi, float mu, const float
     if (B <= 0 || B > plan->cfg.max_tokens || T < 1) return CS_ERR_SHAPE;
     if (!isfinite(mu) || !(mu > 0.f)) return CS_ERR_NONFINITE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cs_status s = launch_check_support(plan, support0, B, st);
-    if (s != CS_OK) return s;
-    return launch_recover(plan, Phi, mu, y, B, support, z, resid, false, st, T, support0, z0);
+    RecoverOptions o;
+    o.T = T; o.sup0 = support0; o.z0 = z0; o.check = support0;
+    return launch_recover(plan, Phi, mu, y, B, support, z, resid, false, st, o);
 }
 
 cs_status cs_support_drift(cs_plan *plan, const int32_t *support_prev, const int32_t *support_cur, int32_t B,
@@ -218,15 +216,33 @@ static cs_status check_options(const cs_plan *plan, const cs_step_options *o, bo
     return CS_OK;
 }
 
-// The estimator an options struct asks for, on y; gram_ready: plan->gram holds this Phi's matrix.
+// The estimator an options struct asks for, on y, with the check of the previous supports and the drift against
+// them; gram_ready: plan->gram holds this Phi's matrix; decode: see RecoverOptions (CS_SOLVER_IHT only).
 static cs_status recover_with(cs_plan *plan, const float *Phi, float mu, const float *y, int B, const cs_step_options *o,
-                              int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st) {
+                              int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st, bool decode = false,
+                              bool norm = false) {
     const int T = o->T < 0 ? plan->cfg.T : o->T;
-    if (o->solver == CS_SOLVER_NIHT) return launch_niht(plan, Phi, mu, y, B, T, support, z, resid, st);
-    if (o->solver == CS_SOLVER_OMP) return launch_omp(plan, Phi, y, B, support, z, resid, st);
-    return launch_recover(plan, Phi, mu, y, B, support, z, resid, gram_ready, st, T,
-                          o->warm_start ? o->support_prev : nullptr, o->warm_start ? o->z_prev : nullptr, o->gamma,
-                          o->gamma > 0.f ? o->support_prev : nullptr, o->gamma > 0.f ? o->z_prev : nullptr);
+    if (o->solver == CS_SOLVER_IHT) {
+        RecoverOptions r;
+        r.T = T; r.gamma = o->gamma; r.decode = decode; r.norm = norm;
+        if (o->warm_start) { r.sup0 = o->support_prev; r.z0 = o->z_prev; }
+        if (o->gamma > 0.f) { r.sup_prev = o->support_prev; r.z_prev = o->z_prev; }
+        r.check = o->support_prev; r.delta = o->delta_out; r.drift = o->drift_out;
+        // the supports may overwrite the previous ones, which the drift needs
+        if (support == o->support_prev) r.delta = nullptr, r.drift = nullptr;
+        cs_status s = launch_recover(plan, Phi, mu, y, B, support, z, resid, gram_ready, st, r);
+        if (s != CS_OK || support != o->support_prev) return s;
+    } else {
+        cs_status s = CS_OK;
+        if (o->support_prev != nullptr) s = launch_check_support(plan, o->support_prev, B, st);
+        if (s == CS_OK)
+            s = o->solver == CS_SOLVER_NIHT ? launch_niht(plan, Phi, mu, y, B, T, support, z, resid, st)
+                                            : launch_omp(plan, Phi, y, B, support, z, resid, st);
+        if (s != CS_OK) return s;
+    }
+    if (o->delta_out != nullptr || o->drift_out != nullptr)
+        return launch_support_drift(plan, o->support_prev, support, B, o->delta_out, o->drift_out, st);
+    return CS_OK;
 }
 
 cs_status cs_recover_ex(cs_plan *plan, const float *Phi, float mu, const float *y, int32_t B,
@@ -238,15 +254,7 @@ cs_status cs_recover_ex(cs_plan *plan, const float *Phi, float mu, const float *
     cs_status s = check_options(plan, opt, false);
     if (s != CS_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (opt->support_prev != nullptr) {
-        s = launch_check_support(plan, opt->support_prev, B, st);
-        if (s != CS_OK) return s;
-    }
-    s = recover_with(plan, Phi, mu, y, B, opt, support, z, resid, false, st);
-    if (s != CS_OK) return s;
-    if (opt->delta_out != nullptr || opt->drift_out != nullptr)
-        s = launch_support_drift(plan, opt->support_prev, support, B, opt->delta_out, opt->drift_out, st);
-    return s;
+    return recover_with(plan, Phi, mu, y, B, opt, support, z, resid, false, st);
 }
 
 cs_status cs_sketch_srht(cs_plan *plan, const uint32_t *sign_bits, const int32_t *rows, const float *h, int32_t B,
@@ -270,40 +278,11 @@ static cs_status check_weights(const cs_layer *L) {
     return CS_OK;
 }
 
-extern "C++" {
-static bool use_decode_mma(const cs_plan *plan, int B) { return plan->mma_ok && B >= plan->mma_min_tokens && B <= 128; }
-
-// Tensor-core decode path from the crossover batch (mma_min_tokens) up to 128 tokens.  The gate/up
-// GEMM needs no supports (at these batch sizes the union of the supports is, to within a group or two, every group), so it runs on the
-// caller's stream while `side_work` -- sketch / recovery / bucketing -- runs on the plan's second
-// stream; the two join before the activations are masked and the down GEMM starts.
-// gamma != NULL: h is the un-normalised x and the operand split applies the RMSNorm itself.
-template <typename SideWork>
-static cs_status exec_decode_overlapped(cs_plan *plan, const cs_layer *layer, const float *h, int B,
-                                        const float *residual, float *out, cudaStream_t st, SideWork side_work,
-                                        const float *gamma = nullptr) {
-    __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
-    __nv_bfloat16 *x_lo = x_hi + (size_t)plan->cfg.max_tokens * plan->cfg.d;
-    CS_CUDA_TRY(plan, cudaEventRecord(plan->ev_fork, st));
-    CS_CUDA_TRY(plan, cudaStreamWaitEvent(plan->side, plan->ev_fork, 0));
-    cs_status s = side_work(plan->side);
-    if (s != CS_OK) return s;
-    CS_CUDA_TRY(plan, cudaEventRecord(plan->ev_join, plan->side));
-    // f32 activations go in as two bf16 parts so that the result keeps f32-level accuracy
-    s = gamma != nullptr ? launch_norm_split_bf16(plan, h, gamma, B, x_hi, x_lo, st)
-                         : launch_split_bf16(plan, h, x_hi, x_lo, (size_t)B * plan->cfg.d, st);
-    if (s != CS_OK) return s;
-    s = launch_decode_gateup(plan, layer, x_hi, x_lo, B, false, st);
-    if (s != CS_OK) return s;
-    CS_CUDA_TRY(plan, cudaStreamWaitEvent(st, plan->ev_join, 0));
-    s = launch_decode_mask(plan, B, st);
-    if (s != CS_OK) return s;
-    return launch_decode_down(plan, layer, B, true, residual, out, st);
+static bool use_decode_mma(const cs_plan *plan, int B) {
+    return plan->mma_ok && B >= plan->mma_min_tokens && B <= kDecodeMaxTokens;
 }
 
-}  // extern "C++"
-
-// Dispatch of the actuator by batch size: gather GEMV, tensor-core decode path, or (more than 128
+// Dispatch of the actuator by batch size: gather GEMV, tensor-core decode path, or (more than kDecodeMaxTokens
 // tokens) the token-tiled grouped GEMMs over the union list.
 // check: the supports come from the caller and are validated on the device (inside the gather
 // kernel, or by a small kernel ahead of the tensor-core paths).
@@ -311,28 +290,17 @@ static cs_status exec_dispatch(cs_plan *plan, const cs_layer *layer, const float
                                int B, const float *residual, float *out, bool check, cudaStream_t st) {
     if (!plan->mma_ok || B < plan->mma_min_tokens)
         return launch_ffn_gather(plan, layer, h, support, B, residual, out, check, st);
+    if (use_decode_mma(plan, B)) {
+        cs_status s = launch_decode_prep(plan, h, support, B, check, st);
+        if (s != CS_OK) return s;
+        return launch_decode_ffn(plan, layer, B, false, false, residual, out, st);
+    }
     if (check) {
         cs_status s = launch_check_support(plan, support, B, st);
         if (s != CS_OK) return s;
     }
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
     __nv_bfloat16 *x_lo = x_hi + (size_t)plan->cfg.max_tokens * plan->cfg.d;
-    if (use_decode_mma(plan, B)) {
-        // The supports are known before the GEMMs here.  While the batch is small enough that a fair share
-        // of the groups is in nobody's support (expected unused fraction (1 - k/G)^B of about 8 % or more),
-        // the buckets are formed first and gate/up runs over the union list only, with the membership masks
-        // applied in its epilogue; beyond that the union is (nearly) every group and bucketing runs beside
-        // the dense gate/up GEMM instead.
-        if (2 * B * plan->cfg.k <= 5 * plan->G) {
-            cs_status s = launch_bucket(plan, support, B, st);
-            if (s == CS_OK) s = launch_split_bf16(plan, h, x_hi, x_lo, (size_t)B * plan->cfg.d, st);
-            if (s == CS_OK) s = launch_decode_gateup(plan, layer, x_hi, x_lo, B, true, st);
-            if (s == CS_OK) s = launch_decode_down(plan, layer, B, false, residual, out, st);
-            return s;
-        }
-        return exec_decode_overlapped(plan, layer, h, B, residual, out, st,
-                                      [&](cudaStream_t side) { return launch_bucket(plan, support, B, side); });
-    }
     cs_status s = launch_split_bf16(plan, h, x_hi, x_lo, (size_t)B * plan->cfg.d, st);
     if (s != CS_OK) return s;
     s = launch_bucket(plan, support, B, st);
@@ -377,16 +345,14 @@ cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, in
     const float *n = norm ? plan->n_buf : x;
     int32_t *sup = support_out != nullptr ? support_out : plan->sup_buf;
     if (use_decode_mma(plan, B)) {
-        // sketch, recovery and bucketing run beside the gate/up GEMM; with a normalisation the GEMM's
-        // operand split normalises for itself, so that it does not wait for the sketch kernel either
-        return exec_decode_overlapped(plan, layer, x, B, layer->add_residual ? x : nullptr, x_out, st,
-                                      [&](cudaStream_t side) {
-            cs_status r = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, norm ? plan->n_buf : nullptr,
-                                        layer->Phi, layer->mu, side);
-            if (r == CS_OK) r = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z_out, resid_out, true, side);
-            if (r == CS_OK) r = launch_bucket(plan, sup, B, side);
-            return r;
-        }, layer->rms_gamma);
+        // The sketch launch also splits the activations; the recovery runs beside the gate/up GEMM, which needs the
+        // supports only in its epilogue.
+        s = launch_sketch_slices(plan, layer, x, B, st);
+        RecoverOptions o;
+        o.decode = true; o.norm = norm;
+        if (s == CS_OK) s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z_out, resid_out, true, st, o);
+        if (s == CS_OK) s = launch_decode_ffn(plan, layer, B, true, norm, layer->add_residual ? x : nullptr, x_out, st);
+        return s;
     }
     const bool gather = !plan->mma_ok || B < plan->mma_min_tokens;
     if (gather && plan->speculative && sketch_recover_ok(plan) && !plan->timing) {
@@ -431,13 +397,11 @@ cs_status cs_layer_step_ex(cs_plan *plan, const cs_layer *layer, const float *x,
     const bool norm = layer->rms_gamma != nullptr;
     if (srht && norm) return CS_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (opt->support_prev != nullptr) {
-        s = launch_check_support(plan, opt->support_prev, B, st);
-        if (s != CS_OK) return s;
-    }
     const float *n = norm ? plan->n_buf : x;
     const float *residual = layer->add_residual ? x : nullptr;
     if (opt->reuse_support) {   // no estimation this step: the previous supports execute
+        s = launch_check_support(plan, opt->support_prev, B, st);
+        if (s != CS_OK) return s;
         if (norm) {   // the sketch kernel also forms the normalised input
             s = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, plan->n_buf, nullptr, 0.f, st);
             if (s != CS_OK) return s;
@@ -447,17 +411,19 @@ cs_status cs_layer_step_ex(cs_plan *plan, const cs_layer *layer, const float *x,
                                               cudaMemcpyDeviceToDevice, st));
         return exec_dispatch(plan, layer, n, opt->support_prev, B, residual, x_out, false, st);
     }
+    int32_t *sup = support_out != nullptr ? support_out : plan->sup_buf;
+    if (use_decode_mma(plan, B) && !srht && opt->solver == CS_SOLVER_IHT) {   // as in cs_layer_step
+        s = launch_sketch_slices(plan, layer, x, B, st);
+        if (s == CS_OK) s = recover_with(plan, layer->Phi, layer->mu, plan->y_buf, B, opt, sup, z_out, resid_out, true, st, true, norm);
+        if (s == CS_OK) s = launch_decode_ffn(plan, layer, B, true, norm, residual, x_out, st);
+        return s;
+    }
     if (srht) s = launch_sketch_srht(plan, opt->srht_sign, opt->srht_rows, x, B, plan->y_buf, st);
     else s = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, norm ? plan->n_buf : nullptr, layer->Phi,
                            layer->mu, st);
     if (s != CS_OK) return s;
-    int32_t *sup = support_out != nullptr ? support_out : plan->sup_buf;
     s = recover_with(plan, layer->Phi, layer->mu, plan->y_buf, B, opt, sup, z_out, resid_out, !srht, st);
     if (s != CS_OK) return s;
-    if (opt->delta_out != nullptr || opt->drift_out != nullptr) {
-        s = launch_support_drift(plan, opt->support_prev, sup, B, opt->delta_out, opt->drift_out, st);
-        if (s != CS_OK) return s;
-    }
     return exec_dispatch(plan, layer, n, sup, B, residual, x_out, false, st);
 }
 
@@ -515,14 +481,14 @@ cs_status cs_layer_step_host(cs_plan *plan, const cs_layer *layer, const float *
     // copy engine.
     const float *x_alias = nullptr;
     float *out_alias = nullptr;
-    if (bytes <= (pdl_for(plan, B) ? kZeroCopyBytes : kZeroCopyBytesLarge)) {
+    if (bytes <= (use_decode_mma(plan, B) ? kZeroCopyBytesLarge : kZeroCopyBytes)) {
         x_alias = static_cast<const float *>(device_alias(x_host));
         out_alias = static_cast<float *>(device_alias(x_out_host));
         if (x_alias == nullptr || out_alias == nullptr || !aligned16(x_alias) || !aligned16(out_alias)) x_alias = nullptr;
     }
     if (x_alias != nullptr) {
         const int n4 = (int)(bytes / 16);
-        launch_pdl(pdl_for(plan, B), stage_in_kernel, dim3((n4 + 255) / 256), dim3(256), 0, st,
+        launch_pdl(true, stage_in_kernel, dim3((n4 + 255) / 256), dim3(256), 0, st,
                    reinterpret_cast<const float4 *>(x_alias), reinterpret_cast<float4 *>(plan->x_host_in), n4);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());

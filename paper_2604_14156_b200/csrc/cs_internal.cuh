@@ -18,6 +18,7 @@ constexpr int kGatherMaxTokens = 16; // tokens per gather launch (scratch for pa
 constexpr int kSlotTableSlots = 32;  // slots per token of the recovery's slot table (small-batch step) ...
 constexpr int kSlotTablePitch = 40;  // ... and ints per token: the slots, then a word that says "final"
 constexpr int kReduceGroups = 32;    // partial-sum groups of the deterministic cross-CTA reduction
+constexpr int kDecodeMaxTokens = 256;   // largest decode batch of exec_decode.cu; larger ones take the 128-token tiles of exec_mma.cu
 constexpr int kMmaMinTokens = 16;    // decode batches at least this large always run on the tensor cores; a plan
                                      // lowers the bound by its G / k (cs_plan_set_crossover overrides it)
 
@@ -50,13 +51,13 @@ struct cs_plan {
     cs::DeviceStatus *status;  // device status word
     // tensor-core path (bf16 weights, 128-channel groups, d a multiple of 256)
     uint32_t *mask;      // [max_tokens, 4] membership bits: bit g of token t
-    uint32_t *gmask;     // [G, 4] membership bits the other way round: bit t of group g (t < 128)
     int32_t *counts;     // [G] tokens per group
     int32_t *offsets;    // [G + 1]
     int32_t *token_ids;  // [max_tokens * k] tokens of each group, ascending
     int32_t *glist;      // [G] groups with a non-empty bucket, ascending
     int32_t *nu;         // [1] their number
     void *x_bf16;        // [2][max_tokens, d] bf16 activations: rounded value, then remainder
+    float *rscale;       // [max_tokens] RMSNorm row scales, applied behind the gate/up GEMM
     void *act;           // [2][max_tokens, d_ff] bf16 SwiGLU activations over the group list (value, remainder)
     float *mma_partial;  // [slices, padded tokens, d] f32 partial down projections
     int speculative;     // small batches, on the recovery's first iterate: 1 = start the weight stream, 2 = warm L2 only
@@ -68,8 +69,6 @@ struct cs_plan {
     float *x_host_in;  // [max_tokens, d] staging for the host-buffer entry point
     float *x_host_out; // [max_tokens, d]
     cudaEvent_t ev[2 * CS_STAGE_COUNT];  // start/stop per stage
-    cudaStream_t side;                   // second stream: recovery runs beside the gate/up GEMM
-    cudaEvent_t ev_fork, ev_join;
     int timing;
     int stage_seen[CS_STAGE_COUNT];
     int nx_max;
@@ -112,12 +111,25 @@ struct StageTimer {
 // Phi != NULL: the launch also forms the recovery's matrix I - mu Phi^T Phi (plan->gram) in spare CTAs.
 cs_status launch_sketch(cs_plan *plan, const float *S, const float *x, const float *gamma, int B,
                         float *y, float *n_out, const float *Phi, float mu, cudaStream_t st);
+// The sensor in front of launch_decode_ffn: partial sketches per slice of columns (and of the squares, for the RMSNorm),
+// the two bf16 token matrices, and plan->gram.  The recovery adds the partials up.
+cs_status launch_sketch_slices(cs_plan *plan, const cs_layer *L, const float *x, int B, cudaStream_t st);
+struct RecoverOptions {
+    int T = -1;                                             // iterations; < 0: the plan's
+    const int32_t *sup0 = nullptr; const float *z0 = nullptr;   // warm start
+    float gamma = 0.f;                                      // temporal term towards (sup_prev, z_prev)
+    const int32_t *sup_prev = nullptr; const float *z_prev = nullptr;
+    const int32_t *check = nullptr;                         // supports to validate (ascending, distinct, in range) ...
+    int32_t *delta = nullptr; float *drift = nullptr;       // ... and the drift of the result against them
+    // launch_sketch_slices came before and launch_decode_ffn comes next: take the sketch from the partials (writing it
+    // to plan->y_buf), write the membership masks (plan->mask) and, with norm, the RMSNorm's row scales (plan->rscale), and
+    // let the dependents start only when the launches before the recovery are complete.
+    bool decode = false, norm = false;
+};
 // gram_ready: plan->gram already holds this Phi's matrix (the sketch launch before formed it).
 cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float *y, int B,
                          int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st,
-                         int T = -1 /* the plan's */, const int32_t *sup0 = nullptr, const float *z0 = nullptr,
-                         float gamma = 0.f /* temporal term */, const int32_t *sup_prev = nullptr,
-                         const float *z_prev = nullptr);
+                         const RecoverOptions &opt = RecoverOptions());
 // the other estimators (solvers.cu)
 cs_status prepare_solvers(cs_plan *plan);
 cs_status launch_niht(cs_plan *plan, const float *Phi, float mu_fallback, const float *y, int B, int T,
@@ -157,26 +169,22 @@ cs_status prepare_ffn_mma(cs_plan *plan);
 cs_status launch_bucket(cs_plan *plan, const int32_t *support, int B, cudaStream_t st, int32_t *counts = nullptr,
                         int32_t *offsets = nullptr, int32_t *token_ids = nullptr);
 cs_status launch_split_bf16(cs_plan *plan, const float *x, void *y_hi, void *y_lo, size_t n, cudaStream_t st);
-cs_status launch_norm_split_bf16(cs_plan *plan, const float *x, const float *gamma, int B, void *y_hi, void *y_lo,
-                                 cudaStream_t st);
 cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const void *X_lo, int M, const int32_t *glist,
                          const int32_t *ng_dev, int ng_host, const uint32_t *mask, const float *residual,
                          float *out_f32, void *out_bf16, cudaStream_t st);
-cs_status launch_decode_gateup(cs_plan *plan, const cs_layer *L, const void *X, const void *X_lo, int B,
-                               bool masked, cudaStream_t st);
-cs_status launch_decode_mask(cs_plan *plan, int B, cudaStream_t st);
-cs_status launch_decode_down(cs_plan *plan, const cs_layer *L, int B, bool act_by_group, const float *residual,
-                             float *out, cudaStream_t st);
+// decode batches of at most kDecodeMaxTokens tokens on the tensor cores (exec_decode.cu)
+cs_status prepare_decode(cs_plan *plan);
+int decode_slices(const cs_plan *plan);
+cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *support, int B, bool check, cudaStream_t st);
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, bool x_ready, bool rscale, const float *residual, float *out,
+                            cudaStream_t st);
 cs_status launch_prompt_mean(cs_plan *plan, const void *H, int n, float *hbar, cudaStream_t st);
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may start while its
 // predecessor in the stream is still running (its CTAs become resident, run their prologue and
 // then block in pdl_wait until the predecessor's writes are complete and visible).  Kernels call
 // pdl_launch_dependents early so that their successor can do the same.  Both are no-ops for a
-// kernel launched the ordinary way (pdl = false).  Only the small-batch chain uses it: its kernels are
-// a few microseconds long and launch latency matters; with the large tensor-core kernels early-resident
-// dependents measurably slowed the step down.
-inline bool pdl_for(const cs_plan *plan, int B) { return !(plan->mma_ok && B >= plan->mma_min_tokens); }
+// kernel launched the ordinary way (pdl = false).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -211,6 +219,21 @@ inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim
     cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
+
+// The partial sketches share plan->mma_partial with the down GEMM, whose first store comes after the recovery:
+// y [d / 64][B, m], then the squares [d / 64][B].  (d / 64) (m + 1) B <= 2 d B floats.
+inline float *sketch_partials(const cs_plan *plan) { return plan->mma_partial; }
+inline float *sketch_square_partials(const cs_plan *plan, int B) {
+    return plan->mma_partial + (size_t)(plan->cfg.d / 64) * B * plan->cfg.m;
+}
+
+// The small kernels around the large ones ask for the large ones' split of L1 and shared memory.  An SM changes its split
+// only when it is empty, so with the default split a CTA of 200 KB does not start beside a running recovery: at 64
+// tokens half of the gate/up CTAs then began 12 us late, when the last recovery on their SM had ended.
+template <typename Fn> inline cudaError_t prefer_shared(Fn *kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+cs_status prepare_recover(cs_plan *plan);
 
 // ---- small device helpers -------------------------------------------------------------------
 // Rows 2*blk and 2*blk+1 of M = I - mu Phi^T Phi by a CTA of kGramThreads threads.  M is stored
@@ -252,6 +275,15 @@ __device__ __forceinline__ uint4 ldg_stream(const void *p) {
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                  : "l"(p));
     return r;
+}
+
+// Four floats as bf16 values and bf16 remainders: hi = round(x), lo = round(x - hi).
+__device__ __forceinline__ void split4(float a, float b, float c, float e, uint2 &hi, uint2 &lo) {
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(a, b), h1 = __floats2bfloat162_rn(c, e);
+    const __nv_bfloat162 l0 = __floats2bfloat162_rn(a - __low2float(h0), b - __high2float(h0));
+    const __nv_bfloat162 l1 = __floats2bfloat162_rn(c - __low2float(h1), e - __high2float(h1));
+    hi.x = *reinterpret_cast<const uint32_t *>(&h0); hi.y = *reinterpret_cast<const uint32_t *>(&h1);
+    lo.x = *reinterpret_cast<const uint32_t *>(&l0); lo.y = *reinterpret_cast<const uint32_t *>(&l1);
 }
 
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }

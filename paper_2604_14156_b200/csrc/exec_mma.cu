@@ -25,151 +25,14 @@
 // (one elected lane), warps 2-5 run the epilogue (one warp per 32 TMEM lanes).  Every wait on an
 // mbarrier is bounded; a wait that runs out records CS_ERR_TIMEOUT in the plan's status word and the
 // CTA drains and exits.
-#include <cuda.h>
-
 #include <algorithm>
 #include <vector>
 
-#include "cs_internal.cuh"
+#include "mma_core.cuh"
 
 namespace cs {
 
 namespace {
-
-constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int kMaxStages = 8;
-constexpr int kABytes = BM * BK * 2;   // 16 KB
-constexpr int kBBytes = BN * BK * 2;   // 32 KB
-constexpr int kRingBytesMma = 4 * (kABytes + kBBytes);   // 192 KB of operand tiles
-constexpr int kMmaThreads = 192;
-// Epilogue warps come in slices of four (a warp may read the tensor-memory lane quarter warp % 4); a kernel
-// launched with 64 + 128 S threads drains its accumulators with S slices, each taking every S-th chunk.
-constexpr int kSwapMaxThreads = 64 + 4 * 128;
-constexpr int kTileThreads = kSwapMaxThreads;   // the 128-token-tile kernels: four slices
-constexpr uint32_t kSpinLimit = 1u << 20;
-constexpr size_t kMmaSmem = 1024 + (size_t)kRingBytesMma + 256;
-
-struct Barriers {
-    uint64_t full[kMaxStages];
-    uint64_t empty[kMaxStages];
-    uint64_t acc_ready;
-    uint32_t tmem_base;
-    uint32_t aborted;
-};
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// Bounded wait on a phase parity.  Returns false (after flagging the timeout) if the limit is hit.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Barriers *bars, DeviceStatus *status) {
-    const uint32_t addr = smem_u32(bar);
-    for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\n"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            "selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-        if (done) return true;
-        if (*reinterpret_cast<volatile uint32_t *>(&bars->aborted)) return false;
-    }
-    bars->aborted = 1;
-    atomicCAS(&status->code, 0, (int)CS_ERR_TIMEOUT);
-    return false;
-}
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// 32 consecutive f32 columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptors (version 1, 128-byte swizzle).  Offsets are in 16-byte units.
-//   K-major:  rows 128 bytes apart, 8-row atoms 1024 bytes apart (SBO); LBO unused.
-//   MN-major: 64-element blocks `lbo_bytes` apart (LBO), 8-row k groups 1024 bytes apart (SBO).
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t lbo_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3ffff) >> 4);
-    d |= (uint64_t)(lbo_bytes >> 4) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;   // descriptor version
-    d |= (uint64_t)2 << 61;   // SWIZZLE_128B
-    return d;
-}
-// Instruction descriptor: bf16 x bf16 -> f32, M = 128, N = 256; b_mn = B operand is N-major.
-__host__ __device__ constexpr uint32_t make_idesc(bool b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) |
-           ((uint32_t)(BM >> 4) << 24);
-}
-
-// General form: N columns, either operand MN-major.
-__device__ __forceinline__ uint32_t make_idesc_rt(int n, bool a_mn, bool b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
-           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-}
-// 16 consecutive f32 columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-}
-// Barriers + tensor memory of `ncols` columns (a power of two >= 32), owned by warp 1.
-__device__ __forceinline__ void setup_cta(Barriers *bars, int warp, uint32_t ncols) {
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxStages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
-        mbar_init(&bars->acc_ready, 1);
-        bars->aborted = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&bars->tmem_base)), "r"(ncols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-}
-__device__ __forceinline__ void teardown_cta(Barriers *bars, int warp, uint32_t ncols) {
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(bars->tmem_base), "r"(ncols) : "memory");
-    }
-}
 
 // SPLIT: the activation operand comes as two bf16 matrices (high part and remainder, whose sum
 // carries ~16 mantissa bits), each stage holds both A tiles and every MMA is issued twice.  The
@@ -241,8 +104,6 @@ __device__ __forceinline__ void mma_loop(const Tiles<SPLIT> &t, int kblocks, Dev
     }
     tc_commit(&t.bars->acc_ready);
 }
-
-__device__ __forceinline__ float silu_f(float x) { return x / (1.f + __expf(-x)); }
 
 }  // namespace
 
@@ -808,297 +669,6 @@ ffn_down_wide_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_co
 }
 
 
-// ---- decode batches of at most 128 tokens: weights on the M side -------------------------------
-// With few tokens the cheap orientation is the transposed one: the 128 channel rows of a weight
-// block are the MMA's M operand and the tokens its N columns (N = batch rounded up to 16), so an
-// instruction costs in proportion to the batch instead of a fixed 256 columns.
-//   gate/up:  D_g[128 ch, N] = W_gate[g rows] X^T,  D_u likewise;  actT[slot*128 + ch, token] = silu(D_g) D_u
-//   down:     D[128 out columns, N] = Wd_t[slice rows, 128 columns]^T actT[slice rows, tokens]
-// actT is stored channel-major (tokens contiguous, pitch 128), which makes it an N-major B operand for
-// the down GEMM; the Wd_t tile is the M-major A operand.
-template <bool SPLIT>
-__global__ void __launch_bounds__(kSwapMaxThreads, 1)
-ffn_gateup_swap_kernel(const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u,
-                       const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
-                       const int32_t *__restrict__ glist, const int32_t *__restrict__ ng_dev, int N, int d,
-                       const uint32_t *__restrict__ gmask, __nv_bfloat16 *__restrict__ actT,
-                       __nv_bfloat16 *__restrict__ actT_lo, DeviceStatus *status) {
-    extern __shared__ uint8_t smem_raw[];
-    // glist == NULL: one CTA per group of the layer, activations stored at the group's own index and
-    // left unmasked (the supports are still being recovered on another stream; mask_act_kernel
-    // applies them afterwards).
-    const int gi = blockIdx.x;
-    if (glist != nullptr && gi >= *ng_dev) return;
-    const int g = glist != nullptr ? glist[gi] : gi;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    Barriers *bars = reinterpret_cast<Barriers *>(base + kRingBytesMma);
-    const int xbytes = N * 128;                                    // X tile: N tokens x 64 k
-    const int stage_bytes = 2 * kABytes + (SPLIT ? 2 : 1) * xbytes;
-    const int stages = min(6, kRingBytesMma / stage_bytes);
-    const int NB = (SPLIT ? 2 : 1) * N;                            // columns per accumulator
-    const uint32_t tcols = 2 * NB <= 256 ? 256u : 512u;
-    setup_cta(bars, warp, tcols);
-    const int kblocks = d / BK;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            // Weights are parameters: the first ring of weight tiles is requested before the wait for the
-            // kernel that produces the token tiles (programmatic dependent launch), so the stream from
-            // HBM starts while that kernel is still running.
-            const int pre = min(stages, kblocks);
-            for (int kb = 0; kb < pre; ++kb) {
-                uint8_t *st = base + (size_t)kb * stage_bytes;
-                mbar_expect_tx(&bars->full[kb], stage_bytes);
-                tma_load_2d(st, &tm_g, kb * BK, g * 128, &bars->full[kb]);
-                tma_load_2d(st + kABytes, &tm_u, kb * BK, g * 128, &bars->full[kb]);
-            }
-            pdl_wait();
-            for (int kb = 0; kb < pre; ++kb) {
-                uint8_t *st = base + (size_t)kb * stage_bytes;
-                tma_load_2d(st + 2 * kABytes, &tm_x, kb * BK, 0, &bars->full[kb]);
-                if (SPLIT) tma_load_2d(st + 2 * kABytes + xbytes, &tm_x_lo, kb * BK, 0, &bars->full[kb]);
-            }
-            for (int kb = pre; kb < kblocks; ++kb) {
-                const int s = kb % stages;
-                if (!mbar_wait(&bars->empty[s], ((kb / stages) - 1) & 1, bars, status)) break;
-                uint8_t *st = base + (size_t)s * stage_bytes;
-                mbar_expect_tx(&bars->full[s], stage_bytes);
-                tma_load_2d(st, &tm_g, kb * BK, g * 128, &bars->full[s]);
-                tma_load_2d(st + kABytes, &tm_u, kb * BK, g * 128, &bars->full[s]);
-                tma_load_2d(st + 2 * kABytes, &tm_x, kb * BK, 0, &bars->full[s]);
-                if (SPLIT) tma_load_2d(st + 2 * kABytes + xbytes, &tm_x_lo, kb * BK, 0, &bars->full[s]);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_rt(NB, false, false);
-            const uint32_t tmem = bars->tmem_base;
-            bool ok = true;
-            int s = 0, ph = 0;
-            for (int kb = 0; kb < kblocks && ok; ++kb, ++s) {
-                if (s == stages) { s = 0; ph ^= 1; }
-                ok = mbar_wait(&bars->full[s], ph, bars, status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_g = smem_u32(base + (size_t)s * stage_bytes), a_u = a_g + kABytes;
-                const uint32_t x0 = a_g + 2 * kABytes;
-#pragma unroll
-                for (int k4 = 0; k4 < BK / 16; ++k4) {
-                    // x_hi and x_lo tiles are adjacent: one B operand of NB rows gives W x_hi in the first
-                    // N columns and W x_lo in the next N, at the cost of a single instruction
-                    const uint64_t bd = desc_sw128(x0 + k4 * 32, 16);
-                    tc_mma(tmem, desc_sw128(a_g + k4 * 32, 16), bd, idesc, (kb | k4) != 0);
-                    tc_mma(tmem + NB, desc_sw128(a_u + k4 * 32, 16), bd, idesc, (kb | k4) != 0);
-                }
-                tc_commit(&bars->empty[s]);
-            }
-            if (ok) tc_commit(&bars->acc_ready);
-        }
-    } else {
-        // Warps 2.. are the epilogue: four consecutive warps cover the four lane quarters of tensor memory
-        // (a warp may read quarter warp % 4), and each such slice of four warps takes every nslice-th
-        // chunk of 16 tokens, so the accumulators drain in one or two rounds instead of N / 16 (measured at
-        // 64 tokens: 1.5 us instead of 4.6 us after the last MMA).
-        const int q = warp & 3, ch = q * 32 + lane;
-        const int slice = (warp - 2) >> 2, nslice = ((int)(blockDim.x >> 5) - 2) >> 2;
-        pdl_wait();   // nothing is stored before the kernels before this one are complete
-        if (mbar_wait(&bars->acc_ready, 0, bars, status)) {
-            tc_fence_after();
-            const uint32_t tbase = bars->tmem_base + ((uint32_t)(q * 32) << 16);
-            const uint4 gm = gmask != nullptr ? *reinterpret_cast<const uint4 *>(gmask + (size_t)g * 4)
-                                              : make_uint4(~0u, ~0u, ~0u, ~0u);
-            const uint32_t gw[4] = {gm.x, gm.y, gm.z, gm.w};
-            const size_t row = ((size_t)gi * 128 + ch) * 128;
-#pragma unroll 1
-            for (int c = slice; c < N / 16; c += nslice) {
-                uint32_t gv[16], uv[16];
-                tc_ld16(tbase + c * 16, gv);
-                tc_ld16(tbase + NB + c * 16, uv);
-                if (SPLIT) {   // add the x_lo halves
-                    uint32_t g2[16], u2[16];
-                    tc_ld16(tbase + N + c * 16, g2);
-                    tc_ld16(tbase + NB + N + c * 16, u2);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        gv[j] = __float_as_uint(__uint_as_float(gv[j]) + __uint_as_float(g2[j]));
-                        uv[j] = __float_as_uint(__uint_as_float(uv[j]) + __uint_as_float(u2[j]));
-                    }
-                } else {
-                    tc_wait_ld();
-                }
-                const uint32_t bits = gw[(c * 16) >> 5] >> ((c * 16) & 31);
-                uint32_t hi[8], lo[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float k0 = (bits >> (2 * j)) & 1u ? 1.f : 0.f, k1 = (bits >> (2 * j + 1)) & 1u ? 1.f : 0.f;
-                    const float a0 = silu_f(__uint_as_float(gv[2 * j])) * __uint_as_float(uv[2 * j]) * k0;
-                    const float a1 = silu_f(__uint_as_float(gv[2 * j + 1])) * __uint_as_float(uv[2 * j + 1]) * k1;
-                    const __nv_bfloat162 p = __floats2bfloat162_rn(a0, a1);
-                    hi[j] = *reinterpret_cast<const uint32_t *>(&p);
-                    if (SPLIT) {
-                        const __nv_bfloat162 r = __floats2bfloat162_rn(a0 - __low2float(p), a1 - __high2float(p));
-                        lo[j] = *reinterpret_cast<const uint32_t *>(&r);
-                    }
-                }
-                uint4 *dst = reinterpret_cast<uint4 *>(actT + row + c * 16);
-                dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                dst[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
-                if (SPLIT) {
-                    uint4 *dl = reinterpret_cast<uint4 *>(actT_lo + row + c * 16);
-                    dl[0] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                    dl[1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
-                }
-            }
-        }
-    }
-    teardown_cta(bars, warp, tcols);
-}
-
-// grid (d / 128 / CPC, slices).  partial [slice][128 tokens][d].  A CTA owns CPC adjacent tiles of
-// 128 output columns, which share every activation tile: these kernels are bound by the bytes the SMs
-// take in, from DRAM and L2 alike (about 6.5 TB/s in all), and with one column tile per CTA the
-// activation tiles that every CTA fetches again are as many bytes as the weights.
-template <bool SPLIT, int CPC>
-__global__ void __launch_bounds__(kSwapMaxThreads, 1)
-ffn_down_swap_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_constant__ CUtensorMap tm_act,
-                     const __grid_constant__ CUtensorMap tm_act_lo, const int32_t *__restrict__ glist,
-                     const int32_t *__restrict__ ng_dev, int N, int B, int d, int act_by_group,
-                     float *__restrict__ partial, DeviceStatus *status) {
-    extern __shared__ uint8_t smem_raw[];
-    const int c0 = blockIdx.x * 128 * CPC, z = blockIdx.y, Z = gridDim.y;
-    const int ng = *ng_dev;
-    const int gi0 = (int)(((long long)ng * z) / Z), gi1 = (int)(((long long)ng * (z + 1)) / Z);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    Barriers *bars = reinterpret_cast<Barriers *>(base + kRingBytesMma);
-    const int nblk = (N + 63) / 64;                                // token blocks of 64
-    const int bbytes = nblk * 64 * BK * 2;                         // actT tile: 64 k rows x tokens
-    const int stage_bytes = CPC * kABytes + (SPLIT ? 2 : 1) * bbytes;
-    const int stages = min(6, kRingBytesMma / stage_bytes);
-    const int NB = SPLIT ? 2 * nblk * 64 : N;                      // MMA columns: value blocks then remainder blocks
-    const uint32_t tcols = CPC * NB <= 128 ? 128u : CPC * NB <= 256 ? 256u : 512u;
-    setup_cta(bars, warp, tcols);
-    const int kblocks = (gi1 - gi0) * 2;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            auto load_w = [&](int kb, int s) {   // weight tile of column tile j / 2: two blocks of 64 columns
-                const int wrow = glist[gi0 + (kb >> 1)] * 128 + (kb & 1) * BK;
-                uint8_t *st = base + (size_t)s * stage_bytes;
-#pragma unroll
-                for (int j = 0; j < 2 * CPC; ++j)
-                    tma_load_2d(st + j * (64 * BK * 2), &tm_wd, c0 + j * 64, wrow, &bars->full[s]);
-            };
-            auto load_act = [&](int kb, int s) {
-                const int gi = gi0 + (kb >> 1);
-                const int arow = (act_by_group ? glist[gi] : gi) * 128 + (kb & 1) * BK;
-                uint8_t *st = base + (size_t)s * stage_bytes;
-                for (int i = 0; i < nblk; ++i) {
-                    tma_load_2d(st + CPC * kABytes + i * (64 * BK * 2), &tm_act, i * 64, arow, &bars->full[s]);
-                    if (SPLIT) tma_load_2d(st + CPC * kABytes + bbytes + i * (64 * BK * 2), &tm_act_lo, i * 64, arow, &bars->full[s]);
-                }
-            };
-            // as in the gate/up kernel: the first ring of weight tiles goes out before the wait for the
-            // kernel that completes the activations (the group list was final before that kernel began)
-            const int pre = min(stages, kblocks);
-            for (int kb = 0; kb < pre; ++kb) { mbar_expect_tx(&bars->full[kb], stage_bytes); load_w(kb, kb); }
-            pdl_wait();
-            for (int kb = 0; kb < pre; ++kb) load_act(kb, kb);
-            for (int kb = pre; kb < kblocks; ++kb) {
-                const int s = kb % stages;
-                if (!mbar_wait(&bars->empty[s], ((kb / stages) - 1) & 1, bars, status)) break;
-                mbar_expect_tx(&bars->full[s], stage_bytes);
-                load_w(kb, s);
-                load_act(kb, s);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0 && kblocks > 0) {
-            const uint32_t idesc = make_idesc_rt(NB, true, true);
-            const uint32_t tmem = bars->tmem_base;
-            bool ok = true;
-            int s = 0, ph = 0;
-            for (int kb = 0; kb < kblocks && ok; ++kb, ++s) {
-                if (s == stages) { s = 0; ph ^= 1; }
-                ok = mbar_wait(&bars->full[s], ph, bars, status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a0 = smem_u32(base + (size_t)s * stage_bytes), b0 = a0 + CPC * kABytes;
-#pragma unroll
-                for (int k4 = 0; k4 < BK / 16; ++k4) {   // remainder blocks follow the value blocks: one operand
-                    const uint64_t bd = desc_sw128(b0 + k4 * 2048, 64 * BK * 2);
-#pragma unroll
-                    for (int ct = 0; ct < CPC; ++ct)
-                        tc_mma(tmem + ct * NB, desc_sw128(a0 + ct * kABytes + k4 * 2048, 64 * BK * 2), bd, idesc, (kb | k4) != 0);
-                }
-                tc_commit(&bars->empty[s]);
-            }
-            if (ok) tc_commit(&bars->acc_ready);
-        }
-    } else {
-        const int q = warp & 3;                     // epilogue slices as in the gate/up kernel
-        const int slice = (warp - 2) >> 2, nslice = ((int)(blockDim.x >> 5) - 2) >> 2;
-        pdl_wait();   // nothing is stored before the kernels before this one are complete
-        if (kblocks == 0) {
-            for (int ct = 0; ct < CPC; ++ct) {
-                float *dst = partial + (size_t)z * 128 * d + c0 + ct * 128 + q * 32 + lane;
-                for (int tkn = slice; tkn < B; tkn += nslice) dst[(size_t)tkn * d] = 0.f;
-            }
-        } else if (mbar_wait(&bars->acc_ready, 0, bars, status)) {
-            tc_fence_after();
-            for (int ct = 0; ct < CPC; ++ct) {
-                const uint32_t tbase = bars->tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ct * NB);
-                float *dst = partial + (size_t)z * 128 * d + c0 + ct * 128 + q * 32 + lane;
-#pragma unroll 1
-                for (int c = slice; c < N / 16; c += nslice) {
-                    uint32_t v[16];
-                    tc_ld16(tbase + c * 16, v);
-                    if (SPLIT) {
-                        uint32_t v2[16];
-                        tc_ld16(tbase + nblk * 64 + c * 16, v2);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v2[j]));
-                    } else {
-                        tc_wait_ld();
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int tkn = c * 16 + j;
-                        if (tkn < B) dst[(size_t)tkn * d] = __uint_as_float(v[j]);
-                    }
-                }
-            }
-        }
-    }
-    teardown_cta(bars, warp, tcols);
-}
-
-
-// Zeroes the activations of (group, token) pairs outside the supports: row r of actT belongs to
-// group r / 128; bit t of gmask[group] says whether token t owns the group.  One thread per row
-// and 8-token chunk, for the value and the remainder matrix.
-__global__ void mask_act_kernel(__nv_bfloat16 *__restrict__ actT, __nv_bfloat16 *__restrict__ actT_lo,
-                                const uint32_t *__restrict__ gmask, int rows, int N) {
-    pdl_launch_dependents();   // the down GEMM may start streaming its weights
-    const int chunks = N / 8;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * chunks) return;
-    const int r = i / chunks, c = i - r * chunks;
-    const uint32_t bits = (gmask[(size_t)(r >> 7) * 4 + ((c * 8) >> 5)] >> ((c * 8) & 31)) & 0xffu;
-    if (bits == 0xffu) return;
-    const uint32_t m0 = (bits & 1u ? 0xffffu : 0u) | (bits & 2u ? 0xffff0000u : 0u);
-    const uint32_t m1 = (bits & 4u ? 0xffffu : 0u) | (bits & 8u ? 0xffff0000u : 0u);
-    const uint32_t m2 = (bits & 16u ? 0xffffu : 0u) | (bits & 32u ? 0xffff0000u : 0u);
-    const uint32_t m3 = (bits & 64u ? 0xffffu : 0u) | (bits & 128u ? 0xffff0000u : 0u);
-    uint4 *p = reinterpret_cast<uint4 *>(actT + (size_t)r * 128 + c * 8);
-    uint4 v = *p; v.x &= m0; v.y &= m1; v.z &= m2; v.w &= m3; *p = v;
-    uint4 *q = reinterpret_cast<uint4 *>(actT_lo + (size_t)r * 128 + c * 8);
-    uint4 w = *q; w.x &= m0; w.y &= m1; w.z &= m2; w.w &= m3; *q = w;
-}
-
 // out[m, :] = residual[m, :] + sum_z partial[z, m, :], slices added in index order.
 template <typename OutT>
 __global__ void reduce_slices_kernel(const float *__restrict__ partial, int Z, int M, int m_pad, int d,
@@ -1126,57 +696,13 @@ __global__ void reduce_slices_kernel(const float *__restrict__ partial, int Z, i
 // x = y_hi + y_lo with both parts bf16: y_hi = round(x), y_lo = round(x - y_hi).
 __global__ void split_bf16_kernel(const float *__restrict__ x, __nv_bfloat16 *__restrict__ y_hi,
                                   __nv_bfloat16 *__restrict__ y_lo, size_t n4) {
-    pdl_launch_dependents();   // the gate/up GEMM may start streaming its weights
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
     const float4 v = reinterpret_cast<const float4 *>(x)[i];
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-    const __nv_bfloat162 l0 = __floats2bfloat162_rn(v.x - __low2float(h0), v.y - __high2float(h0));
-    const __nv_bfloat162 l1 = __floats2bfloat162_rn(v.z - __low2float(h1), v.w - __high2float(h1));
     uint2 p, q;
-    p.x = *reinterpret_cast<const uint32_t *>(&h0); p.y = *reinterpret_cast<const uint32_t *>(&h1);
-    q.x = *reinterpret_cast<const uint32_t *>(&l0); q.y = *reinterpret_cast<const uint32_t *>(&l1);
+    split4(v.x, v.y, v.z, v.w, p, q);
     reinterpret_cast<uint2 *>(y_hi)[i] = p;
     reinterpret_cast<uint2 *>(y_lo)[i] = q;
-}
-
-// The same with the RMSNorm of the stacked workload in front: n = x * rsqrt(mean(x^2) + eps) * gamma,
-// one CTA per token.  The GEMM's operand does not have to wait for the sketch kernel, which forms the
-// same n for itself on the other stream.
-constexpr int kNormSplitThreads = 256;
-__global__ void __launch_bounds__(kNormSplitThreads)
-norm_split_bf16_kernel(const float *__restrict__ x, const float *__restrict__ gamma, float eps, int d,
-                       __nv_bfloat16 *__restrict__ y_hi, __nv_bfloat16 *__restrict__ y_lo) {
-    __shared__ float red[kNormSplitThreads / 32];
-    pdl_launch_dependents();   // the gate/up GEMM may start streaming its weights
-    const int t = blockIdx.x, tid = threadIdx.x;
-    const float4 *xr = reinterpret_cast<const float4 *>(x + (size_t)t * d);
-    const float4 *gr = reinterpret_cast<const float4 *>(gamma);
-    float ss = 0.f;
-    for (int c = tid; c < d / 4; c += kNormSplitThreads) {
-        const float4 v = xr[c];
-        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-    }
-    ss = warp_sum(ss);
-    if ((tid & 31) == 0) red[tid >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < kNormSplitThreads / 32; ++w) tot += red[w];
-    const float rscale = rsqrtf(tot / (float)d + eps);
-    for (int c = tid; c < d / 4; c += kNormSplitThreads) {
-        float4 v = xr[c];
-        const float4 g = gr[c];
-        v.x = v.x * g.x * rscale; v.y = v.y * g.y * rscale; v.z = v.z * g.z * rscale; v.w = v.w * g.w * rscale;
-        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-        const __nv_bfloat162 l0 = __floats2bfloat162_rn(v.x - __low2float(h0), v.y - __high2float(h0));
-        const __nv_bfloat162 l1 = __floats2bfloat162_rn(v.z - __low2float(h1), v.w - __high2float(h1));
-        uint2 p, q;
-        p.x = *reinterpret_cast<const uint32_t *>(&h0); p.y = *reinterpret_cast<const uint32_t *>(&h1);
-        q.x = *reinterpret_cast<const uint32_t *>(&l0); q.y = *reinterpret_cast<const uint32_t *>(&l1);
-        reinterpret_cast<uint2 *>(y_hi + (size_t)t * d)[c] = p;
-        reinterpret_cast<uint2 *>(y_lo + (size_t)t * d)[c] = q;
-    }
 }
 
 // ---- bucketing: supports [B,k] -> membership masks, per-group token lists, union list ------------
@@ -1187,7 +713,7 @@ constexpr int kBucketSmemTokens = 2048;   // masks of this many tokens are kept 
 
 __global__ void __launch_bounds__(1024)
 bucket_kernel(const int32_t *__restrict__ support, int B, int k, int G, uint32_t *__restrict__ mask,
-              uint32_t *__restrict__ gmask, int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
+              int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
               int32_t *__restrict__ token_ids, int32_t *__restrict__ glist, int32_t *__restrict__ nu) {
     extern __shared__ uint32_t mask_s[];            // [min(B, kBucketSmemTokens)][4]
     __shared__ int warp_tot[kMaxG / 32], warp_used[kMaxG / 32];
@@ -1217,8 +743,7 @@ bucket_kernel(const int32_t *__restrict__ support, int B, int k, int G, uint32_t
     auto member = [&](int t) -> bool {
         return ((t < Bs ? mask_s[(size_t)t * 4 + word] : mask[(size_t)t * 4 + word]) & bit) != 0u;
     };
-    // the transposed mask (bit t of group g) for the first 128 tokens, in four scalar words, and the
-    // bucket size
+    // bit t of group g for the first 128 tokens, in four scalar words, and the bucket size
     uint32_t w0 = 0u, w1 = 0u, w2 = 0u, w3 = 0u;
     int cnt = 0;
     if (g < G) {
@@ -1255,7 +780,6 @@ bucket_kernel(const int32_t *__restrict__ support, int B, int k, int G, uint32_t
         counts[g] = cnt;
         offsets[g] = off;
         if (used) glist[uoff] = g;
-        *reinterpret_cast<uint4 *>(gmask + (size_t)g * 4) = make_uint4(w0, w1, w2, w3);
         int o = off;   // tokens of the bucket in ascending order: walk the set bits, then the tail
         auto emit = [&](uint32_t wd, int t0) {
             while (wd) { token_ids[o++] = t0 + __ffs(wd) - 1; wd &= wd - 1; }
@@ -1268,39 +792,6 @@ bucket_kernel(const int32_t *__restrict__ support, int B, int k, int G, uint32_t
 }
 
 // ---- host side ----------------------------------------------------------------------------------
-namespace {
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (fn == nullptr) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
-// bf16 matrix [outer, inner] row-major with `ld` elements per row; box = [box_outer rows, 64 columns].
-bool make_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld, uint32_t box_outer) {
-    EncodeTiledFn fn = encode_fn();
-    if (fn == nullptr) return false;
-    const cuuint64_t dims[2] = {inner, outer};
-    const cuuint64_t strides[1] = {ld * 2};
-    const cuuint32_t box[2] = {64, box_outer};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-}  // namespace
-
 // How many of the pair slots a mixed launch runs as paired tiles: CTAs are handed out in index order to
 // whichever SM is free first, pairs first.  Measured on B200, a pair takes about 1.8 single-tile times
 // (both kinds are bound by what shared memory can serve: the tensor pipe reads 12 KB of operands per
@@ -1339,15 +830,13 @@ cs_status prepare_ffn_mma(cs_plan *plan) {
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_swap_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_swap_kernel<true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     return CS_OK;
 }
 
 cs_status launch_bucket(cs_plan *plan, const int32_t *support, int B, cudaStream_t st, int32_t *counts,
                         int32_t *offsets, int32_t *token_ids) {
     const size_t smem = (size_t)min(B, kBucketSmemTokens) * 16;
-    bucket_kernel<<<1, 1024, smem, st>>>(support, B, plan->cfg.k, plan->G, plan->mask, plan->gmask,
+    bucket_kernel<<<1, 1024, smem, st>>>(support, B, plan->cfg.k, plan->G, plan->mask,
                                       counts ? counts : plan->counts, offsets ? offsets : plan->offsets,
                                       token_ids ? token_ids : plan->token_ids, plan->glist, plan->nu);
     plan->launches++;
@@ -1445,90 +934,6 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
     return CS_OK;
 }
 
-
-// Decode batches from the crossover batch up to 128 tokens in three launches that the caller orders
-// (the gate/up GEMM can run while the supports are still being recovered on another stream):
-//   launch_decode_gateup(masked = false)  every group of the layer, activations unmasked, stored at the
-//                                         group's own index;   (masked = true: union list + masks)
-//   launch_decode_mask                    zeroes the (group, token) pairs outside the supports
-//   launch_decode_down                    down GEMM over the union list, slice reduction, residual
-static bool decode_maps(cs_plan *plan, const cs_layer *L, const void *X, const void *X_lo, int B, int N,
-                        CUtensorMap *tm) {
-    const cs_config &c = plan->cfg;
-    __nv_bfloat16 *actT = static_cast<__nv_bfloat16 *>(plan->act);
-    __nv_bfloat16 *actT_lo = actT + (size_t)plan->G * 128 * 128;
-    return make_map(&tm[0], L->W_gate, c.d, c.d_ff, c.d, 128) && make_map(&tm[1], L->W_up, c.d, c.d_ff, c.d, 128) &&
-           make_map(&tm[2], X ? X : plan->x_bf16, c.d, B, c.d, N) &&
-           make_map(&tm[3], X_lo ? X_lo : plan->x_bf16, c.d, B, c.d, N) &&
-           make_map(&tm[4], L->Wd_t, c.d, c.d_ff, c.d, BK) &&
-           make_map(&tm[5], actT, 128, (uint64_t)plan->G * 128, 128, BK) &&
-           make_map(&tm[6], actT_lo, 128, (uint64_t)plan->G * 128, 128, BK);
-}
-
-cs_status launch_decode_gateup(cs_plan *plan, const cs_layer *L, const void *X, const void *X_lo, int B,
-                               bool masked, cudaStream_t st) {
-    const cs_config &c = plan->cfg;
-    const int N = (B + 15) / 16 * 16;
-    __nv_bfloat16 *actT = static_cast<__nv_bfloat16 *>(plan->act);
-    __nv_bfloat16 *actT_lo = actT + (size_t)plan->G * 128 * 128;
-    CUtensorMap tm[7];
-    if (!decode_maps(plan, L, X, X_lo, B, N, tm)) return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
-    StageTimer timer(plan, CS_STAGE_EXEC, st);
-    const int threads = 64 + 128 * min(4, N / 16);   // one epilogue slice per chunk of 16 tokens, at most four
-    launch_pdl(true, ffn_gateup_swap_kernel<true>, dim3(plan->G), dim3(threads), kMmaSmem, st,
-               tm[0], tm[1], tm[2], tm[3], masked ? (const int32_t *)plan->glist : (const int32_t *)nullptr,
-               (const int32_t *)plan->nu, N, c.d, masked ? (const uint32_t *)plan->gmask : (const uint32_t *)nullptr,
-               actT, actT_lo, plan->status);
-    plan->launches++;
-    CS_CUDA_TRY(plan, cudaGetLastError());
-    return CS_OK;
-}
-
-cs_status launch_decode_mask(cs_plan *plan, int B, cudaStream_t st) {
-    const int N = (B + 15) / 16 * 16;
-    __nv_bfloat16 *actT = static_cast<__nv_bfloat16 *>(plan->act);
-    __nv_bfloat16 *actT_lo = actT + (size_t)plan->G * 128 * 128;
-    const int rows = plan->G * 128, total = rows * (N / 8);
-    mask_act_kernel<<<(total + 255) / 256, 256, 0, st>>>(actT, actT_lo, plan->gmask, rows, N);
-    plan->launches++;
-    CS_CUDA_TRY(plan, cudaGetLastError());
-    return CS_OK;
-}
-
-cs_status launch_decode_down(cs_plan *plan, const cs_layer *L, int B, bool act_by_group, const float *residual,
-                             float *out, cudaStream_t st) {
-    const cs_config &c = plan->cfg;
-    const int N = (B + 15) / 16 * 16;
-    CUtensorMap tm[7];
-    if (!decode_maps(plan, L, nullptr, nullptr, B, N, tm)) return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
-    const int Z = max(1, min(plan->sm_count / (c.d / 256), 8));   // two column tiles per CTA (d is a multiple of 256)
-    {
-        StageTimer timer(plan, CS_STAGE_EXEC2, st);
-        const int threads = 64 + 128 * min(4, N / 16);
-        launch_pdl(true, ffn_down_swap_kernel<true, 2>, dim3(c.d / 256, Z), dim3(threads), kMmaSmem, st,
-                   tm[4], tm[5], tm[6], (const int32_t *)plan->glist, (const int32_t *)plan->nu, N, B, c.d,
-                   act_by_group ? 1 : 0, plan->mma_partial, plan->status);
-        plan->launches++;
-        CS_CUDA_TRY(plan, cudaGetLastError());
-    }
-    {
-        StageTimer timer(plan, CS_STAGE_REDUCE, st);
-        const size_t total4 = (size_t)B * c.d / 4;
-        reduce_slices_kernel<float><<<(int)((total4 + 255) / 256), 256, 0, st>>>(plan->mma_partial, Z, B, 128, c.d, residual, out);
-        plan->launches++;
-        CS_CUDA_TRY(plan, cudaGetLastError());
-    }
-    return CS_OK;
-}
-
-cs_status launch_norm_split_bf16(cs_plan *plan, const float *x, const float *gamma, int B, void *y_hi, void *y_lo,
-                                 cudaStream_t st) {
-    norm_split_bf16_kernel<<<B, kNormSplitThreads, 0, st>>>(x, gamma, plan->cfg.rms_eps, plan->cfg.d,
-                                                            static_cast<__nv_bfloat16 *>(y_hi), static_cast<__nv_bfloat16 *>(y_lo));
-    plan->launches++;
-    CS_CUDA_TRY(plan, cudaGetLastError());
-    return CS_OK;
-}
 
 cs_status launch_split_bf16(cs_plan *plan, const float *x, void *y_hi, void *y_lo, size_t n, cudaStream_t st) {
     const size_t n4 = n / 4;

@@ -54,6 +54,7 @@ template <int NW, int KC> struct RecoverSmem {
     static constexpr int GP = 32 * NW;                 // padded number of entries = pitch of M
     static constexpr int NV = KC > 0 ? KC * 8 : GP;    // length of the iterate as the mat-vec reads it
     alignas(16) float key[GP];        // |v| of the current iterate
+    alignas(16) float part[GP];       // partial sums while y is put together
     alignas(16) float red[kMaxM];     // residual r of the two-step form; partial sums of the residual norm
     alignas(16) float val[2][NV];     // the iterate, by iteration parity: slot values, or dense z
     int idx[NV];                      // list form: entry held by each slot (the support, in slot order)
@@ -163,20 +164,20 @@ __device__ __forceinline__ void recover_load_phi(const float *__restrict__ Phi, 
 // Runs the recovery of one token.  g = this thread's entry (0 .. 32*NW-1); all 32*NW threads call it
 // together and synchronise on named barrier BAR.  M: where the entries of I - mu Phi^T Phi come from
 // (the dense form reads whole rows of the global matrix, whose pitch must be 32 * NW).  phc: the thread's column of Phi when m <= 32
-// (recover_load_phi), unused otherwise.  y, gram, sup0, z0 may come from the kernel before: they are
+// (recover_load_phi), unused otherwise.  load_y(s) fills s.y[0 .. m).  y, gram, sup0, z0 may come from the kernel before: they are
 // read with dependent loads, after the caller's wait.  table_ready() is called once by every thread
 // when the slot table s.idx first holds a support worth acting on (that of the first iterate, or the
 // start's own when T == 0 or the start is warm); from then on s.idx always holds k valid groups and changes only where the
 // support changes: slot_changed(slot, g) is called by the thread whose entry g has just taken `slot`.
 // table_final() is called once by every thread after the last iteration, before the outputs are
-// written.
-template <int NW, int KC, int BAR, typename MSource, typename TableReady, typename SlotChanged, typename TableFinal>
+// written.  mask (may be NULL): NW words of membership bits.
+template <int NW, int KC, int BAR, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
 __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int g, const float *__restrict__ Phi,
-                                              const MSource M, float mu, const float *__restrict__ y, int m, int G, int k, int T, int32_t *__restrict__ support,
+                                              const MSource M, float mu, LoadY load_y, int m, int G, int k, int T, int32_t *__restrict__ support,
                                               float *__restrict__ z_out, float *__restrict__ resid_out,
                                               const int32_t *__restrict__ sup0, const float *__restrict__ z0,
                                               const float tgamma, const int32_t *__restrict__ sup_prev,
-                                              const float *__restrict__ z_prev, DeviceStatus *status, const float (&phc)[32], TableReady table_ready,
+                                              const float *__restrict__ z_prev, uint32_t *__restrict__ mask, DeviceStatus *status, const float (&phc)[32], TableReady table_ready,
                                               SlotChanged slot_changed, TableFinal table_final) {
     constexpr int GP = 32 * NW;
     constexpr int NV = RecoverSmem<NW, KC>::NV;
@@ -200,7 +201,7 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
             mreg[4 * j] = q.x; mreg[4 * j + 1] = q.y; mreg[4 * j + 2] = q.z; mreg[4 * j + 3] = q.w;
         }
     }
-    for (int row = g; row < m; row += GP) s.y[row] = ld_dep(y + row);
+    load_y(s);   // s.y, complete at the next barrier
     // z_0 = 0 with the support the order assigns to an all-zero vector (indices 0..k-1), or, warm
     // started, the k-sparse iterate handed in (sup0 ascending and distinct, z0 its values).
     const bool warm = sup0 != nullptr;
@@ -412,7 +413,10 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
     }
     // ascending index order: a kept entry goes to position (number of kept entries with a lower index)
     const unsigned kb = __ballot_sync(0xffffffffu, kept);
-    if (lane == 0) s.cnt[warp] = __popc(kb);
+    if (lane == 0) {
+        s.cnt[warp] = __popc(kb);
+        if (mask != nullptr) mask[warp] = kb;   // membership bits of this warp's 32 groups
+    }
     bar_sync<BAR, GP>();
     if (kept) {
         int o = __popc(kb & lt_mask);

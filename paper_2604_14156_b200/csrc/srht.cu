@@ -70,7 +70,7 @@ cs_status launch_sketch_srht(cs_plan *plan, const uint32_t *sign_bits, const int
     const size_t smem = (size_t)d * sizeof(float);
 #define CS_SRHT_CASE(E)                                                                                       \
     case E * kSrhtThreads:                                                                                    \
-        launch_pdl(pdl_for(plan, B), srht_kernel<E>, dim3(B), dim3(kSrhtThreads), smem, st, sign_bits, rows, h, m, y); \
+        launch_pdl(true, srht_kernel<E>, dim3(B), dim3(kSrhtThreads), smem, st, sign_bits, rows, h, m, y); \
         break
     switch (d) {
         CS_SRHT_CASE(1); CS_SRHT_CASE(2); CS_SRHT_CASE(4); CS_SRHT_CASE(8); CS_SRHT_CASE(16); CS_SRHT_CASE(32);

@@ -1,0 +1,25 @@
+"""GPU parity of the tensor-core decode path (up to 256 tokens) at the sizes where its tiling can go wrong."""
+import pytest
+
+from gen import workloads as W
+from parity_util import compare_layer_step, make_plan
+
+pytestmark = pytest.mark.gpu
+
+
+# Token tiles: packed value / remainder rows up to 64 tokens, two operands up to 128, two accumulators up to 256, and the
+# first batch beyond.  Channel tiles: d_ff that the tiles of 8 x SM-share channels do not divide, and fewer channels than
+# SMs x 8.  k small against G leaves groups out of every support.
+@pytest.mark.parametrize("B", [2, 8, 15, 63, 64, 65, 127, 128, 129, 192, 193, 256, 257])
+@pytest.mark.parametrize("d,G,m,k,norm", [(512, 13, 9, 3, True), (768, 101, 35, 11, False)])
+def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
+    base = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"]
+    cfg = base.with_(n_layers=1, d=d, d_ff=128 * G, m=m, k=k, T=6, B=B, index=300 + B)
+    L = W.make_layer(cfg, device="cuda:0")
+    tk = W.make_tokens(cfg, L.A)
+    plan = make_plan(cfg)
+    plan.set_crossover(2)
+    # output bound: 1e-4 (parity_util), f32 accumulation of bf16 value + remainder products
+    rep, _, _ = compare_layer_step(cfg, L, plan, tk.h)
+    assert rep.excused <= max(1, B // 16), rep
+    plan.close()
