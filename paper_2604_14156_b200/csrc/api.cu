@@ -113,7 +113,6 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
         const size_t slice_rows = (size_t)128 * (p->sm_count / max(1, cfg->d / 256) + 1);
         const size_t decode_rows = (size_t)decode_slices(p) * min(nt, (size_t)kDecodeMaxTokens);
         alloc((void **)&p->mma_partial, max(max(slice_rows, max(decode_rows, 2 * min(nt, (size_t)kDecodeMaxTokens))), m_pad) * cfg->d * sizeof(float));
-        alloc((void **)&p->rscale, nt * sizeof(float));
     }
     alloc((void **)&p->x_host_in, nt * cfg->d * sizeof(float));
     alloc((void **)&p->x_host_out, nt * cfg->d * sizeof(float));
@@ -144,7 +143,7 @@ cs_status cs_plan_destroy(cs_plan *p) {
     cudaFree(p->resid_buf); cudaFree(p->fb_flags); cudaFree(p->fb_list); cudaFree(p->fb_count); cudaFree(p->hbar); cudaFree(p->colsum);
     cudaFree(p->status); cudaFree(p->x_host_in); cudaFree(p->x_host_out);
     cudaFree(p->mask); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
-    cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial); cudaFree(p->rscale);
+    cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial);
     for (int i = 0; i < 2 * CS_STAGE_COUNT; ++i)
         if (p->ev[i] != nullptr) cudaEventDestroy(p->ev[i]);
     delete p;
@@ -216,33 +215,32 @@ static cs_status check_options(const cs_plan *plan, const cs_step_options *o, bo
     return CS_OK;
 }
 
+// The options of the fixed-step iteration as launch_recover takes them.
+static RecoverOptions iht_options(const cs_plan *plan, const cs_step_options *o) {
+    RecoverOptions r;
+    r.T = o->T < 0 ? plan->cfg.T : o->T; r.gamma = o->gamma;
+    if (o->warm_start) { r.sup0 = o->support_prev; r.z0 = o->z_prev; }
+    if (o->gamma > 0.f) { r.sup_prev = o->support_prev; r.z_prev = o->z_prev; }
+    r.check = o->support_prev;
+    r.delta = o->delta_out; r.drift = o->drift_out;
+    return r;
+}
+
 // The estimator an options struct asks for, on y, with the check of the previous supports and the drift against
-// them; gram_ready: plan->gram holds this Phi's matrix; decode: see RecoverOptions (CS_SOLVER_IHT only).
+// them; gram_ready: plan->gram holds this Phi's matrix.
 static cs_status recover_with(cs_plan *plan, const float *Phi, float mu, const float *y, int B, const cs_step_options *o,
-                              int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st, bool decode = false,
-                              bool norm = false) {
+                              int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st) {
     const int T = o->T < 0 ? plan->cfg.T : o->T;
-    if (o->solver == CS_SOLVER_IHT) {
-        RecoverOptions r;
-        r.T = T; r.gamma = o->gamma; r.decode = decode; r.norm = norm;
-        if (o->warm_start) { r.sup0 = o->support_prev; r.z0 = o->z_prev; }
-        if (o->gamma > 0.f) { r.sup_prev = o->support_prev; r.z_prev = o->z_prev; }
-        r.check = o->support_prev; r.delta = o->delta_out; r.drift = o->drift_out;
-        // the supports may overwrite the previous ones, which the drift needs
-        if (support == o->support_prev) r.delta = nullptr, r.drift = nullptr;
-        cs_status s = launch_recover(plan, Phi, mu, y, B, support, z, resid, gram_ready, st, r);
-        if (s != CS_OK || support != o->support_prev) return s;
-    } else {
-        cs_status s = CS_OK;
-        if (o->support_prev != nullptr) s = launch_check_support(plan, o->support_prev, B, st);
-        if (s == CS_OK)
-            s = o->solver == CS_SOLVER_NIHT ? launch_niht(plan, Phi, mu, y, B, T, support, z, resid, st)
-                                            : launch_omp(plan, Phi, y, B, support, z, resid, st);
-        if (s != CS_OK) return s;
-    }
-    if (o->delta_out != nullptr || o->drift_out != nullptr)
-        return launch_support_drift(plan, o->support_prev, support, B, o->delta_out, o->drift_out, st);
-    return CS_OK;
+    if (o->solver == CS_SOLVER_IHT)
+        return launch_recover(plan, Phi, mu, y, B, support, z, resid, gram_ready, st, iht_options(plan, o));
+    cs_status s = CS_OK;
+    if (o->support_prev != nullptr) s = launch_check_support(plan, o->support_prev, B, st);
+    if (s == CS_OK)
+        s = o->solver == CS_SOLVER_NIHT ? launch_niht(plan, Phi, mu, y, B, T, support, z, resid, st)
+                                        : launch_omp(plan, Phi, y, B, support, z, resid, st);
+    if (s == CS_OK && (o->delta_out != nullptr || o->drift_out != nullptr))
+        s = launch_support_drift(plan, o->support_prev, support, B, o->delta_out, o->drift_out, st);
+    return s;
 }
 
 cs_status cs_recover_ex(cs_plan *plan, const float *Phi, float mu, const float *y, int32_t B,
@@ -293,7 +291,7 @@ static cs_status exec_dispatch(cs_plan *plan, const cs_layer *layer, const float
     if (use_decode_mma(plan, B)) {
         cs_status s = launch_decode_prep(plan, h, support, B, check, st);
         if (s != CS_OK) return s;
-        return launch_decode_ffn(plan, layer, B, false, false, residual, out, st);
+        return launch_decode_ffn(plan, layer, B, nullptr, false, false, residual, out, st);
     }
     if (check) {
         cs_status s = launch_check_support(plan, support, B, st);
@@ -329,6 +327,23 @@ cs_status cs_bucket(cs_plan *plan, const int32_t *support, int32_t B, int32_t *c
     return launch_bucket(plan, support, B, st, counts, offsets, token_ids);
 }
 
+// One step on the tensor cores: the sketch launch also splits the activations, the recovery runs inside the gate/up
+// launch (or, for k beyond its list form, as a launch in front of it).
+static cs_status decode_step(cs_plan *plan, const cs_layer *layer, const float *x, int B, RecoverOptions &o, float *x_out,
+                             int32_t *sup, float *z, float *resid, cudaStream_t st) {
+    const float *residual = layer->add_residual ? x : nullptr;
+    o.decode = true; o.norm = layer->rms_gamma != nullptr;
+    cs_status s = launch_sketch_slices(plan, layer, x, B, st);
+    if (s != CS_OK) return s;
+    if (decode_recovers(plan)) {
+        const RecoverArgs ra = recover_args(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z, resid, o);
+        return launch_decode_ffn(plan, layer, B, &ra, false, o.norm, residual, x_out, st);
+    }
+    s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z, resid, true, st, o);
+    if (s != CS_OK) return s;
+    return launch_decode_ffn(plan, layer, B, nullptr, true, o.norm, residual, x_out, st);
+}
+
 cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, int32_t B, float *x_out,
                         int32_t *support_out, float *z_out, float *resid_out, void *stream) {
     if (plan == nullptr || x == nullptr || x_out == nullptr) return CS_ERR_NULL;
@@ -345,14 +360,8 @@ cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, in
     const float *n = norm ? plan->n_buf : x;
     int32_t *sup = support_out != nullptr ? support_out : plan->sup_buf;
     if (use_decode_mma(plan, B)) {
-        // The sketch launch also splits the activations; the recovery runs beside the gate/up GEMM, which needs the
-        // supports only in its epilogue.
-        s = launch_sketch_slices(plan, layer, x, B, st);
         RecoverOptions o;
-        o.decode = true; o.norm = norm;
-        if (s == CS_OK) s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z_out, resid_out, true, st, o);
-        if (s == CS_OK) s = launch_decode_ffn(plan, layer, B, true, norm, layer->add_residual ? x : nullptr, x_out, st);
-        return s;
+        return decode_step(plan, layer, x, B, o, x_out, sup, z_out, resid_out, st);
     }
     const bool gather = !plan->mma_ok || B < plan->mma_min_tokens;
     if (gather && plan->speculative && sketch_recover_ok(plan) && !plan->timing) {
@@ -370,9 +379,13 @@ cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, in
         if (s != CS_OK) return s;
         return launch_ffn_gather_spec(plan, layer, n, B, layer->add_residual ? x : nullptr, x_out, st);
     }
-    s = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, norm ? plan->n_buf : nullptr, layer->Phi, layer->mu, st);
-    if (s != CS_OK) return s;
-    s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z_out, resid_out, true, st);
+    if (B <= kSenseMaxTokens) {
+        s = launch_sense_recover(plan, layer->S, layer->Phi, layer->mu, x, layer->rms_gamma, B, norm ? plan->n_buf : nullptr, sup, z_out,
+                                 resid_out, st);
+    } else {
+        s = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, norm ? plan->n_buf : nullptr, layer->Phi, layer->mu, st);
+        if (s == CS_OK) s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z_out, resid_out, true, st);
+    }
     if (s != CS_OK) return s;
     // supports produced by the recovery are valid by construction: no device check here
     return exec_dispatch(plan, layer, n, sup, B, layer->add_residual ? x : nullptr, x_out, false, st);
@@ -413,10 +426,14 @@ cs_status cs_layer_step_ex(cs_plan *plan, const cs_layer *layer, const float *x,
     }
     int32_t *sup = support_out != nullptr ? support_out : plan->sup_buf;
     if (use_decode_mma(plan, B) && !srht && opt->solver == CS_SOLVER_IHT) {   // as in cs_layer_step
-        s = launch_sketch_slices(plan, layer, x, B, st);
-        if (s == CS_OK) s = recover_with(plan, layer->Phi, layer->mu, plan->y_buf, B, opt, sup, z_out, resid_out, true, st, true, norm);
-        if (s == CS_OK) s = launch_decode_ffn(plan, layer, B, true, norm, residual, x_out, st);
-        return s;
+        RecoverOptions o = iht_options(plan, opt);
+        return decode_step(plan, layer, x, B, o, x_out, sup, z_out, resid_out, st);
+    }
+    if (B <= kSenseMaxTokens && !srht && opt->solver == CS_SOLVER_IHT) {
+        s = launch_sense_recover(plan, layer->S, layer->Phi, layer->mu, x, layer->rms_gamma, B, norm ? plan->n_buf : nullptr, sup, z_out,
+                                 resid_out, st, iht_options(plan, opt));
+        if (s != CS_OK) return s;
+        return exec_dispatch(plan, layer, n, sup, B, residual, x_out, false, st);
     }
     if (srht) s = launch_sketch_srht(plan, opt->srht_sign, opt->srht_rows, x, B, plan->y_buf, st);
     else s = launch_sketch(plan, layer->S, x, layer->rms_gamma, B, plan->y_buf, norm ? plan->n_buf : nullptr, layer->Phi,
@@ -551,9 +568,7 @@ cs_status cs_prompt_support(cs_plan *plan, const float *S, const float *Phi, flo
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cs_status s = launch_prompt_mean(plan, H, n, plan->hbar, st);
     if (s != CS_OK) return s;
-    s = launch_sketch(plan, S, plan->hbar, nullptr, 1, plan->y_buf, nullptr, Phi, mu, st);
-    if (s != CS_OK) return s;
-    return launch_recover(plan, Phi, mu, plan->y_buf, 1, support, z, resid, true, st);
+    return launch_sense_recover(plan, S, Phi, mu, plan->hbar, nullptr, 1, nullptr, support, z, resid, st);
 }
 
 cs_status cs_ffn_exec_shared(cs_plan *plan, const cs_layer *layer, const void *H, int32_t n,

@@ -57,7 +57,6 @@ struct cs_plan {
     int32_t *glist;      // [G] groups with a non-empty bucket, ascending
     int32_t *nu;         // [1] their number
     void *x_bf16;        // [2][max_tokens, d] bf16 activations: rounded value, then remainder
-    float *rscale;       // [max_tokens] RMSNorm row scales, applied behind the gate/up GEMM
     void *act;           // [2][max_tokens, d_ff] bf16 SwiGLU activations over the group list (value, remainder)
     float *mma_partial;  // [slices, padded tokens, d] f32 partial down projections
     int speculative;     // small batches, on the recovery's first iterate: 1 = start the weight stream, 2 = warm L2 only
@@ -114,6 +113,27 @@ cs_status launch_sketch(cs_plan *plan, const float *S, const float *x, const flo
 // The sensor in front of launch_decode_ffn: partial sketches per slice of columns (and of the squares, for the RMSNorm),
 // the two bf16 token matrices, and plan->gram.  The recovery adds the partials up.
 cs_status launch_sketch_slices(cs_plan *plan, const cs_layer *L, const float *x, int B, cudaStream_t st);
+// The sketch of a token as launch_sketch_slices leaves it: partial sums per slice of 64 columns.
+struct SketchParts {
+    const float *y, *ss;       // [slices][B, m] and, with an RMSNorm, of the squares [slices][B]
+    int slices, B, d;
+    float eps;
+    float *y_out;              // [B, m]
+};
+struct RecoverArgs {
+    const float *Phi, *gram, *y;
+    float mu, tgamma;          // tgamma = 2 mu gamma of the temporal term
+    int m, G, k, T, B;
+    int32_t *support;
+    float *z, *resid;
+    const int32_t *sup0; const float *z0;
+    const int32_t *sup_prev; const float *z_prev;
+    const int32_t *check;
+    int32_t *delta; float *drift;
+    uint32_t *mask;
+    SketchParts parts;
+    cs::DeviceStatus *status;
+};
 struct RecoverOptions {
     int T = -1;                                             // iterations; < 0: the plan's
     const int32_t *sup0 = nullptr; const float *z0 = nullptr;   // warm start
@@ -121,15 +141,22 @@ struct RecoverOptions {
     const int32_t *sup_prev = nullptr; const float *z_prev = nullptr;
     const int32_t *check = nullptr;                         // supports to validate (ascending, distinct, in range) ...
     int32_t *delta = nullptr; float *drift = nullptr;       // ... and the drift of the result against them
-    // launch_sketch_slices came before and launch_decode_ffn comes next: take the sketch from the partials (writing it
-    // to plan->y_buf), write the membership masks (plan->mask) and, with norm, the RMSNorm's row scales (plan->rscale), and
-    // let the dependents start only when the launches before the recovery are complete.
+    // launch_sketch_slices came before and the decode GEMMs come next: take the sketch from the partials (writing it to
+    // plan->y_buf; norm: with the RMSNorm's row scale), write the membership masks (plan->mask), and (as a launch of its
+    // own) let the dependents start when the launches before the recovery are complete.
     bool decode = false, norm = false;
 };
+RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const float *y, int B, int32_t *support, float *z,
+                         float *resid, const RecoverOptions &o);
 // gram_ready: plan->gram already holds this Phi's matrix (the sketch launch before formed it).
 cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float *y, int B,
                          int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st,
                          const RecoverOptions &opt = RecoverOptions());
+// Sensor and estimator in one launch, a cluster of CTAs per token, for at most kSenseMaxTokens tokens.
+constexpr int kSenseMaxTokens = 16;
+cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,
+                               float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st,
+                               const RecoverOptions &opt = RecoverOptions());
 // the other estimators (solvers.cu)
 cs_status prepare_solvers(cs_plan *plan);
 cs_status launch_niht(cs_plan *plan, const float *Phi, float mu_fallback, const float *y, int B, int T,
@@ -176,8 +203,12 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
 cs_status prepare_decode(cs_plan *plan);
 int decode_slices(const cs_plan *plan);
 cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *support, int B, bool check, cudaStream_t st);
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, bool x_ready, bool rscale, const float *residual, float *out,
-                            cudaStream_t st);
+// recover != NULL and decode_recovers(): the recovery runs inside the gate/up launch; otherwise the launches before have
+// left the masks (plan->mask).  norm: the row scales come from the sketch's partial squares.  x_ready: the launch directly
+// before this one triggers its dependents only when the token matrices are complete.
+bool decode_recovers(const cs_plan *plan);
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool x_ready, bool norm,
+                            const float *residual, float *out, cudaStream_t st);
 cs_status launch_prompt_mean(cs_plan *plan, const void *H, int n, float *hbar, cudaStream_t st);
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may start while its
@@ -266,6 +297,15 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// L2 policy of the weights, which are read once: first to leave L2, so that they do not push out the activations, S and
+// Phi, and the kernels' own code, which after a 270 MB step without this is fetched from HBM again (7B step at 64
+// tokens 63.8 -> 60.0 us, 200 tokens 135 -> 121).
+__device__ __forceinline__ uint64_t policy_evict_first() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
 }
 
 // 16-byte read-only streaming load (weights are read once per step: keep them out of L1).

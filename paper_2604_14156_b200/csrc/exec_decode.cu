@@ -23,11 +23,15 @@
 // without work and took 39.7 us for 180 MB at 64 tokens).  The down GEMM has d / 256 column tiles times
 // as many list slices as fill the SMs, cut at 64-channel k blocks.
 //
-// Chain: gate/up does not need the supports until its epilogue.  In a step the launch before it is the recovery,
-// which triggers its programmatic dependents as soon as the kernels before IT have completed; gate/up then streams
-// while the recovery runs beside it on the same SMs and waits for it (griddepcontrol.wait) only when the accumulators
-// are complete.  The down kernel requests its first ring of weights before it waits for the activations.
+// Supports: gate/up computes every channel of every token and the down GEMM leaves out what a token's support does not
+// hold, by the instruction's lane mask (lanes = tokens, so a k block's mask is its group's membership bits; the
+// accumulators are zeroed first and only ever added to).  So nothing waits for the recovery before the down GEMM,
+// and the recovery runs inside the gate/up launch, in four warps of each CTA that take the tokens in turn.
+// A step is then sketch -> gate/up (+ recovery) -> down -> reduction, each started early (programmatic dependent
+// launch) and streaming its weights before it waits for what the launch before produces.  With the recovery as a launch
+// ahead of gate/up the weight stream began 5.4 us after the step, in this form while the sketch still runs.
 #include "mma_core.cuh"
+#include "recover_core.cuh"
 
 namespace cs {
 
@@ -36,8 +40,8 @@ namespace {
 constexpr int kEpiWarps = 8;                         // two per quarter of the tensor-memory lanes
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kDecThreads = 64 + kEpiThreads;        // + TMA warp, MMA warp
-constexpr int kDecRing = 208 * 1024;                 // operand ring; what is left of the 227 KB holds the recovery's CTAs
-constexpr size_t kDecSmem = 1024 + (size_t)kDecRing + 256;
+constexpr int kRecNW = kMaxG / 32, kRecThreads = 32 * kRecNW;   // the recovery's warps of a gate/up CTA
+constexpr int kDecRing = 208 * 1024;                 // operand ring at most
 constexpr int kDecMaxSlices = 20;
 constexpr int kDecBN = 256;                          // output columns of a down tile
 
@@ -71,9 +75,15 @@ __device__ __forceinline__ void load_tokens(const TokenTile &t, uint8_t *dst, co
     }
 }
 // Ring stages: [tokens][weights] each; what the MMA reads past the tokens of the last stage stays inside the ring.
-__device__ __forceinline__ int ring_stages(const TokenTile &t, int wbytes) {
-    return min(kMaxStages, (kDecRing - max(0, t.over - wbytes)) / (t.bytes + wbytes));
+__host__ __device__ inline int ring_stages(const TokenTile &t, int wbytes) {
+    const int over = t.over > wbytes ? t.over - wbytes : 0, n = (kDecRing - over) / (t.bytes + wbytes);
+    return n < kMaxStages ? n : kMaxStages;
 }
+__host__ __device__ inline int ring_bytes(const TokenTile &t, int wbytes) {
+    return ring_stages(t, wbytes) * (t.bytes + wbytes) + (t.over > wbytes ? t.over - wbytes : 0);
+}
+// No more shared memory than the ring needs: the sketch of the step behind fits beside it.
+inline size_t decode_smem(const TokenTile &t, int wbytes) { return 1024 + (size_t)ring_bytes(t, wbytes) + sizeof(Barriers); }
 __device__ __forceinline__ int token_tx_bytes(const TokenTile &t) { return 2 * t.nbox * t.box * BK * 2; }
 
 __device__ __forceinline__ void prefetch_map(const CUtensorMap *m) {
@@ -116,35 +126,44 @@ template <bool PACK> __device__ __forceinline__ float4 row4(const float *s, int 
 }
 
 // One k block of MMAs: token operand at a0 (remainders at a0 + lo_off) against the N operand given by bdesc(k4).
+// lanes != NULL: the 128-bit lane mask of each 128-token tile (a set bit leaves that lane of the accumulator alone).
 template <bool PACK, int MT, typename BDesc>
-__device__ __forceinline__ void mma_kblock(uint32_t tmem, uint32_t a0, uint32_t lo_off, uint32_t idesc, bool first, BDesc bdesc) {
+__device__ __forceinline__ void mma_kblock(uint32_t tmem, uint32_t a0, uint32_t lo_off, uint32_t idesc, bool first, BDesc bdesc,
+                                           const uint4 *lanes = nullptr) {
 #pragma unroll
     for (int k4 = 0; k4 < BK / 16; ++k4) {
         const uint64_t bd = bdesc(k4);
 #pragma unroll
         for (int t = 0; t < MT; ++t) {
             const uint32_t a = a0 + t * kABytes + k4 * 32;
-            tc_mma(tmem + t * 256, desc_sw128(a, 16), bd, idesc, !first || k4 != 0);
-            if (!PACK) tc_mma(tmem + t * 256, desc_sw128(a + lo_off, 16), bd, idesc, 1);
+            if (lanes != nullptr) {
+                tc_mma_lanes(tmem + t * 256, desc_sw128(a, 16), bd, idesc, lanes[t]);
+                if (!PACK) tc_mma_lanes(tmem + t * 256, desc_sw128(a + lo_off, 16), bd, idesc, lanes[t]);
+            } else {
+                tc_mma(tmem + t * 256, desc_sw128(a, 16), bd, idesc, !first || k4 != 0);
+                if (!PACK) tc_mma(tmem + t * 256, desc_sw128(a + lo_off, 16), bd, idesc, 1);
+            }
         }
     }
 }
 
 // ---- gate / up ------------------------------------------------------------------------------------------
-// CTA x: channels [x R, x R + R).  x_ready: the token matrices were complete before this launch could begin.
-template <bool PACK, int MT>
-__global__ void __launch_bounds__(kDecThreads, 2)
+// CTA x: channels [x R, x R + R), and with KC > 0 (slots of the recovery's list form, in units of 8) the recovery of tokens
+// x, x + gridDim.x, ...  x_ready: the token matrices were complete before this launch could begin (KC == 0 only).
+template <bool PACK, int MT, int KC>
+__global__ void __launch_bounds__(kDecThreads + kRecThreads, 1)
 decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
                      const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u, int B, int R, int d,
-                     int d_ff, int x_ready, const int32_t *mask, const float *rscale,
+                     int d_ff, int x_ready, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
                      __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ act_lo, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
+    __shared__ float rscale_s[MT * BM];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    Barriers *bars = reinterpret_cast<Barriers *>(base + kDecRing);
     const TokenTile tt = token_tile(PACK, MT, B);
     const int c0 = blockIdx.x * R;
     const int wbytes = 2 * R * BK * 2;                   // gate rows then up rows
+    Barriers *bars = reinterpret_cast<Barriers *>(base + ring_bytes(tt, wbytes));
     const int stage_bytes = tt.bytes + wbytes;
     const int stages = ring_stages(tt, wbytes);
     const uint32_t tcols = MT == 2 ? 512u : 256u;
@@ -155,15 +174,16 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     if (warp == 0) {
         if (lane == 0) {
             const int tx = wbytes + token_tx_bytes(tt);
+            const uint64_t once = policy_evict_first();
             auto load_w = [&](int kb, int s) {
                 uint8_t *w = base + (size_t)s * stage_bytes + tt.bytes;
-                tma_load_2d(w, &tm_g, kb * BK, c0, &bars->full[s]);
-                tma_load_2d(w + wbytes / 2, &tm_u, kb * BK, c0, &bars->full[s]);
+                tma_load_2d(w, &tm_g, kb * BK, c0, &bars->full[s], once);
+                tma_load_2d(w + wbytes / 2, &tm_u, kb * BK, c0, &bars->full[s], once);
             };
             // weights are parameters: the first ring is requested before anything is waited for
             const int pre = min(stages, kblocks);
             for (int kb = 0; kb < pre; ++kb) { mbar_expect_tx(&bars->full[kb], tx); load_w(kb, kb); }
-            if (!x_ready) pdl_wait();
+            if (KC > 0 || !x_ready) pdl_wait();
             for (int kb = 0; kb < pre; ++kb) load_tokens(tt, base + (size_t)kb * stage_bytes, &tm_x, &tm_x_lo, kb * BK, &bars->full[kb]);
             int s = 0, ph = 0;
             for (int kb = pre; kb < kblocks; ++kb) {
@@ -191,14 +211,32 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             }
             if (ok) tc_commit(&bars->acc_ready);
         }
-    } else {
-        const bool ok = mbar_wait(&bars->acc_ready, 0, bars, status);
+    } else if (warp < kDecThreads / 32) {
+        const int et = threadIdx.x - 64, r4 = R / 4;
+        pdl_wait();   // the row squares; and nothing is stored before the kernels before this one are complete
+        if (KC == 0) pdl_launch_dependents();   // the supports are final: the down kernel reads them before its own wait
+        for (int t = et; t < MT * BM; t += kEpiThreads) {
+            float rs = 1.f;
+            if (ss_part != nullptr && t < B) {
+                float q = 0.f;
+                for (int i = 0; i < d / 64; i += 16) {   // d is a multiple of 256
+                    float v[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) v[u] = i + u < d / 64 ? ld_dep(ss_part + (size_t)(i + u) * B + t) : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) q += v[u];
+                }
+                rs = rsqrtf(q / (float)d + eps);
+            }
+            rscale_s[t] = rs;
+        }
+        // one warp polls, the others sleep at the barrier behind it
+        if (warp == 2) mbar_wait(&bars->acc_ready, 0, bars, status);
+        epi_sync();
+        const bool ok = *reinterpret_cast<volatile uint32_t *>(&bars->aborted) == 0u && mbar_wait(&bars->acc_ready, 0, bars, status);
         tc_fence_after();
-        pdl_wait();                  // the supports (and the row scales) are final
-        pdl_launch_dependents();     // the down kernel reads the supports before its own wait
         float *dump = reinterpret_cast<float *>(base);   // the ring is free: every load has been consumed
         const int P = ((2 * R + 31) & ~31) + 4;
-        const int et = threadIdx.x - 64, r4 = R / 4;
 #pragma unroll 1
         for (int t = 0; t < MT; ++t) {
             const int t0 = t * BM, rows = min(B - t0, PACK ? 64 : BM);
@@ -206,26 +244,38 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             if (ok) dump_tile<PACK>(bars->tmem_base + t * 256, 2 * R / 16, dump, P, rows, warp, lane);
             epi_sync();
             if (ok) {
+#pragma unroll 2
                 for (int i = et; i < rows * r4; i += kEpiThreads) {
                     const int r = i / r4, c = (i - r * r4) * 4, ch = c0 + c;
                     if (ch >= d_ff) continue;
                     const float4 g = row4<PACK>(dump, P, r, c), u = row4<PACK>(dump, P, r, R + c);
-                    const int grp = ch >> 7;
-                    const bool in = ((uint32_t)ld_dep(mask + (size_t)(t0 + r) * 4 + (grp >> 5)) >> (grp & 31)) & 1u;
-                    float a[4] = {0.f, 0.f, 0.f, 0.f};
-                    if (in) {
-                        const float sc = rscale != nullptr ? ld_dep(rscale + t0 + r) : 1.f;
-                        a[0] = silu_f(g.x * sc) * (u.x * sc); a[1] = silu_f(g.y * sc) * (u.y * sc);
-                        a[2] = silu_f(g.z * sc) * (u.z * sc); a[3] = silu_f(g.w * sc) * (u.w * sc);
-                    }
+                    const float sc = rscale_s[t0 + r];
                     uint2 hi, lo;
-                    split4(a[0], a[1], a[2], a[3], hi, lo);
+                    split4(silu_f(g.x * sc) * (u.x * sc), silu_f(g.y * sc) * (u.y * sc), silu_f(g.z * sc) * (u.z * sc),
+                           silu_f(g.w * sc) * (u.w * sc), hi, lo);
                     const size_t off = (size_t)(t0 + r) * d_ff + ch;
                     *reinterpret_cast<uint2 *>(act + off) = hi;
                     *reinterpret_cast<uint2 *>(act_lo + off) = lo;
                 }
             }
         }
+    } else if constexpr (KC > 0) {
+        constexpr int kRecBar = 3;
+        __shared__ RecoverSmem<kRecNW, KC> rs;
+        const int g = threadIdx.x - kDecThreads;
+        float phc[32];
+        if (ra.m <= 32) recover_load_phi<kRecNW>(ra.Phi, ra.m, ra.G, g, phc);
+        const GramSource M{ra.gram, gram_pitch(ra.G)};
+        pdl_wait();   // the partial sketches and M come from the kernel before
+        for (int t = blockIdx.x; t < B; t += gridDim.x) {
+            recover_row<kRecNW, KC, kRecBar>(
+                rs, ra, M, [&](auto &sm) { y_from_parts<kRecNW, kRecBar>(sm, ra.parts, g, t, ra.m); }, ra.mask, g, t, phc);
+            bar_sync<kRecBar, kRecThreads>();
+        }
+        // the down kernel reads the masks before its own wait
+        __threadfence();
+        bar_sync<kRecBar, kRecThreads>();
+        if (g == 0) pdl_launch_dependents();
     }
     teardown_cta(bars, warp, tcols);
 }
@@ -240,12 +290,14 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
                    int d, float *__restrict__ partial, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t union_s[4];
+    __shared__ int glist_s[kMaxG];                          // groups of this slice, in list order
+    __shared__ __align__(16) uint32_t out_s[kMaxG][4 * MT]; // tokens whose support does not hold them: the lane masks
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    Barriers *bars = reinterpret_cast<Barriers *>(base + kDecRing);
     const TokenTile tt = token_tile(PACK, MT, B);
     const int col0 = blockIdx.x * kDecBN, z = blockIdx.y, Z = gridDim.y;
     constexpr int wbytes = kDecBN * BK * 2;
+    Barriers *bars = reinterpret_cast<Barriers *>(base + ring_bytes(tt, wbytes));
     const int stage_bytes = tt.bytes + wbytes;
     const int stages = ring_stages(tt, wbytes);
     const uint32_t tcols = MT == 2 ? 512u : 256u;
@@ -253,8 +305,9 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
     if (threadIdx.x == 0) { prefetch_map(&tm_wd); prefetch_map(&tm_act); prefetch_map(&tm_act_lo); }
     if (threadIdx.x < 4) union_s[threadIdx.x] = 0u;
     setup_cta(bars, warp, tcols);
+    // The masks were final, and visible, before this launch could begin (see the gate/up kernel's trigger).
     int ng = G;
-    if (use_union) {   // the supports were final before this launch could begin (see the gate/up kernel's trigger)
+    if (use_union) {
         for (int t = threadIdx.x; t < B; t += kDecThreads) {
             const uint4 m = ld_l2(mask + (size_t)t * 4);
             if (m.x) atomicOr(&union_s[0], m.x);
@@ -267,86 +320,102 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
     }
     const int nk = 2 * ng;
     const int k0 = (int)((long long)nk * z / Z), kblocks = (int)((long long)nk * (z + 1) / Z) - k0;
+    const int l0 = k0 >> 1, nl = kblocks > 0 ? ((k0 + kblocks - 1) >> 1) - l0 + 1 : 0;   // list entries of this slice
+    if (threadIdx.x < G) {
+        const int g = threadIdx.x;
+        int pos = g;
+        bool in = true;
+        if (use_union) {
+            in = (union_s[g >> 5] >> (g & 31)) & 1u;
+            pos = __popc(union_s[g >> 5] & ((1u << (g & 31)) - 1u));
+            for (int w = 0; w < (g >> 5); ++w) pos += __popc(union_s[w]);
+        }
+        if (in && pos >= l0 && pos < l0 + nl) glist_s[pos - l0] = g;
+    }
+    __syncthreads();
 
     if (warp == 0) {
         if (lane == 0) {
             const int tx = wbytes + token_tx_bytes(tt);
-            // walks the channels of the list's k blocks: two per group
-            struct Walk { int word; uint32_t bits; int g; bool half; };
-            auto start = [&](int k) {
-                Walk w{0, 0u, k >> 1, (k & 1) != 0};
-                if (use_union) {
-                    int skip = k >> 1;
-                    while (w.word < 3 && skip >= __popc(union_s[w.word])) skip -= __popc(union_s[w.word++]);
-                    w.bits = union_s[w.word];
-                    while (skip-- > 0) w.bits &= w.bits - 1;
-                    w.g = 32 * w.word + __ffs(w.bits) - 1;
-                }
-                return w;
-            };
-            auto channel = [](const Walk &w) { return w.g * 128 + (w.half ? BK : 0); };
-            auto advance = [&](Walk &w) {
-                if (!w.half) { w.half = true; return; }
-                w.half = false;
-                if (!use_union) { ++w.g; return; }
-                w.bits &= w.bits - 1;
-                while (w.bits == 0u && w.word < 3) w.bits = union_s[++w.word];
-                w.g = 32 * w.word + __ffs(w.bits) - 1;
-            };
+            const uint64_t once = policy_evict_first();
+            auto channel = [&](int kb) { return glist_s[((k0 + kb) >> 1) - l0] * 128 + ((k0 + kb) & 1) * BK; };
             auto load_w = [&](int ch, int s) {
                 uint8_t *w = base + (size_t)s * stage_bytes + tt.bytes;
 #pragma unroll
                 for (int j = 0; j < kDecBN / 64; ++j)
-                    tma_load_2d(w + j * (64 * BK * 2), &tm_wd, col0 + j * 64, ch, &bars->full[s]);
+                    tma_load_2d(w + j * (64 * BK * 2), &tm_wd, col0 + j * 64, ch, &bars->full[s], once);
             };
             const int pre = min(stages, kblocks);
-            if (kblocks > 0) {
-                Walk w = start(k0), wa = w;
-                for (int kb = 0; kb < pre; ++kb, advance(w)) { mbar_expect_tx(&bars->full[kb], tx); load_w(channel(w), kb); }
-                pdl_wait();   // the activations
-                for (int kb = 0; kb < pre; ++kb, advance(wa))
-                    load_tokens(tt, base + (size_t)kb * stage_bytes, &tm_act, &tm_act_lo, channel(wa), &bars->full[kb]);
-                int s = 0, ph = 0;
-                for (int kb = pre; kb < kblocks; ++kb, advance(w)) {
-                    if (!mbar_wait(&bars->empty[s], ph, bars, status)) break;
-                    mbar_expect_tx(&bars->full[s], tx);
-                    load_w(channel(w), s);
-                    load_tokens(tt, base + (size_t)s * stage_bytes, &tm_act, &tm_act_lo, channel(w), &bars->full[s]);
-                    if (++s == stages) { s = 0; ph ^= 1; }
-                }
+            for (int kb = 0; kb < pre; ++kb) { mbar_expect_tx(&bars->full[kb], tx); load_w(channel(kb), kb); }
+            pdl_wait();   // the activations
+            for (int kb = 0; kb < pre; ++kb)
+                load_tokens(tt, base + (size_t)kb * stage_bytes, &tm_act, &tm_act_lo, channel(kb), &bars->full[kb]);
+            int s = 0, ph = 0;
+            for (int kb = pre; kb < kblocks; ++kb) {
+                if (!mbar_wait(&bars->empty[s], ph, bars, status)) break;
+                mbar_expect_tx(&bars->full[s], tx);
+                load_w(channel(kb), s);
+                load_tokens(tt, base + (size_t)s * stage_bytes, &tm_act, &tm_act_lo, channel(kb), &bars->full[s]);
+                if (++s == stages) { s = 0; ph ^= 1; }
             }
         }
     } else if (warp == 1) {
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads + 32) : "memory");   // accumulators zeroed, lane masks in place
+        tc_fence_after();
         if (lane == 0 && kblocks > 0) {
             constexpr uint32_t idesc = make_idesc(true);
             const uint32_t tmem = bars->tmem_base;
             bool ok = true;
             int s = 0, ph = 0;
             for (int kb = 0; kb < kblocks; ++kb) {
+                const uint4 *lanes = reinterpret_cast<const uint4 *>(out_s[((k0 + kb) >> 1) - l0]);
                 ok = mbar_wait(&bars->full[s], ph, bars, status);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(base + (size_t)s * stage_bytes), w0 = a0 + tt.bytes;
-                mma_kblock<PACK, MT>(tmem, a0, tt.lo_off, idesc, kb == 0,
-                                     [&](int k4) { return desc_sw128(w0 + k4 * 2048, 64 * BK * 2); });
+                mma_kblock<PACK, MT>(tmem, a0, tt.lo_off, idesc, false,
+                                     [&](int k4) { return desc_sw128(w0 + k4 * 2048, 64 * BK * 2); }, lanes);
                 tc_commit(&bars->empty[s]);
                 if (++s == stages) { s = 0; ph ^= 1; }
             }
             if (ok) tc_commit(&bars->acc_ready);
         }
     } else {
-        const bool ok = kblocks > 0 && mbar_wait(&bars->acc_ready, 0, bars, status);
+        const int ew = warp - 2, q = warp & 3, et = threadIdx.x - 64;
+        // lane masks: epilogue warp w holds the membership words of tokens 32 w .. 32 w + 31
+        if (ew < (PACK ? 2 : 4 * MT)) {
+            const int t = 32 * ew + lane;
+            const uint4 m = t < B ? ld_l2(mask + (size_t)t * 4) : make_uint4(0u, 0u, 0u, 0u);
+            for (int i = 0; i < nl; ++i) {
+                const int g = glist_s[i], w = g >> 5;
+                const uint32_t word = w == 0 ? m.x : w == 1 ? m.y : w == 2 ? m.z : m.w;
+                const uint32_t out = ~__ballot_sync(0xffffffffu, (word >> (g & 31)) & 1u);
+                if (lane == 0) {
+                    out_s[i][ew] = out;
+                    if (PACK) out_s[i][ew + 2] = out;   // the remainder rows of the same tokens
+                }
+            }
+        }
+        for (int c = ew >> 2; c < MT * 256 / 16; c += kEpiWarps / 4)
+            tc_st16_zero(bars->tmem_base + ((uint32_t)(q * 32) << 16) + c * 16);
+        tc_wait_st();
+        tc_fence_before();
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads + 32) : "memory");
+        if (warp == 2 && kblocks > 0) mbar_wait(&bars->acc_ready, 0, bars, status);
+        epi_sync();
+        const bool ok = kblocks > 0 && *reinterpret_cast<volatile uint32_t *>(&bars->aborted) == 0u &&
+                        mbar_wait(&bars->acc_ready, 0, bars, status);
         tc_fence_after();
         pdl_wait();   // nothing is stored before the kernels before this one are complete
         float *dump = reinterpret_cast<float *>(base);
         constexpr int P = kDecBN + 4;
-        const int et = threadIdx.x - 64;
 #pragma unroll 1
         for (int t = 0; t < MT; ++t) {
             const int t0 = t * BM, rows = min(B - t0, PACK ? 64 : BM);
             if (t > 0) epi_sync();
             if (ok) dump_tile<PACK>(bars->tmem_base + t * 256, kDecBN / 16, dump, P, rows, warp, lane);
             epi_sync();
+#pragma unroll 2
             for (int i = et; i < rows * (kDecBN / 4); i += kEpiThreads) {
                 const int r = i / (kDecBN / 4), c = (i % (kDecBN / 4)) * 4;
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);   // an empty slice contributes zero
@@ -412,11 +481,24 @@ decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ supp
     if (tid < 4) mask[(size_t)t * 4 + tid] = (int)m_s[tid];
 }
 
-typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, int, const int32_t *,
-                         const float *, __nv_bfloat16 *, __nv_bfloat16 *, DeviceStatus *);
+typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, int, const float *, float,
+                         RecoverArgs, __nv_bfloat16 *, __nv_bfloat16 *, DeviceStatus *);
 typedef void (*DownFn)(CUtensorMap, CUtensorMap, CUtensorMap, const int32_t *, int, int, int, int, float *, DeviceStatus *);
 
+// The recovery's list form in three lengths (24, 32, 56 slots); 0: no recovery inside the launch.
+int gateup_kc(const cs_plan *plan) { return plan->cfg.k <= 24 ? 3 : plan->cfg.k <= 32 ? 4 : 7; }
+template <bool PACK, int MT> GateUpFn gateup_fn_kc(int kc) {
+    return kc == 0 ? decode_gateup_kernel<PACK, MT, 0> : kc == 3 ? decode_gateup_kernel<PACK, MT, 3>
+         : kc == 4 ? decode_gateup_kernel<PACK, MT, 4> : decode_gateup_kernel<PACK, MT, 7>;
+}
+GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators
+    return form == 0 ? gateup_fn_kc<true, 1>(kc) : form == 1 ? gateup_fn_kc<false, 1>(kc) : gateup_fn_kc<false, 2>(kc);
+}
+DownFn down_fn(int form) { return form == 0 ? decode_down_kernel<true, 1> : form == 1 ? decode_down_kernel<false, 1> : decode_down_kernel<false, 2>; }
+
 }  // namespace
+
+bool decode_recovers(const cs_plan *plan) { return plan->cfg.k <= 56; }
 
 int decode_slices(const cs_plan *plan) {   // list slices of the down GEMM: one CTA per SM
     const int tiles = plan->cfg.d / kDecBN;
@@ -426,13 +508,12 @@ int decode_slices(const cs_plan *plan) {   // list slices of the down GEMM: one 
 cs_status prepare_decode(cs_plan *plan) {
     CS_CUDA_TRY(plan, prefer_shared(decode_prep_kernel));
     CS_CUDA_TRY(plan, prefer_shared(decode_reduce_kernel));
-    const int smem = (int)kDecSmem;
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_gateup_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_gateup_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_gateup_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_down_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_down_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(decode_down_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int smem = 1024 + kDecRing + (int)sizeof(Barriers);
+    for (int form = 0; form < 3; ++form) {
+        CS_CUDA_TRY(plan, cudaFuncSetAttribute(gateup_fn(form, 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CS_CUDA_TRY(plan, cudaFuncSetAttribute(gateup_fn(form, gateup_kc(plan)), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        CS_CUDA_TRY(plan, cudaFuncSetAttribute(down_fn(form), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    }
     return CS_OK;
 }
 
@@ -446,14 +527,11 @@ cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *suppo
     return CS_OK;
 }
 
-// The three launches of the actuator.  The token matrices (plan->x_bf16), the masks (plan->mask) and, with rscale, the row
-// scales (plan->rscale) come from the launches before; x_ready: the launch directly before this one triggers its
-// dependents only after the matrices are complete.
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, bool x_ready, bool rscale, const float *residual, float *out,
-                            cudaStream_t st) {
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool x_ready, bool norm,
+                            const float *residual, float *out, cudaStream_t st) {
     const cs_config &c = plan->cfg;
     const bool pack = B <= 64;
-    const int mt = B <= BM ? 1 : 2;
+    const int mt = B <= BM ? 1 : 2, form = pack ? 0 : mt;
     const TokenTile tt = token_tile(pack, mt, B);
     const int R = min(128, ((c.d_ff + plan->sm_count - 1) / plan->sm_count + 7) & ~7);
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16), *x_lo = x_hi + (size_t)c.max_tokens * c.d;
@@ -466,10 +544,10 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, bool x_read
         return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
-        const GateUpFn fn = pack ? decode_gateup_kernel<true, 1> : mt == 1 ? decode_gateup_kernel<false, 1> : decode_gateup_kernel<false, 2>;
-        launch_pdl(true, fn, dim3((c.d_ff + R - 1) / R), dim3(kDecThreads), kDecSmem, st, tm_x, tm_x_lo, tm_g, tm_u, B, R, c.d, c.d_ff,
-                   x_ready ? 1 : 0, (const int32_t *)plan->mask, rscale ? (const float *)plan->rscale : (const float *)nullptr, act, act_lo,
-                   plan->status);
+        launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3((c.d_ff + R - 1) / R),
+                   dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), decode_smem(tt, 2 * R * BK * 2), st, tm_x, tm_x_lo, tm_g,
+                   tm_u, B, R, c.d, c.d_ff, x_ready ? 1 : 0, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
+                   c.rms_eps, recover != nullptr ? *recover : RecoverArgs{}, act, act_lo, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }
@@ -479,9 +557,8 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, bool x_read
         // Expected number of groups in nobody's support, G (1 - k/G)^B: below a quarter group the list is every group and
         // the masks need not be read.
         const bool use_union = (float)plan->G * powf(1.f - (float)c.k / plan->G, (float)B) > 0.25f;
-        const DownFn fn = pack ? decode_down_kernel<true, 1> : mt == 1 ? decode_down_kernel<false, 1> : decode_down_kernel<false, 2>;
-        launch_pdl(true, fn, dim3(c.d / kDecBN, Z), dim3(kDecThreads), kDecSmem, st, tm_wd, tm_act, tm_act_lo, (const int32_t *)plan->mask,
-                   use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
+        launch_pdl(true, down_fn(form), dim3(c.d / kDecBN, Z), dim3(kDecThreads), decode_smem(tt, kDecBN * BK * 2), st, tm_wd, tm_act,
+                   tm_act_lo, (const int32_t *)plan->mask, use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }

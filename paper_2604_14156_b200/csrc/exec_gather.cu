@@ -62,9 +62,10 @@ __device__ __forceinline__ int ld_acquire(const int32_t *p) {
     return v;
 }
 
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
+// Weights: read once, first to leave L2, so that S, Phi and the kernels' code stay there from step to step.
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src, uint64_t policy) {
     const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem_src) : "memory");
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "l"(policy) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() {
@@ -99,6 +100,7 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
     const int rows_total = k << lb;
     const int nrows = (rows_total - bx + nx - 1) / nx;     // rows bx, bx + nx, ...
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t once = policy_evict_first();
     auto cta_sync = [] {   // the streaming warps only
         if constexpr (SPEC) bar_sync<1, kGatherThreads>(); else __syncthreads();
     };
@@ -209,8 +211,8 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
 #pragma unroll
         for (int j = 0; j < kUnitChunks; ++j) {
             if (FULL || (seg * kUnitChunks + j) * 32 + lane < chunks) {
-                cp_async16(dst + j * 32, pg + j * 32 * E);
-                cp_async16(dst + (kUnitChunks + j) * 32, pu + j * 32 * E);
+                cp_async16(dst + j * 32, pg + j * 32 * E, once);
+                cp_async16(dst + (kUnitChunks + j) * 32, pu + j * 32 * E, once);
             }
         }
     };
@@ -314,7 +316,7 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
             uint4 *dst = wring + issue_stage * (CPT * 32);
 #pragma unroll
             for (int j = 0; j < CPT; ++j)
-                if (FULL || tid + j * kGatherThreads < chunks) cp_async16(dst + j * 32, p + j * kGatherThreads * E);
+                if (FULL || tid + j * kGatherThreads < chunks) cp_async16(dst + j * 32, p + j * kGatherThreads * E, once);
         }
         cp_async_commit();
         ++issue_r;
@@ -550,6 +552,7 @@ static cudaError_t gather_attrs_all(bool fused_too) {
 
 cs_status prepare_ffn_gather(cs_plan *plan) {
     CS_CUDA_TRY(plan, gather_attrs_all(true));
+    CS_CUDA_TRY(plan, prefer_shared(reduce_partials_kernel));
     return CS_OK;
 }
 

@@ -11,129 +11,202 @@ __global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restr
     gram_rows(Phi, mu, m, G, blockIdx.x, gram);
 }
 
-// Support drift between consecutive decoding steps (Sec. 11): Delta_t = |S_t symmetric-difference
-// S_{t-1}|.  Both rows are ascending and distinct, so entry j of the new row is looked up in the old
-// one by bisection; the rows have k entries each, so the symmetric difference is twice the misses.
-// Called by a whole CTA of at least k threads.
-__device__ __forceinline__ void drift_row(const int32_t *p, const int32_t *cur, int k, int j, int t, int32_t *drift, float *ratio) {
-    int missing = 0;
-    if (j < k) {
-        const int e = ld_dep(cur + j);
-        int lo = 0, hi = k;                       // first index whose entry is >= e
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (ld_dep(p + mid) < e) lo = mid + 1; else hi = mid;
-        }
-        missing = !(lo < k && ld_dep(p + lo) == e);
-    }
-    const int n = __syncthreads_count(missing);
-    if (j == 0) {
-        if (drift != nullptr) drift[t] = 2 * n;
-        // D_t = |S_t sym.diff S_{t-1}| / |S_t union S_{t-1}| (Sec. 15): both rows have k entries, so the union has k + n
-        if (ratio != nullptr) ratio[t] = (float)(2 * n) / (float)(k + n);
-    }
-}
-
-// The previous supports of a recovery: validated (ascending, distinct, in range), and the drift against them.
-struct RecoverDrift {
-    const int32_t *prev;
-    int32_t *delta;
-    float *ratio;
-};
-
-// The sketch of a token as launch_sketch_slices leaves it: partial sums per slice of columns.
-struct SketchParts {
-    const float *y, *ss;       // [slices][B, m] and, with an RMSNorm, [slices][B]; y == NULL: the sketch is given
-    int slices, B, d;
-    float eps;
-    float *y_out, *rscale;     // [B, m], [B]
-};
-
-// s.y of token t from the partials: thread g adds the slices of one row in its share of the slices, the shares are added
-// in order; the row scale is folded in.
-template <int NW, typename Smem>
-__device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int g, int t, int m) {
-    constexpr int GP = 32 * NW;
-    const int shares = GP / m < 1 ? 1 : GP / m;            // threads per row (m <= 64 <= 2 GP)
-    for (int row0 = 0; row0 < m; row0 += GP) {             // one round unless m > GP
-        const int row = row0 + g % m, share = g / m;
-        float a = 0.f;
-        if (row < m && share < shares) {
-            const int n = (p.slices + shares - 1) / shares, lo = share * n, hi = min(p.slices, lo + n);
-            const float *src = p.y + (size_t)t * m + row;
-            for (int i = lo; i < hi; i += 16) {
-                float v[16];
-#pragma unroll
-                for (int u = 0; u < 16; ++u) v[u] = i + u < hi ? ld_dep(src + (size_t)(i + u) * p.B * m) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 16; ++u) a += v[u];
-            }
-        }
-        if (m > GP) { if (row < m) s.y[row] = a; }
-        else s.part[g] = a;
-    }
-    float rs = 1.f;
-    if (p.ss != nullptr) {   // every warp for itself
-        float q = 0.f;
-        for (int i = g & 31; i < p.slices; i += 32) q += ld_dep(p.ss + (size_t)i * p.B + t);
-        rs = rsqrtf(warp_sum(q) / (float)p.d + p.eps);
-        if (g == 0) p.rscale[t] = rs;
-    }
-    bar_sync<0, GP>();
-    for (int row = g; row < m; row += GP) {
-        float a = 0.f;
-        if (m > GP) a = s.y[row];
-        else for (int sh = 0; sh < shares; ++sh) a += s.part[sh * m + row];
-        a *= rs;
-        s.y[row] = a;
-        p.y_out[(size_t)t * m + row] = a;
-    }
-}
-
 // NW = warps = ceil(G / 32).  KC = ceil(k / 8) for k <= 56 (list form), 0 otherwise (dense form).
 // DECODE: the form of RecoverOptions::decode.
 template <int NW, int KC, bool DECODE>
-__global__ void __launch_bounds__(32 * NW)
-recover_kernel(const float *__restrict__ Phi, const float *__restrict__ gram, float mu, const float *__restrict__ y,
-               int m, int G, int k, int T, int32_t *__restrict__ support, float *__restrict__ z_out,
-               float *__restrict__ resid_out, const int32_t *__restrict__ sup0, const float *__restrict__ z0,
-               float tgamma, const int32_t *__restrict__ sup_prev, const float *__restrict__ z_prev, uint32_t *__restrict__ mask,
-               SketchParts parts, RecoverDrift drift, DeviceStatus *status) {
+__global__ void __launch_bounds__(32 * NW) recover_kernel(const __grid_constant__ RecoverArgs a) {
     __shared__ RecoverSmem<NW, KC> s;
-    const int g = threadIdx.x, t = blockIdx.x;
+    const int g = threadIdx.x;
     if (!DECODE) pdl_launch_dependents();
     // Phi is a parameter: this thread's column is requested before the wait for the kernel that
     // produces y and M, when it fits 32 registers
     float phc[32];
-    if (m <= 32) recover_load_phi<NW>(Phi, m, G, g, phc);
+    if (a.m <= 32) recover_load_phi<NW>(a.Phi, a.m, a.G, g, phc);
     pdl_wait();   // y and M come from the kernel before
     // The decode GEMMs read what the kernels before this one wrote without a wait of their own, and wait for the
     // supports behind their main loop.
     if (DECODE) pdl_launch_dependents();
-    if (drift.prev != nullptr && g < k) {
-        const int32_t *p = drift.prev + (size_t)t * k + g;
-        const int e = ld_dep(p);
-        if (e < 0 || e >= G || (g > 0 && ld_dep(p - 1) >= e)) atomicCAS(&status->code, 0, (int)CS_ERR_SUPPORT);
-    }
-    recover_token<NW, KC, 0>(s, g, Phi, GramSource{gram, 32 * NW}, mu,
-                             [&](auto &sm) {
-                                 if constexpr (DECODE) y_from_parts<NW>(sm, parts, g, t, m);
-                                 else for (int row = g; row < m; row += 32 * NW) sm.y[row] = ld_dep(y + (size_t)t * m + row);
-                             }, m, G, k, T, support + (size_t)t * k,
-                             z_out != nullptr ? z_out + (size_t)t * k : nullptr,
-                             resid_out != nullptr ? resid_out + t : nullptr,
-                             sup0 != nullptr ? sup0 + (size_t)t * k : nullptr, z0 != nullptr ? z0 + (size_t)t * k : nullptr,
-                             tgamma, sup_prev != nullptr ? sup_prev + (size_t)t * k : nullptr,
-                             z_prev != nullptr ? z_prev + (size_t)t * k : nullptr,
-                             DECODE ? mask + (size_t)t * 4 : nullptr, status, phc, [] {}, [](int, int) {}, [] {});
-    if (drift.delta != nullptr || drift.ratio != nullptr) {
-        __syncthreads();   // the support row is written
-        drift_row(drift.prev + (size_t)t * k, support + (size_t)t * k, k, g, t, drift.delta, drift.ratio);
-    }
+    const int t = blockIdx.x;
+    recover_row<NW, KC, 0>(
+        s, a, GramSource{a.gram, 32 * NW},
+        [&](auto &sm) {
+            if constexpr (DECODE) y_from_parts<NW, 0>(sm, a.parts, g, t, a.m);
+            else for (int i = g; i < a.m; i += 32 * NW) sm.y[i] = ld_dep(a.y + (size_t)t * a.m + i);
+        },
+        DECODE ? a.mask : nullptr, g, t, phc);
 }
 
-typedef void (*RecoverFn)(const float *, const float *, float, const float *, int, int, int, int, int32_t *, float *, float *,
-                          const int32_t *, const float *, float, const int32_t *, const float *, uint32_t *, SketchParts, RecoverDrift, DeviceStatus *);
+// ---- sensor and estimator of a token in one launch (small batches, the prompt's mean) ------------------------
+// A cluster of eight CTAs per token.  CTA r takes the columns [r d / 8, (r + 1) d / 8) of S and x.  Its part of S is in
+// shared memory before the wait for the kernel that produces x, and so are Phi and M = I - mu Phi^T Phi in that of
+// CTA 0 (every CTA forms an eighth of M), so between x and the sketch lie one load of x, the dot products, and one
+// exchange over distributed shared memory; CTA 0 then runs the iteration with every operand in its shared memory.
+// Bound by latency.  As two launches, with M formed by the first and read from L2 by the second, the pair took
+// 15 us of a step at 7B, batch 1 (to the gather kernel), in this form 11.5 us.
+constexpr int kSenseCtas = 8;
+constexpr int kSenseThreads = 256;
+constexpr int kSenseWarps = kSenseThreads / 32;
+constexpr int kSenseMaxChunks = kMaxD / kSenseCtas / 4 / 32;   // float4 columns per lane
+constexpr int kSenseSmem = 220 * 1024;                         // dynamic, at most
+
+struct SenseArgs {
+    const float *S, *x, *gamma;
+    float eps;
+    int d, s_rows;        // s_rows: rows of S that fit in shared memory (the others are read after the wait)
+    float *y_out, *n_out;
+};
+
+__device__ __forceinline__ uint32_t remote_smem(const void *p, uint32_t rank) {   // the same place in CTA `rank` of the cluster
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_remote(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <int NW, int KC>
+__global__ void __cluster_dims__(kSenseCtas, 1, 1) __launch_bounds__(kSenseThreads, 1)
+sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant__ RecoverArgs a) {
+    constexpr int GP = 32 * NW;
+    extern __shared__ float4 sense_s[];
+    __shared__ RecoverSmem<NW, KC> rs;
+    __shared__ float part_s[kSenseCtas][kMaxM], ss_s[kSenseCtas];
+    const int t = blockIdx.x / kSenseCtas, rank = blockIdx.x % kSenseCtas;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m = a.m, G = a.G, d = sa.d;
+    const int nc = d / (4 * kSenseCtas);            // float4 columns of this CTA
+    const size_t col0 = (size_t)rank * nc * 4;
+    float *M_s = reinterpret_cast<float *>(sense_s), *phi_s = M_s + G * GP;
+    float4 *S_s = reinterpret_cast<float4 *>(phi_s + m * (GP + 4));
+    pdl_launch_dependents();
+    cluster_arrive();                               // matched below: every CTA of the cluster has started
+    // this lane's chunks of this warp's rows of S: no other thread reads them
+    for (int r = warp; r < sa.s_rows; r += kSenseWarps)
+        for (int c = lane; c < nc; c += 32) {
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(S_s + r * nc + c);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(sa.S + (size_t)r * d + col0 + 4 * c) : "memory");
+        }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    float4 gm[kSenseMaxChunks];
+    if (sa.gamma != nullptr) {
+#pragma unroll
+        for (int j = 0; j < kSenseMaxChunks; ++j)
+            if (lane + 32 * j < nc) gm[j] = __ldg(reinterpret_cast<const float4 *>(sa.gamma + col0) + lane + 32 * j);
+    }
+    for (int i = tid; i < m * GP; i += kSenseThreads) {
+        const int row = i / GP, g = i - row * GP;
+        phi_s[row * (GP + 4) + g] = g < G ? __ldg(a.Phi + row * G + g) : 0.f;
+    }
+    __syncthreads();
+    float phc[32];
+    if (rank == 0 && m <= 32 && tid < GP) {
+#pragma unroll
+        for (int row = 0; row < 32; ++row) phc[row] = row < m ? phi_s[row * (GP + 4) + tid] : 0.f;
+    }
+    cluster_wait();
+    // M in blocks of 2 x 4 entries, each summed as gram_rows sums it; every eighth row pair is this CTA's
+    const uint32_t M0 = remote_smem(M_s, 0);
+    for (int b = tid; b < ((G + 1) / 2 - rank + kSenseCtas - 1) / kSenseCtas * (GP / 4); b += kSenseThreads) {
+        const int i0 = (b / (GP / 4) * kSenseCtas + rank) * 2, j0 = b % (GP / 4) * 4;
+        float s0[2][4] = {}, s1[2][4] = {};
+        auto add = [&](int row, float (&s)[2][4]) {
+            const float2 p = *reinterpret_cast<const float2 *>(phi_s + row * (GP + 4) + i0);
+            const float4 q = *reinterpret_cast<const float4 *>(phi_s + row * (GP + 4) + j0);
+            s[0][0] = fmaf(p.x, q.x, s[0][0]); s[0][1] = fmaf(p.x, q.y, s[0][1]); s[0][2] = fmaf(p.x, q.z, s[0][2]); s[0][3] = fmaf(p.x, q.w, s[0][3]);
+            s[1][0] = fmaf(p.y, q.x, s[1][0]); s[1][1] = fmaf(p.y, q.y, s[1][1]); s[1][2] = fmaf(p.y, q.z, s[1][2]); s[1][3] = fmaf(p.y, q.w, s[1][3]);
+        };
+        int row = 0;
+#pragma unroll 4
+        for (; row + 1 < m; row += 2) { add(row, s0); add(row + 1, s1); }
+        if (row < m) add(row, s0);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (i0 + u >= G) break;
+            float o[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) o[v] = j0 + v < G ? (i0 + u == j0 + v ? 1.f : 0.f) - a.mu * (s0[u][v] + s1[u][v]) : 0.f;
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(M0 + 4u * ((i0 + u) * GP + j0)), "f"(o[0]), "f"(o[1]),
+                         "f"(o[2]), "f"(o[3]) : "memory");
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    pdl_wait();   // x may be the previous kernel's output
+    float4 xv[kSenseMaxChunks];
+    float ss = 0.f;
+#pragma unroll
+    for (int j = 0; j < kSenseMaxChunks; ++j)
+        xv[j] = lane + 32 * j < nc ? ld_dep4(sa.x + (size_t)t * d + col0 + 4 * (lane + 32 * j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < kSenseMaxChunks; ++j) {
+        ss += xv[j].x * xv[j].x + xv[j].y * xv[j].y + xv[j].z * xv[j].z + xv[j].w * xv[j].w;
+        if (sa.gamma != nullptr && lane + 32 * j < nc) { xv[j].x *= gm[j].x; xv[j].y *= gm[j].y; xv[j].z *= gm[j].z; xv[j].w *= gm[j].w; }
+    }
+#pragma unroll 1
+    for (int r0 = warp; r0 < m; r0 += 4 * kSenseWarps) {   // four rows at a time: their reductions interleave
+        float acc[4] = {};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + q * kSenseWarps;
+            if (r >= m) break;
+#pragma unroll
+            for (int j = 0; j < kSenseMaxChunks; ++j) {
+                const int c = lane + 32 * j;
+                if (c >= nc) break;
+                const float4 s = r < sa.s_rows ? S_s[r * nc + c] : __ldg(reinterpret_cast<const float4 *>(sa.S + (size_t)r * d + col0) + c);
+                acc[q] = fmaf(s.x, xv[j].x, acc[q]); acc[q] = fmaf(s.y, xv[j].y, acc[q]);
+                acc[q] = fmaf(s.z, xv[j].z, acc[q]); acc[q] = fmaf(s.w, xv[j].w, acc[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = warp_sum(acc[q]);
+        if (lane < 4) {
+            const int r = r0 + lane * kSenseWarps;
+            const float v = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+            if (r < m) st_remote(remote_smem(&part_s[rank][r], 0), v);
+        }
+    }
+    if (warp == 0 && sa.gamma != nullptr) {
+        ss = warp_sum(ss);
+        if (lane < kSenseCtas) st_remote(remote_smem(&ss_s[rank], lane), ss);
+    }
+    cluster_arrive();
+    cluster_wait();
+    float rscale = 1.f;
+    if (sa.gamma != nullptr) {
+        float tot = 0.f;
+#pragma unroll
+        for (int r = 0; r < kSenseCtas; ++r) tot += ss_s[r];
+        rscale = rsqrtf(tot / (float)d + sa.eps);
+    }
+    if (sa.n_out != nullptr && warp == kSenseWarps - 1) {
+#pragma unroll
+        for (int j = 0; j < kSenseMaxChunks; ++j)
+            if (lane + 32 * j < nc)
+                *reinterpret_cast<float4 *>(sa.n_out + (size_t)t * d + col0 + 4 * (lane + 32 * j)) =
+                    make_float4(xv[j].x * rscale, xv[j].y * rscale, xv[j].z * rscale, xv[j].w * rscale);
+    }
+    if (rank != 0 || tid >= GP) return;
+    const int g = tid;
+    recover_row<NW, KC, 1>(
+        rs, a, SharedSource<GP>{M_s, phi_s, G},
+        [&](auto &sm) {
+            for (int i = g; i < m; i += GP) {
+                float y = 0.f;
+#pragma unroll
+                for (int r = 0; r < kSenseCtas; ++r) y += part_s[r][i];
+                y *= rscale;
+                sm.y[i] = y;
+                sa.y_out[(size_t)t * m + i] = y;
+            }
+        },
+        nullptr, g, t, phc);
+}
+typedef void (*SenseFn)(SenseArgs, RecoverArgs);
+
+typedef void (*RecoverFn)(RecoverArgs);
 static int recover_kc(int k) { return k <= 56 ? (k + 7) / 8 : 0; }
 template <int NW, bool DECODE> static RecoverFn recover_fn_kc(int k) {
     switch (recover_kc(k)) {
@@ -155,7 +228,63 @@ template <bool DECODE> static RecoverFn recover_fn(int G, int k) {
         default: return recover_fn_kc<4, DECODE>(k);
     }
 }
+RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const float *y, int B, int32_t *support, float *z,
+                         float *resid, const RecoverOptions &o) {
+    const cs_config &c = plan->cfg;
+    RecoverArgs a{};
+    a.Phi = Phi; a.gram = plan->gram; a.y = y; a.mu = mu; a.tgamma = 2.f * mu * o.gamma;
+    a.m = c.m; a.G = plan->G; a.k = c.k; a.T = o.T < 0 ? c.T : o.T; a.B = B;
+    a.support = support; a.z = z; a.resid = resid;
+    a.sup0 = o.sup0; a.z0 = o.z0; a.sup_prev = o.sup_prev; a.z_prev = o.z_prev;
+    a.check = o.check; a.delta = o.delta; a.drift = o.drift;
+    if (o.decode) {
+        a.mask = plan->mask;
+        a.parts = SketchParts{sketch_partials(plan), o.norm ? sketch_square_partials(plan, B) : nullptr, c.d / 64, B, c.d, c.rms_eps,
+                              plan->y_buf};
+    }
+    a.status = plan->status;
+    return a;
+}
+
+template <int NW> static SenseFn sense_fn_kc(int k) {
+    switch (recover_kc(k)) {
+        case 1: return sense_recover_kernel<NW, 1>;
+        case 2: return sense_recover_kernel<NW, 2>;
+        case 3: return sense_recover_kernel<NW, 3>;
+        case 4: return sense_recover_kernel<NW, 4>;
+        case 5: return sense_recover_kernel<NW, 5>;
+        case 6: return sense_recover_kernel<NW, 6>;
+        case 7: return sense_recover_kernel<NW, 7>;
+        default: return sense_recover_kernel<NW, 0>;
+    }
+}
+static SenseFn sense_fn(int G, int k) {
+    switch ((G + 31) / 32) {
+        case 1: return sense_fn_kc<1>(k);
+        case 2: return sense_fn_kc<2>(k);
+        case 3: return sense_fn_kc<3>(k);
+        default: return sense_fn_kc<4>(k);
+    }
+}
+
+cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,
+                               float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st, const RecoverOptions &o) {
+    const cs_config &c = plan->cfg;
+    const int GP = gram_pitch(plan->G), row_bytes = c.d / kSenseCtas * 4;
+    const int fixed = (plan->G * GP + c.m * (GP + 4)) * 4;
+    SenseArgs sa{S, x, gamma, c.rms_eps, c.d, min(c.m, (kSenseSmem - fixed) / row_bytes), plan->y_buf, n_out};
+    {
+        StageTimer timer(plan, CS_STAGE_SKETCH, st);
+        launch_pdl(true, sense_fn(plan->G, c.k), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)sa.s_rows * row_bytes, st,
+                   sa, recover_args(plan, Phi, mu, nullptr, B, support, z, resid, o));
+    }
+    plan->launches++;
+    CS_CUDA_TRY(plan, cudaGetLastError());
+    return CS_OK;
+}
+
 cs_status prepare_recover(cs_plan *plan) {
+    CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
     CS_CUDA_TRY(plan, prefer_shared(recover_fn<true>(plan->G, plan->cfg.k)));
     return CS_OK;
 }
@@ -170,13 +299,8 @@ cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float 
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }
-    SketchParts parts{};
-    if (o.decode)
-        parts = SketchParts{sketch_partials(plan), o.norm ? sketch_square_partials(plan, B) : nullptr, c.d / 64, B, c.d, c.rms_eps,
-                            plan->y_buf, plan->rscale};
-    launch_pdl(true, o.decode ? recover_fn<true>(G, c.k) : recover_fn<false>(G, c.k), dim3(B), dim3(gram_pitch(G)), 0, st, Phi, (const float *)plan->gram, mu, y, c.m, G, c.k,
-               o.T < 0 ? c.T : o.T, support, z, resid, o.sup0, o.z0, 2.f * mu * o.gamma, o.sup_prev, o.z_prev,
-               o.decode ? plan->mask : (uint32_t *)nullptr, parts, RecoverDrift{o.check, o.delta, o.drift}, plan->status);
+    launch_pdl(true, o.decode ? recover_fn<true>(G, c.k) : recover_fn<false>(G, c.k), dim3(B), dim3(gram_pitch(G)), 0, st,
+               recover_args(plan, Phi, mu, y, B, support, z, resid, o));
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
     return CS_OK;
@@ -187,7 +311,7 @@ __global__ void __launch_bounds__(kDriftThreads)
 support_drift_kernel(const int32_t *__restrict__ prev, const int32_t *__restrict__ cur, int k,
                      int32_t *__restrict__ drift, float *__restrict__ ratio) {
     const int t = blockIdx.x;
-    drift_row(prev + (size_t)t * k, cur + (size_t)t * k, k, threadIdx.x, t, drift, ratio);
+    drift_row<0, kDriftThreads>(prev + (size_t)t * k, cur + (size_t)t * k, k, threadIdx.x, t, drift, ratio);
 }
 
 cs_status launch_support_drift(cs_plan *plan, const int32_t *prev, const int32_t *cur, int B, int32_t *drift,

@@ -58,7 +58,7 @@ template <int NW, int KC> struct RecoverSmem {
     alignas(16) float red[kMaxM];     // residual r of the two-step form; partial sums of the residual norm
     alignas(16) float val[2][NV];     // the iterate, by iteration parity: slot values, or dense z
     int idx[NV];                      // list form: entry held by each slot (the support, in slot order)
-    float y[kMaxM];
+    alignas(16) float y[kMaxM];       // zero past m
     uint32_t mm[2][2][4];             // per parity: min kept key / max other key, per warp
     int sum[4];                       // rank sums per warp
     int cnt[4];                       // entries that left the support (or, at the end, kept entries) per warp
@@ -83,6 +83,15 @@ struct GramSource {
         return ld_dep(gram + (size_t)j * pitch + g);
     }
     __device__ __forceinline__ float phi(const float *Phi, int row, int col, int G) const { return __ldg(Phi + row * G + col); }
+    // row g, padded to GP entries (M is symmetric: column g as well)
+    template <int GP> __device__ __forceinline__ void row(int g, float (&mreg)[GP]) const {
+        const float *src = gram + (size_t)g * GP;
+#pragma unroll
+        for (int j = 0; j < GP / 4; ++j) {
+            const float4 q = ld_dep4(src + 4 * j);
+            mreg[4 * j] = q.x; mreg[4 * j + 1] = q.y; mreg[4 * j + 2] = q.z; mreg[4 * j + 3] = q.w;
+        }
+    }
     // the entries of all k slots: independent loads, issued together (tid: unused)
     template <int NR> __device__ __forceinline__ void fill(const int *idx, int k, int, int g, const float (&own)[32],
                                                            float (&mreg)[NR]) const {
@@ -96,6 +105,28 @@ struct GramSource {
 #pragma unroll
         for (int j = 0; j < NR; ++j)
             if ((chg >> j) & 1ull) mreg[j] = get(idx[j], g, own);
+    }
+};
+//   SharedSource: the matrix in shared memory, [G][GP], columns past G zero, and Phi beside it, [m][GP + 4].
+template <int GP_> struct SharedSource {
+    const float *M_s, *phi_s;
+    int G;
+    __device__ __forceinline__ float phi(const float *, int row, int col, int) const { return phi_s[row * (GP_ + 4) + col]; }
+    template <int GP> __device__ __forceinline__ void row(int g, float (&mreg)[GP]) const {
+#pragma unroll
+        for (int j = 0; j < GP; ++j) mreg[j] = j < G ? M_s[j * GP + g] : 0.f;
+    }
+    template <int NR> __device__ __forceinline__ void fill(const int *idx, int k, int, int g, const float (&)[32],
+                                                           float (&mreg)[NR]) const {
+#pragma unroll
+        for (int j = 0; j < NR; ++j)
+            if (j < k) mreg[j] = M_s[idx[j] * GP_ + g];
+    }
+    template <int NR> __device__ __forceinline__ void reload(unsigned long long chg, const int *idx, int g,
+                                                             const float (&)[32], float (&mreg)[NR]) const {
+#pragma unroll
+        for (int j = 0; j < NR; ++j)
+            if ((chg >> j) & 1ull) mreg[j] = M_s[idx[j] * GP_ + g];
     }
 };
 template <int BAR_A, int BAR_B, int THREADS> struct PhiSource {
@@ -193,15 +224,9 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
 #pragma unroll
         for (int j = 0; j < NR; ++j) mreg[j] = 0.f;
     }
-    if constexpr (KC == 0) {   // row g of M (M is symmetric: row g is the column that multiplies into entry g)
-        const float *src = M.gram + (size_t)gm * GP;
-#pragma unroll
-        for (int j = 0; j < GP / 4; ++j) {
-            const float4 q = ld_dep4(src + 4 * j);
-            mreg[4 * j] = q.x; mreg[4 * j + 1] = q.y; mreg[4 * j + 2] = q.z; mreg[4 * j + 3] = q.w;
-        }
-    }
+    if constexpr (KC == 0) M.template row<GP>(gm, mreg);   // row g of M: what multiplies into entry g
     load_y(s);   // s.y, complete at the next barrier
+    for (int i = m + g; i < kMaxM; i += GP) s.y[i] = 0.f;
     // z_0 = 0 with the support the order assigns to an all-zero vector (indices 0..k-1), or, warm
     // started, the k-sparse iterate handed in (sup0 ascending and distinct, z0 its values).
     const bool warm = sup0 != nullptr;
@@ -233,10 +258,7 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
         }
     }
     if constexpr (KC > 0) {
-        if (warm) {   // the entries that go with the warm list
-#pragma unroll
-            for (int j = 0; j < NR; ++j) mreg[j] = M.get(s.idx[j], gm, phc);
-        }
+        if (warm) M.fill(s.idx, k, g, gm, phc, mreg);   // the entries that go with the warm list
     }
     // c_g = mu sum_i Phi[i,g] y_i
     float cg = 0.f;
@@ -244,22 +266,20 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
         for (int row = 0; row < 32; row += 4) {   // rows past m hold zeros
-            const float y0 = row < m ? s.y[row] : 0.f, y1 = row + 1 < m ? s.y[row + 1] : 0.f;
-            const float y2 = row + 2 < m ? s.y[row + 2] : 0.f, y3 = row + 3 < m ? s.y[row + 3] : 0.f;
-            a0 = fmaf(phc[row], y0, a0); a1 = fmaf(phc[row + 1], y1, a1);
-            a2 = fmaf(phc[row + 2], y2, a2); a3 = fmaf(phc[row + 3], y3, a3);
+            const float4 yq = *reinterpret_cast<const float4 *>(s.y + row);
+            a0 = fmaf(phc[row], yq.x, a0); a1 = fmaf(phc[row + 1], yq.y, a1);
+            a2 = fmaf(phc[row + 2], yq.z, a2); a3 = fmaf(phc[row + 3], yq.w, a3);
         }
         cg = mu * ((a0 + a1) + (a2 + a3));
     } else if (valid) {
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        const float *pcol = Phi + g;
         int row = 0;
 #pragma unroll 4
         for (; row + 3 < m; row += 4) {
-            a0 = fmaf(__ldg(pcol + row * G), s.y[row], a0); a1 = fmaf(__ldg(pcol + (row + 1) * G), s.y[row + 1], a1);
-            a2 = fmaf(__ldg(pcol + (row + 2) * G), s.y[row + 2], a2); a3 = fmaf(__ldg(pcol + (row + 3) * G), s.y[row + 3], a3);
+            a0 = fmaf(M.phi(Phi, row, g, G), s.y[row], a0); a1 = fmaf(M.phi(Phi, row + 1, g, G), s.y[row + 1], a1);
+            a2 = fmaf(M.phi(Phi, row + 2, g, G), s.y[row + 2], a2); a3 = fmaf(M.phi(Phi, row + 3, g, G), s.y[row + 3], a3);
         }
-        for (; row < m; ++row) a0 = fmaf(__ldg(pcol + row * G), s.y[row], a0);
+        for (; row < m; ++row) a0 = fmaf(M.phi(Phi, row, g, G), s.y[row], a0);
         cg = mu * ((a0 + a1) + (a2 + a3));
     }
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -434,6 +454,95 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
         const int parts = KC > 0 ? NW : m;   // per-warp sums in the list form, per-row squares in the dense form
         for (int i = 0; i < parts; ++i) ss += s.red[i];
         *resid_out = sqrtf(ss);
+    }
+}
+
+// Support drift between consecutive decoding steps (Sec. 11): Delta_t = |S_t symmetric-difference
+// S_{t-1}|.  Both rows are ascending and distinct, so entry j of the new row is looked up in the old
+// one by bisection; the rows have k entries each, so the symmetric difference is twice the misses.
+// Called by the N >= k threads that meet on named barrier BAR, j = 0 .. N - 1.
+template <int BAR, int N>
+__device__ __forceinline__ void drift_row(const int32_t *p, const int32_t *cur, int k, int j, int t, int32_t *drift, float *ratio) {
+    int missing = 0;
+    if (j < k) {
+        const int e = ld_dep(cur + j);
+        int lo = 0, hi = k;                       // first index whose entry is >= e
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (ld_dep(p + mid) < e) lo = mid + 1; else hi = mid;
+        }
+        missing = !(lo < k && ld_dep(p + lo) == e);
+    }
+    int n;
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %1, 0;\nbarrier.cta.red.popc.aligned.u32 %0, %2, %3, p;\n}"
+                 : "=r"(n) : "r"(missing), "n"(BAR), "n"(N) : "memory");
+    if (j == 0) {
+        if (drift != nullptr) drift[t] = 2 * n;
+        // D_t = |S_t sym.diff S_{t-1}| / |S_t union S_{t-1}| (Sec. 15): both rows have k entries, so the union has k + n
+        if (ratio != nullptr) ratio[t] = (float)(2 * n) / (float)(k + n);
+    }
+}
+
+// s.y of token t from the partial sketches: thread g adds the slices of one row in its share of the slices, the shares
+// are added in order; the RMSNorm's row scale is folded in.
+template <int NW, int BAR, typename Smem>
+__device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int g, int t, int m) {
+    constexpr int GP = 32 * NW;
+    const int shares = GP / m < 1 ? 1 : GP / m;            // threads per row (m <= 64 <= 2 GP)
+    for (int row0 = 0; row0 < m; row0 += GP) {             // one round unless m > GP
+        const int row = row0 + g % m, share = g / m;
+        float a = 0.f;
+        if (row < m && share < shares) {
+            const int n = (p.slices + shares - 1) / shares, lo = share * n, hi = min(p.slices, lo + n);
+            const float *src = p.y + (size_t)t * m + row;
+            for (int i = lo; i < hi; i += 16) {
+                float v[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) v[u] = i + u < hi ? ld_dep(src + (size_t)(i + u) * p.B * m) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 16; ++u) a += v[u];
+            }
+        }
+        if (m > GP) { if (row < m) s.y[row] = a; }
+        else s.part[g] = a;
+    }
+    float rs = 1.f;
+    if (p.ss != nullptr) {   // every warp for itself
+        float q = 0.f;
+        for (int i = g & 31; i < p.slices; i += 32) q += ld_dep(p.ss + (size_t)i * p.B + t);
+        rs = rsqrtf(warp_sum(q) / (float)p.d + p.eps);
+    }
+    bar_sync<BAR, GP>();
+    for (int row = g; row < m; row += GP) {
+        float a = 0.f;
+        if (m > GP) a = s.y[row];
+        else for (int sh = 0; sh < shares; ++sh) a += s.part[sh * m + row];
+        a *= rs;
+        s.y[row] = a;
+        p.y_out[(size_t)t * m + row] = a;
+    }
+}
+
+// Token t of a batch, by the 32 * NW threads that meet on named barrier BAR: the check of the previous support, the
+// iteration, the outputs, the drift.  load_y as in recover_token; mask: [B, 4] membership bits, or NULL.
+template <int NW, int KC, int BAR, typename MSource, typename LoadY>
+__device__ __forceinline__ void recover_row(RecoverSmem<NW, KC> &s, const RecoverArgs &a, const MSource M, LoadY load_y,
+                                            uint32_t *mask, int g, int t, const float (&phc)[32]) {
+    const size_t row = (size_t)t * a.k;
+    if (a.check != nullptr && g < a.k) {
+        const int32_t *p = a.check + row + g;
+        const int e = ld_dep(p);
+        if (e < 0 || e >= a.G || (g > 0 && ld_dep(p - 1) >= e)) atomicCAS(&a.status->code, 0, (int)CS_ERR_SUPPORT);
+    }
+    recover_token<NW, KC, BAR>(
+        s, g, a.Phi, M, a.mu, load_y, a.m, a.G, a.k, a.T, a.support + row, a.z != nullptr ? a.z + row : nullptr,
+        a.resid != nullptr ? a.resid + t : nullptr, a.sup0 != nullptr ? a.sup0 + row : nullptr,
+        a.z0 != nullptr ? a.z0 + row : nullptr, a.tgamma, a.sup_prev != nullptr ? a.sup_prev + row : nullptr,
+        a.z_prev != nullptr ? a.z_prev + row : nullptr, mask != nullptr ? mask + (size_t)t * 4 : nullptr, a.status, phc, [] {},
+        [](int, int) {}, [] {});
+    if (a.delta != nullptr || a.drift != nullptr) {
+        bar_sync<BAR, 32 * NW>();   // the support row is written
+        drift_row<BAR, 32 * NW>(a.check + row, a.support + row, a.k, g, t, a.delta, a.drift);
     }
 }
 

@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kSketchThreads)
 sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, const float *__restrict__ gamma, int m, int d, int B,
                      float *__restrict__ y_part, float *__restrict__ ss_part, __nv_bfloat16 *__restrict__ x_hi,
                      __nv_bfloat16 *__restrict__ x_lo, const float *__restrict__ Phi, float mu, int G, float *__restrict__ gram) {
-    __shared__ float4 xs[kSliceTokens * kSlicePitch / 4], Ss[kMaxM * kSlicePitch / 4];
+    extern __shared__ float4 slice_s[];   // x rows, then S rows: small enough to sit beside a decode GEMM's CTA
     const int slices = d / kSliceCols, tiles = (B + kSliceTokens - 1) / kSliceTokens;
     const int tid = threadIdx.x;
     pdl_launch_dependents();
@@ -222,6 +222,7 @@ sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, c
     }
     const int sl = (int)blockIdx.x % slices, t0 = (int)blockIdx.x / slices * kSliceTokens;
     const int nt = min(kSliceTokens, B - t0), c0 = sl * kSliceCols;
+    float4 *xs = slice_s, *Ss = slice_s + min(kSliceTokens, B) * (kSlicePitch / 4);
     const int q = tid & 15, r0 = tid >> 4;        // 16 threads per row of 64 columns
     constexpr int RS = kSketchThreads / 16;       // rows per round
     for (int r = r0; r < m; r += RS)              // S is a parameter: before the wait
@@ -239,8 +240,8 @@ sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, c
         const int r = r0 + i * RS;
         float ss = v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
         v[i].x *= gm.x; v[i].y *= gm.y; v[i].z *= gm.z; v[i].w *= gm.w;
-        xs[r * (kSlicePitch / 4) + q] = v[i];
         if (r < nt) {
+            xs[r * (kSlicePitch / 4) + q] = v[i];
             uint2 hi, lo;
             split4(v[i].x, v[i].y, v[i].z, v[i].w, hi, lo);
             const size_t o = ((size_t)(t0 + r) * d + c0) / 4 + q;
@@ -257,7 +258,7 @@ sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, c
     // 2 tokens x 4 rows per thread, rows m4 apart and tokens nt2 apart (neighbouring threads: neighbouring rows)
     const int m4 = (m + 3) / 4, nt2 = (nt + 1) / 2;
     for (int i = tid; i < m4 * nt2; i += kSketchThreads) {
-        const int rr = i % m4, ta = i / m4, tb = min(ta + nt2, kSliceTokens - 1);
+        const int rr = i % m4, ta = i / m4, tb = min(ta + nt2, nt - 1);
         float acc[2][4] = {};
 #pragma unroll 4
         for (int c = 0; c < kSliceCols / 4; ++c) {
@@ -287,8 +288,8 @@ cs_status launch_sketch_slices(cs_plan *plan, const cs_layer *L, const float *x,
     StageTimer timer(plan, CS_STAGE_SKETCH, st);
     const int slices = c.d / kSliceCols, tiles = (B + kSliceTokens - 1) / kSliceTokens;
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
-    launch_pdl(true, sketch_slices_kernel, dim3(slices * tiles + gram_blocks(plan->G)), dim3(kSketchThreads), 0, st, L->S, x,
-               L->rms_gamma, c.m, c.d, B, sketch_partials(plan), sketch_square_partials(plan, B), x_hi,
+    launch_pdl(true, sketch_slices_kernel, dim3(slices * tiles + gram_blocks(plan->G)), dim3(kSketchThreads),
+               (size_t)(min(kSliceTokens, B) + c.m) * kSlicePitch * sizeof(float), st, L->S, x, L->rms_gamma, c.m, c.d, B, sketch_partials(plan), sketch_square_partials(plan, B), x_hi,
                x_hi + (size_t)c.max_tokens * c.d, L->Phi, L->mu, plan->G, plan->gram);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
