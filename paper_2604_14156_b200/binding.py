@@ -125,13 +125,15 @@ def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str, shape=None) -
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     return t.data_ptr()
 
 
 def _stream(stream) -> int:
     if stream is None:
+        if torch.cuda.is_initialized():   # the handle itself: building a Stream object takes 3 us of a 24 us call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
@@ -146,6 +148,7 @@ class Plan:
         self.G = d_ff // group if group > 0 else 0
         self.w_dtype = w_dtype
         self.max_tokens = max_tokens
+        self._templates = {}
         code = {torch.float32: CS_F32, torch.bfloat16: CS_BF16}.get(w_dtype, -1)
         cfg = _Config(d, d_ff, group, m, k, T, code, max_tokens, rms_eps)
         handle = ctypes.c_void_p()
@@ -154,6 +157,19 @@ class Plan:
         if st != 0:
             raise CSError(st, "cs_plan_create")
         self.handle = handle
+
+    def outputs(self, B: int, device):
+        """New (support [B,k], z [B,k], resid [B]) for a call's outputs.  Allocated like empty templates that are kept per
+        batch size: half the host time of naming shape, type and device each time."""
+        t = self._templates.get((B, device))
+        if t is None:
+            if len(self._templates) >= 64:
+                self._templates.clear()
+            t = (torch.empty((B, self.k), dtype=torch.int32, device=device),
+                 torch.empty((B, self.k), dtype=torch.float32, device=device),
+                 torch.empty((B,), dtype=torch.float32, device=device))
+            self._templates[(B, device)] = t
+        return torch.empty_like(t[0]), torch.empty_like(t[1]), torch.empty_like(t[2])
 
     def check(self, st: int, where: str):
         if st != 0:
@@ -219,6 +235,7 @@ class Layer:
             _ptr(W_up, plan.w_dtype, "W_up", (plan.d_ff, plan.d)),
             _ptr(Wd_t, plan.w_dtype, "Wd_t", (plan.d_ff, plan.d)),
             _ptr(rms_gamma, torch.float32, "rms_gamma", (plan.d,)), float(mu), int(bool(add_residual)))
+        self.ref = ctypes.byref(self.c)
         self.mu = float(mu)
         self.S, self.Phi = S, Phi
 
@@ -235,9 +252,7 @@ def cs_sketch(plan: Plan, S, h, y=None, stream=None):
 def cs_recover(plan: Plan, Phi, mu: float, y, stream=None):
     B = y.shape[0]
     dev = y.device
-    support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-    z = torch.empty((B, plan.k), dtype=torch.float32, device=dev)
-    resid = torch.empty((B,), dtype=torch.float32, device=dev)
+    support, z, resid = plan.outputs(B, dev)
     plan.check(plan.lib.cs_recover(plan.handle, _ptr(Phi, torch.float32, "Phi", (plan.m, plan.G)), float(mu),
                                    _ptr(y, torch.float32, "y", (B, plan.m)), B, support.data_ptr(),
                                    z.data_ptr(), resid.data_ptr(), _stream(stream)), "cs_recover")
@@ -248,9 +263,7 @@ def cs_recover_warm(plan: Plan, Phi, mu: float, y, T: int, support0, z0, stream=
     """T iterations from the k-sparse iterate (support0, z0) instead of zero; returns (support, z, resid)."""
     B = y.shape[0]
     dev = y.device
-    support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-    z = torch.empty((B, plan.k), dtype=torch.float32, device=dev)
-    resid = torch.empty((B,), dtype=torch.float32, device=dev)
+    support, z, resid = plan.outputs(B, dev)
     plan.check(plan.lib.cs_recover_warm(plan.handle, _ptr(Phi, torch.float32, "Phi", (plan.m, plan.G)), float(mu),
                                         _ptr(y, torch.float32, "y", (B, plan.m)), B, int(T),
                                         _ptr(support0, torch.int32, "support0", (B, plan.k)),
@@ -303,9 +316,7 @@ class StepOptions:
 def cs_recover_ex(plan: Plan, Phi, mu: float, y, options: StepOptions, stream=None):
     B = y.shape[0]
     dev = y.device
-    support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-    z = torch.empty((B, plan.k), dtype=torch.float32, device=dev)
-    resid = torch.empty((B,), dtype=torch.float32, device=dev)
+    support, z, resid = plan.outputs(B, dev)
     plan.check(plan.lib.cs_recover_ex(plan.handle, _ptr(Phi, torch.float32, "Phi", (plan.m, plan.G)), float(mu),
                                       _ptr(y, torch.float32, "y", (B, plan.m)), B, ctypes.byref(options.c),
                                       support.data_ptr(), z.data_ptr(), resid.data_ptr(), _stream(stream)), "cs_recover_ex")
@@ -327,10 +338,11 @@ def cs_layer_step_ex(plan: Plan, layer: Layer, x, options: StepOptions, x_out=No
     B = x.shape[0]
     dev = x.device
     x_out = torch.empty_like(x) if x_out is None else x_out
-    support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-    z = torch.zeros((B, plan.k), dtype=torch.float32, device=dev)
-    resid = torch.zeros((B,), dtype=torch.float32, device=dev)
-    plan.check(plan.lib.cs_layer_step_ex(plan.handle, ctypes.byref(layer.c), _ptr(x, torch.float32, "x", (B, plan.d)), B,
+    support, z, resid = plan.outputs(B, dev)
+    if options.c.reuse_support:   # no estimation: the call leaves these two alone
+        z.zero_()
+        resid.zero_()
+    plan.check(plan.lib.cs_layer_step_ex(plan.handle, layer.ref, _ptr(x, torch.float32, "x", (B, plan.d)), B,
                                          ctypes.byref(options.c), _ptr(x_out, torch.float32, "x_out", (B, plan.d)),
                                          support.data_ptr(), z.data_ptr(), resid.data_ptr(), _stream(stream)),
                "cs_layer_step_ex")
@@ -343,12 +355,10 @@ def cs_layer_step_fallback(plan: Plan, dense: Plan, layer: Layer, x, tau: float,
     B = x.shape[0]
     dev = x.device
     x_out = torch.empty_like(x)
-    support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-    z = torch.empty((B, plan.k), dtype=torch.float32, device=dev)
-    resid = torch.empty((B,), dtype=torch.float32, device=dev)
+    support, z, resid = plan.outputs(B, dev)
     flags = torch.empty((B,), dtype=torch.int32, device=dev)
     n = ctypes.c_int32(0)
-    plan.check(plan.lib.cs_layer_step_fallback(plan.handle, dense.handle, ctypes.byref(layer.c),
+    plan.check(plan.lib.cs_layer_step_fallback(plan.handle, dense.handle, layer.ref,
                                                _ptr(x, torch.float32, "x", (B, plan.d)), B,
                                                None if options is None else ctypes.byref(options.c), float(tau),
                                                x_out.data_ptr(), support.data_ptr(), z.data_ptr(), resid.data_ptr(),
@@ -359,7 +369,7 @@ def cs_layer_step_fallback(plan: Plan, dense: Plan, layer: Layer, x, tau: float,
 def cs_uds_budget(plan: Plan, logits, m_base: float, gamma: float, m_min: int, m_max: int, stream=None):
     """Entropy of softmax(logits[t]) and the budget clip(floor(m_base (1 + gamma H)), m_min, m_max); returns (m_t, H)."""
     B, V = logits.shape
-    H = torch.empty((B,), dtype=torch.float32, device=logits.device)
+    H = logits.new_empty((B,))
     m_t = torch.empty((B,), dtype=torch.int32, device=logits.device)
     plan.check(plan.lib.cs_uds_budget(plan.handle, _ptr(logits, torch.float32, "logits", (B, V)), B, V, float(m_base),
                                       float(gamma), int(m_min), int(m_max), H.data_ptr(), m_t.data_ptr(),
@@ -370,7 +380,7 @@ def cs_uds_budget(plan: Plan, logits, m_base: float, gamma: float, m_min: int, m
 def cs_ffn_exec(plan: Plan, layer: Layer, h, support, residual=None, out=None, stream=None):
     B = h.shape[0]
     out = torch.empty((B, plan.d), dtype=torch.float32, device=h.device) if out is None else out
-    plan.check(plan.lib.cs_ffn_exec(plan.handle, ctypes.byref(layer.c), _ptr(h, torch.float32, "h", (B, plan.d)),
+    plan.check(plan.lib.cs_ffn_exec(plan.handle, layer.ref, _ptr(h, torch.float32, "h", (B, plan.d)),
                                     _ptr(support, torch.int32, "support", (B, plan.k)), B,
                                     _ptr(residual, torch.float32, "residual", (B, plan.d)),
                                     _ptr(out, torch.float32, "out", (B, plan.d)), _stream(stream)), "cs_ffn_exec")
@@ -392,7 +402,7 @@ def cs_ffn_exec_static(d: int, d_ff: int, group: int, k: int, layer: Layer, h, s
     cfg = _Config(d, d_ff, group, 1, k, 0, code, 1, 1e-5)
     B = h.shape[0]
     out = torch.empty((B, d), dtype=torch.float32, device=h.device) if out is None else out
-    st = lib.cs_ffn_exec_static(ctypes.byref(cfg), ctypes.byref(layer.c), _ptr(h, torch.float32, "h", (B, d)),
+    st = lib.cs_ffn_exec_static(ctypes.byref(cfg), layer.ref, _ptr(h, torch.float32, "h", (B, d)),
                                 _ptr(support, torch.int32, "support", (B, k)), B,
                                 _ptr(residual, torch.float32, "residual", (B, d)),
                                 _ptr(out, torch.float32, "out", (B, d)), _stream(stream))
@@ -421,10 +431,8 @@ def cs_layer_step(plan: Plan, layer: Layer, x, x_out=None, want_aux: bool = True
     x_out = torch.empty_like(x) if x_out is None else x_out
     support = z = resid = None
     if want_aux:
-        support = torch.empty((B, plan.k), dtype=torch.int32, device=dev)
-        z = torch.empty((B, plan.k), dtype=torch.float32, device=dev)
-        resid = torch.empty((B,), dtype=torch.float32, device=dev)
-    plan.check(plan.lib.cs_layer_step(plan.handle, ctypes.byref(layer.c), _ptr(x, torch.float32, "x", (B, plan.d)), B,
+        support, z, resid = plan.outputs(B, dev)
+    plan.check(plan.lib.cs_layer_step(plan.handle, layer.ref, _ptr(x, torch.float32, "x", (B, plan.d)), B,
                                       _ptr(x_out, torch.float32, "x_out", (B, plan.d)),
                                       None if support is None else support.data_ptr(),
                                       None if z is None else z.data_ptr(),
@@ -439,7 +447,7 @@ def cs_layer_step_host(plan: Plan, layer: Layer, x_host, x_out_host, support_hos
     for t, name in ((x_host, "x_host"), (x_out_host, "x_out_host")):
         if t.is_cuda or t.dtype != torch.float32 or not t.is_contiguous() or tuple(t.shape) != (B, plan.d):
             raise TypeError(f"{name} must be a contiguous CPU float32 tensor of shape ({B}, {plan.d})")
-    plan.check(plan.lib.cs_layer_step_host(plan.handle, ctypes.byref(layer.c), x_host.data_ptr(), B,
+    plan.check(plan.lib.cs_layer_step_host(plan.handle, layer.ref, x_host.data_ptr(), B,
                                            x_out_host.data_ptr(),
                                            None if support_host is None else support_host.data_ptr(),
                                            _stream(stream)), "cs_layer_step_host")
@@ -449,9 +457,8 @@ def cs_layer_step_host(plan: Plan, layer: Layer, x_host, x_out_host, support_hos
 def cs_prompt_support(plan: Plan, S, Phi, mu: float, H, stream=None):
     n = H.shape[0]
     dev = H.device
-    support = torch.empty((plan.k,), dtype=torch.int32, device=dev)
-    z = torch.empty((plan.k,), dtype=torch.float32, device=dev)
-    resid = torch.empty((1,), dtype=torch.float32, device=dev)
+    support, z, resid = plan.outputs(1, dev)
+    support, z = support.view(-1), z.view(-1)
     plan.check(plan.lib.cs_prompt_support(plan.handle, _ptr(S, torch.float32, "S", (plan.m, plan.d)),
                                           _ptr(Phi, torch.float32, "Phi", (plan.m, plan.G)), float(mu),
                                           _ptr(H, torch.bfloat16, "H", (n, plan.d)), n, support.data_ptr(),
@@ -462,7 +469,7 @@ def cs_prompt_support(plan: Plan, S, Phi, mu: float, H, stream=None):
 def cs_ffn_exec_shared(plan: Plan, layer: Layer, H, support, out=None, stream=None):
     n = H.shape[0]
     out = torch.empty_like(H) if out is None else out
-    plan.check(plan.lib.cs_ffn_exec_shared(plan.handle, ctypes.byref(layer.c),
+    plan.check(plan.lib.cs_ffn_exec_shared(plan.handle, layer.ref,
                                            _ptr(H, torch.bfloat16, "H", (n, plan.d)), n,
                                            _ptr(support, torch.int32, "support", (plan.k,)),
                                            _ptr(out, torch.bfloat16, "out", (n, plan.d)), _stream(stream)),
