@@ -75,7 +75,6 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device);
     const size_t nt = (size_t)cfg->max_tokens;
     p->nx_max = max(p->sm_count, (cfg->k * cfg->group + kGatherMaxRows - 1) / kGatherMaxRows);
-    p->mean_row_blocks = 32;
     auto alloc = [&](void **ptr, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(ptr, bytes);
     };
@@ -90,8 +89,7 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     alloc((void **)&p->fb_count, sizeof(int32_t));
     alloc((void **)&p->slot_table, nt * kSlotTablePitch * sizeof(int32_t));
     alloc((void **)&p->ticket, nt * sizeof(unsigned));
-    alloc((void **)&p->hbar, (size_t)cfg->d * sizeof(float));
-    alloc((void **)&p->colsum, (size_t)p->mean_row_blocks * cfg->d * sizeof(float));
+    alloc((void **)&p->colsum, (size_t)kMeanRowBlocks * cfg->d * sizeof(float));
     alloc((void **)&p->status, sizeof(DeviceStatus));
     p->mma_ok = cfg->w_dtype == CS_BF16 && cfg->group == 128 && cfg->d % 256 == 0;
     // The gather path streams B * k groups, the tensor-core path every group once: it takes over where
@@ -123,6 +121,7 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     if (e == cudaSuccess) e = cudaMemset(p->slot_table, 0, nt * kSlotTablePitch * sizeof(int32_t));
     if (e == cudaSuccess && prepare_sketch(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && prepare_recover(p) != CS_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess && prepare_prompt(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && prepare_solvers(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && prepare_ffn_gather(p) != CS_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess && p->mma_ok && prepare_ffn_mma(p) != CS_OK) e = cudaErrorUnknown;
@@ -140,7 +139,7 @@ cs_status cs_plan_destroy(cs_plan *p) {
     if (p == nullptr) return CS_ERR_NULL;
     cudaFree(p->n_buf); cudaFree(p->y_buf); cudaFree(p->sup_buf);
     cudaFree(p->partial); cudaFree(p->gram); cudaFree(p->slot_table); cudaFree(p->ticket);
-    cudaFree(p->resid_buf); cudaFree(p->fb_flags); cudaFree(p->fb_list); cudaFree(p->fb_count); cudaFree(p->hbar); cudaFree(p->colsum);
+    cudaFree(p->resid_buf); cudaFree(p->fb_flags); cudaFree(p->fb_list); cudaFree(p->fb_count); cudaFree(p->colsum);
     cudaFree(p->status); cudaFree(p->x_host_in); cudaFree(p->x_host_out);
     cudaFree(p->mask); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
     cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial);
@@ -566,9 +565,10 @@ cs_status cs_prompt_support(cs_plan *plan, const float *S, const float *Phi, flo
     if (!isfinite(mu) || !(mu > 0.f)) return CS_ERR_NONFINITE;
     if (!aligned16(S) || !aligned16(H)) return CS_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cs_status s = launch_prompt_mean(plan, H, n, plan->hbar, st);
+    int blocks = 0;
+    cs_status s = launch_prompt_colsum(plan, H, n, &blocks, st);
     if (s != CS_OK) return s;
-    return launch_sense_recover(plan, S, Phi, mu, plan->hbar, nullptr, 1, nullptr, support, z, resid, st);
+    return launch_sense_recover(plan, S, Phi, mu, plan->colsum, nullptr, 1, nullptr, support, z, resid, st, RecoverOptions(), blocks, n);
 }
 
 cs_status cs_ffn_exec_shared(cs_plan *plan, const cs_layer *layer, const void *H, int32_t n,
@@ -579,9 +579,7 @@ cs_status cs_ffn_exec_shared(cs_plan *plan, const cs_layer *layer, const void *H
     if (n <= 0 || n > plan->cfg.max_tokens) return CS_ERR_SHAPE;
     if (!plan->mma_ok || !aligned16(H) || !aligned16(out)) return CS_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    s = launch_check_support(plan, support, 1, st);
-    if (s != CS_OK) return s;
-    return launch_ffn_mma(plan, layer, H, nullptr, n, support, nullptr, plan->cfg.k, nullptr, nullptr, nullptr, out, st);
+    return launch_ffn_mma(plan, layer, H, nullptr, n, support, nullptr, plan->cfg.k, nullptr, nullptr, nullptr, out, st);   // checks the support
 }
 
 cs_status cs_last_device_status(cs_plan *plan, void *stream, int32_t *code) {

@@ -46,8 +46,7 @@ struct cs_plan {
     int32_t *fb_count;    // [1] their number
     int32_t *slot_table;  // [max_tokens, kSlotTablePitch] small-batch step: slot -> group of the recovery in flight
     unsigned *ticket;     // [max_tokens] arrival counters of the sketch CTAs (zero between launches)
-    float *hbar;       // [d] mean prompt hidden state
-    float *colsum;     // [mean_row_blocks, d]
+    float *colsum;     // [kMeanRowBlocks, d] column sums of a prompt's hidden states, per block of rows
     cs::DeviceStatus *status;  // device status word
     // tensor-core path (bf16 weights, 128-channel groups, d a multiple of 256)
     uint32_t *mask;      // [max_tokens, 4] membership bits: bit g of token t
@@ -62,16 +61,15 @@ struct cs_plan {
     int speculative;     // small batches, on the recovery's first iterate: 1 = start the weight stream, 2 = warm L2 only
     int mma_ok;          // shape qualifies for the tensor-core path
     int mma_min_tokens;  // smallest decode batch that takes it
-    int mma_slices;      // most list slices the down GEMM is split into
     int last_slices;
     int pair_key_ng, pair_key_mtiles, pair_count;   // prompt gate/up: paired-tile count of the last shape seen
+    int mma_slices;      // most list slices the down GEMM is split into
     float *x_host_in;  // [max_tokens, d] staging for the host-buffer entry point
     float *x_host_out; // [max_tokens, d]
     cudaEvent_t ev[2 * CS_STAGE_COUNT];  // start/stop per stage
     int timing;
     int stage_seen[CS_STAGE_COUNT];
     int nx_max;
-    int mean_row_blocks;
     int64_t launches;
     char cuda_error[256];
 };
@@ -152,11 +150,12 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
 cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float *y, int B,
                          int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st,
                          const RecoverOptions &opt = RecoverOptions());
-// Sensor and estimator in one launch, a cluster of CTAs per token, for at most kSenseMaxTokens tokens.
+// Sensor and estimator in one launch, a cluster of CTAs per token, for at most kSenseMaxTokens tokens.  blocks > 0: one
+// token whose x is the sum of `blocks` rows [blocks, d] divided by n (a prompt's mean hidden state).
 constexpr int kSenseMaxTokens = 16;
 cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,
                                float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st,
-                               const RecoverOptions &opt = RecoverOptions());
+                               const RecoverOptions &opt = RecoverOptions(), int blocks = 0, int n = 1);
 // the other estimators (solvers.cu)
 cs_status prepare_solvers(cs_plan *plan);
 cs_status launch_niht(cs_plan *plan, const float *Phi, float mu_fallback, const float *y, int B, int T,
@@ -209,7 +208,10 @@ cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *suppo
 bool decode_recovers(const cs_plan *plan);
 cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool x_ready, bool norm,
                             const float *residual, float *out, cudaStream_t st);
-cs_status launch_prompt_mean(cs_plan *plan, const void *H, int n, float *hbar, cudaStream_t st);
+// Column sums of H per block of rows (plan->colsum); *blocks = their number.
+constexpr int kMeanRowBlocks = 16;
+cs_status prepare_prompt(cs_plan *plan);
+cs_status launch_prompt_colsum(cs_plan *plan, const void *H, int n, int *blocks, cudaStream_t st);
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may start while its
 // predecessor in the stream is still running (its CTAs become resident, run their prologue and
@@ -306,15 +308,6 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
-}
-
-// 16-byte read-only streaming load (weights are read once per step: keep them out of L1).
-__device__ __forceinline__ uint4 ldg_stream(const void *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-                 : "l"(p));
-    return r;
 }
 
 // Four floats as bf16 values and bf16 remainders: hi = round(x), lo = round(x - hi).

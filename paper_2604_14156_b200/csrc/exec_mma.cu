@@ -186,6 +186,14 @@ ffn_gateup_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     epilogue_done(t, warp);
 }
 
+// A support given by the caller: ascending, hence distinct, and in range.
+__device__ __forceinline__ void check_list(const int32_t *glist, int ng, int G, DeviceStatus *status) {
+    const int j = threadIdx.x;
+    if (j >= ng) return;
+    const int g = ld_dep(glist + j);
+    if (g < 0 || g >= G || (j > 0 && ld_dep(glist + j - 1) >= g)) atomicCAS(&status->code, 0, (int)CS_ERR_SUPPORT);
+}
+
 // ---- gate / up for one shared support (the prompt-level variant): single and paired token tiles ---------
 // A 128 x 256 tile with both operands streamed per 64-wide k block takes in 0.0117 bytes per flop, which at
 // the rate of the tensor pipe is more than the SMs can take in from L2 (the kernel above sits at 13.5 TB/s
@@ -197,7 +205,7 @@ ffn_gateup_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 // Pair slot q = (group q % ng, token tiles 2 (q / ng) and 2 (q / ng) + 1).
 __global__ void __launch_bounds__(kTileThreads, 1)
 ffn_gateup_tiles_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_g,
-                        const __grid_constant__ CUtensorMap tm_u, const int32_t *__restrict__ glist, int ng, int n_pair,
+                        const __grid_constant__ CUtensorMap tm_u, const int32_t *glist, int ng, int G, int n_pair,
                         int mtiles, int M, int d, int act_ld, __nv_bfloat16 *__restrict__ act, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     const int c = blockIdx.x;
@@ -206,7 +214,10 @@ ffn_gateup_tiles_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_c
     const int gi = q % ng, mt0 = 2 * (q / ng) + (pair ? 0 : ((c - n_pair) & 1));
     if (mt0 >= mtiles) return;                                   // the odd half of a last, incomplete pair slot
     const int ntile = (pair && mt0 + 1 < mtiles) ? 2 : 1;
-    const int g = glist[gi];
+    pdl_wait();   // the support, and H
+    pdl_launch_dependents();
+    if (c == 0) check_list(glist, ng, G, status);
+    const int g = ld_dep(glist + gi);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     Barriers *bars = reinterpret_cast<Barriers *>(base + kRingBytesMma);
@@ -349,7 +360,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
 // two slots later, once all epilogue warps of BOTH CTAs have arrived on its `acc_empty` barrier in the even CTA.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTileThreads, 1)
 ffn_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_g,
-                       const __grid_constant__ CUtensorMap tm_u, const int32_t *__restrict__ glist, int ng, int slots,
+                       const __grid_constant__ CUtensorMap tm_u, const int32_t *glist, int ng, int G, int slots,
                        int M, int d, int act_ld, __nv_bfloat16 *__restrict__ act, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t rank = cluster_ctarank();                  // 0: gate half, issues the MMAs; 1: up half
@@ -377,6 +388,9 @@ ffn_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
     tc_fence_after();
     const int kblocks = d / BK;
 
+    pdl_wait();   // the support, and H
+    pdl_launch_dependents();
+    if (blockIdx.x == 0) check_list(glist, ng, G, status);
     if (warp == 0) {
         if (lane == 0) {
             const uint32_t full0 = map_to_cta(smem_u32(&bars->full[0]), 0);   // the even CTA's full barriers
@@ -384,7 +398,7 @@ ffn_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
             int s = 0, ph = 1, it = 0;
             bool ok = true;
             for (int q = c0; q < slots && ok; q += nc) {
-                const int g = glist[q % ng], mt = 2 * (q / ng) + (int)rank;
+                const int g = ld_dep(glist + q % ng), mt = 2 * (q / ng) + (int)rank;
                 for (int kb = 0; kb < kblocks; ++kb, ++s, ++it) {
                     if (s == kPairStages) { s = 0; ph ^= 1; }
                     if (it >= kPairStages && !mbar_wait(&bars->empty[s], ph, bars, status)) { ok = false; break; }
@@ -474,7 +488,7 @@ ffn_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
 template <bool SPLIT>
 __global__ void __launch_bounds__(kTileThreads, 1)
 ffn_down_mma_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_act_lo,
-                    const __grid_constant__ CUtensorMap tm_wd, const int32_t *__restrict__ glist,
+                    const __grid_constant__ CUtensorMap tm_wd, const int32_t *glist,
                     const int32_t *__restrict__ ng_dev, int ng_host, int M, int m_pad, int d,
                     float *__restrict__ partial, const float *residual, float *out_f32,
                     __nv_bfloat16 *__restrict__ out_bf16, DeviceStatus *status) {
@@ -487,9 +501,11 @@ ffn_down_mma_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
     const Tiles<SPLIT> t = carve<SPLIT>(smem_raw);
     prologue(t, warp, lane);
     const int kblocks = (gi1 - gi0) * 2;   // two 64-row k blocks per 128-channel group
+    pdl_launch_dependents();
 
     if (warp == 0) {
         if (lane == 0) {
+            pdl_wait();   // the activations
             for (int kb = 0; kb < kblocks; ++kb) {
                 const int s = kb % kStages;
                 if (kb >= kStages && !mbar_wait(&t.bars->empty[s], ((kb / kStages) - 1) & 1, t.bars, status)) break;
@@ -506,6 +522,7 @@ ffn_down_mma_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
     } else if (warp == 1) {
         if (lane == 0 && kblocks > 0) mma_loop<true, SPLIT>(t, kblocks, status);
     } else {
+        pdl_wait();   // nothing is stored before the kernels before this one are complete
         const int q = warp & 3;
         const int slice = (warp - 2) >> 2, nslice = ((int)(blockDim.x >> 5) - 2) >> 2;
         const int row = q * 32 + lane, m = mt * BM + row;
@@ -574,7 +591,7 @@ constexpr int kWideStages = kRingBytesMma / kWideStage;  // 3
 
 __global__ void __launch_bounds__(kTileThreads, 1)
 ffn_down_wide_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_wd,
-                     const int32_t *__restrict__ glist, const int32_t *__restrict__ ng_dev, int ng_host, int M, int d,
+                     const int32_t *glist, const int32_t *__restrict__ ng_dev, int ng_host, int M, int d,
                      const float *residual, float *out_f32, __nv_bfloat16 *__restrict__ out_bf16, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     const int nt = blockIdx.x, mt = blockIdx.y;
@@ -584,9 +601,11 @@ ffn_down_wide_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_co
     Barriers *bars = reinterpret_cast<Barriers *>(base + kRingBytesMma);
     setup_cta(bars, warp, 512);
     const int kblocks = ng * 2;   // two 64-row k blocks per 128-channel group
+    pdl_launch_dependents();
 
     if (warp == 0) {
         if (lane == 0) {
+            pdl_wait();   // the activations
             for (int kb = 0; kb < kblocks; ++kb) {
                 const int s = kb % kWideStages;
                 if (kb >= kWideStages && !mbar_wait(&bars->empty[s], ((kb / kWideStages) - 1) & 1, bars, status)) break;
@@ -622,6 +641,7 @@ ffn_down_wide_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_co
             if (ok) tc_commit(&bars->acc_ready);
         }
     } else {
+        pdl_wait();   // nothing is stored before the kernels before this one are complete
         const int q = warp & 3;
         const int slice = (warp - 2) >> 2, nslice = ((int)(blockDim.x >> 5) - 2) >> 2;
         const int m = mt * BM + q * 32 + lane;
@@ -885,12 +905,12 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
             // one shared support and no gain from paired tiles (measured at k = 27 of 108 groups, 2048 tokens:
             // 214 us for the GEMM pair against 223 us with single tiles; with paired tiles in play, k = 11 and
             // 54, the mixed launch below is faster): CTA pairs, one M = 256 instruction over two token tiles
-            ffn_gateup_pair_kernel<<<dim3(2 * min(slots, plan->sm_count / 2)), kTileThreads, kMmaSmem, st>>>(
-                tm_x, tm_g, tm_u, glist, ng_host, slots, M, c.d, act_ld, act, plan->status);
+            launch_pdl(true, ffn_gateup_pair_kernel, dim3(2 * min(slots, plan->sm_count / 2)), dim3(kTileThreads), kMmaSmem, st, tm_x, tm_g,
+                       tm_u, glist, ng_host, plan->G, slots, M, c.d, act_ld, act, plan->status);
         } else if (n_pair > 0) {
             // one shared support, its size known on the host: paired and single token tiles in one launch
-            ffn_gateup_tiles_kernel<<<dim3(n_pair + 2 * (slots - n_pair)), kTileThreads, kMmaSmem, st>>>(
-                tm_x, tm_g, tm_u, glist, ng_host, n_pair, mtiles, M, c.d, act_ld, act, plan->status);
+            launch_pdl(true, ffn_gateup_tiles_kernel, dim3(n_pair + 2 * (slots - n_pair)), dim3(kTileThreads), kMmaSmem, st, tm_x, tm_g, tm_u,
+                       glist, ng_host, plan->G, n_pair, mtiles, M, c.d, act_ld, act, plan->status);
         } else
             ffn_gateup_mma_kernel<false><<<dim3(grid_g, mtiles), kTileThreads, kMmaSmem, st>>>(
                 tm_x, tm_x_lo, tm_g, tm_u, glist, ng_dev, ng_host, M, c.d, act_ld, mask, act, act_lo, plan->status);
@@ -905,16 +925,16 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
         const bool wide = !split && Z == 1 && c.d % BNW == 0 && ng_host > 0 &&
                           ((mtiles * (c.d / BNW) + sms - 1) / sms) * BNW < ((mtiles * ntiles + sms - 1) / sms) * BN;
         if (wide)
-            ffn_down_wide_kernel<<<dim3(c.d / BNW, mtiles), kTileThreads, kMmaSmem, st>>>(
-                tm_act, tm_wd, glist, ng_dev, ng_host, M, c.d, residual, out_f32, static_cast<__nv_bfloat16 *>(out_bf16), plan->status);
+            launch_pdl(true, ffn_down_wide_kernel, dim3(c.d / BNW, mtiles), dim3(kTileThreads), kMmaSmem, st, tm_act, tm_wd, glist, ng_dev,
+                       ng_host, M, c.d, residual, out_f32, static_cast<__nv_bfloat16 *>(out_bf16), plan->status);
         else if (split)
             ffn_down_mma_kernel<true><<<dim3(ntiles, mtiles, Z), kTileThreads, kMmaSmem, st>>>(
                 tm_act, tm_act_lo, tm_wd, glist, ng_dev, ng_host, M, m_pad, c.d, plan->mma_partial, residual, out_f32,
                 static_cast<__nv_bfloat16 *>(out_bf16), plan->status);
         else
-            ffn_down_mma_kernel<false><<<dim3(ntiles, mtiles, Z), kTileThreads, kMmaSmem, st>>>(
-                tm_act, tm_act_lo, tm_wd, glist, ng_dev, ng_host, M, m_pad, c.d, plan->mma_partial, residual, out_f32,
-                static_cast<__nv_bfloat16 *>(out_bf16), plan->status);
+            launch_pdl(true, ffn_down_mma_kernel<false>, dim3(ntiles, mtiles, Z), dim3(kTileThreads), kMmaSmem, st, tm_act, tm_act_lo, tm_wd,
+                       glist, ng_dev, ng_host, M, m_pad, c.d, plan->mma_partial, residual, out_f32, static_cast<__nv_bfloat16 *>(out_bf16),
+                       plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
         plan->last_slices = Z;

@@ -42,18 +42,21 @@ __global__ void __launch_bounds__(32 * NW) recover_kernel(const __grid_constant_
 // CTA 0 (every CTA forms an eighth of M), so between x and the sketch lie one load of x, the dot products, and one
 // exchange over distributed shared memory; CTA 0 then runs the iteration with every operand in its shared memory.
 // Bound by latency.  As two launches, with M formed by the first and read from L2 by the second, the pair took
-// 15 us of a step at 7B, batch 1 (to the gather kernel), in this form 11.5 us.
+// 15 us of a step at 7B, batch 1 (to the gather kernel), in this form 10 us (26.1 us for the step against 29.8).
 constexpr int kSenseCtas = 8;
 constexpr int kSenseThreads = 256;
 constexpr int kSenseWarps = kSenseThreads / 32;
 constexpr int kSenseMaxChunks = kMaxD / kSenseCtas / 4 / 32;   // float4 columns per lane
 constexpr int kSenseSmem = 220 * 1024;                         // dynamic, at most
+constexpr int kSenseExtra = 1;                                 // rows of S a warp keeps in registers
 
 struct SenseArgs {
     const float *S, *x, *gamma;
     float eps;
     int d, s_rows;        // s_rows: rows of S that fit in shared memory (the others are read after the wait)
     float *y_out, *n_out;
+    int blocks;           // > 0: x is [blocks, d], and what is sensed is the sum of its rows times inv_n
+    float inv_n;
 };
 
 __device__ __forceinline__ uint32_t remote_smem(const void *p, uint32_t rank) {   // the same place in CTA `rank` of the cluster
@@ -79,42 +82,59 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     const int m = a.m, G = a.G, d = sa.d;
     const int nc = d / (4 * kSenseCtas);            // float4 columns of this CTA
     const size_t col0 = (size_t)rank * nc * 4;
-    float *M_s = reinterpret_cast<float *>(sense_s), *phi_s = M_s + G * GP;
-    float4 *S_s = reinterpret_cast<float4 *>(phi_s + m * (GP + 4));
+    const int pitch = (G + 3) & ~3, ppitch = pitch + 4;
+    float *M_s = reinterpret_cast<float *>(sense_s), *phi_s = M_s + G * pitch;
+    float4 *S_s = reinterpret_cast<float4 *>(phi_s + m * ppitch);
     pdl_launch_dependents();
     cluster_arrive();                               // matched below: every CTA of the cluster has started
     // this lane's chunks of this warp's rows of S: no other thread reads them
     for (int r = warp; r < sa.s_rows; r += kSenseWarps)
+#pragma unroll 4
         for (int c = lane; c < nc; c += 32) {
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(S_s + r * nc + c);
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(sa.S + (size_t)r * d + col0 + 4 * c) : "memory");
         }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    float4 gm[kSenseMaxChunks];
-    if (sa.gamma != nullptr) {
+    const int nch = (nc + 31) / 32;
+    // rows of S without a place there: the warp's next in registers, what is left in L2 at least
+    float4 ex[kSenseExtra][kSenseMaxChunks];
+    const int x0 = sa.s_rows + ((warp - sa.s_rows) & (kSenseWarps - 1));   // this warp's first such row
+#pragma unroll
+    for (int q = 0; q < kSenseExtra; ++q)
 #pragma unroll
         for (int j = 0; j < kSenseMaxChunks; ++j)
-            if (lane + 32 * j < nc) gm[j] = __ldg(reinterpret_cast<const float4 *>(sa.gamma + col0) + lane + 32 * j);
-    }
-    for (int i = tid; i < m * GP; i += kSenseThreads) {
-        const int row = i / GP, g = i - row * GP;
-        phi_s[row * (GP + 4) + g] = g < G ? __ldg(a.Phi + row * G + g) : 0.f;
+            if (x0 + q * kSenseWarps < m && j < nch)
+                ex[q][j] = __ldg(reinterpret_cast<const float4 *>(sa.S + (size_t)(x0 + q * kSenseWarps) * d + col0) + min(lane + 32 * j, nc - 1));
+    for (int r = sa.s_rows + kSenseExtra * kSenseWarps + tid; r < m; r += kSenseThreads)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(sa.S + (size_t)r * d + col0), "r"(nc * 16) : "memory");
+    for (int i0 = tid; i0 < m * GP; i0 += 8 * kSenseThreads) {   // eight loads in flight: addresses clamped, no branches
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = min(i0 + u * kSenseThreads, m * GP - 1);
+            v[u] = __ldg(a.Phi + i / GP * G + min(i % GP, G - 1));
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * kSenseThreads, g = i % GP;
+            if (i < m * GP && g < pitch) phi_s[i / GP * ppitch + g] = g < G ? v[u] : 0.f;
+        }
     }
     __syncthreads();
     float phc[32];
     if (rank == 0 && m <= 32 && tid < GP) {
 #pragma unroll
-        for (int row = 0; row < 32; ++row) phc[row] = row < m ? phi_s[row * (GP + 4) + tid] : 0.f;
+        for (int row = 0; row < 32; ++row) phc[row] = row < m && tid < G ? phi_s[row * ppitch + tid] : 0.f;
     }
     cluster_wait();
     // M in blocks of 2 x 4 entries, each summed as gram_rows sums it; every eighth row pair is this CTA's
     const uint32_t M0 = remote_smem(M_s, 0);
-    for (int b = tid; b < ((G + 1) / 2 - rank + kSenseCtas - 1) / kSenseCtas * (GP / 4); b += kSenseThreads) {
-        const int i0 = (b / (GP / 4) * kSenseCtas + rank) * 2, j0 = b % (GP / 4) * 4;
+    for (int b = tid; b < ((G + 1) / 2 - rank + kSenseCtas - 1) / kSenseCtas * (pitch / 4); b += kSenseThreads) {
+        const int i0 = (b / (pitch / 4) * kSenseCtas + rank) * 2, j0 = b % (pitch / 4) * 4;
         float s0[2][4] = {}, s1[2][4] = {};
         auto add = [&](int row, float (&s)[2][4]) {
-            const float2 p = *reinterpret_cast<const float2 *>(phi_s + row * (GP + 4) + i0);
-            const float4 q = *reinterpret_cast<const float4 *>(phi_s + row * (GP + 4) + j0);
+            const float2 p = *reinterpret_cast<const float2 *>(phi_s + row * ppitch + i0);
+            const float4 q = *reinterpret_cast<const float4 *>(phi_s + row * ppitch + j0);
             s[0][0] = fmaf(p.x, q.x, s[0][0]); s[0][1] = fmaf(p.x, q.y, s[0][1]); s[0][2] = fmaf(p.x, q.z, s[0][2]); s[0][3] = fmaf(p.x, q.w, s[0][3]);
             s[1][0] = fmaf(p.y, q.x, s[1][0]); s[1][1] = fmaf(p.y, q.y, s[1][1]); s[1][2] = fmaf(p.y, q.z, s[1][2]); s[1][3] = fmaf(p.y, q.w, s[1][3]);
         };
@@ -128,45 +148,89 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
             float o[4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) o[v] = j0 + v < G ? (i0 + u == j0 + v ? 1.f : 0.f) - a.mu * (s0[u][v] + s1[u][v]) : 0.f;
-            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(M0 + 4u * ((i0 + u) * GP + j0)), "f"(o[0]), "f"(o[1]),
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(M0 + 4u * ((i0 + u) * pitch + j0)), "f"(o[0]), "f"(o[1]),
                          "f"(o[2]), "f"(o[3]) : "memory");
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     pdl_wait();   // x may be the previous kernel's output
-    float4 xv[kSenseMaxChunks];
+    float4 xv[kSenseMaxChunks], gm[kSenseMaxChunks];
     float ss = 0.f;
+    if (sa.gamma != nullptr) {
 #pragma unroll
-    for (int j = 0; j < kSenseMaxChunks; ++j)
-        xv[j] = lane + 32 * j < nc ? ld_dep4(sa.x + (size_t)t * d + col0 + 4 * (lane + 32 * j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < kSenseMaxChunks; ++j)
+            if (j < nch) gm[j] = __ldg(reinterpret_cast<const float4 *>(sa.gamma + col0) + min(lane + 32 * j, nc - 1));
+    }
+    if (sa.blocks > 0) {   // every column is summed once, for all warps
+        float4 *sum_s = S_s + sa.s_rows * nc;
+        for (int c = tid; c < nc; c += kSenseThreads) {
+            float4 v[kMeanRowBlocks], s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int b = 0; b < kMeanRowBlocks; ++b)
+                v[b] = b < sa.blocks ? ld_dep4(sa.x + (size_t)b * d + col0 + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int b = 0; b < kMeanRowBlocks; ++b) { s.x += v[b].x; s.y += v[b].y; s.z += v[b].z; s.w += v[b].w; }
+            sum_s[c] = make_float4(s.x * sa.inv_n, s.y * sa.inv_n, s.z * sa.inv_n, s.w * sa.inv_n);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kSenseMaxChunks; ++j) xv[j] = lane + 32 * j < nc ? sum_s[lane + 32 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+#pragma unroll
+        for (int j = 0; j < kSenseMaxChunks; ++j)
+            xv[j] = lane + 32 * j < nc ? ld_dep4(sa.x + (size_t)t * d + col0 + 4 * (lane + 32 * j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 #pragma unroll
     for (int j = 0; j < kSenseMaxChunks; ++j) {
         ss += xv[j].x * xv[j].x + xv[j].y * xv[j].y + xv[j].z * xv[j].z + xv[j].w * xv[j].w;
-        if (sa.gamma != nullptr && lane + 32 * j < nc) { xv[j].x *= gm[j].x; xv[j].y *= gm[j].y; xv[j].z *= gm[j].z; xv[j].w *= gm[j].w; }
+        if (sa.gamma != nullptr && j < nch) { xv[j].x *= gm[j].x; xv[j].y *= gm[j].y; xv[j].z *= gm[j].z; xv[j].w *= gm[j].w; }
     }
-#pragma unroll 1
-    for (int r0 = warp; r0 < m; r0 += 4 * kSenseWarps) {   // four rows at a time: their reductions interleave
-        float acc[4] = {};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * kSenseWarps;
-            if (r >= m) break;
-#pragma unroll
-            for (int j = 0; j < kSenseMaxChunks; ++j) {
-                const int c = lane + 32 * j;
-                if (c >= nc) break;
-                const float4 s = r < sa.s_rows ? S_s[r * nc + c] : __ldg(reinterpret_cast<const float4 *>(sa.S + (size_t)r * d + col0) + c);
-                acc[q] = fmaf(s.x, xv[j].x, acc[q]); acc[q] = fmaf(s.y, xv[j].y, acc[q]);
-                acc[q] = fmaf(s.z, xv[j].z, acc[q]); acc[q] = fmaf(s.w, xv[j].w, acc[q]);
-            }
-        }
+    auto dot = [](const float4 &s, const float4 &v, float a) { return fmaf(s.w, v.w, fmaf(s.z, v.z, fmaf(s.y, v.y, fmaf(s.x, v.x, a)))); };
+    // four rows: their reductions interleave; lane q stores row q's
+    auto finish = [&](float (&acc)[4], int r0, int end) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q] = warp_sum(acc[q]);
         if (lane < 4) {
             const int r = r0 + lane * kSenseWarps;
             const float v = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
-            if (r < m) st_remote(remote_smem(&part_s[rank][r], 0), v);
+            if (r < end) st_remote(remote_smem(&part_s[rank][r], 0), v);
         }
+    };
+    // (columns past nc repeat the last one with x = 0, rows past the last repeat it and are not stored)
+#pragma unroll 1
+    for (int r0 = warp; r0 < sa.s_rows; r0 += 4 * kSenseWarps) {
+        float acc[4] = {};
+        const float4 *row[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) row[q] = S_s + min(r0 + q * kSenseWarps, r0 + (sa.s_rows - 1 - r0) / kSenseWarps * kSenseWarps) * nc;
+#pragma unroll
+        for (int j = 0; j < kSenseMaxChunks; ++j) {
+            if (j >= nch) break;
+            const int c = min(lane + 32 * j, nc - 1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q] = dot(row[q][c], xv[j], acc[q]);
+        }
+        finish(acc, r0, sa.s_rows);
+    }
+#pragma unroll 1
+    for (int r0 = x0; r0 < m; r0 += 4 * kSenseWarps) {
+        float acc[4] = {};
+        if (r0 == x0) {
+#pragma unroll
+            for (int q = 0; q < kSenseExtra; ++q)
+#pragma unroll
+                for (int j = 0; j < kSenseMaxChunks; ++j)
+                    if (x0 + q * kSenseWarps < m && j < nch) acc[q] = dot(ex[q][j], xv[j], acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + q * kSenseWarps;
+            if (r >= m || (r0 == x0 && q < kSenseExtra)) continue;
+#pragma unroll
+            for (int j = 0; j < kSenseMaxChunks; ++j)
+                if (j < nch) acc[q] = dot(__ldg(reinterpret_cast<const float4 *>(sa.S + (size_t)r * d + col0) + min(lane + 32 * j, nc - 1)), xv[j], acc[q]);
+        }
+        finish(acc, r0, m);
     }
     if (warp == 0 && sa.gamma != nullptr) {
         ss = warp_sum(ss);
@@ -191,7 +255,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     if (rank != 0 || tid >= GP) return;
     const int g = tid;
     recover_row<NW, KC, 1>(
-        rs, a, SharedSource<GP>{M_s, phi_s, G},
+        rs, a, SharedSource{M_s, phi_s, G, pitch},
         [&](auto &sm) {
             for (int i = g; i < m; i += GP) {
                 float y = 0.f;
@@ -268,14 +332,15 @@ static SenseFn sense_fn(int G, int k) {
 }
 
 cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,
-                               float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st, const RecoverOptions &o) {
+                               float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st, const RecoverOptions &o, int blocks,
+                               int n) {
     const cs_config &c = plan->cfg;
-    const int GP = gram_pitch(plan->G), row_bytes = c.d / kSenseCtas * 4;
-    const int fixed = (plan->G * GP + c.m * (GP + 4)) * 4;
-    SenseArgs sa{S, x, gamma, c.rms_eps, c.d, min(c.m, (kSenseSmem - fixed) / row_bytes), plan->y_buf, n_out};
+    const int pitch = (plan->G + 3) & ~3, row_bytes = c.d / kSenseCtas * 4;
+    const int fixed = (plan->G * pitch + c.m * (pitch + 4)) * 4;
+    SenseArgs sa{S, x, gamma, c.rms_eps, c.d, min(c.m, (kSenseSmem - fixed) / row_bytes - 1), plan->y_buf, n_out, blocks, 1.f / (float)n};
     {
         StageTimer timer(plan, CS_STAGE_SKETCH, st);
-        launch_pdl(true, sense_fn(plan->G, c.k), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)sa.s_rows * row_bytes, st,
+        launch_pdl(true, sense_fn(plan->G, c.k), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)(sa.s_rows + (blocks > 0)) * row_bytes, st,
                    sa, recover_args(plan, Phi, mu, nullptr, B, support, z, resid, o));
     }
     plan->launches++;

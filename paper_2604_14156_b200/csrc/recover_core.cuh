@@ -57,7 +57,7 @@ template <int NW, int KC> struct RecoverSmem {
     alignas(16) float part[GP];       // partial sums while y is put together
     alignas(16) float red[kMaxM];     // residual r of the two-step form; partial sums of the residual norm
     alignas(16) float val[2][NV];     // the iterate, by iteration parity: slot values, or dense z
-    int idx[NV];                      // list form: entry held by each slot (the support, in slot order)
+    alignas(16) int idx[NV];          // list form: entry held by each slot (the support, in slot order)
     alignas(16) float y[kMaxM];       // zero past m
     uint32_t mm[2][2][4];             // per parity: min kept key / max other key, per warp
     int sum[4];                       // rank sums per warp
@@ -77,6 +77,7 @@ template <int NW, int KC> struct RecoverSmem {
 //   of the first support are formed together with 32 * NW helper threads (PhiSource::help), which
 //   take every other slot and hand their values over through shared memory.
 struct GramSource {
+    static constexpr bool kRefill = false;
     const float *gram;
     int pitch;
     __device__ __forceinline__ float get(int j, int g, const float (&)[32]) const {
@@ -107,29 +108,30 @@ struct GramSource {
             if ((chg >> j) & 1ull) mreg[j] = get(idx[j], g, own);
     }
 };
-//   SharedSource: the matrix in shared memory, [G][GP], columns past G zero, and Phi beside it, [m][GP + 4].
-template <int GP_> struct SharedSource {
+//   SharedSource: the matrix in shared memory, [G][pitch], and Phi beside it, [m][pitch + 4], pitch = G rounded up to 4
+//   (threads past G read what follows their row, and nobody reads them).
+//   A change of the support reads the entries of all slots again: that takes 0.1 us, less than finding out which changed.
+struct SharedSource {
+    static constexpr bool kRefill = true;
     const float *M_s, *phi_s;
-    int G;
-    __device__ __forceinline__ float phi(const float *, int row, int col, int) const { return phi_s[row * (GP_ + 4) + col]; }
+    int G, pitch;
+    __device__ __forceinline__ float phi(const float *, int row, int col, int) const { return phi_s[row * (pitch + 4) + col]; }
     template <int GP> __device__ __forceinline__ void row(int g, float (&mreg)[GP]) const {
 #pragma unroll
-        for (int j = 0; j < GP; ++j) mreg[j] = j < G ? M_s[j * GP + g] : 0.f;
+        for (int j = 0; j < GP; ++j) mreg[j] = j < G ? M_s[j * pitch + g] : 0.f;
     }
-    template <int NR> __device__ __forceinline__ void fill(const int *idx, int k, int, int g, const float (&)[32],
-                                                           float (&mreg)[NR]) const {
+    // (slots past k hold entry 0, and the value 0)
+    template <int NR> __device__ __forceinline__ void fill(const int *idx, int, int, int g, const float (&)[32], float (&mreg)[NR]) const {
 #pragma unroll
-        for (int j = 0; j < NR; ++j)
-            if (j < k) mreg[j] = M_s[idx[j] * GP_ + g];
-    }
-    template <int NR> __device__ __forceinline__ void reload(unsigned long long chg, const int *idx, int g,
-                                                             const float (&)[32], float (&mreg)[NR]) const {
-#pragma unroll
-        for (int j = 0; j < NR; ++j)
-            if ((chg >> j) & 1ull) mreg[j] = M_s[idx[j] * GP_ + g];
+        for (int j = 0; j < NR; j += 4) {
+            const int4 e = *reinterpret_cast<const int4 *>(idx + j);
+            mreg[j] = M_s[e.x * pitch + g]; mreg[j + 1] = M_s[e.y * pitch + g];
+            mreg[j + 2] = M_s[e.z * pitch + g]; mreg[j + 3] = M_s[e.w * pitch + g];
+        }
     }
 };
 template <int BAR_A, int BAR_B, int THREADS> struct PhiSource {
+    static constexpr bool kRefill = false;
     const float4 *phiT_s;   // shared memory, [G][8] float4
     float mu;
     float *fill_s;          // shared memory, [slots][THREADS / 2]
@@ -385,17 +387,20 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
             kept = kept_new;
             if (kept) s.val[par ^ 1][slot] = v;
             unsigned long long chg = 0ull;   // slots whose entry changed
-            if (first) {
-                chg = k >= 64 ? ~0ull : (1ull << k) - 1ull;
-            } else {
+            if constexpr (!MSource::kRefill) {
+                if (first) {
+                    chg = k >= 64 ? ~0ull : (1ull << k) - 1ull;
+                } else {
 #pragma unroll
-                for (int w = 0; w < NW; ++w)
-                    for (int i = 0; i < s.cnt[w]; ++i) chg |= 1ull << s.vac[w][i];
+                    for (int w = 0; w < NW; ++w)
+                        for (int i = 0; i < s.cnt[w]; ++i) chg |= 1ull << s.vac[w][i];
+                }
             }
             bar_sync<BAR, GP>();
             if (first) table_ready();   // the table holds the first iterate's support
-            if (first) M.fill(s.idx, k, g, gm, phc, mreg);   // the entries of all k slots
-            else M.reload(chg, s.idx, gm, phc, mreg);        // those of the slots that changed hands
+            if constexpr (MSource::kRefill) M.fill(s.idx, k, g, gm, phc, mreg);
+            else if (first) M.fill(s.idx, k, g, gm, phc, mreg);   // the entries of all k slots
+            else M.reload(chg, s.idx, gm, phc, mreg);             // those of the slots that changed hands
         }
     }
     table_final();
@@ -408,8 +413,13 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
             float ss = 0.f;
             for (int row = g; row < m; row += GP) {
                 float a = 0.f;
-#pragma unroll 8
-                for (int j = 0; j < k; ++j) a = fmaf(M.phi(Phi, row, s.idx[j], G), s.val[T & 1][j], a);
+#pragma unroll 4
+                for (int j = 0; j < NV; j += 4) {   // slots past k hold zeros
+                    const int4 e = *reinterpret_cast<const int4 *>(s.idx + j);
+                    const float4 v4 = *reinterpret_cast<const float4 *>(s.val[T & 1] + j);
+                    a = fmaf(M.phi(Phi, row, e.x, G), v4.x, a); a = fmaf(M.phi(Phi, row, e.y, G), v4.y, a);
+                    a = fmaf(M.phi(Phi, row, e.z, G), v4.z, a); a = fmaf(M.phi(Phi, row, e.w, G), v4.w, a);
+                }
                 const float r = s.y[row] - a;
                 ss = fmaf(r, r, ss);
             }

@@ -1,0 +1,41 @@
+"""GPU parity of the launch that senses and recovers a token on a cluster of CTAs, at the sizes where its split can go wrong."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2604_14156_b200 as cs
+from gen import workloads as W
+from parity_util import compare_layer_step, make_plan, recovery_matches
+
+pytestmark = pytest.mark.gpu
+
+
+# d: slices of two float4 columns, a ragged and a full last chunk per lane, the widest; m: fewer rows than warps, odd, rows of S
+# that do not fit in shared memory beside a large M (8192 x 64); G: padded to 4, all four warps; k: the list form's lengths
+# and the dense form; 16 and 17 tokens: the last batch on clusters and the first beyond.
+@pytest.mark.parametrize("d,G,m,k,B,norm", [(64, 2, 1, 1, 1, False), (192, 5, 5, 2, 16, True), (320, 33, 7, 9, 17, False),
+                                            (4096, 50, 33, 24, 2, True), (5120, 108, 64, 57, 1, False), (8192, 128, 64, 32, 2, True)])
+def test_layer_step_sense_cluster_edges(d, G, m, k, B, norm):
+    cfg = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"].with_(
+        n_layers=1, w_dtype="f32", d=d, d_ff=64 * G, group=64, m=m, k=k, T=7, B=B, index=400 + G)
+    L = W.make_layer(cfg, device="cuda:0")
+    tk = W.make_tokens(cfg, L.A)
+    plan = make_plan(cfg)
+    rep, _, _ = compare_layer_step(cfg, L, plan, tk.h)   # output bound 1e-5 (parity_util): f32 weights
+    assert rep.excused <= max(1, B // 16), rep
+    plan.close()
+
+
+# prompt lengths around the row blocks (16) and the rows a CTA has in flight (64): remainders, fewer rows than blocks
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 63, 65, 1025])
+def test_prompt_support_row_block_edges(n):
+    cfg = W.CONFIGS["l2_13b_prompt"].with_(B=n, d=320, d_ff=128 * 20, k=6, m=40, index=430)
+    L = W.make_layer(cfg, device="cuda:0")
+    tk = W.make_tokens(cfg, L.A)
+    plan = cs.Plan(cfg.d, cfg.d_ff, cfg.group, cfg.m, cfg.k, cfg.T, torch.bfloat16, n, cfg.rms_eps)
+    sup, z, resid = cs.cs_prompt_support(plan, L.S, L.Phi, L.mu, tk.h.to("cuda:0"))
+    y, ref = oracle.prompt_support(L.S.cpu(), L.Phi.cpu(), tk.h, cfg.k, cfg.T, L.mu)
+    recovery_matches(sup.cpu().numpy(), z.cpu().numpy(), float(resid.cpu()[0]), ref, L.Phi.cpu().numpy(), np.asarray(y))
+    assert plan.device_status() == 0
+    plan.close()
