@@ -23,3 +23,15 @@ def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
     rep, _, _ = compare_layer_step(cfg, L, plan, tk.h)
     assert rep.excused <= max(1, B // 16), rep
     plan.close()
+
+
+# Gather path, rows per CTA at its bound: four tokens of 55 groups are 96 rows for each of 37 CTAs, of 56 groups one CTA more
+# a token; and few rows for many CTAs.
+@pytest.mark.parametrize("k,B", [(55, 4), (56, 4), (60, 3), (1, 3)])
+def test_gather_rows_per_cta_edges(k, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(d=256, d_ff=64 * 64, group=64, m=20, k=k, T=5, B=B, w_dtype="f32", index=360 + k)
+    L = W.make_layer(cfg, device="cuda:0")
+    tk = W.make_tokens(cfg, L.A)
+    plan = make_plan(cfg)
+    compare_layer_step(cfg, L, plan, tk.h)   # output bound 1e-5 (parity_util): f32 weights
+    plan.close()
