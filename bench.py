@@ -45,9 +45,9 @@ UNIT = "tokens/s"
 # ncu captures summarised under profiles/, keyed by (workload, k).  An entry is removed when its
 # kernel changes and comes back with the next capture; a missing entry reports null.
 NCU_TRAFFIC = {
-    ("l2_7b_b1", 22): 69.24e6 + 1.34e6,                       # ffn_gather_kernel
-    ("l2_7b_b64", 22): 181.44e6 + 3.52e6 + 95.85e6 + 3.53e6,  # ffn_gateup_swap_kernel + ffn_down_swap_kernel
-    ("l2_13b_prompt", 27): 211.12e6 + 12.08e6 + 56.08e6 + 5.21e6,  # ffn_gateup_pair_kernel + ffn_down_wide_kernel
+    ("l2_7b_b1", 22): 69.25e6 + 0.20e6,                       # ffn_gather_kernel
+    ("l2_7b_b64", 22): 182.17e6 + 1.14e6 + 93.04e6 + 1.04e6,  # decode_gateup_kernel + decode_down_kernel
+    ("l2_13b_prompt", 27): 205.4e6 + 8.30e6 + 54.6e6 + 2.65e6,  # ffn_gateup_pair_kernel + ffn_down_wide_kernel
 }
 GRAPH_STEPS = 64          # most steps captured per CUDA graph
 N_TOKEN_BATCHES = 16      # distinct input batches rotated through
@@ -291,8 +291,8 @@ def bench_decode(cfg, args, K, Wm, rank, world, local, dev, primary):
     tokens_per_s = cfg.B * world / (step_us * 1e-6)
     ab = algorithmic_bytes(cfg, union)
     peak, _, peak_kind = peaks()
-    mma = cfg.B >= plan.crossover and cfg.B <= 128 and cfg.w_dtype == "bf16" and cfg.group == 128 and cfg.d % 256 == 0
-    big = cfg.B > 128 and cfg.w_dtype == "bf16" and cfg.group == 128 and cfg.d % 256 == 0
+    mma = cfg.B >= plan.crossover and cfg.B <= 256 and cfg.w_dtype == "bf16" and cfg.group == 128 and cfg.d % 256 == 0
+    big = cfg.B > 256 and cfg.w_dtype == "bf16" and cfg.group == 128 and cfg.d % 256 == 0
     # the actuator reads the active weights and the hidden state and writes the output
     kernel_bytes = ab["weights"] + cfg.B * cfg.d * 4 * 2
     achieved = kernel_bytes / (exec_only_us * 1e-6) / 1e9
@@ -319,7 +319,7 @@ def bench_decode(cfg, args, K, Wm, rank, world, local, dev, primary):
         "clocks": clocks.summary(),
         "region_ms": {"median": ms_region, "min": min(times), "max": max(times)},
         "roofline": {"bound": "hbm",
-                     "kernel": ("ffn_gateup_swap_kernel + ffn_down_swap_kernel" if mma else
+                     "kernel": ("decode_gateup_kernel + decode_down_kernel" if mma else
                                 "ffn_gateup_mma_kernel + ffn_down_mma_kernel" if big else "ffn_gather_kernel"),
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_kind": peak_kind, "frac_of_8tbs_nominal": achieved / 8000.0,
@@ -331,7 +331,9 @@ def bench_decode(cfg, args, K, Wm, rank, world, local, dev, primary):
                      "traffic": NCU_TRAFFIC.get((cfg.name, cfg.k)) if cfg.B == W.CONFIGS[cfg.name].B else None},
         "stages_us": {"sketch": stage_ms[0] * 1e3, "recover": stage_ms[1] * 1e3, "exec": stage_ms[2] * 1e3,
                       "exec_down": stage_ms[4] * 1e3, "reduce": stage_ms[3] * 1e3, "step_net": step_us,
-                      "note": "stage figures are event brackets inside one-step graphs (2-4 us of record overhead each)",
+                      "note": "stage figures are event brackets inside one-step graphs (2-4 us of record overhead each); "
+                              "from the crossover batch on the recovery runs inside the gate/up launch (exec), below "
+                              "it inside the sketch's",
                       "measure_recover_per_token": mr_us / cfg.B,
                       "measure_recover_share_of_step": mr_us / step_us if step_us > 0 else None,
                       "exec_only_step": exec_only_us,
