@@ -278,8 +278,8 @@ cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, in
 /*
  * cs_layer_step with options (opt == NULL: cs_layer_step itself): another estimator, a warm start and
  * the temporal term from the previous step's result, the structured sensor, the drift against the
- * previous supports, or no estimation at all (reuse_support).  The stages run one after the other on
- * `stream` (the overlap of cs_layer_step's default path is not used).  With srht_sign / srht_rows the
+ * previous supports, or no estimation at all (reuse_support).  CS_SOLVER_IHT with the dense sketch takes
+ * cs_layer_step's launches; otherwise the stages run one after the other on `stream`.  With srht_sign / srht_rows the
  * layer must have no RMSNorm (rms_gamma == NULL) and layer->S is not read.
  */
 cs_status cs_layer_step_ex(cs_plan *plan, const cs_layer *layer, const float *x, int32_t B,
