@@ -87,7 +87,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     float4 *S_s = reinterpret_cast<float4 *>(phi_s + m * ppitch);
     pdl_launch_dependents();
     cluster_arrive();                               // matched below: every CTA of the cluster has started
-    // this lane's chunks of this warp's rows of S: no other thread reads them
+    // this lane's chunks of this warp's rows of S (read by this warp only)
     for (int r = warp; r < sa.s_rows; r += kSenseWarps)
 #pragma unroll 4
         for (int c = lane; c < nc; c += 32) {
@@ -152,7 +152,10 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
                          "f"(o[2]), "f"(o[3]) : "memory");
         }
     }
+    // A lane's wait covers its own copies; when nc is not a multiple of 32 the lanes past the end read the last column, which
+    // another lane copied (their x is zero, but zero times what shared memory held before could be NaN).
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
     pdl_wait();   // x may be the previous kernel's output
     float4 xv[kSenseMaxChunks], gm[kSenseMaxChunks];
     float ss = 0.f;

@@ -6,7 +6,7 @@ import torch
 import oracle
 import paper_2604_14156_b200 as cs
 from gen import workloads as W
-from parity_util import compare_layer_step, make_plan, recovery_matches
+from parity_util import compare_layer_step, device_layer, make_plan, recovery_matches
 
 pytestmark = pytest.mark.gpu
 
@@ -38,4 +38,24 @@ def test_prompt_support_row_block_edges(n):
     y, ref = oracle.prompt_support(L.S.cpu(), L.Phi.cpu(), tk.h, cfg.k, cfg.T, L.mu)
     recovery_matches(sup.cpu().numpy(), z.cpu().numpy(), float(resid.cpu()[0]), ref, L.Phi.cpu().numpy(), np.asarray(y))
     assert plan.device_status() == 0
+    plan.close()
+
+
+# d / 32 float4 columns per CTA that 32 lanes do not divide: lanes past the end read a column that another lane copied.  A layer
+# whose S is all NaN leaves NaN in every byte of shared memory such a read could find too early.
+@pytest.mark.parametrize("d", [192, 256, 1088, 2304, 5376])
+def test_sense_cluster_ragged_columns_after_nan_sketch(d):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(n_layers=1, w_dtype="f32", d=d, d_ff=64 * 20, group=64, m=30, k=6, T=5, B=4, index=440)
+    L = W.make_layer(cfg, device="cuda:0")
+    x = W.make_tokens(cfg, L.A).h.to("cuda:0")
+    plan = make_plan(cfg)
+    good = device_layer(plan, L)
+    bad = cs.Layer(plan, torch.full_like(L.S, float("nan")), L.Phi, L.W_gate, L.W_up, L.Wd_t, L.mu)
+    ref = [t.clone() for t in cs.cs_layer_step(plan, good, x)]
+    assert plan.device_status() == 0 and all(torch.isfinite(t).all() for t in ref)
+    for _ in range(20):
+        cs.cs_layer_step(plan, bad, x)
+        for a, b in zip(cs.cs_layer_step(plan, good, x), ref):
+            assert torch.equal(a, b)
+    plan.device_status()   # the NaN layer's report
     plan.close()
