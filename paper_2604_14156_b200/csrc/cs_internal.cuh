@@ -51,6 +51,7 @@ struct cs_plan {
     cs::DeviceStatus *status;  // device status word
     // tensor-core path (bf16 weights, 128-channel groups, d a multiple of 256)
     uint32_t *mask;      // [max_tokens, 4] membership bits: bit g of token t
+    unsigned *recovered; // [1] decode step: gate/up CTAs whose recoveries are done
     int32_t *counts;     // [G] tokens per group
     int32_t *offsets;    // [G + 1]
     int32_t *token_ids;  // [max_tokens * k] tokens of each group, ascending
@@ -130,6 +131,7 @@ struct RecoverArgs {
     const int32_t *check;
     int32_t *delta; float *drift;
     uint32_t *mask;
+    unsigned *recovered;       // decode batches: counts the CTAs whose recoveries are done
     SketchParts parts;
     cs::DeviceStatus *status;
 };
@@ -141,8 +143,7 @@ struct RecoverOptions {
     const int32_t *check = nullptr;                         // supports to validate (ascending, distinct, in range) ...
     int32_t *delta = nullptr; float *drift = nullptr;       // ... and the drift of the result against them
     // launch_sketch_slices came before and the decode GEMMs come next: take the sketch from the partials (writing it to
-    // plan->y_buf; norm: with the RMSNorm's row scale), write the membership masks (plan->mask), and (as a launch of its
-    // own) let the dependents start when the launches before the recovery are complete.
+    // plan->y_buf; norm: with the RMSNorm's row scale) and write the membership masks (plan->mask).
     bool decode = false, norm = false;
 };
 RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const float *y, int B, int32_t *support, float *z,
@@ -204,10 +205,9 @@ cs_status prepare_decode(cs_plan *plan);
 int decode_slices(const cs_plan *plan);
 cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *support, int B, bool check, cudaStream_t st);
 // recover != NULL and decode_recovers(): the recovery runs inside the gate/up launch; otherwise the launches before have
-// left the masks (plan->mask).  norm: the row scales come from the sketch's partial squares.  x_ready: the launch directly
-// before this one triggers its dependents only when the token matrices are complete.
+// left the masks (plan->mask).  norm: the row scales come from the sketch's partial squares.
 bool decode_recovers(const cs_plan *plan);
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool x_ready, bool norm,
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool norm,
                             const float *residual, float *out, cudaStream_t st);
 // Column sums of H per block of rows (plan->colsum); *blocks = their number.
 constexpr int kMeanRowBlocks = 16;

@@ -30,6 +30,9 @@
 // A step is then sketch -> gate/up (+ recovery) -> down -> reduction, each started early (programmatic dependent
 // launch) and streaming its weights before it waits for what the launch before produces.  With the recovery as a launch
 // ahead of gate/up the weight stream began 5.4 us after the step, in this form while the sketch still runs.
+// What an earlier launch of the step wrote is read behind a launch's own wait, since a trigger orders nothing in memory.  The
+// one exception are the masks in the down launch: the recoveries count themselves (release), and a CTA that finds the
+// count complete (acquire) may read them at once; a CTA that does not waits first.
 #include "mma_core.cuh"
 #include "recover_core.cuh"
 
@@ -149,12 +152,12 @@ __device__ __forceinline__ void mma_kblock(uint32_t tmem, uint32_t a0, uint32_t 
 
 // ---- gate / up ------------------------------------------------------------------------------------------
 // CTA x: channels [x R, x R + R), and with KC > 0 (slots of the recovery's list form, in units of 8) the recovery of tokens
-// x, x + gridDim.x, ...  x_ready: the token matrices were complete before this launch could begin (KC == 0 only).
+// x, x + gridDim.x, ...
 template <bool PACK, int MT, int KC>
 __global__ void __launch_bounds__(kDecThreads + kRecThreads, 1)
 decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
                      const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u, int B, int R, int d,
-                     int d_ff, int x_ready, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
+                     int d_ff, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
                      __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ act_lo, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ float rscale_s[MT * BM];
@@ -183,7 +186,7 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             // weights are parameters: the first ring is requested before anything is waited for
             const int pre = min(stages, kblocks);
             for (int kb = 0; kb < pre; ++kb) { mbar_expect_tx(&bars->full[kb], tx); load_w(kb, kb); }
-            if (KC > 0 || !x_ready) pdl_wait();
+            pdl_wait();   // the token matrices
             for (int kb = 0; kb < pre; ++kb) load_tokens(tt, base + (size_t)kb * stage_bytes, &tm_x, &tm_x_lo, kb * BK, &bars->full[kb]);
             int s = 0, ph = 0;
             for (int kb = pre; kb < kblocks; ++kb) {
@@ -214,7 +217,7 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     } else if (warp < kDecThreads / 32) {
         const int et = threadIdx.x - 64, r4 = R / 4;
         pdl_wait();   // the row squares; and nothing is stored before the kernels before this one are complete
-        if (KC == 0) pdl_launch_dependents();   // the supports are final: the down kernel reads them before its own wait
+        if (KC == 0) pdl_launch_dependents();
         for (int t = et; t < MT * BM; t += kEpiThreads) {
             float rs = 1.f;
             if (ss_part != nullptr && t < B) {
@@ -272,24 +275,26 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                 rs, ra, M, [&](auto &sm) { y_from_parts<kRecNW, kRecBar>(sm, ra.parts, g, t, ra.m); }, ra.mask, g, t, phc);
             bar_sync<kRecBar, kRecThreads>();
         }
-        // the down kernel reads the masks before its own wait
-        __threadfence();
-        bar_sync<kRecBar, kRecThreads>();
-        if (g == 0) pdl_launch_dependents();
+        // this CTA's masks are written (the barrier that ends the loop, or no token at all)
+        if (g == 0) {
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ra.recovered) : "memory");
+            pdl_launch_dependents();
+        }
     }
     teardown_cta(bars, warp, tcols);
 }
 
 // ---- down -----------------------------------------------------------------------------------------------
 // grid (d / 256, slices).  The list is every group (use_union == 0) or the groups that are in some token's support; slice z
-// takes the 64-channel k blocks [z nk / Z, (z + 1) nk / Z) of it.
+// takes the 64-channel k blocks [z nk / Z, (z + 1) nk / Z) of it.  recovered: count of the gate/up CTAs whose recoveries are done
+// (set to zero by the step's sketch), complete at `recoveries` (0: the masks come from elsewhere).
 template <bool PACK, int MT>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_constant__ CUtensorMap tm_act,
-                   const __grid_constant__ CUtensorMap tm_act_lo, const int32_t *mask, int use_union, int B, int G,
-                   int d, float *__restrict__ partial, DeviceStatus *status) {
+                   const __grid_constant__ CUtensorMap tm_act_lo, const int32_t *mask, const unsigned *recovered,
+                   unsigned recoveries, int use_union, int B, int G, int d, float *__restrict__ partial, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint32_t union_s[4];
+    __shared__ uint32_t union_s[4], masks_s;
     __shared__ int glist_s[kMaxG];                          // groups of this slice, in list order
     __shared__ __align__(16) uint32_t out_s[kMaxG][4 * MT]; // tokens whose support does not hold them: the lane masks
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -304,8 +309,14 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
     pdl_launch_dependents();
     if (threadIdx.x == 0) { prefetch_map(&tm_wd); prefetch_map(&tm_act); prefetch_map(&tm_act_lo); }
     if (threadIdx.x < 4) union_s[threadIdx.x] = 0u;
+    if (threadIdx.x == 64) {
+        unsigned n = 0u;
+        if (recoveries != 0u) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(recovered) : "memory");
+        masks_s = recoveries != 0u && n == recoveries;
+    }
     setup_cta(bars, warp, tcols);
-    // The masks were final, and visible, before this launch could begin (see the gate/up kernel's trigger).
+    const bool masks_ready = masks_s != 0u;   // (behind a barrier, as the masks of the other threads' reads)
+    if (use_union && !masks_ready) pdl_wait();
     int ng = G;
     if (use_union) {
         for (int t = threadIdx.x; t < B; t += kDecThreads) {
@@ -382,6 +393,10 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
         }
     } else {
         const int ew = warp - 2, q = warp & 3, et = threadIdx.x - 64;
+        for (int c = ew >> 2; c < MT * 256 / 16; c += kEpiWarps / 4)
+            tc_st16_zero(bars->tmem_base + ((uint32_t)(q * 32) << 16) + c * 16);
+        tc_wait_st();
+        if (!masks_ready) pdl_wait();
         // lane masks: epilogue warp w holds the membership words of tokens 32 w .. 32 w + 31
         if (ew < (PACK ? 2 : 4 * MT)) {
             const int t = 32 * ew + lane;
@@ -396,9 +411,6 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
                 }
             }
         }
-        for (int c = ew >> 2; c < MT * 256 / 16; c += kEpiWarps / 4)
-            tc_st16_zero(bars->tmem_base + ((uint32_t)(q * 32) << 16) + c * 16);
-        tc_wait_st();
         tc_fence_before();
         asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads + 32) : "memory");
         if (warp == 2 && kblocks > 0) mbar_wait(&bars->acc_ready, 0, bars, status);
@@ -481,9 +493,10 @@ decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ supp
     if (tid < 4) mask[(size_t)t * 4 + tid] = (int)m_s[tid];
 }
 
-typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, int, const float *, float,
+typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, const float *, float,
                          RecoverArgs, __nv_bfloat16 *, __nv_bfloat16 *, DeviceStatus *);
-typedef void (*DownFn)(CUtensorMap, CUtensorMap, CUtensorMap, const int32_t *, int, int, int, int, float *, DeviceStatus *);
+typedef void (*DownFn)(CUtensorMap, CUtensorMap, CUtensorMap, const int32_t *, const unsigned *, unsigned, int, int, int, int, float *,
+                       DeviceStatus *);
 
 // The recovery's list form in three lengths (24, 32, 56 slots); 0: no recovery inside the launch.
 int gateup_kc(const cs_plan *plan) { return plan->cfg.k <= 24 ? 3 : plan->cfg.k <= 32 ? 4 : 7; }
@@ -527,13 +540,14 @@ cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *suppo
     return CS_OK;
 }
 
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool x_ready, bool norm,
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool norm,
                             const float *residual, float *out, cudaStream_t st) {
     const cs_config &c = plan->cfg;
     const bool pack = B <= 64;
     const int mt = B <= BM ? 1 : 2, form = pack ? 0 : mt;
     const TokenTile tt = token_tile(pack, mt, B);
     const int R = min(128, ((c.d_ff + plan->sm_count - 1) / plan->sm_count + 7) & ~7);
+    const int gateup_ctas = (c.d_ff + R - 1) / R;
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16), *x_lo = x_hi + (size_t)c.max_tokens * c.d;
     __nv_bfloat16 *act = static_cast<__nv_bfloat16 *>(plan->act), *act_lo = act + (size_t)c.max_tokens * c.d_ff;
     CUtensorMap tm_g, tm_u, tm_x, tm_x_lo, tm_wd, tm_act, tm_act_lo;
@@ -544,9 +558,9 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
         return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
-        launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3((c.d_ff + R - 1) / R),
+        launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
                    dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), decode_smem(tt, 2 * R * BK * 2), st, tm_x, tm_x_lo, tm_g,
-                   tm_u, B, R, c.d, c.d_ff, x_ready ? 1 : 0, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
+                   tm_u, B, R, c.d, c.d_ff, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
                    c.rms_eps, recover != nullptr ? *recover : RecoverArgs{}, act, act_lo, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
@@ -558,7 +572,8 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
         // the masks need not be read.
         const bool use_union = (float)plan->G * powf(1.f - (float)c.k / plan->G, (float)B) > 0.25f;
         launch_pdl(true, down_fn(form), dim3(c.d / kDecBN, Z), dim3(kDecThreads), decode_smem(tt, kDecBN * BK * 2), st, tm_wd, tm_act,
-                   tm_act_lo, (const int32_t *)plan->mask, use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
+                   tm_act_lo, (const int32_t *)plan->mask, (const unsigned *)plan->recovered,
+                   recover != nullptr ? (unsigned)gateup_ctas : 0u, use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }

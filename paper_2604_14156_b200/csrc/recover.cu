@@ -17,15 +17,12 @@ template <int NW, int KC, bool DECODE>
 __global__ void __launch_bounds__(32 * NW) recover_kernel(const __grid_constant__ RecoverArgs a) {
     __shared__ RecoverSmem<NW, KC> s;
     const int g = threadIdx.x;
-    if (!DECODE) pdl_launch_dependents();
+    pdl_launch_dependents();
     // Phi is a parameter: this thread's column is requested before the wait for the kernel that
     // produces y and M, when it fits 32 registers
     float phc[32];
     if (a.m <= 32) recover_load_phi<NW>(a.Phi, a.m, a.G, g, phc);
     pdl_wait();   // y and M come from the kernel before
-    // The decode GEMMs read what the kernels before this one wrote without a wait of their own, and wait for the
-    // supports behind their main loop.
-    if (DECODE) pdl_launch_dependents();
     const int t = blockIdx.x;
     recover_row<NW, KC, 0>(
         s, a, GramSource{a.gram, 32 * NW},
@@ -305,7 +302,7 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
     a.sup0 = o.sup0; a.z0 = o.z0; a.sup_prev = o.sup_prev; a.z_prev = o.z_prev;
     a.check = o.check; a.delta = o.delta; a.drift = o.drift;
     if (o.decode) {
-        a.mask = plan->mask;
+        a.mask = plan->mask; a.recovered = plan->recovered;
         a.parts = SketchParts{sketch_partials(plan), o.norm ? sketch_square_partials(plan, B) : nullptr, c.d / 64, B, c.d, c.rms_eps,
                               plan->y_buf};
     }

@@ -1,8 +1,11 @@
 """GPU parity of the tensor-core decode path (up to 256 tokens) at the sizes where its tiling can go wrong."""
 import pytest
+import torch
+
+import paper_2604_14156_b200 as cs
 
 from gen import workloads as W
-from parity_util import compare_layer_step, make_plan
+from parity_util import compare_layer_step, device_layer, make_plan
 
 pytestmark = pytest.mark.gpu
 
@@ -34,4 +37,30 @@ def test_gather_rows_per_cta_edges(k, B):
     tk = W.make_tokens(cfg, L.A)
     plan = make_plan(cfg)
     compare_layer_step(cfg, L, plan, tk.h)   # output bound 1e-5 (parity_util): f32 weights
+    plan.close()
+
+
+# Steps on changing tokens, launched without a pause: masks, token matrices or supports of the step before would show in the
+# bits.  Few groups per token (the down GEMM's list is the union), nearly all groups in use, and the recovery as a launch
+# of its own (k > 56); one, two and four 64-row boxes of tokens.
+@pytest.mark.parametrize("k", [3, 40, 60])
+@pytest.mark.parametrize("B", [5, 64, 130, 256])
+def test_back_to_back_steps_on_changing_tokens(k, B):
+    cfg = W.CONFIGS["l3_8b_stack"].with_(n_layers=1, d=1024, d_ff=128 * 100, m=40, k=k, T=6, B=B, index=460)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    plan.set_crossover(2)
+    lay = device_layer(plan, L)
+    h = W.make_tokens(cfg, L.A).h.to("cuda:0")
+    xs = [h.roll(i, 0) * (1.0 + i) + 0.1 * i for i in range(4)]
+    alone = []
+    for x in xs:
+        torch.cuda.synchronize()
+        alone.append([t.clone() for t in cs.cs_layer_step(plan, lay, x)])
+    torch.cuda.synchronize()
+    runs = [cs.cs_layer_step(plan, lay, xs[i % 4]) for i in range(24)]
+    for i, run in enumerate(runs):
+        for a, b in zip(run, alone[i % 4]):
+            assert torch.equal(a, b), i
+    assert plan.device_status() == 0
     plan.close()
