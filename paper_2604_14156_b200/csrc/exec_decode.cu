@@ -498,11 +498,12 @@ typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int
 typedef void (*DownFn)(CUtensorMap, CUtensorMap, CUtensorMap, const int32_t *, const unsigned *, unsigned, int, int, int, int, float *,
                        DeviceStatus *);
 
-// The recovery's list form in three lengths (24, 32, 56 slots); 0: no recovery inside the launch.
-int gateup_kc(const cs_plan *plan) { return plan->cfg.k <= 24 ? 3 : plan->cfg.k <= 32 ? 4 : 7; }
+// The recovery's list form in four lengths (24, 32, 56, 64 slots); 0: no recovery inside the launch.
+int gateup_kc(const cs_plan *plan) { return plan->cfg.k <= 24 ? 3 : plan->cfg.k <= 32 ? 4 : plan->cfg.k <= 56 ? 7 : 8; }
 template <bool PACK, int MT> GateUpFn gateup_fn_kc(int kc) {
     return kc == 0 ? decode_gateup_kernel<PACK, MT, 0> : kc == 3 ? decode_gateup_kernel<PACK, MT, 3>
-         : kc == 4 ? decode_gateup_kernel<PACK, MT, 4> : decode_gateup_kernel<PACK, MT, 7>;
+         : kc == 4 ? decode_gateup_kernel<PACK, MT, 4> : kc == 7 ? decode_gateup_kernel<PACK, MT, 7>
+         : decode_gateup_kernel<PACK, MT, 8>;
 }
 GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators
     return form == 0 ? gateup_fn_kc<true, 1>(kc) : form == 1 ? gateup_fn_kc<false, 1>(kc) : gateup_fn_kc<false, 2>(kc);
@@ -511,7 +512,9 @@ DownFn down_fn(int form) { return form == 0 ? decode_down_kernel<true, 1> : form
 
 }  // namespace
 
-bool decode_recovers(const cs_plan *plan) { return plan->cfg.k <= 56; }
+// Half of the most groups.  With k = 64 slots a recovery inside gate/up costs what one with 56 does (108 groups, k = 60: 3 tokens
+// 72 to 75 us a step, 64 tokens 81 to 87; with the recovery as a launch of its own 89 and 95); a longer list does not fit the registers.
+bool decode_recovers(const cs_plan *plan) { return plan->cfg.k <= 64; }
 
 int decode_slices(const cs_plan *plan) {   // list slices of the down GEMM: one CTA per SM
     const int tiles = plan->cfg.d / kDecBN;

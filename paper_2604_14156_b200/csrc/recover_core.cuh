@@ -11,13 +11,13 @@
 //     token) and  M = I - mu Phi^T Phi  (once per layer, gram_rows).  Since z has exactly k
 //     non-zeros, one iteration is k multiply-adds per entry instead of the two mat-vecs through
 //     the m-dimensional residual, and nothing but z crosses threads.
-//   - Thread g owns entry g of v and z.  In the list form (k <= 56) z is a list of k slots in shared
+//   - Thread g owns entry g of v and z.  In the list form (k <= 56, inside the decode GEMM k <= 64) z is a list of k slots in shared
 //     memory, read by broadcast: slot j holds the value of entry idx[j], and the thread keeps the k
 //     matrix entries M[idx[j], g] that go with the list in registers, so the mat-vec has no indexed
 //     load.  Slots are stable: an entry that stays in the support keeps its slot, an entry that
 //     enters takes the slot of one that left, and only the matrix entries of those slots are fetched
 //     again.  (In the first iteration from z = 0 the slots are handed out by rank, which lists the
-//     support by decreasing magnitude.)  For k > 56 z is a dense vector and the thread keeps its
+//     support by decreasing magnitude.)  For larger k z is a dense vector and the thread keeps its
 //     whole row of M.
 //   - H_k is exact under the total order (|v| descending, group index ascending), but most
 //     iterations do not change the support, which is the case exactly when every kept |v| exceeds
@@ -49,7 +49,7 @@ template <int ID, int N> __device__ __forceinline__ void bar_arrive() {
     asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(N) : "memory");
 }
 
-// NW = warps = ceil(G / 32).  KC = ceil(k / 8) for k <= 56 (list form); KC = 0: any k, dense form.
+// NW = warps = ceil(G / 32).  KC >= ceil(k / 8), at most 8 (list form); KC = 0: any k, dense form.
 template <int NW, int KC> struct RecoverSmem {
     static constexpr int GP = 32 * NW;                 // padded number of entries = pitch of M
     static constexpr int NV = KC > 0 ? KC * 8 : GP;    // length of the iterate as the mat-vec reads it
