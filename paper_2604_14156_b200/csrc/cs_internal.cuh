@@ -13,7 +13,7 @@ constexpr int kMaxG = 128;        // groups per layer
 constexpr int kMaxM = 64;         // sketch rows
 constexpr int kMaxD = 8192;       // hidden size
 constexpr int kGatherThreads = 512;
-constexpr int kGatherMaxRows = 96;   // channel rows one gather CTA owns at most: one CTA per SM up to four tokens of 22 groups
+constexpr int kGatherMaxRows = 160;  // channel rows one gather CTA owns at most (what its tables hold beside 192 KB of rings)
 constexpr int kStaticMaxRows = 32;   // the same bound of the entry without a plan (part of its stated limit)
 constexpr int kGatherMaxTokens = 16; // tokens per gather launch (scratch for partial sums)
 constexpr int kSlotTableSlots = 32;  // slots per token of the recovery's slot table (small-batch step) ...

@@ -46,7 +46,6 @@ constexpr int kUnitChunks = 4;                             // chunks per lane, m
 constexpr int kUnitBytes = 2 * kUnitChunks * 32 * 16;      // gate + up: 4 KB
 constexpr int kUnitStages = kWarpRing / kUnitBytes;        // 3 units in flight per warp
 constexpr int kLaneSlots = kWarpRing / (32 * 16);          // 24 chunks per lane in the down phase
-constexpr int kMaxSegs = kMaxD * 4 / (kUnitChunks * 32 * 16);  // 16 (f32 rows of 8192)
 
 constexpr int kSpecThreads = kGatherThreads + 32;   // the streaming warps + the warp that follows the slot table
 constexpr uint32_t kFollowLimit = 1u << 16;         // polls of the table after which the following warp gives up
@@ -85,6 +84,8 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
     constexpr int DR = kLaneSlots / CPT;               // down rows in flight per thread
     constexpr int kSegElems = kUnitChunks * 32 * E;    // elements of one row segment
     extern __shared__ __align__(16) uint4 ring[];      // [kGatherWarps][kWarpRing / 16]
+    // segments of a row, at most 4 CPT: tables no larger than the row needs, so that a small step's next sensing launch fits beside
+    constexpr int kMaxSegs = CPT * kGatherThreads / (kUnitChunks * 32);
     __shared__ float red[kGatherMaxRows][kMaxSegs][2];
     __shared__ float a_s[kGatherMaxRows];
     __shared__ int chan_s[kGatherMaxRows];
@@ -481,10 +482,16 @@ static void launch_gather_kernel(dim3 grid, cudaStream_t st, int cpt, int chunks
 #undef CS_GATHER_CASE
 }
 
-// CTAs per token: one CTA per SM for all tokens in flight, never more than kGatherMaxRows rows per CTA.  (With at most 32
-// rows two tokens of 2816 rows were 176 CTAs and three 264, two waves of 148: 44.7 and 47.1 us a step, four tokens 63.4; now 33.5, 42.2 and 48.1.)
+// CTAs per token.  An SM holds one CTA (192 KB of rings), so the launch takes whole waves: as many CTAs as fit into the fewest
+// waves that leave no CTA more than kGatherMaxRows rows.  A few CTAs past a wave cost a whole CTA's time, and tokens of
+// one wave meet in L2 where they share groups.  One step, with max(SMs / tokens, rows / 96) CTAs per token and so: 8B layer, 4
+// tokens (38 CTAs each and 37) 79.0 and 52.7 us; d = 5120, 11 of 108 groups, 10 tokens 122.6 and 73.9; 22 groups in f32, 5 tokens
+// 109.0 and 81.5, 8 tokens 132 and 110 (a bound of 128 rows there: 146, two waves of four tokens).  Sizes that filled one wave
+// before keep their grid (7B, 1 to 4 tokens: 22.5, 31.3, 39.6, 44.9).  (22 groups in f32, 9 tokens: 143 and 149, the one size
+// measured where two whole waves are behind a partly filled second one.)
 static int gather_nx(int sm_count, int nb, int rows_total, int nx_max) {
-    int nx = max(sm_count / nb, (rows_total + kGatherMaxRows - 1) / kGatherMaxRows);
+    int nx = sm_count / nb;
+    for (int waves = 2; nx * kGatherMaxRows < rows_total && nx < nx_max; ++waves) nx = sm_count * waves / nb;
     return max(1, min(nx, min(rows_total, nx_max)));
 }
 

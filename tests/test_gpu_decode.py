@@ -28,8 +28,7 @@ def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
     plan.close()
 
 
-# Gather path, rows per CTA at its bound: four tokens of 55 groups are 96 rows for each of 37 CTAs, of 56 groups one CTA more
-# a token; and few rows for many CTAs.
+# Gather path: few rows for many CTAs, and three or four tokens of 55 to 60 groups.
 @pytest.mark.parametrize("k,B", [(55, 4), (56, 4), (60, 3), (1, 3)])
 def test_gather_rows_per_cta_edges(k, B):
     cfg = W.CONFIGS["l2_7b_b64"].with_(d=256, d_ff=64 * 64, group=64, m=20, k=k, T=5, B=B, w_dtype="f32", index=360 + k)
@@ -37,6 +36,53 @@ def test_gather_rows_per_cta_edges(k, B):
     tk = W.make_tokens(cfg, L.A)
     plan = make_plan(cfg)
     compare_layer_step(cfg, L, plan, tk.h)   # output bound 1e-5 (parity_util): f32 weights
+    plan.close()
+
+
+# Gather path, rows per CTA at the bound of 160: four tokens of 92 groups are 160 rows for each of 37 CTAs, of 93 groups two
+# waves of CTAs; eight of 45 groups one wave; sixteen of 128 groups, several waves.
+@pytest.mark.parametrize("k,B", [(92, 4), (93, 4), (45, 8), (128, 16)])
+def test_gather_rows_per_cta_bound(k, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(d=256, d_ff=64 * 128, group=64, m=20, k=k, T=5, B=B, w_dtype="f32", index=380 + k)
+    L = W.make_layer(cfg, device="cuda:0")
+    tk = W.make_tokens(cfg, L.A)
+    plan = make_plan(cfg)
+    compare_layer_step(cfg, L, plan, tk.h)   # output bound 1e-5 (parity_util): f32 weights
+    plan.close()
+
+
+def _replay_us(fn, calls=16, replays=20):
+    """Median microseconds of a call, captured back to back."""
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        fn()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(calls):
+            fn()
+    times = []
+    for _ in range(replays):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record(); graph.replay(); b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) * 1e3 / calls)
+    return sorted(times)[replays // 2]
+
+
+def test_gather_grid_has_no_nearly_empty_wave():
+    """Four tokens of the 8B layer are a third more rows than three (measured 1.2 times the time); a few CTAs past a whole wave
+    of them made it 1.7 times."""
+    cfg = W.CONFIGS["l3_8b_stack"].with_(n_layers=1, B=4)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    lay = device_layer(plan, L)
+    h = W.make_tokens(cfg, L.A).h.to("cuda:0")
+    us = {}
+    for B in (3, 4):
+        x, out = h[:B].contiguous(), torch.empty((B, cfg.d), device="cuda:0")
+        us[B] = _replay_us(lambda: cs.cs_layer_step(plan, lay, x, out, want_aux=False))
+    assert plan.crossover > 4 and us[4] <= 1.45 * us[3], us
     plan.close()
 
 
