@@ -380,7 +380,7 @@ cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, in
         if (s != CS_OK) return s;
         return launch_ffn_gather_spec(plan, layer, n, B, layer->add_residual ? x : nullptr, x_out, st);
     }
-    if (B <= kSenseMaxTokens) {
+    if (B <= plan->sense_tokens) {
         s = launch_sense_recover(plan, layer->S, layer->Phi, layer->mu, x, layer->rms_gamma, B, norm ? plan->n_buf : nullptr, sup, z_out,
                                  resid_out, st);
     } else {
@@ -430,7 +430,7 @@ cs_status cs_layer_step_ex(cs_plan *plan, const cs_layer *layer, const float *x,
         RecoverOptions o = iht_options(plan, opt);
         return decode_step(plan, layer, x, B, o, x_out, sup, z_out, resid_out, st);
     }
-    if (B <= kSenseMaxTokens && !srht && opt->solver == CS_SOLVER_IHT) {
+    if (B <= plan->sense_tokens && !srht && opt->solver == CS_SOLVER_IHT) {
         s = launch_sense_recover(plan, layer->S, layer->Phi, layer->mu, x, layer->rms_gamma, B, norm ? plan->n_buf : nullptr, sup, z_out,
                                  resid_out, st, iht_options(plan, opt));
         if (s != CS_OK) return s;

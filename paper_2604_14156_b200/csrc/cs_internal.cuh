@@ -60,6 +60,7 @@ struct cs_plan {
     void *x_bf16;        // [2][max_tokens, d] bf16 activations: rounded value, then remainder
     void *act;           // [2][max_tokens, d_ff] bf16 SwiGLU activations over the group list (value, remainder)
     float *mma_partial;  // [slices, padded tokens, d] f32 partial down projections
+    int sense_tokens;    // up to this many tokens sensor and estimator are one launch (launch_sense_recover)
     int speculative;     // small batches, on the recovery's first iterate: 1 = start the weight stream, 2 = warm L2 only
     int mma_ok;          // shape qualifies for the tensor-core path
     int mma_min_tokens;  // smallest decode batch that takes it
@@ -152,7 +153,7 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
 cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float *y, int B,
                          int32_t *support, float *z, float *resid, bool gram_ready, cudaStream_t st,
                          const RecoverOptions &opt = RecoverOptions());
-// Sensor and estimator in one launch, a cluster of CTAs per token, for at most kSenseMaxTokens tokens.  blocks > 0: one
+// Sensor and estimator in one launch, a cluster of CTAs per token, for at most plan->sense_tokens tokens.  blocks > 0: one
 // token whose x is the sum of `blocks` rows [blocks, d] divided by n (a prompt's mean hidden state).
 constexpr int kSenseMaxTokens = 16;
 cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,

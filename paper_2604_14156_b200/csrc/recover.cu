@@ -11,7 +11,7 @@ __global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restr
     gram_rows(Phi, mu, m, G, blockIdx.x, gram);
 }
 
-// NW = warps = ceil(G / 32).  KC = ceil(k / 8) for k <= 56 (list form), 0 otherwise (dense form).
+// NW = warps = ceil(G / 32).  KC = ceil(k / 8) for k <= 64 (list form), 0 otherwise (dense form).
 // DECODE: the form of RecoverOptions::decode.
 template <int NW, int KC, bool DECODE>
 __global__ void __launch_bounds__(32 * NW) recover_kernel(const __grid_constant__ RecoverArgs a) {
@@ -271,7 +271,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
 typedef void (*SenseFn)(SenseArgs, RecoverArgs);
 
 typedef void (*RecoverFn)(RecoverArgs);
-static int recover_kc(int k) { return k <= 56 ? (k + 7) / 8 : 0; }
+static int recover_kc(int k) { return k <= 64 ? (k + 7) / 8 : 0; }
 template <int NW, bool DECODE> static RecoverFn recover_fn_kc(int k) {
     switch (recover_kc(k)) {
         case 1: return recover_kernel<NW, 1, DECODE>;
@@ -281,6 +281,7 @@ template <int NW, bool DECODE> static RecoverFn recover_fn_kc(int k) {
         case 5: return recover_kernel<NW, 5, DECODE>;
         case 6: return recover_kernel<NW, 6, DECODE>;
         case 7: return recover_kernel<NW, 7, DECODE>;
+        case 8: return recover_kernel<NW, 8, DECODE>;
         default: return recover_kernel<NW, 0, DECODE>;
     }
 }
@@ -319,6 +320,7 @@ template <int NW> static SenseFn sense_fn_kc(int k) {
         case 5: return sense_recover_kernel<NW, 5>;
         case 6: return sense_recover_kernel<NW, 6>;
         case 7: return sense_recover_kernel<NW, 7>;
+        case 8: return sense_recover_kernel<NW, 8>;
         default: return sense_recover_kernel<NW, 0>;
     }
 }
@@ -348,8 +350,25 @@ cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, 
     return CS_OK;
 }
 
+// Up to how many tokens the sensing launch takes over from the sketch and recovery launches: as many clusters as the device
+// holds at once (15 of eight CTAs on B200; the sixteenth costs 2.5 us of a 15 us step).  None where a CTA's part of S is
+// above 128 KB, which the cluster reads anew for every token and the sketch launch once for all of them (d = 5120, m = 64, 2 tokens
+// 31.4 us against 28.8; at 8192 x 32 still 23.2 against 23.8 for one token, 34.0 against 32.7 for two), nor for the dense
+// form, whose rows of M every thread first reads from shared memory (128 groups, k = 64 in the dense form, one token 52.9 against 47.0).
+// Below that it saves 0.5 to 1.5 us a step up to three tokens and is even, within 0.5 us, above.
+static int sense_tokens(const cs_plan *plan, int smem) {
+    const cs_config &c = plan->cfg;
+    if ((size_t)c.m * c.d * 4 > (size_t)kSenseCtas * 128 * 1024 || recover_kc(c.k) == 0) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kSenseCtas * kSenseMaxTokens); cfg.blockDim = dim3(kSenseThreads); cfg.dynamicSmemBytes = smem;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, sense_fn(plan->G, c.k), &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return min(clusters, kSenseMaxTokens);
+}
+
 cs_status prepare_recover(cs_plan *plan) {
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
+    plan->sense_tokens = sense_tokens(plan, kSenseSmem);
     CS_CUDA_TRY(plan, prefer_shared(recover_fn<true>(plan->G, plan->cfg.k)));
     return CS_OK;
 }

@@ -11,7 +11,7 @@
 //     token) and  M = I - mu Phi^T Phi  (once per layer, gram_rows).  Since z has exactly k
 //     non-zeros, one iteration is k multiply-adds per entry instead of the two mat-vecs through
 //     the m-dimensional residual, and nothing but z crosses threads.
-//   - Thread g owns entry g of v and z.  In the list form (k <= 56, inside the decode GEMM k <= 64) z is a list of k slots in shared
+//   - Thread g owns entry g of v and z.  In the list form (k <= 64) z is a list of k slots in shared
 //     memory, read by broadcast: slot j holds the value of entry idx[j], and the thread keeps the k
 //     matrix entries M[idx[j], g] that go with the list in registers, so the mat-vec has no indexed
 //     load.  Slots are stable: an entry that stays in the support keeps its slot, an entry that

@@ -27,6 +27,36 @@ def test_layer_step_sense_cluster_edges(d, G, m, k, B, norm):
     plan.close()
 
 
+# What decides between the sensing launch and the sketch and recovery launches: tokens (clusters resident at once, 15 on B200),
+# the bytes of S (128 KB per CTA: 8192 x 32, 8192 x 33), the list form (64 groups).  The dense form and its prompt.
+@pytest.mark.parametrize("d,G,m,k,B", [(256, 16, 8, 4, 12), (256, 16, 8, 4, 15), (256, 16, 8, 4, 16), (8192, 40, 32, 9, 2), (8192, 40, 33, 9, 2),
+                                       (1024, 128, 48, 56, 3), (1024, 128, 48, 57, 3), (1024, 128, 48, 64, 3), (1024, 128, 48, 65, 3),
+                                       (1024, 70, 48, 68, 2), (1024, 128, 48, 128, 2)])
+def test_layer_step_sense_launch_limits(d, G, m, k, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(n_layers=1, w_dtype="f32", d=d, d_ff=64 * G, group=64, m=m, k=k, T=7, B=B, index=480 + k)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    rep, _, _ = compare_layer_step(cfg, L, plan, W.make_tokens(cfg, L.A).h)   # output bound 1e-5 (parity_util): f32 weights
+    assert rep.excused <= max(1, B // 16), rep
+    plan.close()
+
+
+def test_sense_launch_is_taken_up_to_the_resident_clusters():
+    """Launches of a step: sense + gather + reduction, or sketch + recovery + gather + reduction."""
+    def launches(**kw):
+        cfg = W.CONFIGS["tiny_f32"].with_(**kw)
+        L = W.make_layer(cfg, device="cuda:0")
+        plan = make_plan(cfg)
+        lay, x = device_layer(plan, L), W.make_tokens(cfg, L.A).h.to("cuda:0")
+        before = plan.launches
+        cs.cs_layer_step(plan, lay, x)
+        n = plan.launches - before
+        plan.close()
+        return n
+    assert launches(B=1) == 3 and launches(B=8) == 3 and launches(B=16) == 4
+    assert launches(B=2, d=8192, m=33, d_ff=64 * 40) == 4 and launches(B=2, d_ff=64 * 128, m=48, k=65) == 4
+
+
 # prompt lengths around the row blocks (16) and the rows a CTA has in flight (64): remainders, fewer rows than blocks
 @pytest.mark.parametrize("n", [1, 15, 16, 17, 63, 65, 1025])
 def test_prompt_support_row_block_edges(n):
