@@ -97,7 +97,7 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     // 4 and 5 tokens at G / k = 3.9).
     p->mma_min_tokens = max(2, min(kMmaMinTokens, (int)ceilf(1.15f * (float)p->G / (float)cfg->k)));
     alloc((void **)&p->mask, nt * 4 * sizeof(uint32_t));
-    alloc((void **)&p->recovered, sizeof(unsigned));
+    alloc((void **)&p->mask_count, sizeof(unsigned));
     alloc((void **)&p->counts, (size_t)kMaxG * sizeof(int32_t));
     alloc((void **)&p->offsets, (size_t)(kMaxG + 1) * sizeof(int32_t));
     alloc((void **)&p->token_ids, nt * cfg->k * sizeof(int32_t));
@@ -118,7 +118,7 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     for (int i = 0; i < 2 * CS_STAGE_COUNT; ++i)
         if (e == cudaSuccess) e = cudaEventCreate(&p->ev[i]);
     if (e == cudaSuccess) e = cudaMemset(p->status, 0, sizeof(DeviceStatus));
-    if (e == cudaSuccess) e = cudaMemset(p->recovered, 0, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemset(p->mask_count, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(p->ticket, 0, nt * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(p->slot_table, 0, nt * kSlotTablePitch * sizeof(int32_t));
     if (e == cudaSuccess && prepare_sketch(p) != CS_OK) e = cudaErrorUnknown;
@@ -143,7 +143,7 @@ cs_status cs_plan_destroy(cs_plan *p) {
     cudaFree(p->partial); cudaFree(p->gram); cudaFree(p->slot_table); cudaFree(p->ticket);
     cudaFree(p->resid_buf); cudaFree(p->fb_flags); cudaFree(p->fb_list); cudaFree(p->fb_count); cudaFree(p->colsum);
     cudaFree(p->status); cudaFree(p->x_host_in); cudaFree(p->x_host_out);
-    cudaFree(p->mask); cudaFree(p->recovered); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
+    cudaFree(p->mask); cudaFree(p->mask_count); cudaFree(p->counts); cudaFree(p->offsets); cudaFree(p->token_ids); cudaFree(p->glist);
     cudaFree(p->nu); cudaFree(p->x_bf16); cudaFree(p->act); cudaFree(p->mma_partial);
     for (int i = 0; i < 2 * CS_STAGE_COUNT; ++i)
         if (p->ev[i] != nullptr) cudaEventDestroy(p->ev[i]);
@@ -292,7 +292,7 @@ static cs_status exec_dispatch(cs_plan *plan, const cs_layer *layer, const float
     if (use_decode_mma(plan, B)) {
         cs_status s = launch_decode_prep(plan, h, support, B, check, st);
         if (s != CS_OK) return s;
-        return launch_decode_ffn(plan, layer, B, nullptr, false, residual, out, st);
+        return launch_decode_ffn(plan, layer, B, nullptr, true, false, residual, out, st);
     }
     if (check) {
         cs_status s = launch_check_support(plan, support, B, st);
@@ -338,11 +338,11 @@ static cs_status decode_step(cs_plan *plan, const cs_layer *layer, const float *
     if (s != CS_OK) return s;
     if (decode_recovers(plan)) {
         const RecoverArgs ra = recover_args(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z, resid, o);
-        return launch_decode_ffn(plan, layer, B, &ra, o.norm, residual, x_out, st);
+        return launch_decode_ffn(plan, layer, B, &ra, false, o.norm, residual, x_out, st);
     }
     s = launch_recover(plan, layer->Phi, layer->mu, plan->y_buf, B, sup, z, resid, true, st, o);
     if (s != CS_OK) return s;
-    return launch_decode_ffn(plan, layer, B, nullptr, o.norm, residual, x_out, st);
+    return launch_decode_ffn(plan, layer, B, nullptr, false, o.norm, residual, x_out, st);
 }
 
 cs_status cs_layer_step(cs_plan *plan, const cs_layer *layer, const float *x, int32_t B, float *x_out,

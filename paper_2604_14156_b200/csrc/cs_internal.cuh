@@ -40,7 +40,7 @@ struct cs_plan {
     float *y_buf;      // [max_tokens, m]
     int32_t *sup_buf;  // [max_tokens, k]
     float *partial;    // [kGatherMaxTokens, nx_max, d] partial down-projections of the gather path
-    float *gram;       // [G, pitch] I - mu Phi^T Phi of the layer being recovered, pitch = 32 ceil(G/32)
+    float *gram;       // [G, pitch] I - mu Phi^T Phi of the layer being mask_count, pitch = 32 ceil(G/32)
     float *resid_buf;     // [max_tokens] residual norms when the caller wants none (confidence fallback)
     int32_t *fb_flags;    // [max_tokens] confidence fallback: 1 = the token's recovery is not trusted
     int32_t *fb_list;     // [max_tokens] those tokens, ascending
@@ -51,7 +51,7 @@ struct cs_plan {
     cs::DeviceStatus *status;  // device status word
     // tensor-core path (bf16 weights, 128-channel groups, d a multiple of 256)
     uint32_t *mask;      // [max_tokens, 4] membership bits: bit g of token t
-    unsigned *recovered; // [1] decode step: gate/up CTAs whose recoveries are done
+    unsigned *mask_count; // [1] decode batches: CTAs that have written their masks
     int32_t *counts;     // [G] tokens per group
     int32_t *offsets;    // [G + 1]
     int32_t *token_ids;  // [max_tokens * k] tokens of each group, ascending
@@ -132,7 +132,7 @@ struct RecoverArgs {
     const int32_t *check;
     int32_t *delta; float *drift;
     uint32_t *mask;
-    unsigned *recovered;       // decode batches: counts the CTAs whose recoveries are done
+    unsigned *mask_count;      // decode batches: counts the CTAs whose recoveries are done
     SketchParts parts;
     cs::DeviceStatus *status;
 };
@@ -206,9 +206,9 @@ cs_status prepare_decode(cs_plan *plan);
 int decode_slices(const cs_plan *plan);
 cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *support, int B, bool check, cudaStream_t st);
 // recover != NULL and decode_recovers(): the recovery runs inside the gate/up launch; otherwise the launches before have
-// left the masks (plan->mask).  norm: the row scales come from the sketch's partial squares.
+// left the masks (plan->mask); given: they are those of supports the caller gave (launch_decode_prep).  norm: the row scales come from the sketch's partial squares.
 bool decode_recovers(const cs_plan *plan);
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool norm,
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool given, bool norm,
                             const float *residual, float *out, cudaStream_t st);
 // Column sums of H per block of rows (plan->colsum); *blocks = their number.
 constexpr int kMeanRowBlocks = 16;

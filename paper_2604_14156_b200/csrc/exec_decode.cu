@@ -23,7 +23,7 @@
 // without work and took 39.7 us for 180 MB at 64 tokens).  The down GEMM has d / 256 column tiles times
 // as many list slices as fill the SMs, cut at 64-channel k blocks.
 //
-// Supports: gate/up computes every channel of every token and the down GEMM leaves out what a token's support does not
+// Supports: in a step gate/up computes every channel of every token and the down GEMM leaves out what a token's support does not
 // hold, by the instruction's lane mask (lanes = tokens, so a k block's mask is its group's membership bits; the
 // accumulators are zeroed first and only ever added to).  So nothing waits for the recovery before the down GEMM,
 // and the recovery runs inside the gate/up launch, in four warps of each CTA that take the tokens in turn.
@@ -31,8 +31,8 @@
 // launch) and streaming its weights before it waits for what the launch before produces.  With the recovery as a launch
 // ahead of gate/up the weight stream began 5.4 us after the step, in this form while the sketch still runs.
 // What an earlier launch of the step wrote is read behind a launch's own wait, since a trigger orders nothing in memory.  The
-// one exception are the masks in the down launch: the recoveries count themselves (release), and a CTA that finds the
-// count complete (acquire) may read them at once; a CTA that does not waits first.
+// one exception are the masks in the down launch: the CTAs that write them count themselves (release), and a down CTA that finds
+// the count complete (acquire) may read them at once; one that does not waits first.  The reduction sets the count back.
 #include "mma_core.cuh"
 #include "recover_core.cuh"
 
@@ -100,6 +100,28 @@ __device__ __forceinline__ uint4 ld_l2(const int32_t *p) {
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
+// This CTA's masks are written (and a barrier has joined the threads that wrote them).
+__device__ __forceinline__ void count_masks(unsigned *mask_count) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(mask_count) : "memory");
+}
+// Union of the tokens' supports (their masks are visible): union_s, zero before the barrier that precedes the call, is
+// complete behind the one that follows it.
+__device__ __forceinline__ void collect_union(const int32_t *mask, int B, uint32_t *union_s) {
+    for (int t = threadIdx.x; t < B; t += blockDim.x) {
+        const uint4 m = ld_l2(mask + (size_t)t * 4);
+        if (m.x) atomicOr(&union_s[0], m.x);
+        if (m.y) atomicOr(&union_s[1], m.y);
+        if (m.z) atomicOr(&union_s[2], m.z);
+        if (m.w) atomicOr(&union_s[3], m.w);
+    }
+}
+__device__ __forceinline__ int union_size(const uint32_t *u) { return __popc(u[0]) + __popc(u[1]) + __popc(u[2]) + __popc(u[3]); }
+__device__ __forceinline__ int union_rank(const uint32_t *u, int g) {   // groups of the union below g
+    int n = __popc(u[g >> 5] & ((1u << (g & 31)) - 1u));
+    for (int w = 0; w < (g >> 5); ++w) n += __popc(u[w]);
+    return n;
+}
+
 // The accumulator of one 128-row tile (columns tcol .. tcol + 16 nchunk) into shared memory, row-major with pitch P
 // floats; `rows` rows are wanted (PACK: from each half).
 template <bool PACK>
@@ -153,11 +175,16 @@ __device__ __forceinline__ void mma_kblock(uint32_t tmem, uint32_t a0, uint32_t 
 // ---- gate / up ------------------------------------------------------------------------------------------
 // CTA x: channels [x R, x R + R), and with KC > 0 (slots of the recovery's list form, in units of 8) the recovery of tokens
 // x, x + gridDim.x, ...
+// mask != NULL (KC == 0, MT == 2): the supports were given, and where it makes a CTA's share smaller the channels are those of
+// the groups in use only, in units of 16 that the CTAs share evenly (tm_gu, tm_uu: the weights in boxes of 16 rows).  Groups outside
+// the union keep what `act` held, and the down launch does not read them.
+constexpr int kListRows = 16;
 template <bool PACK, int MT, int KC>
 __global__ void __launch_bounds__(kDecThreads + kRecThreads, 1)
 decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
-                     const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u, int B, int R, int d,
-                     int d_ff, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
+                     const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u,
+                     const __grid_constant__ CUtensorMap tm_gu, const __grid_constant__ CUtensorMap tm_uu, int B, int R, int d, int d_ff,
+                     const int32_t *mask, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
                      __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ act_lo, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ float rscale_s[MT * BM];
@@ -165,16 +192,60 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const TokenTile tt = token_tile(PACK, MT, B);
     const int c0 = blockIdx.x * R;
-    const int wbytes = 2 * R * BK * 2;                   // gate rows then up rows
-    Barriers *bars = reinterpret_cast<Barriers *>(base + ring_bytes(tt, wbytes));
-    const int stage_bytes = tt.bytes + wbytes;
-    const int stages = ring_stages(tt, wbytes);
+    constexpr bool LIST = KC == 0 && MT == 2;
+    __shared__ uint32_t union_s[LIST ? 4 : 1];
+    __shared__ int unit_s[LIST ? BM / kListRows : 1];   // first channel of each unit of this CTA
+    bool by_list = LIST && mask != nullptr;
+    Barriers *bars = reinterpret_cast<Barriers *>(base + (by_list ? kDecRing : ring_bytes(tt, 2 * R * BK * 2)));
     const uint32_t tcols = MT == 2 ? 512u : 256u;
     const int kblocks = d / BK;
     if (threadIdx.x == 0) { prefetch_map(&tm_g); prefetch_map(&tm_u); prefetch_map(&tm_x); prefetch_map(&tm_x_lo); }
+    if (by_list && threadIdx.x < 4) union_s[threadIdx.x] = 0u;
     setup_cta(bars, warp, tcols);
+    int units = 0;
+    if constexpr (LIST) {
+        if (by_list) {
+            pdl_wait();
+            collect_union(mask, B, union_s);
+            __syncthreads();
+            constexpr int kUnits = 128 / kListRows;   // of a group
+            const int total = union_size(union_s) * kUnits, per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
+            by_list = per * kListRows < R;
+            if (by_list) {
+                const int u0 = blockIdx.x * per, g = threadIdx.x;
+                units = max(0, min(per, total - u0));
+                if (g < kMaxG && ((union_s[g >> 5] >> (g & 31)) & 1u)) {
+                    const int first = union_rank(union_s, g) * kUnits;
+                    for (int u = max(first, u0); u < min(first + kUnits, u0 + units); ++u) unit_s[u - u0] = g * 128 + (u - first) * kListRows;
+                }
+                __syncthreads();
+                R = units * kListRows;
+                if (units == 0) { teardown_cta(bars, warp, tcols); return; }
+            }
+        }
+    }
+    const int wbytes = 2 * R * BK * 2;                   // gate rows then up rows
+    const int stage_bytes = tt.bytes + wbytes;
+    const int stages = ring_stages(tt, wbytes);
 
-    if (warp == 0) {
+    if (warp == 0 && by_list) {   // lane u: the gate rows of unit u, lane 16 + u: its up rows (one lane for all: 47 ns a box)
+        const int tx = wbytes + token_tx_bytes(tt), u = lane & 15;
+        const uint64_t once = policy_evict_first();
+        const CUtensorMap *tm_w = lane < 16 ? &tm_gu : &tm_uu;
+        const int w_off = tt.bytes + (lane < 16 ? 0 : wbytes / 2) + u * (kListRows * BK * 2), ch = u < units ? unit_s[u] : 0;
+        int s = 0, ph = 1;
+        for (int kb = 0; kb < kblocks; ++kb) {
+            bool ok = true;
+            if (kb >= stages && lane == 0) ok = mbar_wait(&bars->empty[s], ph, bars, status);
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            uint8_t *st = base + (size_t)s * stage_bytes;
+            if (lane == 0) mbar_expect_tx(&bars->full[s], tx);
+            __syncwarp();
+            if (u < units) tma_load_2d(st + w_off, tm_w, kb * BK, ch, &bars->full[s], once);
+            if (lane == 0) load_tokens(tt, st, &tm_x, &tm_x_lo, kb * BK, &bars->full[s]);
+            if (++s == stages) { s = 0; ph ^= 1; }
+        }
+    } else if (warp == 0) {
         if (lane == 0) {
             const int tx = wbytes + token_tx_bytes(tt);
             const uint64_t once = policy_evict_first();
@@ -249,7 +320,7 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             if (ok) {
 #pragma unroll 2
                 for (int i = et; i < rows * r4; i += kEpiThreads) {
-                    const int r = i / r4, c = (i - r * r4) * 4, ch = c0 + c;
+                    const int r = i / r4, c = (i - r * r4) * 4, ch = by_list ? unit_s[c / kListRows] + c % kListRows : c0 + c;
                     if (ch >= d_ff) continue;
                     const float4 g = row4<PACK>(dump, P, r, c), u = row4<PACK>(dump, P, r, R + c);
                     const float sc = rscale_s[t0 + r];
@@ -277,7 +348,7 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         }
         // this CTA's masks are written (the barrier that ends the loop, or no token at all)
         if (g == 0) {
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ra.recovered) : "memory");
+            count_masks(ra.mask_count);
             pdl_launch_dependents();
         }
     }
@@ -286,13 +357,13 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 
 // ---- down -----------------------------------------------------------------------------------------------
 // grid (d / 256, slices).  The list is every group (use_union == 0) or the groups that are in some token's support; slice z
-// takes the 64-channel k blocks [z nk / Z, (z + 1) nk / Z) of it.  recovered: count of the gate/up CTAs whose recoveries are done
-// (set to zero by the step's sketch), complete at `recoveries` (0: the masks come from elsewhere).
+// takes the 64-channel k blocks [z nk / Z, (z + 1) nk / Z) of it.  mask_count: the CTAs that have written their masks, all of them
+// at mask_ctas (0: not counted).
 template <bool PACK, int MT>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_constant__ CUtensorMap tm_act,
-                   const __grid_constant__ CUtensorMap tm_act_lo, const int32_t *mask, const unsigned *recovered,
-                   unsigned recoveries, int use_union, int B, int G, int d, float *__restrict__ partial, DeviceStatus *status) {
+                   const __grid_constant__ CUtensorMap tm_act_lo, const int32_t *mask, const unsigned *mask_count,
+                   unsigned mask_ctas, int use_union, int B, int G, int d, float *__restrict__ partial, DeviceStatus *status) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t union_s[4], masks_s;
     __shared__ int glist_s[kMaxG];                          // groups of this slice, in list order
@@ -311,23 +382,17 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
     if (threadIdx.x < 4) union_s[threadIdx.x] = 0u;
     if (threadIdx.x == 64) {
         unsigned n = 0u;
-        if (recoveries != 0u) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(recovered) : "memory");
-        masks_s = recoveries != 0u && n == recoveries;
+        if (mask_ctas != 0u) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(mask_count) : "memory");
+        masks_s = mask_ctas != 0u && n == mask_ctas;
     }
     setup_cta(bars, warp, tcols);
     const bool masks_ready = masks_s != 0u;   // (behind a barrier, as the masks of the other threads' reads)
     if (use_union && !masks_ready) pdl_wait();
     int ng = G;
     if (use_union) {
-        for (int t = threadIdx.x; t < B; t += kDecThreads) {
-            const uint4 m = ld_l2(mask + (size_t)t * 4);
-            if (m.x) atomicOr(&union_s[0], m.x);
-            if (m.y) atomicOr(&union_s[1], m.y);
-            if (m.z) atomicOr(&union_s[2], m.z);
-            if (m.w) atomicOr(&union_s[3], m.w);
-        }
+        collect_union(mask, B, union_s);
         __syncthreads();
-        ng = __popc(union_s[0]) + __popc(union_s[1]) + __popc(union_s[2]) + __popc(union_s[3]);
+        ng = union_size(union_s);
     }
     const int nk = 2 * ng;
     const int k0 = (int)((long long)nk * z / Z), kblocks = (int)((long long)nk * (z + 1) / Z) - k0;
@@ -338,8 +403,7 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
         bool in = true;
         if (use_union) {
             in = (union_s[g >> 5] >> (g & 31)) & 1u;
-            pos = __popc(union_s[g >> 5] & ((1u << (g & 31)) - 1u));
-            for (int w = 0; w < (g >> 5); ++w) pos += __popc(union_s[w]);
+            pos = union_rank(union_s, g);
         }
         if (in && pos >= l0 && pos < l0 + nl) glist_s[pos - l0] = g;
     }
@@ -442,10 +506,11 @@ decode_down_kernel(const __grid_constant__ CUtensorMap tm_wd, const __grid_const
 // out[t, :] = residual[t, :] + sum_z partial[z, t, :], slices added in index order, all loads of a thread in flight at once.
 constexpr int kReduceThreads = 256;
 __global__ void __launch_bounds__(kReduceThreads)
-decode_reduce_kernel(const float *__restrict__ partial, int Z, int n4, const float *residual, float *out) {
+decode_reduce_kernel(const float *__restrict__ partial, int Z, int n4, const float *residual, float *out, unsigned *mask_count) {
     pdl_launch_dependents();
     const int i = blockIdx.x * kReduceThreads + threadIdx.x;
     pdl_wait();
+    if (i == 0) *mask_count = 0u;
     if (i >= n4) return;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (residual != nullptr) s = ld_dep4(residual + 4 * (size_t)i);
@@ -466,7 +531,7 @@ constexpr int kPrepThreads = 256;
 __global__ void __launch_bounds__(kPrepThreads)
 decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ support, int d, int k, int G,
                    __nv_bfloat16 *__restrict__ x_hi, __nv_bfloat16 *__restrict__ x_lo, int32_t *__restrict__ mask, int check,
-                   DeviceStatus *status) {
+                   unsigned *mask_count, DeviceStatus *status) {
     __shared__ uint32_t m_s[4];
     const int t = blockIdx.x, tid = threadIdx.x;
     pdl_launch_dependents();
@@ -491,9 +556,12 @@ decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ supp
     }
     __syncthreads();
     if (tid < 4) mask[(size_t)t * 4 + tid] = (int)m_s[tid];
+    __syncthreads();
+    if (tid == 0) count_masks(mask_count);
 }
 
-typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, const float *, float,
+typedef void (*GateUpFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int,
+                         const int32_t *, const float *, float,
                          RecoverArgs, __nv_bfloat16 *, __nv_bfloat16 *, DeviceStatus *);
 typedef void (*DownFn)(CUtensorMap, CUtensorMap, CUtensorMap, const int32_t *, const unsigned *, unsigned, int, int, int, int, float *,
                        DeviceStatus *);
@@ -537,13 +605,13 @@ cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *suppo
     const cs_config &c = plan->cfg;
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
     launch_pdl(true, decode_prep_kernel, dim3(B), dim3(kPrepThreads), 0, st, h, support, c.d, c.k, plan->G, h ? x_hi : nullptr,
-               x_hi + (size_t)c.max_tokens * c.d, (int32_t *)plan->mask, check ? 1 : 0, plan->status);
+               x_hi + (size_t)c.max_tokens * c.d, (int32_t *)plan->mask, check ? 1 : 0, plan->mask_count, plan->status);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
     return CS_OK;
 }
 
-cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool norm,
+cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const RecoverArgs *recover, bool given, bool norm,
                             const float *residual, float *out, cudaStream_t st) {
     const cs_config &c = plan->cfg;
     const bool pack = B <= 64;
@@ -553,8 +621,14 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     const int gateup_ctas = (c.d_ff + R - 1) / R;
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16), *x_lo = x_hi + (size_t)c.max_tokens * c.d;
     __nv_bfloat16 *act = static_cast<__nv_bfloat16 *>(plan->act), *act_lo = act + (size_t)c.max_tokens * c.d_ff;
-    CUtensorMap tm_g, tm_u, tm_x, tm_x_lo, tm_wd, tm_act, tm_act_lo;
+    // Given supports, more than 128 tokens: gate/up over the groups in use.  There a channel costs more than its bytes (7B, 200
+    // tokens on the same 22 groups 82.7 us against 128.7, on 44 of the 86 93.2 against 127.6, on all of them 129.4 against 129.5).  Up to 128 tokens
+    // the weights requested ahead of the masks are worth as much as the groups left out (5 to 20 tokens on the same quarter
+    // of the groups 42 to 46 us either way; on independent supports 47 to 54 with every group, 55 to 64 by the list).
+    const bool by_list = given && mt == 2;
+    CUtensorMap tm_g, tm_u, tm_gu = {}, tm_uu = {}, tm_x, tm_x_lo, tm_wd, tm_act, tm_act_lo;
     if (!make_map(&tm_g, L->W_gate, c.d, c.d_ff, c.d, R) || !make_map(&tm_u, L->W_up, c.d, c.d_ff, c.d, R) ||
+        (by_list && (!make_map(&tm_gu, L->W_gate, c.d, c.d_ff, c.d, kListRows) || !make_map(&tm_uu, L->W_up, c.d, c.d_ff, c.d, kListRows))) ||
         !make_map(&tm_x, x_hi, c.d, B, c.d, tt.box) || !make_map(&tm_x_lo, x_lo, c.d, B, c.d, tt.box) ||
         !make_map(&tm_wd, L->Wd_t, c.d, c.d_ff, c.d, BK) || !make_map(&tm_act, act, c.d_ff, B, c.d_ff, tt.box) ||
         !make_map(&tm_act_lo, act_lo, c.d_ff, B, c.d_ff, tt.box))
@@ -562,8 +636,9 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
         launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
-                   dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), decode_smem(tt, 2 * R * BK * 2), st, tm_x, tm_x_lo, tm_g,
-                   tm_u, B, R, c.d, c.d_ff, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
+                   dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), by_list ? 1024 + (size_t)kDecRing + sizeof(Barriers) : decode_smem(tt, 2 * R * BK * 2),
+                   st, tm_x, tm_x_lo, tm_g, tm_u, tm_gu, tm_uu, B, R, c.d, c.d_ff,
+                   by_list ? (const int32_t *)plan->mask : (const int32_t *)nullptr, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
                    c.rms_eps, recover != nullptr ? *recover : RecoverArgs{}, act, act_lo, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
@@ -573,10 +648,10 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
         StageTimer timer(plan, CS_STAGE_EXEC2, st);
         // Expected number of groups in nobody's support, G (1 - k/G)^B: below a quarter group the list is every group and
         // the masks need not be read.
-        const bool use_union = (float)plan->G * powf(1.f - (float)c.k / plan->G, (float)B) > 0.25f;
+        const bool use_union = by_list || (float)plan->G * powf(1.f - (float)c.k / plan->G, (float)B) > 0.25f;
         launch_pdl(true, down_fn(form), dim3(c.d / kDecBN, Z), dim3(kDecThreads), decode_smem(tt, kDecBN * BK * 2), st, tm_wd, tm_act,
-                   tm_act_lo, (const int32_t *)plan->mask, (const unsigned *)plan->recovered,
-                   recover != nullptr ? (unsigned)gateup_ctas : 0u, use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
+                   tm_act_lo, (const int32_t *)plan->mask, (const unsigned *)plan->mask_count,
+                   recover != nullptr ? (unsigned)gateup_ctas : given ? (unsigned)B : 0u, use_union ? 1 : 0, B, plan->G, c.d, plan->mma_partial, plan->status);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }
@@ -584,7 +659,7 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
         StageTimer timer(plan, CS_STAGE_REDUCE, st);
         const int n4 = B * c.d / 4;
         launch_pdl(true, decode_reduce_kernel, dim3((n4 + kReduceThreads - 1) / kReduceThreads), dim3(kReduceThreads), 0, st,
-                   (const float *)plan->mma_partial, Z, n4, residual, out);
+                   (const float *)plan->mma_partial, Z, n4, residual, out, plan->mask_count);
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }

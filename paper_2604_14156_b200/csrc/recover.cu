@@ -303,7 +303,7 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
     a.sup0 = o.sup0; a.z0 = o.z0; a.sup_prev = o.sup_prev; a.z_prev = o.z_prev;
     a.check = o.check; a.delta = o.delta; a.drift = o.drift;
     if (o.decode) {
-        a.mask = plan->mask; a.recovered = plan->recovered;
+        a.mask = plan->mask; a.mask_count = plan->mask_count;
         a.parts = SketchParts{sketch_partials(plan), o.norm ? sketch_square_partials(plan, B) : nullptr, c.d / 64, B, c.d, c.rms_eps,
                               plan->y_buf};
     }

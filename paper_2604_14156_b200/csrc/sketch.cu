@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kSketchThreads)
 sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, const float *__restrict__ gamma, int m, int d, int B,
                      float *__restrict__ y_part, float *__restrict__ ss_part, __nv_bfloat16 *__restrict__ x_hi,
                      __nv_bfloat16 *__restrict__ x_lo, const float *__restrict__ Phi, float mu, int G, float *__restrict__ gram,
-                     unsigned *recovered) {
+                     unsigned *mask_count) {
     extern __shared__ float4 slice_s[];   // x rows, then S rows: small enough to sit beside a decode GEMM's CTA
     const int slices = d / kSliceCols, tiles = (B + kSliceTokens - 1) / kSliceTokens;
     const int tid = threadIdx.x;
@@ -230,7 +230,7 @@ sketch_slices_kernel(const float *__restrict__ S, const float *__restrict__ x, c
         Ss[r * (kSlicePitch / 4) + q] = __ldg(reinterpret_cast<const float4 *>(S + (size_t)r * d + c0) + q);
     const float4 gm = gamma != nullptr ? __ldg(reinterpret_cast<const float4 *>(gamma + c0) + q) : make_float4(1.f, 1.f, 1.f, 1.f);
     pdl_wait();
-    if (blockIdx.x == 0 && tid == 0) *recovered = 0u;   // the recoveries of this step count from here
+    if (blockIdx.x == 0 && tid == 0) *mask_count = 0u;   // the recoveries of this step count from here
     float4 v[kSliceTokens / RS];
 #pragma unroll
     for (int i = 0; i < kSliceTokens / RS; ++i) {
@@ -292,7 +292,7 @@ cs_status launch_sketch_slices(cs_plan *plan, const cs_layer *L, const float *x,
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
     launch_pdl(true, sketch_slices_kernel, dim3(slices * tiles + gram_blocks(plan->G)), dim3(kSketchThreads),
                (size_t)(min(kSliceTokens, B) + c.m) * kSlicePitch * sizeof(float), st, L->S, x, L->rms_gamma, c.m, c.d, B, sketch_partials(plan), sketch_square_partials(plan, B), x_hi,
-               x_hi + (size_t)c.max_tokens * c.d, L->Phi, L->mu, plan->G, plan->gram, plan->recovered);
+               x_hi + (size_t)c.max_tokens * c.d, L->Phi, L->mu, plan->G, plan->gram, plan->mask_count);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
     return CS_OK;

@@ -1,11 +1,13 @@
 """GPU parity of the tensor-core decode path (up to 256 tokens) at the sizes where its tiling can go wrong."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2604_14156_b200 as cs
 
 from gen import workloads as W
-from parity_util import compare_layer_step, device_layer, make_plan
+from parity_util import TIGHT_TOL, compare_layer_step, device_layer, make_plan, rel
 
 pytestmark = pytest.mark.gpu
 
@@ -109,4 +111,47 @@ def test_back_to_back_steps_on_changing_tokens(k, B):
         for a, b in zip(run, alone[i % 4]):
             assert torch.equal(a, b), i
     assert plan.device_status() == 0
+    plan.close()
+
+
+# Given supports; beyond 128 tokens gate/up runs over the groups in use (units of 16 channels shared by the CTAs).  One group, a few,
+# an odd number, every group; fewer units than CTAs (3 groups), several a CTA, and a share no smaller than without the list; the
+# three token forms.  Weights of the other groups are NaN: nothing of them may reach the output.
+@pytest.mark.parametrize("G,k,used", [(3, 1, 1), (3, 2, 3), (40, 2, 5), (101, 3, 7), (101, 3, 101), (128, 6, 33)])
+@pytest.mark.parametrize("B", [4, 33, 64, 65, 129, 193, 256])
+def test_ffn_exec_over_the_groups_in_use(G, k, used, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(d=512, d_ff=128 * G, m=9, k=k, T=4, B=B, index=500 + G)
+    L = W.make_layer(cfg, device="cuda:0")
+    rng = np.random.default_rng(B + used)
+    groups = np.sort(rng.permutation(G)[:used])
+    sup = np.sort(np.stack([rng.permutation(groups)[:k] for _ in range(B)]), axis=1).astype(np.int32)
+    Lc = L.to("cpu")
+    unused = torch.ones(G, dtype=torch.bool); unused[torch.from_numpy(np.unique(sup)).long()] = False
+    rows = unused.repeat_interleave(128).to("cuda:0")
+    for w in (L.W_gate, L.W_up, L.Wd_t):
+        w[rows] = float("nan")
+    h = W.make_tokens(cfg, L.A).h
+    plan = make_plan(cfg)
+    plan.set_crossover(2)
+    out = cs.cs_ffn_exec(plan, device_layer(plan, L), h.to("cuda:0"), torch.from_numpy(sup).to("cuda:0")).cpu().numpy()
+    assert plan.device_status() == 0
+    for t in sorted({0, 1, 63 % B, 64 % B, 127 % B, 128 % B, B // 2, B - 1}):
+        ref = oracle.ffn(Lc.W_gate, Lc.W_up, Lc.Wd_t, cfg.group, h[t].double().numpy(), sup[t])
+        assert rel(out[t], ref) <= TIGHT_TOL["bf16"], t   # f32 activations (parity_util)
+    plan.close()
+
+
+def test_ffn_exec_time_follows_the_groups_in_use():
+    """200 tokens on the same 6 of 86 groups stream a fourteenth of the weights of 200 tokens on all of them."""
+    cfg = W.CONFIGS["l2_7b_b64"].with_(B=200, k=6)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    lay = device_layer(plan, L)
+    h = W.make_tokens(cfg, L.A).h.to("cuda:0")
+    out = torch.empty_like(h)
+    us = {}
+    for name, stride in (("six", 0), ("all", 6)):
+        sup = torch.stack([(torch.arange(6) + stride * t) % 86 for t in range(200)]).sort(dim=1).values.int().to("cuda:0")
+        us[name] = _replay_us(lambda: cs.cs_ffn_exec(plan, lay, h, sup, out=out))
+    assert us["six"] <= 0.75 * us["all"], us
     plan.close()
