@@ -879,6 +879,23 @@ def test_layer_step_host_matches_device_entry(name, B, pinned):
     plan.close()
 
 
+def test_layer_step_host_beyond_the_decode_batches_crosses_the_bus_in_the_kernels():
+    """300 page-locked tokens of 2.4 MB: a staging launch more than the device entry, and its result bit for bit."""
+    cfg = W.CONFIGS["l2_7b_b64"].with_(B=300, d=2048, d_ff=128 * 24, k=6, m=12)
+    L = _layer(cfg)
+    plan = make_plan(cfg)
+    lay = device_layer(plan, L)
+    x = W.make_tokens(cfg, L.A).h
+    n0 = plan.launches
+    ref = cs.cs_layer_step(plan, lay, x.to(DEV))[0].cpu()
+    n1 = plan.launches
+    out = torch.empty_like(x).pin_memory()
+    cs.cs_layer_step_host(plan, lay, x.pin_memory(), out)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref) and plan.launches - n1 == n1 - n0 + 1
+    plan.close()
+
+
 def test_layer_step_host_chained_through_one_buffer():
     """Three layers chained through ONE pinned buffer with no synchronisation in between: layer i stores
     its result into the buffer layer i + 1 reads, so the staging load must respect stream order."""
