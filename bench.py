@@ -329,13 +329,14 @@ def bench_decode(cfg, args, K, Wm, rank, world, local, dev, primary):
                                        "partial-sum reduction around them, so an upper bound of the kernels' own time"),
                      "bracket_us": (stage_ms[2] + stage_ms[4]) * 1e3,
                      "traffic": NCU_TRAFFIC.get((cfg.name, cfg.k)) if cfg.B == W.CONFIGS[cfg.name].B else None},
-        "stages_us": {"sketch": stage_ms[0] * 1e3, "recover": stage_ms[1] * 1e3, "exec": stage_ms[2] * 1e3,
+        "stages_us": {"sketch": stage_ms[0] * 1e3, "recover": stage_ms[1] * 1e3 or None, "exec": stage_ms[2] * 1e3,
                       "exec_down": stage_ms[4] * 1e3, "reduce": stage_ms[3] * 1e3, "step_net": step_us,
-                      "note": "stage figures are event brackets inside one-step graphs (2-4 us of record overhead each); "
-                              "from the crossover batch on the recovery runs inside the gate/up launch (exec), below "
-                              "it inside the sketch's",
-                      "measure_recover_per_token": mr_us / cfg.B,
-                      "measure_recover_share_of_step": mr_us / step_us if step_us > 0 else None,
+                      "note": "stage figures are event brackets inside one-step graphs (2-4 us of record overhead each, so "
+                              "those of a short step add up to more than the step); from the crossover batch on the recovery "
+                              "runs inside the gate/up launch (exec), below it inside the sketch's, and recover is then null",
+                      # what the brackets show of measure + recover: not the part inside gate/up
+                      "measure_recover_per_token": mr_us / cfg.B if not mma else None,
+                      "measure_recover_share_of_step": mr_us / step_us if step_us > 0 and not mma else None,
                       "exec_only_step": exec_only_us,
                       # what sketch + recovery leave on the critical path: net step minus the actuator alone
                       "measure_recover_exposed_us": max(0.0, step_us - exec_only_us),
@@ -440,7 +441,7 @@ def bench_prompt(cfg, args, K, Wm, rank, world, local, dev, primary):
                      "duration_from": "cs_ffn_exec_shared on a given support, timed like the step (CUDA events, median of repeats)",
                      "bracket_us": stage_ms[2] * 1e3,
                      "traffic": NCU_TRAFFIC.get((cfg.name, cfg.k))},
-        "stages_us": {"mean_sketch": stage_ms[0] * 1e3, "recover": stage_ms[1] * 1e3, "exec": stage_ms[2] * 1e3,
+        "stages_us": {"mean_sketch": stage_ms[0] * 1e3, "recover": stage_ms[1] * 1e3 or None, "exec": stage_ms[2] * 1e3,
                       "reduce": stage_ms[3] * 1e3, "step_net": step_us, "exec_only_step": exec_us,
                       "measure_recover_exposed_share": max(0.0, step_us - exec_us) / step_us},
     }

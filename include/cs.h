@@ -371,7 +371,11 @@ cs_status cs_plan_set_speculative(cs_plan *plan, int32_t on);
  * Stage timing (the paper asks for sensing / recovery overhead to be reported apart from the
  * sparse kernel itself, Sec. 15 metric suite).  While enabled, every launch of a stage is bracketed
  * by CUDA events on the call's stream.  cs_plan_stage_times synchronises `stream` and returns the
- * device time in milliseconds of each stage's kernels in the most recent call that ran it.
+ * device time in milliseconds of each stage's kernels in the most recent call that ran it (0: none since timing was enabled).
+ * A launch that does the work of two stages counts for one of them: cs_layer_step's recovery (and cs_layer_step_ex's with
+ * CS_SOLVER_IHT and the dense sketch, and cs_prompt_support's) is part of CS_STAGE_SKETCH where sensor and estimator are
+ * one launch (small batches, prompts) and of CS_STAGE_EXEC where it runs beside the gate/up GEMM (tensor-core batches of at
+ * most 256 tokens with k <= 64); CS_STAGE_RECOVER then reads 0, whatever an earlier call left there.
  */
 enum { CS_STAGE_SKETCH = 0, CS_STAGE_RECOVER = 1, CS_STAGE_EXEC = 2, CS_STAGE_REDUCE = 3,
        CS_STAGE_EXEC2 = 4 /* down GEMM of the tensor-core decode path */, CS_STAGE_COUNT = 5 };

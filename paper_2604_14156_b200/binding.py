@@ -200,7 +200,8 @@ class Plan:
 
     def stage_times(self, stream=None):
         """Milliseconds of (sketch, recover, exec, reduce, exec2) in the most recent call; exec2 is
-        the down GEMM of the tensor-core decode path (0 otherwise)."""
+        the down GEMM of the tensor-core decode path (0 otherwise), recover is 0 where the recovery is part of
+        the sketch's launch or of exec's (see include/cs.h)."""
         ms = (ctypes.c_float * 5)()
         self.check(self.lib.cs_plan_stage_times(self.handle, _stream(stream), ctypes.byref(ms)),
                    "cs_plan_stage_times")

@@ -635,6 +635,7 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
         return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
+        if (recover != nullptr) plan->stage_seen[CS_STAGE_RECOVER] = 0;   // part of this launch
         launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
                    dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), by_list ? 1024 + (size_t)kDecRing + sizeof(Barriers) : decode_smem(tt, 2 * R * BK * 2),
                    st, tm_x, tm_x_lo, tm_g, tm_u, tm_gu, tm_uu, B, R, c.d, c.d_ff,

@@ -342,6 +342,7 @@ cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, 
     SenseArgs sa{S, x, gamma, c.rms_eps, c.d, min(c.m, (kSenseSmem - fixed) / row_bytes - 1), plan->y_buf, n_out, blocks, 1.f / (float)n};
     {
         StageTimer timer(plan, CS_STAGE_SKETCH, st);
+        plan->stage_seen[CS_STAGE_RECOVER] = 0;   // part of this launch
         launch_pdl(true, sense_fn(plan->G, c.k), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)(sa.s_rows + (blocks > 0)) * row_bytes, st,
                    sa, recover_args(plan, Phi, mu, nullptr, B, support, z, resid, o));
     }

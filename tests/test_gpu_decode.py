@@ -155,3 +155,21 @@ def test_ffn_exec_time_follows_the_groups_in_use():
         us[name] = _replay_us(lambda: cs.cs_ffn_exec(plan, lay, h, sup, out=out))
     assert us["six"] <= 0.75 * us["all"], us
     plan.close()
+
+
+def test_stage_times_of_a_fused_step_forget_an_earlier_recovery():
+    """The recovery inside the sensing launch (3 tokens) or the gate/up launch (40) has no time of its own, not an earlier call's."""
+    cfg = W.CONFIGS["l2_7b_b64"].with_(d=512, d_ff=128 * 20, m=9, k=5, T=6, B=40, index=520)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    lay = device_layer(plan, L)
+    x = W.make_tokens(cfg, L.A).h.to("cuda:0")
+    plan.enable_timing()
+    for B, fused in ((3, 0), (40, 2)):
+        y = cs.cs_sketch(plan, L.S, x[:B].contiguous())
+        cs.cs_recover(plan, L.Phi, L.mu, y)
+        assert plan.stage_times()[1] > 0.0
+        cs.cs_layer_step(plan, lay, x[:B].contiguous())
+        ms = plan.stage_times()
+        assert ms[1] == 0.0 and ms[fused] > 0.0, (B, ms)
+    plan.close()
