@@ -130,10 +130,16 @@ def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str, shape=None) -
     return t.data_ptr()
 
 
+# torch's own accessors of the current stream's handle, which it does not promise to keep; without them the public one serves
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
-        if torch.cuda.is_initialized():   # the handle itself: building a Stream object takes 3 us of a 24 us call
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        # the handle itself: building a Stream object takes 3 us of a 24 us call
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 

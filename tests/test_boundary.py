@@ -66,3 +66,19 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "_LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(ImportError):
         binding.load_library()
+
+
+def test_stream_handle_without_torchs_raw_accessors(monkeypatch):
+    from paper_2604_14156_b200 import binding
+
+    class Current:
+        cuda_stream = 1234
+    monkeypatch.setattr(binding.torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: Current)
+    for name in ("_raw_stream", "_current_device"):
+        with monkeypatch.context() as m:
+            m.setattr(binding, name, None)
+            assert binding._stream(None) == 1234
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 77 + device)
+    monkeypatch.setattr(binding, "_current_device", lambda: 1)
+    assert binding._stream(None) == 78 and binding._stream(Current) == 1234
