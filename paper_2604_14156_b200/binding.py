@@ -165,15 +165,20 @@ class Plan:
         self.handle = handle
 
     def outputs(self, B: int, device):
-        """New (support [B,k], z [B,k], resid [B]) for a call's outputs.  Allocated like empty templates that are kept per
-        batch size: half the host time of naming shape, type and device each time."""
+        """New (support [B,k], z [B,k], resid [B]) for a call's outputs.  Allocated like templates that are kept per batch
+        size: half the host time of naming shape, type and device each time.  A template is one element (strides 0), and none
+        is made during a graph capture, whose memory pool it would keep alive."""
         t = self._templates.get((B, device))
         if t is None:
+            if device.type == "cuda" and torch.cuda.is_current_stream_capturing():
+                return (torch.empty((B, self.k), dtype=torch.int32, device=device),
+                        torch.empty((B, self.k), dtype=torch.float32, device=device),
+                        torch.empty((B,), dtype=torch.float32, device=device))
             if len(self._templates) >= 64:
                 self._templates.clear()
-            t = (torch.empty((B, self.k), dtype=torch.int32, device=device),
-                 torch.empty((B, self.k), dtype=torch.float32, device=device),
-                 torch.empty((B,), dtype=torch.float32, device=device))
+            t = (torch.empty_strided((B, self.k), (0, 0), dtype=torch.int32, device=device),
+                 torch.empty_strided((B, self.k), (0, 0), dtype=torch.float32, device=device),
+                 torch.empty_strided((B,), (0,), dtype=torch.float32, device=device))
             self._templates[(B, device)] = t
         return torch.empty_like(t[0]), torch.empty_like(t[1]), torch.empty_like(t[2])
 

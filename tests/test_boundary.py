@@ -82,3 +82,22 @@ def test_stream_handle_without_torchs_raw_accessors(monkeypatch):
     monkeypatch.setattr(binding, "_raw_stream", lambda device: 77 + device)
     monkeypatch.setattr(binding, "_current_device", lambda: 1)
     assert binding._stream(None) == 78 and binding._stream(Current) == 1234
+
+
+def test_output_templates_hold_one_element_and_give_contiguous_outputs():
+    import torch
+
+    import paper_2604_14156_b200 as cs
+    plan = object.__new__(cs.Plan)
+    plan.handle, plan._templates = None, {}
+    for k in (1, 5, 22):
+        plan.k = k
+        plan._templates.clear()
+        for B in range(1, 130):
+            for _ in range(2):   # a new template, a kept one
+                support, z, resid = plan.outputs(B, torch.device("cpu"))
+                assert support.dtype == torch.int32 and z.dtype == resid.dtype == torch.float32
+                assert support.shape == z.shape == (B, k) and resid.shape == (B,)
+                assert all(t.is_contiguous() and t.untyped_storage().nbytes() == 4 * t.numel() for t in (support, z, resid))
+        assert len(plan._templates) <= 64
+        assert all(t.untyped_storage().nbytes() == 4 for ts in plan._templates.values() for t in ts)
