@@ -1,9 +1,10 @@
 // Actuator, tensor-core regime for decode batches of at most kDecodeMaxTokens tokens with independent supports.
 //
-//   decode_gateup_kernel   act[t, c] = silu(n_t . W_gate[c]) (n_t . W_up[c]) for every channel c, zero where the
-//                          channel's group is not in the token's support
-//   decode_down_kernel     partial[z, t, :] = sum over the channels of list slice z of act[t, c] Wd_t[c, :]
-//   reduce_slices_kernel   out = residual + sum_z partial
+//   decode_gateup_kernel   act[t, c] = silu(n_t . W_gate[c]) (n_t . W_up[c]) for every token t and channel c, in its support
+//                          or not
+//   decode_down_kernel     partial[z, t, :] = sum over the channels of list slice z that are in t's support of
+//                          act[t, c] Wd_t[c, :]
+//   decode_reduce_kernel   out = residual + sum_z partial
 //
 // Both GEMMs put the tokens on the M side of the MMA and stream the weights as its N operand: at these batch sizes
 // the step is bound by the weight bytes (HBM), and what limits a kernel before that is shared memory, which every
@@ -526,7 +527,7 @@ decode_reduce_kernel(const float *__restrict__ partial, int Z, int n4, const flo
 }
 
 // ---- given supports: operand split and membership masks (one CTA per token) --------------------------------
-// check: validates the support row (ascending, distinct, in range).  x_hi == NULL: masks only.
+// check: validates the support row (ascending, distinct, in range).
 constexpr int kPrepThreads = 256;
 __global__ void __launch_bounds__(kPrepThreads)
 decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ support, int d, int k, int G,
@@ -545,14 +546,12 @@ decode_prep_kernel(const float *__restrict__ h, const int32_t *__restrict__ supp
         if (check && (!in || (tid > 0 && ld_dep(support + (size_t)t * k + tid - 1) >= g)))
             atomicCAS(&status->code, 0, (int)CS_ERR_SUPPORT);
     }
-    if (x_hi != nullptr) {
-        for (int c = tid; c < d / 4; c += kPrepThreads) {
-            const float4 v = ld_dep4(h + (size_t)t * d + 4 * (size_t)c);
-            uint2 hi, lo;
-            split4(v.x, v.y, v.z, v.w, hi, lo);
-            reinterpret_cast<uint2 *>(x_hi + (size_t)t * d)[c] = hi;
-            reinterpret_cast<uint2 *>(x_lo + (size_t)t * d)[c] = lo;
-        }
+    for (int c = tid; c < d / 4; c += kPrepThreads) {
+        const float4 v = ld_dep4(h + (size_t)t * d + 4 * (size_t)c);
+        uint2 hi, lo;
+        split4(v.x, v.y, v.z, v.w, hi, lo);
+        reinterpret_cast<uint2 *>(x_hi + (size_t)t * d)[c] = hi;
+        reinterpret_cast<uint2 *>(x_lo + (size_t)t * d)[c] = lo;
     }
     __syncthreads();
     if (tid < 4) mask[(size_t)t * 4 + tid] = (int)m_s[tid];
@@ -604,7 +603,7 @@ cs_status prepare_decode(cs_plan *plan) {
 cs_status launch_decode_prep(cs_plan *plan, const float *h, const int32_t *support, int B, bool check, cudaStream_t st) {
     const cs_config &c = plan->cfg;
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16);
-    launch_pdl(true, decode_prep_kernel, dim3(B), dim3(kPrepThreads), 0, st, h, support, c.d, c.k, plan->G, h ? x_hi : nullptr,
+    launch_pdl(true, decode_prep_kernel, dim3(B), dim3(kPrepThreads), 0, st, h, support, c.d, c.k, plan->G, x_hi,
                x_hi + (size_t)c.max_tokens * c.d, (int32_t *)plan->mask, check ? 1 : 0, plan->mask_count, plan->status);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());

@@ -9,12 +9,10 @@
 //   then out = residual + sum over slices of P (reduce_slices_kernel).
 //
 // The same kernels serve both uses of the paper's method: the prompt-level variant (one support
-// shared by every token: list = that support, no mask) and large decode batches with independent
-// supports (list = union of the supports, mask = which token owns which group).  With at most 128
-// tokens a single 128-row MMA tile holds every token, so "bucketing tokens by group" costs nothing
-// extra: the bucket of a group is the set of rows whose mask bit is set, and rows outside the bucket
-// are zeroed in the epilogue.  (Smaller MMA tiles would not be cheaper: the instruction's cost is
-// set by the 128-row weight operand it reads from shared memory.)
+// shared by every token: list = that support, no mask; its gate/up kernels are ffn_gateup_tiles_kernel and
+// ffn_gateup_pair_kernel) and decode batches of more than 256 tokens with independent supports (list =
+// union of the supports, mask = which token owns which group: the rows of a tile that do not own the
+// group are zeroed in the epilogue).  Smaller decode batches take exec_decode.cu.
 //
 // Operand layouts (all 128-byte swizzled, written by TMA, read through shared-memory descriptors):
 //   X, act, W_gate, W_up tiles are K-major: [rows][64 k] with 128-byte rows, 8-row swizzle atoms.
@@ -107,14 +105,14 @@ __device__ __forceinline__ void mma_loop(const Tiles<SPLIT> &t, int kblocks, Dev
 
 }  // namespace
 
-// ---- gate / up --------------------------------------------------------------------------------
-template <bool SPLIT>
+// ---- gate / up over a union list, f32 activations as two bf16 parts ------------------------------
 __global__ void __launch_bounds__(kTileThreads, 1)
 ffn_gateup_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
                       const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u,
                       const int32_t *__restrict__ glist, const int32_t *__restrict__ ng_dev, int ng_host, int M,
                       int d, int act_ld, const uint32_t *__restrict__ mask, __nv_bfloat16 *__restrict__ act,
                       __nv_bfloat16 *__restrict__ act_lo, DeviceStatus *status) {
+    constexpr bool SPLIT = true;
     constexpr int kStages = Ring<SPLIT>::kStages;
     extern __shared__ uint8_t smem_raw[];
     const int gi = blockIdx.x, mt = blockIdx.y;
@@ -846,8 +844,7 @@ cs_status prepare_ffn_mma(cs_plan *plan) {
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
+    CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_gateup_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(ffn_down_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmem));
     return CS_OK;
@@ -864,8 +861,8 @@ cs_status launch_bucket(cs_plan *plan, const int32_t *support, int B, cudaStream
     return CS_OK;
 }
 
-// X [M, d] bf16 (plus X_lo, the bf16 remainder, when split precision is wanted); list / count on the
-// device (ng_dev) or count on the host; mask may be NULL.  Writes out [M, d] as f32 (out_f32) or bf16
+// X [M, d] bf16 with X_lo, its bf16 remainder: the list, its length (ng_dev) and the masks are on the device.  Without X_lo: one
+// support shared by all rows, its length known on the host (ng_host; ng_dev and mask NULL).  Writes out [M, d] as f32 (out_f32) or bf16
 // (out_bf16), plus residual (f32, may be NULL).
 cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const void *X_lo, int M,
                          const int32_t *glist, const int32_t *ng_dev, int ng_host, const uint32_t *mask,
@@ -888,8 +885,7 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
     // schedule of this shape, computed once); none leaves the launch to the single-tile kernel.
     int n_pair = 0;
     const int slots = ng_host * ((mtiles + 1) / 2);
-    const bool shared = !split && ng_dev == nullptr && mask == nullptr && ng_host > 0;
-    if (shared) {
+    if (!split) {
         if (plan->pair_key_ng != ng_host || plan->pair_key_mtiles != mtiles) {
             plan->pair_count = best_pair_count(slots, mtiles, ng_host, plan->sm_count);
             plan->pair_key_ng = ng_host; plan->pair_key_mtiles = mtiles;
@@ -899,21 +895,19 @@ cs_status launch_ffn_mma(cs_plan *plan, const cs_layer *L, const void *X, const 
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
         if (split)
-            ffn_gateup_mma_kernel<true><<<dim3(grid_g, mtiles), kTileThreads, kMmaSmem, st>>>(
+            ffn_gateup_mma_kernel<<<dim3(grid_g, mtiles), kTileThreads, kMmaSmem, st>>>(
                 tm_x, tm_x_lo, tm_g, tm_u, glist, ng_dev, ng_host, M, c.d, act_ld, mask, act, act_lo, plan->status);
-        else if (shared && n_pair == 0) {
+        else if (n_pair == 0) {
             // one shared support and no gain from paired tiles (measured at k = 27 of 108 groups, 2048 tokens:
             // 214 us for the GEMM pair against 223 us with single tiles; with paired tiles in play, k = 11 and
             // 54, the mixed launch below is faster): CTA pairs, one M = 256 instruction over two token tiles
             launch_pdl(true, ffn_gateup_pair_kernel, dim3(2 * min(slots, plan->sm_count / 2)), dim3(kTileThreads), kMmaSmem, st, tm_x, tm_g,
                        tm_u, glist, ng_host, plan->G, slots, M, c.d, act_ld, act, plan->status);
-        } else if (n_pair > 0) {
+        } else {
             // one shared support, its size known on the host: paired and single token tiles in one launch
             launch_pdl(true, ffn_gateup_tiles_kernel, dim3(n_pair + 2 * (slots - n_pair)), dim3(kTileThreads), kMmaSmem, st, tm_x, tm_g, tm_u,
                        glist, ng_host, plan->G, n_pair, mtiles, M, c.d, act_ld, act, plan->status);
-        } else
-            ffn_gateup_mma_kernel<false><<<dim3(grid_g, mtiles), kTileThreads, kMmaSmem, st>>>(
-                tm_x, tm_x_lo, tm_g, tm_u, glist, ng_dev, ng_host, M, c.d, act_ld, mask, act, act_lo, plan->status);
+        }
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
         // slices: fill the machine when one token tile cannot (decode), one slice otherwise (prompt)

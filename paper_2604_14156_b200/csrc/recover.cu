@@ -12,7 +12,7 @@ __global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restr
 }
 
 // NW = warps = ceil(G / 32).  KC = ceil(k / 8) for k <= 64 (list form), 0 otherwise (dense form).
-// DECODE: the form of RecoverOptions::decode.
+// DECODE: the form of RecoverOptions::decode (dense).
 template <int NW, int KC, bool DECODE>
 __global__ void __launch_bounds__(32 * NW) recover_kernel(const __grid_constant__ RecoverArgs a) {
     __shared__ RecoverSmem<NW, KC> s;
@@ -272,27 +272,29 @@ typedef void (*SenseFn)(SenseArgs, RecoverArgs);
 
 typedef void (*RecoverFn)(RecoverArgs);
 static int recover_kc(int k) { return k <= 64 ? (k + 7) / 8 : 0; }
-template <int NW, bool DECODE> static RecoverFn recover_fn_kc(int k) {
+template <int NW> static RecoverFn recover_fn_kc(int k) {
     switch (recover_kc(k)) {
-        case 1: return recover_kernel<NW, 1, DECODE>;
-        case 2: return recover_kernel<NW, 2, DECODE>;
-        case 3: return recover_kernel<NW, 3, DECODE>;
-        case 4: return recover_kernel<NW, 4, DECODE>;
-        case 5: return recover_kernel<NW, 5, DECODE>;
-        case 6: return recover_kernel<NW, 6, DECODE>;
-        case 7: return recover_kernel<NW, 7, DECODE>;
-        case 8: return recover_kernel<NW, 8, DECODE>;
-        default: return recover_kernel<NW, 0, DECODE>;
+        case 1: return recover_kernel<NW, 1, false>;
+        case 2: return recover_kernel<NW, 2, false>;
+        case 3: return recover_kernel<NW, 3, false>;
+        case 4: return recover_kernel<NW, 4, false>;
+        case 5: return recover_kernel<NW, 5, false>;
+        case 6: return recover_kernel<NW, 6, false>;
+        case 7: return recover_kernel<NW, 7, false>;
+        case 8: return recover_kernel<NW, 8, false>;
+        default: return recover_kernel<NW, 0, false>;
     }
 }
-template <bool DECODE> static RecoverFn recover_fn(int G, int k) {
+static RecoverFn recover_fn(int G, int k) {
     switch ((G + 31) / 32) {
-        case 1: return recover_fn_kc<1, DECODE>(k);
-        case 2: return recover_fn_kc<2, DECODE>(k);
-        case 3: return recover_fn_kc<3, DECODE>(k);
-        default: return recover_fn_kc<4, DECODE>(k);
+        case 1: return recover_fn_kc<1>(k);
+        case 2: return recover_fn_kc<2>(k);
+        case 3: return recover_fn_kc<3>(k);
+        default: return recover_fn_kc<4>(k);
     }
 }
+// In front of the decode GEMMs, which take over up to 64 groups per token: the dense form, 65 groups at least.
+static RecoverFn recover_decode_fn(int G) { return G <= 96 ? recover_kernel<3, 0, true> : recover_kernel<4, 0, true>; }
 RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const float *y, int B, int32_t *support, float *z,
                          float *resid, const RecoverOptions &o) {
     const cs_config &c = plan->cfg;
@@ -370,7 +372,7 @@ static int sense_tokens(const cs_plan *plan, int smem) {
 cs_status prepare_recover(cs_plan *plan) {
     CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
     plan->sense_tokens = sense_tokens(plan, kSenseSmem);
-    CS_CUDA_TRY(plan, prefer_shared(recover_fn<true>(plan->G, plan->cfg.k)));
+    if (!decode_recovers(plan)) CS_CUDA_TRY(plan, prefer_shared(recover_decode_fn(plan->G)));
     return CS_OK;
 }
 
@@ -384,7 +386,7 @@ cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float 
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }
-    launch_pdl(true, o.decode ? recover_fn<true>(G, c.k) : recover_fn<false>(G, c.k), dim3(B), dim3(gram_pitch(G)), 0, st,
+    launch_pdl(true, o.decode ? recover_decode_fn(G) : recover_fn(G, c.k), dim3(B), dim3(gram_pitch(G)), 0, st,
                recover_args(plan, Phi, mu, y, B, support, z, resid, o));
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());

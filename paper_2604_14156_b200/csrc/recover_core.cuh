@@ -498,24 +498,22 @@ __device__ __forceinline__ void drift_row(const int32_t *p, const int32_t *cur, 
 template <int NW, int BAR, typename Smem>
 __device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int g, int t, int m) {
     constexpr int GP = 32 * NW;
-    const int shares = GP / m < 1 ? 1 : GP / m;            // threads per row (m <= 64 <= 2 GP)
-    for (int row0 = 0; row0 < m; row0 += GP) {             // one round unless m > GP
-        const int row = row0 + g % m, share = g / m;
-        float a = 0.f;
-        if (row < m && share < shares) {
-            const int n = (p.slices + shares - 1) / shares, lo = share * n, hi = min(p.slices, lo + n);
-            const float *src = p.y + (size_t)t * m + row;
-            for (int i = lo; i < hi; i += 16) {
-                float v[16];
+    static_assert(GP >= kMaxM, "a thread per row at least");
+    const int shares = GP / m;                             // threads per row
+    const int row = g % m, share = g / m;
+    float a = 0.f;
+    if (share < shares) {
+        const int n = (p.slices + shares - 1) / shares, lo = share * n, hi = min(p.slices, lo + n);
+        const float *src = p.y + (size_t)t * m + row;
+        for (int i = lo; i < hi; i += 16) {
+            float v[16];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) v[u] = i + u < hi ? ld_dep(src + (size_t)(i + u) * p.B * m) : 0.f;
+            for (int u = 0; u < 16; ++u) v[u] = i + u < hi ? ld_dep(src + (size_t)(i + u) * p.B * m) : 0.f;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) a += v[u];
-            }
+            for (int u = 0; u < 16; ++u) a += v[u];
         }
-        if (m > GP) { if (row < m) s.y[row] = a; }
-        else s.part[g] = a;
     }
+    s.part[g] = a;
     float rs = 1.f;
     if (p.ss != nullptr) {   // every warp for itself
         float q = 0.f;
@@ -523,13 +521,12 @@ __device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int 
         rs = rsqrtf(warp_sum(q) / (float)p.d + p.eps);
     }
     bar_sync<BAR, GP>();
-    for (int row = g; row < m; row += GP) {
-        float a = 0.f;
-        if (m > GP) a = s.y[row];
-        else for (int sh = 0; sh < shares; ++sh) a += s.part[sh * m + row];
-        a *= rs;
-        s.y[row] = a;
-        p.y_out[(size_t)t * m + row] = a;
+    if (g < m) {
+        float y = 0.f;
+        for (int sh = 0; sh < shares; ++sh) y += s.part[sh * m + g];
+        y *= rs;
+        s.y[g] = y;
+        p.y_out[(size_t)t * m + g] = y;
     }
 }
 
