@@ -629,6 +629,23 @@ def test_ffn_exec_tensor_path_matches_oracle(B):
         assert err <= OUT_TOL["bf16"] and err <= TIGHT_TOL["bf16"], (t, err)
 
 
+def test_ffn_exec_beyond_the_decode_batches_matches_oracle():
+    """300 tokens at the 7B shape: bucketing, union list and the split-precision grouped GEMMs; tokens of all three 128-token tiles
+    and their edges."""
+    cfg = W.CONFIGS["l2_7b_b64"].with_(B=300)
+    L = _layer(cfg)
+    Lc = L.to("cpu")
+    tk = W.make_tokens(cfg, L.A)
+    plan = make_plan(cfg)
+    res = rng.normal(cfg.seed, (79,), (300, cfg.d), dtype=torch.float32)
+    out = cs.cs_ffn_exec(plan, device_layer(plan, L), tk.h.to(DEV), tk.planted.to(DEV), residual=res.to(DEV)).cpu().numpy()
+    assert plan.device_status() == 0
+    for t in (0, 1, 64, 127, 128, 190, 255, 256, 257, 298, 299):
+        ref = oracle.ffn(Lc.W_gate, Lc.W_up, Lc.Wd_t, cfg.group, tk.h[t], tk.planted[t])
+        assert rel(out[t].astype(np.float64) - res[t].double().numpy(), ref) <= TIGHT_TOL["bf16"], t
+    plan.close()
+
+
 @pytest.mark.parametrize("B", [4, 5, 9])
 def test_layer_step_around_the_crossover_batch(B):
     """The fused step on both sides of the batch where the tensor-core path takes over."""

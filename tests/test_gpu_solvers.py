@@ -227,6 +227,38 @@ def test_layer_step_ex_options_match_oracle(name, B):
     plan.close()
 
 
+# Warm start, temporal term and drift inside the decode launches: two accumulators of tokens, the longest list of the recovery, and the
+# recovery as a launch of its own (more than 64 groups).
+@pytest.mark.parametrize("G,k,B", [(40, 9, 10), (40, 9, 150), (100, 60, 33), (100, 50, 200), (100, 70, 20)])
+def test_layer_step_ex_previous_step_on_the_tensor_cores(G, k, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(B=B, d=512, d_ff=128 * G, m=30, k=k, T=8, index=560 + k)
+    L = W.make_layer(cfg, device=DEV)
+    Lc = L.to("cpu")
+    plan = make_plan(cfg)
+    plan.set_crossover(2)
+    lay = device_layer(plan, L)
+    h, h2 = W.make_tokens(cfg, L.A).h, W.make_tokens(cfg, L.A, batch=1).h
+    _, sup0, z0, _ = cs.cs_layer_step(plan, lay, h.to(DEV))
+    x = 0.9 * h + 0.1 * h2
+    opt = cs.StepOptions(plan, B, T=4, support_prev=sup0, z_prev=z0, warm_start=True, gamma=0.25, want_drift=True)
+    out, sup, z, _ = (t.cpu().numpy() for t in cs.cs_layer_step_ex(plan, lay, x.to(DEV), opt))
+    assert plan.device_status() == 0
+    prev = (sup0.cpu().numpy(), z0.cpu().numpy())
+    rs_, rz, _, gaps, ro, _ = _ex_reference(cfg, L, x, "iht", 4, prev=prev, gamma=0.25, warm=True)
+    bad = 0
+    for t in range(B):
+        if np.array_equal(sup[t], rs_[t]):
+            assert rel(out[t], ro[t]) <= TIGHT_TOL["bf16"], t
+            bad += rel(z[t], rz[t]) > Z_TOL
+            assert rel(z[t], rz[t]) <= Z_TOL or gaps[t] <= GAP_TOL, t
+        else:
+            assert gaps[t] <= GAP_TOL, (t, gaps[t])
+            bad += 1
+    assert bad <= max(1, B // 16)
+    assert opt.delta.cpu().numpy().tolist() == oracle.support_drift(prev[0], sup).tolist()
+    plan.close()
+
+
 def test_layer_step_ex_with_the_structured_sensor():
     """SRHT in place of the dense sketch: Phi is the operator applied to the probe's transpose, as S = Phi A is
     for the dense one; d a power of two."""
