@@ -45,9 +45,9 @@ UNIT = "tokens/s"
 # ncu captures summarised under profiles/, keyed by (workload, k).  An entry is removed when its
 # kernel changes and comes back with the next capture; a missing entry reports null.
 NCU_TRAFFIC = {
-    ("l2_7b_b1", 22): 69.25e6 + 0.20e6,                       # ffn_gather_kernel
-    ("l2_7b_b64", 22): 182.17e6 + 1.14e6 + 93.04e6 + 1.04e6,  # decode_gateup_kernel + decode_down_kernel
-    ("l2_13b_prompt", 27): 205.4e6 + 8.30e6 + 54.6e6 + 2.65e6,  # ffn_gateup_pair_kernel + ffn_down_wide_kernel
+    ("l2_7b_b1", 22): 69.25e6 + 0.16e6,                       # ffn_gather_kernel
+    ("l2_7b_b64", 22): 182.17e6 + 0.45e6 + 93.04e6 + 0.46e6,  # decode_gateup_kernel + decode_down_kernel
+    ("l2_13b_prompt", 27): 204.8e6 + 7.50e6 + 58.3e6 + 2.65e6,  # ffn_gateup_pair_kernel + ffn_down_wide_kernel
 }
 GRAPH_STEPS = 64          # most steps captured per CUDA graph
 N_TOKEN_BATCHES = 16      # distinct input batches rotated through

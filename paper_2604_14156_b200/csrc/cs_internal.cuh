@@ -155,7 +155,7 @@ cs_status launch_recover(cs_plan *plan, const float *Phi, float mu, const float 
                          const RecoverOptions &opt = RecoverOptions());
 // Sensor and estimator in one launch, a cluster of CTAs per token, for at most plan->sense_tokens tokens.  blocks > 0: one
 // token whose x is the sum of `blocks` rows [blocks, d] divided by n (a prompt's mean hidden state).
-constexpr int kSenseMaxTokens = 16;
+constexpr int kSenseMaxTokens = 16;   // bound of plan->sense_tokens, see recover.cu
 cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, float mu, const float *x, const float *gamma, int B,
                                float *n_out, int32_t *support, float *z, float *resid, cudaStream_t st,
                                const RecoverOptions &opt = RecoverOptions(), int blocks = 0, int n = 1);
@@ -305,7 +305,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // L2 policy of the weights, which are read once: first to leave L2, so that they do not push out the activations, S and
 // Phi, and the kernels' own code, which after a 270 MB step without this is fetched from HBM again (7B step at 64
-// tokens 63.8 -> 60.0 us, 200 tokens 135 -> 121).
+// tokens 63.8 -> 60.0 us; 200 tokens 135 -> 121 in bursts of a few ms, no gain over a second of load).
 __device__ __forceinline__ uint64_t policy_evict_first() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));

@@ -647,7 +647,8 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     {
         StageTimer timer(plan, CS_STAGE_EXEC2, st);
         // Expected number of groups in nobody's support, G (1 - k/G)^B: below a quarter group the list is every group and
-        // the masks need not be read.
+        // need not be made.  (7B, 5 tokens, 19.6 groups expected: 48.4 us with the union, 52.1 with every group; 8 tokens, 8.1: 51.8
+        // and 53.2; from 11 tokens, 3.3 groups, on the two are equal within the spread, so the line is not critical.)
         const bool use_union = by_list || (float)plan->G * powf(1.f - (float)c.k / plan->G, (float)B) > 0.25f;
         launch_pdl(true, down_fn(form), dim3(c.d / kDecBN, Z), dim3(kDecThreads), decode_smem(tt, kDecBN * BK * 2), st, tm_wd, tm_act,
                    tm_act_lo, (const int32_t *)plan->mask, (const unsigned *)plan->mask_count,
