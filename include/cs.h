@@ -340,8 +340,9 @@ cs_status cs_layer_step_host(cs_plan *plan, const cs_layer *layer, const float *
  * least `tokens` tokens (and at most 256) run on the tensor cores, smaller ones as the gather GEMV.
  * A plan starts at max(2, min(16, ceil(1.15 * G / k))), the point where streaming every group once
  * moves fewer bytes than streaming k groups per token; 1 <= tokens <= 129 (129: from 129 tokens on,
- * the largest value: no batch beyond 128 tokens takes the gather).  Only shapes the tensor-core path supports (bf16 weights, 128-channel groups, d a
- * multiple of 256) are affected.  cs_plan_crossover returns the current value.
+ * the largest value: no batch beyond 128 tokens takes the gather).  Only shapes the tensor-core path
+ * supports (bf16 weights, 128-channel groups, d a multiple of 256) are affected.  cs_plan_crossover
+ * returns the current value.
  */
 cs_status cs_plan_set_crossover(cs_plan *plan, int32_t tokens);
 int32_t cs_plan_crossover(const cs_plan *plan);
