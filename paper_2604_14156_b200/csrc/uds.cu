@@ -2,36 +2,23 @@
 // distribution over the vocabulary, H = -sum_v p_v log p_v with p = softmax(logits), and the
 // measurement budget it sets, m = clip(floor(m_base (1 + gamma H)), m_min, m_max).
 //
-// One pass over the logits.  Every thread keeps the three moments of its elements
-//     M = max l,   Z = sum e^(l - M),   W = sum e^(l - M) (l - M),
-// which merge associatively under a change of M, so the row is split over several CTAs (a single
-// token still uses a good part of the GPU) and folded in a fixed order: per warp by shuffles, per
-// CTA through shared memory, per row by a second small kernel, which ends with
+// One pass over the logits, one launch.  Every thread keeps the three moments of its elements
+//     M = max l,   Z = sum e^(l - M),   W = sum e^(l - M) (l - M);
+// a row is split over a cluster of up to eight CTAs.  Moments are folded by taking the common maximum first, one rescale per
+// thread, then plain sums in a fixed order (warp, CTA, cluster over distributed shared memory); CTA 0 ends with
 //     H = log Z - W / Z.
-// Bandwidth-bound: 4 V bytes per token, read once.
+// Small batches are a latency chain (at 11 tokens of 32000 logits one load round trip and the folds): as two launches, the row's
+// moments merged pairwise with two exponentials a merge and folded by the second launch, 1 x 32000 logits took 5.5 us and 11 x 32000 5.6,
+// now 2.5 and 3.1.  Large ones are bound by HBM and the arithmetic: 64 x 128256 16.7 and 10.8 us, 512 x 128256 66.6 and 54.0 (4.9 TB/s).
 #include "cs_internal.cuh"
 
 namespace cs {
 
 constexpr int kUdsThreads = 512;
-constexpr int kUdsMaxSplits = 32;
-constexpr int kUdsBatch = 8;
-constexpr int kUdsMinSplitElems = kUdsBatch * kUdsThreads;
+constexpr int kUdsWarps = kUdsThreads / 32;
+constexpr int kUdsMaxCtas = 8;   // of a cluster
 
 struct Moments { float M, Z, W; };   // Z == 0: no element yet
-
-__device__ __forceinline__ Moments merge(const Moments &a, const Moments &b) {
-    if (b.Z == 0.f) return a;
-    if (a.Z == 0.f) return b;
-    const float M = fmaxf(a.M, b.M);
-    const float da = a.M - M, db = b.M - M;       // one of them is exactly 0
-    const float sa = expf(da), sb = expf(db);
-    Moments r;
-    r.M = M;
-    r.Z = sa * a.Z + sb * b.Z;
-    r.W = sa * (a.W + da * a.Z) + sb * (b.W + db * b.Z);
-    return r;
-}
 
 // Folds a batch of N elements: one rescale to the batch maximum, then N independent exponentials.
 // Entries of -inf contribute nothing (p = 0, 0 log 0 = 0).
@@ -63,64 +50,78 @@ __device__ __forceinline__ void add_logits(Moments &s, const float (&v)[N]) {
     s.W += w0 + w1;
 }
 
-__device__ __forceinline__ Moments warp_merge(Moments s) {
+// The same moments about a maximum M (>= s.M where s has an element; a NaN of either stays one).
+__device__ __forceinline__ void rescale(Moments &s, float M) {
+    if (s.Z == 0.f) { s.M = M; return; }
+    const float dm = s.M - M, sc = expf(dm);
+    s.W = sc > 0.f || sc != sc ? sc * (s.W + dm * s.Z) : 0.f;
+    s.Z = sc * s.Z;
+    s.M = M;
+}
+// Folds the moments of a warp's lanes: every lane ends with the same bits.
+__device__ __forceinline__ void warp_fold(Moments &s) {
+    float M = s.Z == 0.f ? -INFINITY : s.M;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Moments other;
-        other.M = __shfl_xor_sync(0xffffffffu, s.M, o);
-        other.Z = __shfl_xor_sync(0xffffffffu, s.Z, o);
-        other.W = __shfl_xor_sync(0xffffffffu, s.W, o);
-        // the lower lane's value goes first on both sides, so all lanes end with the same bits
-        s = (threadIdx.x & o) ? merge(other, s) : merge(s, other);
-    }
-    return s;
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    rescale(s, M);
+    s.Z = warp_sum(s.Z);
+    s.W = warp_sum(s.W);
 }
 
-// grid (splits, B): CTA (s, t) folds elements [s * per, min(V, (s + 1) * per)) of row t.
+// grid (CTAs of a row, B), the row's CTAs one cluster: CTA (s, t) takes elements [s * per, min(V, (s + 1) * per)) of row t, N of a
+// thread in flight.  The floor is taken in double precision from the f32 entropy; a NaN entropy (a NaN or +inf logit) asks for m_max.
+template <int N>
 __global__ void __launch_bounds__(kUdsThreads)
-uds_moments_kernel(const float *__restrict__ logits, int V, int per, Moments *__restrict__ part) {
-    __shared__ Moments ws[kUdsThreads / 32];
-    const int t = blockIdx.y, s = blockIdx.x;
+uds_kernel(const float *__restrict__ logits, int V, int per, float m_base, float gamma, int m_min, int m_max, float *__restrict__ H_out,
+           int32_t *__restrict__ m_out) {
+    __shared__ Moments warp_s[kUdsWarps], cta_s[kUdsMaxCtas];
+    const int t = blockIdx.y, s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lo = s * per, hi = min(V, lo + per);
     const float *row = logits + (size_t)t * V;
     Moments acc{0.f, 0.f, 0.f};
     pdl_launch_dependents();
-    // kUdsBatch loads in flight per thread before any of them is used
-    for (int i = lo + threadIdx.x; i < hi; i += kUdsBatch * kUdsThreads) {
-        float v[kUdsBatch];
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // CTA 0 has started, see below
+    pdl_wait();   // the logits may come from the kernel before
+    int i = lo + (int)threadIdx.x;
+    for (int end = lo + N * kUdsThreads; end < hi; end += N * kUdsThreads, i += N * kUdsThreads) {   // whole batches
+        float v[N];
 #pragma unroll
-        for (int j = 0; j < kUdsBatch; ++j) {
+        for (int j = 0; j < N; ++j) v[j] = ld_dep(row + i + j * kUdsThreads);
+        add_logits(acc, v);
+    }
+    if (i < hi) {
+        float v[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
             const int idx = i + j * kUdsThreads;
-            v[j] = idx < hi ? __ldg(row + idx) : -INFINITY;
+            v[j] = ld_dep(row + min(idx, hi - 1));
+            if (idx >= hi) v[j] = -INFINITY;
         }
         add_logits(acc, v);
     }
-    acc = warp_merge(acc);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+    warp_fold(acc);
+    if (lane == 0) warp_s[warp] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        Moments v = threadIdx.x < kUdsThreads / 32 ? ws[threadIdx.x] : Moments{0.f, 0.f, 0.f};
-        v = warp_merge(v);
-        if (threadIdx.x == 0) part[(size_t)t * gridDim.x + s] = v;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (warp == 0) {
+        acc = lane < kUdsWarps ? warp_s[lane] : Moments{0.f, 0.f, 0.f};
+        warp_fold(acc);
+        if (lane == 0) {
+            uint32_t dst;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&cta_s[s])));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(acc.M) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst + 4u), "f"(acc.Z) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst + 8u), "f"(acc.W) : "memory");
+        }
+        __syncwarp();
     }
-}
-
-// One warp per token: folds the splits, then the entropy and the budget.  The floor is taken in
-// double precision from the f32 entropy; a NaN entropy (a NaN or +inf logit) asks for m_max.
-__global__ void __launch_bounds__(32)
-uds_finish_kernel(const Moments *__restrict__ part, int splits, float m_base, float gamma, int m_min, int m_max,
-                  float *__restrict__ H_out, int32_t *__restrict__ m_out) {
-    const int t = blockIdx.x, lane = threadIdx.x;
-    pdl_wait();   // the moments come from the kernel before
-    Moments v{0.f, 0.f, 0.f};
-    if (lane < splits) {
-        const float *p = reinterpret_cast<const float *>(part + (size_t)t * splits + lane);
-        v.M = ld_dep(p); v.Z = ld_dep(p + 1); v.W = ld_dep(p + 2);
-    }
-    v = warp_merge(v);
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (s != 0 || warp != 0) return;
+    acc = lane < (int)gridDim.x ? cta_s[lane] : Moments{0.f, 0.f, 0.f};
+    warp_fold(acc);
     if (lane == 0) {
-        float H = v.Z > 0.f ? fmaxf(logf(v.Z) - v.W / v.Z, 0.f) : (v.Z == 0.f ? 0.f : v.Z);
-        if (v.Z != v.Z || v.W != v.W) H = NAN;
+        float H = acc.Z > 0.f ? fmaxf(logf(acc.Z) - acc.W / acc.Z, 0.f) : (acc.Z == 0.f ? 0.f : acc.Z);
+        if (acc.Z != acc.Z || acc.W != acc.W) H = NAN;
         int m = m_max;
         if (H == H) {
             const double x = floor((double)m_base * (1.0 + (double)gamma * (double)H));
@@ -133,17 +134,22 @@ uds_finish_kernel(const Moments *__restrict__ part, int splits, float m_base, fl
 
 cs_status launch_uds_budget(cs_plan *plan, const float *logits, int B, int V, float m_base, float gamma,
                             int m_min, int m_max, float *H, int32_t *m_t, cudaStream_t st) {
-    int splits = (2 * plan->sm_count + B - 1) / B;   // about two CTAs per SM
-    splits = max(1, min(splits, min(kUdsMaxSplits, V / kUdsMinSplitElems)));
-    const size_t capacity = (size_t)kGatherMaxTokens * plan->nx_max * plan->cfg.d * sizeof(float);
-    while (splits > 1 && (size_t)B * splits * sizeof(Moments) > capacity) --splits;
-    if ((size_t)B * splits * sizeof(Moments) > capacity) return CS_ERR_SHAPE;
-    const int per = (V + splits - 1) / splits;
-    Moments *part = reinterpret_cast<Moments *>(plan->partial);
-    uds_moments_kernel<<<dim3(splits, B), kUdsThreads, 0, st>>>(logits, V, per, part);
-    plan->launches++;
-    CS_CUDA_TRY(plan, cudaGetLastError());
-    launch_pdl(true, uds_finish_kernel, dim3(B), dim3(32), 0, st, (const Moments *)part, splits, m_base, gamma, m_min, m_max, H, m_t);
+    if ((size_t)B * sizeof(Moments) > (size_t)kGatherMaxTokens * plan->nx_max * plan->cfg.d * sizeof(float)) return CS_ERR_SHAPE;
+    // about two CTAs per SM, each with 2048 elements at least
+    int ctas = 1;
+    while (ctas < kUdsMaxCtas && 2 * ctas * B <= 2 * plan->sm_count && V >= 2 * ctas * 2048) ctas *= 2;
+    const int per = (V + ctas - 1) / ctas;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, B); cfg.blockDim = dim3(kUdsThreads); cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ctas; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    // 16 logits of a thread in flight where the CTAs are too few to keep the memory busy with 8
+    const bool deep = per > 8 * kUdsThreads && ctas * B <= 2 * plan->sm_count;
+    cudaLaunchKernelEx(&cfg, deep ? uds_kernel<16> : uds_kernel<8>, logits, V, per, m_base, gamma, m_min, m_max, H, m_t);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
     return CS_OK;

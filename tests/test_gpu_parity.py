@@ -781,6 +781,20 @@ def test_uds_budget_matches_oracle(B, V):
     plan.close()
 
 
+# Rows over clusters of 1, 2, 4 and 8 CTAs (by tokens and by vocabulary), batches of 8 and 16 logits a thread, and rows that end
+# just before, on and behind a batch or a CTA's share.
+@pytest.mark.parametrize("B,V", [(1, 4095), (2, 4097), (2, 8191), (2, 8192), (37, 16385), (38, 4099), (74, 12289), (75, 8193), (149, 33),
+                                 (3, 65537), (9, 32767), (20, 70001)])
+def test_uds_budget_splits_of_a_row(B, V):
+    g = torch.Generator().manual_seed(300 + B + V)
+    logits = torch.randn((B, V), generator=g) * torch.logspace(-1, 1, B)[:, None]
+    logits[0, -1] = 30.0
+    plan = cs.Plan(256, 1024, 64, 8, 4, 4, torch.float32, B, 1e-5)
+    m_t, H = cs.cs_uds_budget(plan, logits.to(DEV), 16.0, 0.75, 8, 64)
+    _check_budget(m_t, H, oracle.uds_budget(logits, 16.0, 0.75, 8, 64), 16.0, 0.75)
+    plan.close()
+
+
 def test_uds_budget_special_rows():
     """Uniform row (H = log V), one dominant logit (H = 0, m = m_base), masked entries (-inf),
     an entirely masked row, a NaN row (m_max), clipping at both ends, H not requested."""
