@@ -52,7 +52,7 @@ struct SenseArgs {
     float eps;
     int d, s_rows;        // s_rows: rows of S that fit in shared memory (the others are read after the wait)
     float *y_out, *n_out;
-    int blocks;           // > 0: x is [blocks, d], and what is sensed is the sum of its rows times inv_n
+    int blocks;           // STAGED: x is [blocks, d], and what is sensed is the sum of its rows times inv_n
     float inv_n;
 };
 
@@ -67,10 +67,16 @@ __device__ __forceinline__ void st_remote(uint32_t addr, float v) {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-template <int NW, int KC>
+// STAGED: x is a prompt's column sums, which every CTA adds up once for all its warps.
+// PLAIN: see recover_row.  NORM: without an RMSNorm, with one, or either (2).  ALL: every row of S has its place in shared memory.
+// What is bound by latency here is also the fetch of code that the weights of the step before have pushed out of the caches around
+// the SMs: what a form never runs is left out of it, so that what it runs lies close together.  One kernel for all of them, and
+// now: 7B, one token 25.6 and 24.6 us a step, three 41.8 and 39.3; 8B, four 58.3 and 54.9; 777 prompt tokens 72.9 and 69.7.
+template <int NW, int KC, bool STAGED, bool PLAIN, int NORM, bool ALL>
 __global__ void __cluster_dims__(kSenseCtas, 1, 1) __launch_bounds__(kSenseThreads, 1)
 sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant__ RecoverArgs a) {
     constexpr int GP = 32 * NW;
+    const bool norm = NORM == 2 ? sa.gamma != nullptr : NORM == 1;
     extern __shared__ float4 sense_s[];
     __shared__ RecoverSmem<NW, KC> rs;
     __shared__ float part_s[kSenseCtas][kMaxM], ss_s[kSenseCtas];
@@ -96,6 +102,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     // rows of S without a place there: the warp's next in registers, what is left in L2 at least
     float4 ex[kSenseExtra][kSenseMaxChunks];
     const int x0 = sa.s_rows + ((warp - sa.s_rows) & (kSenseWarps - 1));   // this warp's first such row
+    if constexpr (!ALL) {
 #pragma unroll
     for (int q = 0; q < kSenseExtra; ++q)
 #pragma unroll
@@ -104,6 +111,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
                 ex[q][j] = __ldg(reinterpret_cast<const float4 *>(sa.S + (size_t)(x0 + q * kSenseWarps) * d + col0) + min(lane + 32 * j, nc - 1));
     for (int r = sa.s_rows + kSenseExtra * kSenseWarps + tid; r < m; r += kSenseThreads)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(sa.S + (size_t)r * d + col0), "r"(nc * 16) : "memory");
+    }
     for (int i0 = tid; i0 < m * GP; i0 += 8 * kSenseThreads) {   // eight loads in flight: addresses clamped, no branches
         float v[8];
 #pragma unroll
@@ -156,12 +164,12 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     pdl_wait();   // x may be the previous kernel's output
     float4 xv[kSenseMaxChunks], gm[kSenseMaxChunks];
     float ss = 0.f;
-    if (sa.gamma != nullptr) {
+    if (norm) {
 #pragma unroll
         for (int j = 0; j < kSenseMaxChunks; ++j)
             if (j < nch) gm[j] = __ldg(reinterpret_cast<const float4 *>(sa.gamma + col0) + min(lane + 32 * j, nc - 1));
     }
-    if (sa.blocks > 0) {   // every column is summed once, for all warps
+    if constexpr (STAGED) {   // every column is summed once, for all warps
         float4 *sum_s = S_s + sa.s_rows * nc;
         for (int c = tid; c < nc; c += kSenseThreads) {
             float4 v[kMeanRowBlocks], s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -183,7 +191,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
 #pragma unroll
     for (int j = 0; j < kSenseMaxChunks; ++j) {
         ss += xv[j].x * xv[j].x + xv[j].y * xv[j].y + xv[j].z * xv[j].z + xv[j].w * xv[j].w;
-        if (sa.gamma != nullptr && j < nch) { xv[j].x *= gm[j].x; xv[j].y *= gm[j].y; xv[j].z *= gm[j].z; xv[j].w *= gm[j].w; }
+        if (norm && j < nch) { xv[j].x *= gm[j].x; xv[j].y *= gm[j].y; xv[j].z *= gm[j].z; xv[j].w *= gm[j].w; }
     }
     auto dot = [](const float4 &s, const float4 &v, float a) { return fmaf(s.w, v.w, fmaf(s.z, v.z, fmaf(s.y, v.y, fmaf(s.x, v.x, a)))); };
     // four rows: their reductions interleave; lane q stores row q's
@@ -212,6 +220,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
         }
         finish(acc, r0, sa.s_rows);
     }
+    if constexpr (!ALL)
 #pragma unroll 1
     for (int r0 = x0; r0 < m; r0 += 4 * kSenseWarps) {
         float acc[4] = {};
@@ -232,14 +241,14 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
         }
         finish(acc, r0, m);
     }
-    if (warp == 0 && sa.gamma != nullptr) {
+    if (warp == 0 && norm) {
         ss = warp_sum(ss);
         if (lane < kSenseCtas) st_remote(remote_smem(&ss_s[rank], lane), ss);
     }
     cluster_arrive();
     cluster_wait();
     float rscale = 1.f;
-    if (sa.gamma != nullptr) {
+    if (norm) {
         float tot = 0.f;
 #pragma unroll
         for (int r = 0; r < kSenseCtas; ++r) tot += ss_s[r];
@@ -254,7 +263,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     }
     if (rank != 0 || tid >= GP) return;
     const int g = tid;
-    recover_row<NW, KC, 1>(
+    recover_row<NW, KC, 1, PLAIN>(
         rs, a, SharedSource{M_s, phi_s, G, pitch},
         [&](auto &sm) {
             for (int i = g; i < m; i += GP) {
@@ -313,25 +322,31 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
     return a;
 }
 
-template <int NW> static SenseFn sense_fn_kc(int k) {
-    switch (recover_kc(k)) {
-        case 1: return sense_recover_kernel<NW, 1>;
-        case 2: return sense_recover_kernel<NW, 2>;
-        case 3: return sense_recover_kernel<NW, 3>;
-        case 4: return sense_recover_kernel<NW, 4>;
-        case 5: return sense_recover_kernel<NW, 5>;
-        case 6: return sense_recover_kernel<NW, 6>;
-        case 7: return sense_recover_kernel<NW, 7>;
-        case 8: return sense_recover_kernel<NW, 8>;
-        default: return sense_recover_kernel<NW, 0>;
+enum SenseKind { kSensePlain, kSensePlainNorm, kSenseOptions, kSenseStaged };
+// The list in steps of 8 slots for a plain step, of 16 for the rest (a longer list holds zeros).  all: every row of S has its place
+// in shared memory.
+template <int NW> static SenseFn sense_fn_kc(int k, SenseKind kind, bool all) {
+    const int kc = recover_kc(k), kc2 = (kc + 1) / 2 * 2;
+#define CS_SENSE(KC, N) if (kc == KC) return sense_recover_kernel<NW, KC, false, true, N, true>
+    if (kind == kSensePlain && all) {
+        CS_SENSE(1, 0); CS_SENSE(2, 0); CS_SENSE(3, 0); CS_SENSE(4, 0);
+        CS_SENSE(5, 0); CS_SENSE(6, 0); CS_SENSE(7, 0); CS_SENSE(8, 0);
+    } else if (kind == kSensePlainNorm && all) {
+        CS_SENSE(1, 1); CS_SENSE(2, 1); CS_SENSE(3, 1); CS_SENSE(4, 1);
+        CS_SENSE(5, 1); CS_SENSE(6, 1); CS_SENSE(7, 1); CS_SENSE(8, 1);
     }
+#undef CS_SENSE
+#define CS_SENSE(KC) if (kc2 == KC) return kind == kSenseStaged ? sense_recover_kernel<NW, KC, true, true, 0, false> : sense_recover_kernel<NW, KC, false, false, 2, false>
+    CS_SENSE(2); CS_SENSE(4); CS_SENSE(6); CS_SENSE(8);
+#undef CS_SENSE
+    return sense_recover_kernel<NW, 0, true, true, 0, false>;   // dense: only a prompt takes it
 }
-static SenseFn sense_fn(int G, int k) {
+static SenseFn sense_fn(int G, int k, SenseKind kind, bool all) {
     switch ((G + 31) / 32) {
-        case 1: return sense_fn_kc<1>(k);
-        case 2: return sense_fn_kc<2>(k);
-        case 3: return sense_fn_kc<3>(k);
-        default: return sense_fn_kc<4>(k);
+        case 1: return sense_fn_kc<1>(k, kind, all);
+        case 2: return sense_fn_kc<2>(k, kind, all);
+        case 3: return sense_fn_kc<3>(k, kind, all);
+        default: return sense_fn_kc<4>(k, kind, all);
     }
 }
 
@@ -345,7 +360,9 @@ cs_status launch_sense_recover(cs_plan *plan, const float *S, const float *Phi, 
     {
         StageTimer timer(plan, CS_STAGE_SKETCH, st);
         plan->stage_seen[CS_STAGE_RECOVER] = 0;   // part of this launch
-        launch_pdl(true, sense_fn(plan->G, c.k), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)(sa.s_rows + (blocks > 0)) * row_bytes, st,
+        const bool plain = o.sup0 == nullptr && o.gamma == 0.f && o.check == nullptr && o.delta == nullptr && o.drift == nullptr;
+        const SenseKind kind = blocks > 0 ? kSenseStaged : !plain ? kSenseOptions : gamma != nullptr ? kSensePlainNorm : kSensePlain;
+        launch_pdl(true, sense_fn(plan->G, c.k, kind, sa.s_rows == c.m), dim3(kSenseCtas * B), dim3(kSenseThreads), (size_t)fixed + (size_t)(sa.s_rows + (blocks > 0)) * row_bytes, st,
                    sa, recover_args(plan, Phi, mu, nullptr, B, support, z, resid, o));
     }
     plan->launches++;
@@ -365,12 +382,13 @@ static int sense_tokens(const cs_plan *plan, int smem) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kSenseCtas * kSenseMaxTokens); cfg.blockDim = dim3(kSenseThreads); cfg.dynamicSmemBytes = smem;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, sense_fn(plan->G, c.k), &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&clusters, sense_fn(plan->G, c.k, kSensePlain, true), &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return min(clusters, kSenseMaxTokens);
 }
 
 cs_status prepare_recover(cs_plan *plan) {
-    CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
+    for (SenseKind kind : {kSensePlain, kSensePlainNorm, kSenseOptions, kSenseStaged})
+        CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k, kind, true), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
     plan->sense_tokens = sense_tokens(plan, kSenseSmem);
     if (!decode_recovers(plan)) CS_CUDA_TRY(plan, prefer_shared(recover_decode_fn(plan->G)));
     return CS_OK;

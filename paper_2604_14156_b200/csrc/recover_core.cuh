@@ -203,13 +203,13 @@ __device__ __forceinline__ void recover_load_phi(const float *__restrict__ Phi, 
 // start's own when T == 0 or the start is warm); from then on s.idx always holds k valid groups and changes only where the
 // support changes: slot_changed(slot, g) is called by the thread whose entry g has just taken `slot`.
 // table_final() is called once by every thread after the last iteration, before the outputs are
-// written.  mask (may be NULL): NW words of membership bits.
-template <int NW, int KC, int BAR, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
+// written.  mask (may be NULL): NW words of membership bits.  PLAIN: neither a warm start nor a temporal term, and no code for them.
+template <int NW, int KC, int BAR, bool PLAIN, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
 __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int g, const float *__restrict__ Phi,
                                               const MSource M, float mu, LoadY load_y, int m, int G, int k, int T, int32_t *__restrict__ support,
                                               float *__restrict__ z_out, float *__restrict__ resid_out,
                                               const int32_t *__restrict__ sup0, const float *__restrict__ z0,
-                                              const float tgamma, const int32_t *__restrict__ sup_prev,
+                                              const float tgamma_, const int32_t *__restrict__ sup_prev,
                                               const float *__restrict__ z_prev, uint32_t *__restrict__ mask, DeviceStatus *status, const float (&phc)[32], TableReady table_ready,
                                               SlotChanged slot_changed, TableFinal table_final) {
     constexpr int GP = 32 * NW;
@@ -231,7 +231,8 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
     for (int i = m + g; i < kMaxM; i += GP) s.y[i] = 0.f;
     // z_0 = 0 with the support the order assigns to an all-zero vector (indices 0..k-1), or, warm
     // started, the k-sparse iterate handed in (sup0 ascending and distinct, z0 its values).
-    const bool warm = sup0 != nullptr;
+    const bool warm = !PLAIN && sup0 != nullptr;
+    const float tgamma = PLAIN ? 0.f : tgamma_;
     s.slot[g] = -1;
     for (int i = g; i < NV; i += GP) { s.val[0][i] = 0.f; s.val[1][i] = 0.f; s.idx[i] = i < k ? i : 0; }
     bar_sync<BAR, GP>();
@@ -532,22 +533,23 @@ __device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int 
 
 // Token t of a batch, by the 32 * NW threads that meet on named barrier BAR: the check of the previous support, the
 // iteration, the outputs, the drift.  load_y as in recover_token; mask: [B, 4] membership bits, or NULL.
-template <int NW, int KC, int BAR, typename MSource, typename LoadY>
+// PLAIN: none of the options.
+template <int NW, int KC, int BAR, bool PLAIN = false, typename MSource, typename LoadY>
 __device__ __forceinline__ void recover_row(RecoverSmem<NW, KC> &s, const RecoverArgs &a, const MSource M, LoadY load_y,
                                             uint32_t *mask, int g, int t, const float (&phc)[32]) {
     const size_t row = (size_t)t * a.k;
-    if (a.check != nullptr && g < a.k) {
+    if (!PLAIN && a.check != nullptr && g < a.k) {
         const int32_t *p = a.check + row + g;
         const int e = ld_dep(p);
         if (e < 0 || e >= a.G || (g > 0 && ld_dep(p - 1) >= e)) atomicCAS(&a.status->code, 0, (int)CS_ERR_SUPPORT);
     }
-    recover_token<NW, KC, BAR>(
+    recover_token<NW, KC, BAR, PLAIN>(
         s, g, a.Phi, M, a.mu, load_y, a.m, a.G, a.k, a.T, a.support + row, a.z != nullptr ? a.z + row : nullptr,
         a.resid != nullptr ? a.resid + t : nullptr, a.sup0 != nullptr ? a.sup0 + row : nullptr,
         a.z0 != nullptr ? a.z0 + row : nullptr, a.tgamma, a.sup_prev != nullptr ? a.sup_prev + row : nullptr,
         a.z_prev != nullptr ? a.z_prev + row : nullptr, mask != nullptr ? mask + (size_t)t * 4 : nullptr, a.status, phc, [] {},
         [](int, int) {}, [] {});
-    if (a.delta != nullptr || a.drift != nullptr) {
+    if (!PLAIN && (a.delta != nullptr || a.drift != nullptr)) {
         bar_sync<BAR, 32 * NW>();   // the support row is written
         drift_row<BAR, 32 * NW>(a.check + row, a.support + row, a.k, g, t, a.delta, a.drift);
     }

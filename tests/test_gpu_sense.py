@@ -27,6 +27,25 @@ def test_layer_step_sense_cluster_edges(d, G, m, k, B, norm):
     plan.close()
 
 
+# A plain step's form of the sensing launch (with or without the RMSNorm, every row of S in shared memory or not: 64 rows of 4096 beside
+# 128 groups are not) against the general one, which a request for the drift takes: the same bits.  List lengths around 8, 16 and 24.
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("d,G,m,k", [(256, 16, 8, 4), (320, 40, 20, 8), (1088, 70, 33, 9), (256, 100, 40, 16), (512, 128, 64, 17), (4096, 128, 64, 24),
+                                     (4096, 128, 64, 25), (256, 128, 30, 64)])
+def test_sense_launch_plain_and_general_forms_agree(d, G, m, k, norm):
+    cfg = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"].with_(n_layers=1, w_dtype="f32", d=d, d_ff=64 * G, group=64, m=m, k=k, T=7, B=3,
+                                                                  index=470 + k)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    lay, x = device_layer(plan, L), W.make_tokens(cfg, L.A).h.to("cuda:0")
+    plain = cs.cs_layer_step(plan, lay, x)
+    opt = cs.StepOptions(plan, 3, support_prev=plain[1].clone(), want_drift=True)
+    for a, b in zip(plain, cs.cs_layer_step_ex(plan, lay, x, opt)):
+        assert torch.equal(a, b)
+    assert not opt.delta.any() and plan.device_status() == 0
+    plan.close()
+
+
 # What decides between the sensing launch and the sketch and recovery launches: tokens (clusters resident at once, 15 on B200),
 # the bytes of S (128 KB per CTA: 8192 x 32, 8192 x 33), the list form (64 groups).  The dense form and its prompt.
 @pytest.mark.parametrize("d,G,m,k,B", [(256, 16, 8, 4, 12), (256, 16, 8, 4, 15), (256, 16, 8, 4, 16), (8192, 40, 32, 9, 2), (8192, 40, 33, 9, 2),
