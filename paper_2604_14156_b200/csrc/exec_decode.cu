@@ -1,6 +1,7 @@
 // Actuator, tensor-core regime for decode batches of at most kDecodeMaxTokens tokens with independent supports.
 //
-//   decode_gateup_kernel   act[t, c] = silu(n_t . W_gate[c]) (n_t . W_up[c]) for every token t and channel c, in its support
+//   decode_gateup_kernel, decode_gateup_pair_kernel
+//                          act[t, c] = silu(n_t . W_gate[c]) (n_t . W_up[c]) for every token t and channel c, in its support
 //                          or not
 //   decode_down_kernel     partial[z, t, :] = sum over the channels of list slice z that are in t's support of
 //                          act[t, c] Wd_t[c, :]
@@ -16,8 +17,8 @@
 // f32 activations enter as two bf16 matrices, rounded value and remainder (16 mantissa bits together).  PACK
 // (at most 64 tokens): values are rows 0.. and remainders rows 64.. of ONE 128-row operand, their products are added in
 // the epilogue.  Otherwise values and remainders are two operands that accumulate into the same tensor-memory
-// columns; MT = 2 (more than 128 tokens) keeps two accumulators.  Rows no token owns hold whatever shared memory
-// held: rows of an MMA do not mix, and those results are never read.
+// columns; MT = 2 (more than 128 tokens) keeps two accumulators (a step's gate/up there runs on pairs of CTAs).  Rows no token
+// owns hold whatever shared memory held: rows of an MMA do not mix, and those results are never read.
 //
 // Balance: the channel tiles of gate/up are not tied to the 128-channel groups.  A CTA takes R channels, R the
 // multiple of 8 that gives every SM one CTA (80 at d_ff = 11008: 138 CTAs on 148 SMs; one CTA per group left 62 SMs
@@ -356,6 +357,180 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     teardown_cta(bars, warp, tcols);
 }
 
+// The same for a step of more than 128 tokens, on pairs of CTAs (a cluster of two): with both accumulators in one CTA every weight tile is
+// read from shared memory by four instructions and every k block moves 228 KB through that port for 20 KB of weights (1.03 us a k block,
+// 68 us at 7B and 200 tokens, the tensor pipe 51 % busy).  Here one instruction has M = 256: each CTA holds half of the tokens (their
+// values and their remainders, 128 rows each) and half of the pair's channels, R of 2 R, gate rows then up rows: 156 KB for the
+// same 20 KB of weights per CTA.  (One step, 7B: 200 tokens 135.5 to 127.0 us, in short bursts 132 to 121, 256 tokens 139 to 127; d = 5120 with 27 of 108
+// groups, 200 tokens 189 to 181; 129 tokens even, 113.9 and 112.6, so every batch beyond 128 tokens takes it.)  Gate accumulates in tensor-memory columns 0 .. 2 R, up from 256 on.  The even CTA's MMA thread issues
+// for both; no multicast load, each CTA fetches its own tiles and signals the even CTA's barrier.
+constexpr int kPairTokenBytes = 2 * kABytes;   // value rows, then remainder rows
+__host__ __device__ inline int gateup_pair_stages(int R) { return min(kMaxStages, kDecRing / (kPairTokenBytes + 2 * R * BK * 2)); }
+template <int KC>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDecThreads + kRecThreads, 1)
+decode_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_lo,
+                          const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_u, int B, int half, int R, int d,
+                          int d_ff, const float *ss_part, float eps, const __grid_constant__ RecoverArgs ra,
+                          __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ act_lo, DeviceStatus *status) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ float rscale_s[BM];
+    __shared__ int acc_ok;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int c0 = (int)(blockIdx.x >> 1) * 2 * R, t0 = (int)rank * half, nt = min(B - t0, half);   // the pair's channels, this CTA's tokens
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int wbytes = 2 * R * BK * 2, stage_bytes = kPairTokenBytes + wbytes, stages = gateup_pair_stages(R), kblocks = d / BK;
+    Barriers *bars = reinterpret_cast<Barriers *>(base + stages * stage_bytes);
+    if (threadIdx.x == 0) {
+        prefetch_map(&tm_g); prefetch_map(&tm_u); prefetch_map(&tm_x); prefetch_map(&tm_x_lo);
+        for (int s = 0; s < stages; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->empty[s], 1); }
+        mbar_init(&bars->acc_ready, 1);
+        bars->aborted = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {   // the same warp of both CTAs allocates for the pair
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&bars->tmem_base)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();        // the peer's barriers exist before anything signals them
+    tc_fence_after();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            const uint32_t full0 = map_to_cta(smem_u32(&bars->full[0]), 0);   // the even CTA's full barriers
+            const int tx = 2 * (wbytes + 2 * half * BK * 2);                   // both CTAs' bytes
+            const uint64_t once = policy_evict_first();
+            auto load_w = [&](int kb, int s) {
+                uint8_t *w = base + (size_t)s * stage_bytes + kPairTokenBytes;
+                if (rank == 0) mbar_expect_tx(&bars->full[s], tx);
+                tma_load_2d_pair(w, &tm_g, kb * BK, c0 + (int)rank * R, full0 + 8u * s, once);
+                tma_load_2d_pair(w + wbytes / 2, &tm_u, kb * BK, c0 + (int)rank * R, full0 + 8u * s, once);
+            };
+            auto load_t = [&](int kb, int s) {
+                uint8_t *t = base + (size_t)s * stage_bytes;
+                tma_load_2d_pair(t, &tm_x, kb * BK, t0, full0 + 8u * s);
+                tma_load_2d_pair(t + kABytes, &tm_x_lo, kb * BK, t0, full0 + 8u * s);
+            };
+            // weights are parameters: the first ring is requested before anything is waited for
+            const int pre = min(stages, kblocks);
+            for (int kb = 0; kb < pre; ++kb) load_w(kb, kb);
+            pdl_wait();   // the token matrices
+            for (int kb = 0; kb < pre; ++kb) load_t(kb, kb);
+            int s = 0, ph = 0;
+            for (int kb = pre; kb < kblocks; ++kb) {
+                if (!mbar_wait(&bars->empty[s], ph, bars, status)) break;
+                load_w(kb, s);
+                load_t(kb, s);
+                if (++s == stages) { s = 0; ph ^= 1; }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && rank == 0) {
+            // bf16 x bf16 -> f32, M = 256, N = 2 R
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * R >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+            const uint32_t tmem = bars->tmem_base;
+            bool ok = true;
+            int s = 0, ph = 0;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                ok = mbar_wait(&bars->full[s], ph, bars, status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t a0 = smem_u32(base + (size_t)s * stage_bytes), w0 = a0 + kPairTokenBytes;
+#pragma unroll
+                for (int k4 = 0; k4 < BK / 16; ++k4) {   // the descriptors' offsets hold in both CTAs' shared memory
+                    const uint64_t hi = desc_sw128(a0 + k4 * 32, 16), lo = desc_sw128(a0 + kABytes + k4 * 32, 16);
+                    const uint64_t g = desc_sw128(w0 + k4 * 32, 16), u = desc_sw128(w0 + wbytes / 2 + k4 * 32, 16);
+                    tc_mma_pair(tmem, hi, g, idesc, (kb | k4) != 0);
+                    tc_mma_pair(tmem, lo, g, idesc, 1);
+                    tc_mma_pair(tmem + 256, hi, u, idesc, (kb | k4) != 0);
+                    tc_mma_pair(tmem + 256, lo, u, idesc, 1);
+                }
+                tc_commit_pair(&bars->empty[s]);
+                if (++s == stages) { s = 0; ph ^= 1; }
+            }
+            if (ok) tc_commit_pair(&bars->acc_ready);
+        }
+    } else if (warp < kDecThreads / 32) {
+        const int et = threadIdx.x - 64, q = warp & 3, sub = (warp - 2) >> 2;
+        pdl_wait();   // the row squares; and nothing is stored before the kernels before this one are complete
+        for (int t = et; t < nt; t += kEpiThreads) {
+            float rs = 1.f;
+            if (ss_part != nullptr) {
+                float sq = 0.f;
+                for (int i = 0; i < d / 64; i += 16) {   // d is a multiple of 256
+                    float v[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) v[u] = i + u < d / 64 ? ld_dep(ss_part + (size_t)(i + u) * B + t0 + t) : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) sq += v[u];
+                }
+                rs = rsqrtf(sq / (float)d + eps);
+            }
+            rscale_s[t] = rs;
+        }
+        if (warp == 2) {   // one warp polls, the others sleep at the barrier behind it
+            const bool ok = mbar_wait(&bars->acc_ready, 0, bars, status);
+            if (lane == 0) acc_ok = ok;
+        }
+        epi_sync();
+        tc_fence_after();
+        // lane = token, eight channels at a time, two warps per lane quarter
+        const int t = q * 32 + lane;
+        const uint32_t tbase = bars->tmem_base + ((uint32_t)(q * 32) << 16);
+        if (acc_ok && q * 32 < nt) {
+            const float sc = t < nt ? rscale_s[t] : 0.f;
+#pragma unroll 1
+            for (int c = 8 * sub; c < 2 * R; c += 16) {
+                uint32_t g[8], u[8];
+                tc_ld8(tbase + c, g);
+                tc_ld8(tbase + 256 + c, u);
+                tc_wait_ld();
+                if (t < nt && c0 + c < d_ff) {
+                    float v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = silu_f(__uint_as_float(g[j]) * sc) * (__uint_as_float(u[j]) * sc);
+                    uint2 h0, l0, h1, l1;
+                    split4(v[0], v[1], v[2], v[3], h0, l0);
+                    split4(v[4], v[5], v[6], v[7], h1, l1);
+                    const size_t off = (size_t)(t0 + t) * d_ff + c0 + c;
+                    *reinterpret_cast<uint4 *>(act + off) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                    *reinterpret_cast<uint4 *>(act_lo + off) = make_uint4(l0.x, l0.y, l1.x, l1.y);
+                }
+            }
+        }
+    } else {
+        constexpr int kRecBar = 3;
+        __shared__ RecoverSmem<kRecNW, KC> rs;
+        const int g = threadIdx.x - kDecThreads;
+        float phc[32];
+        if (ra.m <= 32) recover_load_phi<kRecNW>(ra.Phi, ra.m, ra.G, g, phc);
+        const GramSource M{ra.gram, gram_pitch(ra.G)};
+        pdl_wait();   // the partial sketches and M come from the kernel before
+        for (int t = blockIdx.x; t < B; t += gridDim.x) {
+            recover_row<kRecNW, KC, kRecBar>(
+                rs, ra, M, [&](auto &sm) { y_from_parts<kRecNW, kRecBar>(sm, ra.parts, g, t, ra.m); }, ra.mask, g, t, phc);
+            bar_sync<kRecBar, kRecThreads>();
+        }
+        // this CTA's masks are written (the barrier that ends the loop, or no token at all)
+        if (g == 0) {
+            count_masks(ra.mask_count);
+            pdl_launch_dependents();
+        }
+    }
+    // Neither CTA leaves (or frees tensor memory) while the other may still read its shared memory or signal its barriers; every
+    // wait above is bounded, so both reach this point.
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(bars->tmem_base), "r"(512) : "memory");
+    }
+}
+
 // ---- down -----------------------------------------------------------------------------------------------
 // grid (d / 256, slices).  The list is every group (use_union == 0) or the groups that are in some token's support; slice z
 // takes the 64-channel k blocks [z nk / Z, (z + 1) nk / Z) of it.  mask_count: the CTAs that have written their masks, all of them
@@ -572,8 +747,13 @@ template <bool PACK, int MT> GateUpFn gateup_fn_kc(int kc) {
          : kc == 4 ? decode_gateup_kernel<PACK, MT, 4> : kc == 7 ? decode_gateup_kernel<PACK, MT, 7>
          : decode_gateup_kernel<PACK, MT, 8>;
 }
-GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators
-    return form == 0 ? gateup_fn_kc<true, 1>(kc) : form == 1 ? gateup_fn_kc<false, 1>(kc) : gateup_fn_kc<false, 2>(kc);
+GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators (2: supports known before; a step takes the pair kernel)
+    return form == 0 ? gateup_fn_kc<true, 1>(kc) : form == 1 ? gateup_fn_kc<false, 1>(kc) : decode_gateup_kernel<false, 2, 0>;
+}
+typedef void (*GateUpPairFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, int, const float *, float, RecoverArgs,
+                             __nv_bfloat16 *, __nv_bfloat16 *, DeviceStatus *);
+GateUpPairFn gateup_pair_fn(int kc) {
+    return kc == 3 ? decode_gateup_pair_kernel<3> : kc == 4 ? decode_gateup_pair_kernel<4> : kc == 7 ? decode_gateup_pair_kernel<7> : decode_gateup_pair_kernel<8>;
 }
 DownFn down_fn(int form) { return form == 0 ? decode_down_kernel<true, 1> : form == 1 ? decode_down_kernel<false, 1> : decode_down_kernel<false, 2>; }
 
@@ -592,6 +772,7 @@ cs_status prepare_decode(cs_plan *plan) {
     CS_CUDA_TRY(plan, prefer_shared(decode_prep_kernel));
     CS_CUDA_TRY(plan, prefer_shared(decode_reduce_kernel));
     const int smem = 1024 + kDecRing + (int)sizeof(Barriers);
+    CS_CUDA_TRY(plan, cudaFuncSetAttribute(gateup_pair_fn(gateup_kc(plan)), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     for (int form = 0; form < 3; ++form) {
         CS_CUDA_TRY(plan, cudaFuncSetAttribute(gateup_fn(form, 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         CS_CUDA_TRY(plan, cudaFuncSetAttribute(gateup_fn(form, gateup_kc(plan)), cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -616,8 +797,11 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     const bool pack = B <= 64;
     const int mt = B <= BM ? 1 : 2, form = pack ? 0 : mt;
     const TokenTile tt = token_tile(pack, mt, B);
-    const int R = min(128, ((c.d_ff + plan->sm_count - 1) / plan->sm_count + 7) & ~7);
-    const int gateup_ctas = (c.d_ff + R - 1) / R;
+    const bool pair = recover != nullptr && mt == 2;
+    const int unit = pair ? 16 : 8;   // the instructions take N = 2 R in units of 16, over a pair of CTAs of 32
+    const int R = min(128, ((c.d_ff + plan->sm_count - 1) / plan->sm_count + unit - 1) & ~(unit - 1));
+    const int gateup_ctas = pair ? 2 * ((c.d_ff + 2 * R - 1) / (2 * R)) : (c.d_ff + R - 1) / R;
+    const int half = ((B + 1) / 2 + 7) & ~7;   // pair: tokens of the even CTA
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16), *x_lo = x_hi + (size_t)c.max_tokens * c.d;
     __nv_bfloat16 *act = static_cast<__nv_bfloat16 *>(plan->act), *act_lo = act + (size_t)c.max_tokens * c.d_ff;
     // Given supports, more than 128 tokens: gate/up over the groups in use.  There a channel costs more than its bytes (7B, 200
@@ -635,6 +819,15 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     {
         StageTimer timer(plan, CS_STAGE_EXEC, st);
         if (recover != nullptr) plan->stage_seen[CS_STAGE_RECOVER] = 0;   // part of this launch
+        if (pair) {
+            CUtensorMap tm_h, tm_h_lo;
+            if (!make_map(&tm_h, x_hi, c.d, B, c.d, half) || !make_map(&tm_h_lo, x_lo, c.d, B, c.d, half))
+                return record_cuda(plan, cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
+            launch_pdl(true, gateup_pair_fn(gateup_kc(plan)), dim3(gateup_ctas), dim3(kDecThreads + kRecThreads),
+                       1024 + (size_t)gateup_pair_stages(R) * (kPairTokenBytes + 2 * R * BK * 2) + sizeof(Barriers), st, tm_h, tm_h_lo, tm_g, tm_u, B, half,
+                       R, c.d, c.d_ff, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr, c.rms_eps, *recover, act,
+                       act_lo, plan->status);
+        } else
         launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
                    dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), by_list ? 1024 + (size_t)kDecRing + sizeof(Barriers) : decode_smem(tt, 2 * R * BK * 2),
                    st, tm_x, tm_x_lo, tm_g, tm_u, tm_gu, tm_uu, B, R, c.d, c.d_ff,

@@ -30,6 +30,19 @@ def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
     plan.close()
 
 
+# Pairs of CTAs, more than 128 tokens: halves of the tokens that are no multiple of 8, a last pair whose second CTA has channels past d_ff or
+# none, fewer pairs than SMs, the recovery's list lengths.
+@pytest.mark.parametrize("B,norm", [(131, False), (145, True), (255, False)])
+@pytest.mark.parametrize("d,G,m,k", [(256, 5, 4, 2), (256, 91, 40, 30), (512, 107, 33, 50)])
+def test_layer_step_on_pairs_of_ctas(d, G, m, k, B, norm):
+    cfg = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"].with_(n_layers=1, d=d, d_ff=128 * G, m=m, k=k, T=6, B=B, index=340 + B)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    rep, _, _ = compare_layer_step(cfg, L, plan, W.make_tokens(cfg, L.A).h)   # output bound 1e-4 (parity_util)
+    assert rep.excused <= max(1, B // 16), rep
+    plan.close()
+
+
 # Gather path: few rows for many CTAs, and three or four tokens of 55 to 60 groups.
 @pytest.mark.parametrize("k,B", [(55, 4), (56, 4), (60, 3), (1, 3)])
 def test_gather_rows_per_cta_edges(k, B):
