@@ -357,13 +357,14 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     teardown_cta(bars, warp, tcols);
 }
 
-// The same for a step of more than 128 tokens, on pairs of CTAs (a cluster of two): with both accumulators in one CTA every weight tile is
-// read from shared memory by four instructions and every k block moves 228 KB through that port for 20 KB of weights (1.03 us a k block,
-// 68 us at 7B and 200 tokens, the tensor pipe 51 % busy).  Here one instruction has M = 256: each CTA holds half of the tokens (their
-// values and their remainders, 128 rows each) and half of the pair's channels, R of 2 R, gate rows then up rows: 156 KB for the
-// same 20 KB of weights per CTA.  (One step, 7B: 200 tokens 135.5 to 127.0 us, in short bursts 132 to 121, 256 tokens 139 to 127; d = 5120 with 27 of 108
-// groups, 200 tokens 189 to 181; 129 tokens even, 113.9 and 112.6, so every batch beyond 128 tokens takes it.)  Gate accumulates in tensor-memory columns 0 .. 2 R, up from 256 on.  The even CTA's MMA thread issues
-// for both; no multicast load, each CTA fetches its own tiles and signals the even CTA's barrier.
+// The same for a step of more than 128 tokens, on pairs of CTAs (a cluster of two).  With both accumulators in one CTA every weight tile
+// is read from shared memory by four instructions and every k block moves 228 KB through that port for 20 KB of weights (1.03 us a k
+// block, 68 us at 7B and 200 tokens, the tensor pipe 51 % busy).  Here one instruction has M = 256: each CTA holds half of the tokens
+// (their values and their remainders, 128 rows each) and half of the pair's channels, R of 2 R, gate rows then up rows: 156 KB for the
+// same 20 KB of weights per CTA.  One step, 7B: 200 tokens 135.5 to 127.0 us, in short bursts 132 to 121, 256 tokens 139 to 127; d = 5120
+// with 27 of 108 groups, 200 tokens 189 to 181; 129 tokens 113.9 to 112.6, so every batch beyond 128 tokens takes it.
+// Gate accumulates in tensor-memory columns 0 .. 2 R, up from 256 on.  The even CTA's MMA thread issues for both; no multicast load, each
+// CTA fetches its own tiles and signals the even CTA's barrier.
 constexpr int kPairTokenBytes = 2 * kABytes;   // value rows, then remainder rows
 __host__ __device__ inline int gateup_pair_stages(int R) { return min(kMaxStages, kDecRing / (kPairTokenBytes + 2 * R * BK * 2)); }
 template <int KC>

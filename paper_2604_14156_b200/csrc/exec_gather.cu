@@ -75,7 +75,10 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 // FULL = every row is a whole number of units and of 512-chunk slices: no bounds checks inside.
 // check: the CTAs with blockIdx.x == 0 also validate their token's support row (ascending, distinct).
 // SPEC: `support` is the recovery's slot table, [tokens, kSlotTablePitch], still changing.
-template <typename WT, int CPT, bool FULL, bool SPEC>
+// STEP: the supports of the recovery ahead: neither check nor warm, and no code for them, nor for changing segments where FULL rules
+// them out (the kernel begins with its code cold; 7B step of one token 23.35 and 22.85 us, three 38.7 and 38.1, 8B four 54.8 and 54.2;
+// rows that are not FULL, d = 5120 and 2048: equal).
+template <typename WT, int CPT, bool FULL, bool SPEC, bool STEP>
 __global__ void __launch_bounds__(SPEC ? kSpecThreads : kGatherThreads, 1)
 ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT *__restrict__ Wdt,
                   const float *__restrict__ h, const int32_t *__restrict__ support, int d, int lb, int k, int G,
@@ -142,7 +145,7 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
         // streams them while the remaining iterations run.  Only a hint: whatever the table holds at this
         // moment, nothing but the range check stands between it and the request, and the pass below reads
         // the final support as always.
-        if (warm != nullptr && tid < 3 * k) {
+        if (!STEP && warm != nullptr && tid < 3 * k) {
             const int mat = tid / k, j = tid - mat * k;
             const size_t chunk = ((size_t)d << lb) * sizeof(WT);            // one group's rows are contiguous
             const size_t seg = ((chunk / nx) + 127) & ~(size_t)127;         // this CTA's share of each block
@@ -171,7 +174,7 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
             bad_s[tid] = bad;
             chan_s[tid] = (g << lb) + (R & (b - 1));
         }
-        if (check && bx == 0 && status != nullptr && tid >= kGatherThreads - kMaxG && tid - (kGatherThreads - kMaxG) < k) {
+        if (!STEP && check && bx == 0 && status != nullptr && tid >= kGatherThreads - kMaxG && tid - (kGatherThreads - kMaxG) < k) {
             // the last warps of the first CTA check the row: ascending, hence distinct (the range is checked above)
             const int j = tid - (kGatherThreads - kMaxG);
             if (j > 0 && ld_dep(support + (size_t)t * k + j) <= ld_dep(support + (size_t)t * k + j - 1))
@@ -224,7 +227,7 @@ ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT
     };
     // When the number of segments divides the number of warps, a warp meets the same segment in every
     // unit and its slice of h is loaded once; otherwise it is fetched (from L1) per unit.
-    const bool fixed_seg = kGatherWarps % nseg == 0;
+    const bool fixed_seg = FULL || kGatherWarps % nseg == 0;   // (FULL: 4, 8 or 16 segments)
     float hv[kUnitChunks][E];
     auto load_h = [&](int seg) {
         const float *hp = h_lane + seg * kSegElems;
@@ -467,14 +470,14 @@ cs_status launch_check_support(cs_plan *plan, const int32_t *support, int B, cud
 }
 
 // Picks the instantiation: chunks per thread in the down phase, and whether rows need bounds checks.
-template <typename WT, bool SPEC>
+template <typename WT, bool SPEC, bool STEP>
 static void launch_gather_kernel(dim3 grid, cudaStream_t st, int cpt, int chunks, const WT *Wg, const WT *Wu,
                                  const WT *Wd, const float *h, const int32_t *sup, int d, int b, int k, int G,
                                  float *partial, DeviceStatus *status, int check, const int32_t *warm) {
     const bool full = chunks % kGatherThreads == 0 && (cpt == 1 || cpt == 2 || cpt == 4);
     const int lb = b == 64 ? 6 : 7;
 #define CS_GATHER_CASE(N, F)                                                                              \
-    launch_pdl(true, ffn_gather_kernel<WT, N, F, SPEC>, grid, dim3(SPEC ? kSpecThreads : kGatherThreads), kRingBytes, st, \
+    launch_pdl(true, ffn_gather_kernel<WT, N, F, SPEC, STEP>, grid, dim3(SPEC ? kSpecThreads : kGatherThreads), kRingBytes, st, \
                Wg, Wu, Wd, h, sup, d, lb, k, G, partial, status, check, warm)
     if (cpt <= 1) { if (full) CS_GATHER_CASE(1, true); else CS_GATHER_CASE(1, false); }
     else if (cpt <= 2) { if (full) CS_GATHER_CASE(2, true); else CS_GATHER_CASE(2, false); }
@@ -515,10 +518,13 @@ static cs_status gather_typed(cs_plan *plan, const cs_layer *L, const float *h, 
         {
             StageTimer timer(plan, CS_STAGE_EXEC, st);
             if (spec)
-                launch_gather_kernel<WT, true>(grid, st, cpt, c.d / E, Wg, Wu, Wd, hp, support + (size_t)t0 * kSlotTablePitch,
+                launch_gather_kernel<WT, true, false>(grid, st, cpt, c.d / E, Wg, Wu, Wd, hp, support + (size_t)t0 * kSlotTablePitch,
                                                c.d, c.group, c.k, plan->G, plan->partial, plan->status, 0, nullptr);
+            else if (!check && warm == nullptr)
+                launch_gather_kernel<WT, false, true>(grid, st, cpt, c.d / E, Wg, Wu, Wd, hp, support + (size_t)t0 * c.k, c.d,
+                                                      c.group, c.k, plan->G, plan->partial, plan->status, 0, nullptr);
             else
-                launch_gather_kernel<WT, false>(grid, st, cpt, c.d / E, Wg, Wu, Wd, hp, support + (size_t)t0 * c.k, c.d,
+                launch_gather_kernel<WT, false, false>(grid, st, cpt, c.d / E, Wg, Wu, Wd, hp, support + (size_t)t0 * c.k, c.d,
                                                 c.group, c.k, plan->G, plan->partial, plan->status, check,
                                                 warm != nullptr ? warm + (size_t)t0 * kSlotTablePitch : nullptr);
         }
@@ -537,15 +543,16 @@ static cs_status gather_typed(cs_plan *plan, const cs_layer *L, const float *h, 
 }
 
 // The ring needs more dynamic shared memory than the default limit: opt in once per kernel.
+template <typename WT, int N, bool SPEC, bool STEP>
+static cudaError_t gather_attr() {
+    const cudaError_t e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, true, SPEC, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(ffn_gather_kernel<WT, N, false, SPEC, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+}
 template <typename WT, int N>
 static cudaError_t gather_attrs(bool fused_too) {
-    cudaError_t e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-    if (e == cudaSuccess && fused_too)
-        e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-    if (e == cudaSuccess && fused_too)
-        e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    cudaError_t e = gather_attr<WT, N, false, false>();
+    if (e == cudaSuccess && fused_too) e = gather_attr<WT, N, false, true>();
+    if (e == cudaSuccess && fused_too) e = gather_attr<WT, N, true, false>();
     return e;
 }
 static cudaError_t gather_attrs_all(bool fused_too) {
@@ -620,7 +627,7 @@ static cudaError_t static_launch(const cs_config &c, const cs_layer *L, const fl
     const WT *Wg = static_cast<const WT *>(L->W_gate), *Wu = static_cast<const WT *>(L->W_up),
              *Wd = static_cast<const WT *>(L->Wd_t);
     dim3 grid(nx, B);
-    launch_gather_kernel<WT, false>(grid, st, cpt, c.d / E, Wg, Wu, Wd, h, support, c.d, c.group, c.k, c.d_ff / c.group,
+    launch_gather_kernel<WT, false, false>(grid, st, cpt, c.d / E, Wg, Wu, Wd, h, support, c.d, c.group, c.k, c.d_ff / c.group,
                                     partial, static_cast<DeviceStatus *>(nullptr), 0, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -30,6 +30,19 @@ def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
     plan.close()
 
 
+# Gather path: a step's form of the kernel against the one for given supports, the same bits.  Rows that are whole slices of 512 chunks
+# (one, two and four a thread) and rows that are not.
+@pytest.mark.parametrize("dtype,d", [("bf16", 4096), ("bf16", 8192), ("bf16", 5120), ("bf16", 320), ("f32", 2048), ("f32", 8192), ("f32", 2112), ("f32", 64)])
+def test_gather_step_and_given_supports_agree(dtype, d):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(n_layers=1, w_dtype=dtype, d=d, d_ff=64 * 20, group=64, m=12, k=5, T=6, B=2, index=350)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    lay, x = device_layer(plan, L), W.make_tokens(cfg, L.A).h.to("cuda:0")
+    out, sup, _, _ = cs.cs_layer_step(plan, lay, x)
+    assert torch.equal(cs.cs_ffn_exec(plan, lay, x, sup), out) and plan.device_status() == 0
+    plan.close()
+
+
 # Pairs of CTAs, more than 128 tokens: halves of the tokens that are no multiple of 8, a last pair whose second CTA has channels past d_ff or
 # none, fewer pairs than SMs, the recovery's list lengths.
 @pytest.mark.parametrize("B,norm", [(131, False), (145, True), (255, False)])
