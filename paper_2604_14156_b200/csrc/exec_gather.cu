@@ -555,18 +555,22 @@ static cudaError_t gather_attrs(bool fused_too) {
     if (e == cudaSuccess && fused_too) e = gather_attr<WT, N, true, false>();
     return e;
 }
-static cudaError_t gather_attrs_all(bool fused_too) {
-    cudaError_t e = gather_attrs<__nv_bfloat16, 1>(fused_too);
-    if (e == cudaSuccess) e = gather_attrs<__nv_bfloat16, 2>(fused_too);
-    if (e == cudaSuccess) e = gather_attrs<__nv_bfloat16, 4>(fused_too);
-    if (e == cudaSuccess) e = gather_attrs<float, 1>(fused_too);
-    if (e == cudaSuccess) e = gather_attrs<float, 2>(fused_too);
-    if (e == cudaSuccess) e = gather_attrs<float, 4>(fused_too);
+static cudaError_t gather_attrs_all() {   // for the entry without a plan
+    cudaError_t e = gather_attrs<__nv_bfloat16, 1>(false);
+    if (e == cudaSuccess) e = gather_attrs<__nv_bfloat16, 2>(false);
+    if (e == cudaSuccess) e = gather_attrs<__nv_bfloat16, 4>(false);
+    if (e == cudaSuccess) e = gather_attrs<float, 1>(false);
+    if (e == cudaSuccess) e = gather_attrs<float, 2>(false);
+    if (e == cudaSuccess) e = gather_attrs<float, 4>(false);
     return e;
 }
 
+// Of a plan's own weight type and row width only: each further kernel is loaded and costs plan creation its time.
 cs_status prepare_ffn_gather(cs_plan *plan) {
-    CS_CUDA_TRY(plan, gather_attrs_all(true));
+    const bool bf16 = plan->cfg.w_dtype == CS_BF16;
+    const int cpt = (plan->cfg.d / (bf16 ? 8 : 4) + kGatherThreads - 1) / kGatherThreads;
+    CS_CUDA_TRY(plan, bf16 ? (cpt <= 1 ? gather_attrs<__nv_bfloat16, 1>(true) : cpt <= 2 ? gather_attrs<__nv_bfloat16, 2>(true) : gather_attrs<__nv_bfloat16, 4>(true))
+                           : (cpt <= 1 ? gather_attrs<float, 1>(true) : cpt <= 2 ? gather_attrs<float, 2>(true) : gather_attrs<float, 4>(true)));
     CS_CUDA_TRY(plan, prefer_shared(reduce_partials_kernel));
     return CS_OK;
 }
@@ -611,7 +615,7 @@ static cudaError_t static_setup(int dev) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (e == cudaSuccess) e = gather_attrs_all(false);
+    if (e == cudaSuccess) e = gather_attrs_all();
     if (e != cudaSuccess) return e;
     g_static_sms[dev] = sms;
     g_static_ptr[dev] = static_cast<float *>(p);
