@@ -127,6 +127,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     }
     __syncthreads();
     float phc[32];
+    if (PLAIN && rank == 0 && tid < GP) recover_init(rs, tid, m, a.k);
     if (rank == 0 && m <= 32 && tid < GP) {
 #pragma unroll
         for (int row = 0; row < 32; ++row) phc[row] = row < m && tid < G ? phi_s[row * ppitch + tid] : 0.f;

@@ -194,6 +194,16 @@ __device__ __forceinline__ void recover_load_phi(const float *__restrict__ Phi, 
     for (int row = 0; row < 32; ++row) phc[row] = (valid && row < m) ? __ldg(Phi + row * G + g) : 0.f;
 }
 
+// What a PLAIN recovery starts from, by the same threads, with a barrier between this and recover_token: nothing of it depends on y.
+// (In the sensing launch ahead of the wait for x, and a barrier less behind it: 7B step of one token 22.75 and 22.64 us, 2048-wide
+// layer 15.58 and 15.38, three tokens 21.2 and 20.9.)
+template <int NW, int KC>
+__device__ __forceinline__ void recover_init(RecoverSmem<NW, KC> &s, int g, int m, int k) {
+    constexpr int GP = 32 * NW, NV = RecoverSmem<NW, KC>::NV;
+    for (int i = m + g; i < kMaxM; i += GP) s.y[i] = 0.f;
+    for (int i = g; i < NV; i += GP) { s.val[0][i] = 0.f; s.val[1][i] = 0.f; s.idx[i] = i < k ? i : 0; }
+}
+
 // Runs the recovery of one token.  g = this thread's entry (0 .. 32*NW-1); all 32*NW threads call it
 // together and synchronise on named barrier BAR.  M: where the entries of I - mu Phi^T Phi come from
 // (the dense form reads whole rows of the global matrix, whose pitch must be 32 * NW).  phc: the thread's column of Phi when m <= 32
@@ -203,7 +213,8 @@ __device__ __forceinline__ void recover_load_phi(const float *__restrict__ Phi, 
 // start's own when T == 0 or the start is warm); from then on s.idx always holds k valid groups and changes only where the
 // support changes: slot_changed(slot, g) is called by the thread whose entry g has just taken `slot`.
 // table_final() is called once by every thread after the last iteration, before the outputs are
-// written.  mask (may be NULL): NW words of membership bits.  PLAIN: neither a warm start nor a temporal term, and no code for them.
+// written.  mask (may be NULL): NW words of membership bits.  PLAIN: neither a warm start nor a temporal term, and no code for them
+// (recover_init has run).
 template <int NW, int KC, int BAR, bool PLAIN, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
 __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int g, const float *__restrict__ Phi,
                                               const MSource M, float mu, LoadY load_y, int m, int G, int k, int T, int32_t *__restrict__ support,
@@ -228,13 +239,11 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
     }
     if constexpr (KC == 0) M.template row<GP>(gm, mreg);   // row g of M: what multiplies into entry g
     load_y(s);   // s.y, complete at the next barrier
-    for (int i = m + g; i < kMaxM; i += GP) s.y[i] = 0.f;
     // z_0 = 0 with the support the order assigns to an all-zero vector (indices 0..k-1), or, warm
     // started, the k-sparse iterate handed in (sup0 ascending and distinct, z0 its values).
     const bool warm = !PLAIN && sup0 != nullptr;
     const float tgamma = PLAIN ? 0.f : tgamma_;
-    s.slot[g] = -1;
-    for (int i = g; i < NV; i += GP) { s.val[0][i] = 0.f; s.val[1][i] = 0.f; s.idx[i] = i < k ? i : 0; }
+    if constexpr (!PLAIN) { recover_init(s, g, m, k); s.slot[g] = -1; }
     bar_sync<BAR, GP>();
     if (warm) {
         for (int j = g; j < k; j += GP) {
@@ -246,7 +255,7 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
             else s.val[0][e] = zv;
         }
     }
-    bar_sync<BAR, GP>();
+    if constexpr (!PLAIN) bar_sync<BAR, GP>();
     bool kept = warm ? s.slot[g] >= 0 : g < k;
     int slot = warm ? max(s.slot[g], 0) : g;
     float v = 0.f;

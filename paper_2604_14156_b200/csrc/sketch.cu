@@ -177,6 +177,8 @@ sketch_kernel(const float *__restrict__ S, const float *__restrict__ x, const fl
         }
         const int g = tid;
         const int k = ra.k;
+        recover_init(rs, g, m, k);
+        bar_sync<1, 32 * kSketchRecNW>();
         recover_token<kSketchRecNW, kSketchRecKC, 1, true>(
             rs, g, Phi, src, mu,
             [&](auto &sm) { for (int row = g; row < m; row += 32 * kSketchRecNW) sm.y[row] = ld_dep(y + (size_t)t * m + row); }, m, G, k, ra.T,
