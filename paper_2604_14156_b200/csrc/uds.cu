@@ -27,7 +27,13 @@ __device__ __forceinline__ void add_logits(Moments &s, const float (&v)[N]) {
     float m = v[0];
 #pragma unroll
     for (int j = 1; j < N; ++j) m = fmaxf(m, v[j]);
-    if (m == -INFINITY) return;
+    if (m == -INFINITY) {                         // nothing but -inf, or a NaN among it (fmaxf passes a NaN over)
+        bool nan = false;
+#pragma unroll
+        for (int j = 0; j < N; ++j) nan |= v[j] != v[j];
+        if (nan) s.Z = NAN;                       // (stays one in every fold below)
+        return;
+    }
     if (s.Z == 0.f) {
         s.M = m;
     } else if (m > s.M) {                         // new maximum: rescale what has been summed

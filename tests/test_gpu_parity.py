@@ -830,6 +830,27 @@ def test_uds_budget_special_rows():
     plan.close()
 
 
+# A NaN or +inf logit where everything else a thread folds with it is -inf: masked vocabulary entries, or the padding of a row (or of
+# a CTA's share: from 4096 logits on a row is split) that ends inside a batch of loads.
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("V", [1, 33, 512, 513, 4097, 8193, 32000])
+def test_uds_budget_nan_among_masked_logits(V, bad):
+    where = sorted({0, V // 3, V // 2, V - 2, V - 1} & set(range(V)))
+    L = torch.full((3 * len(where) + 1, V), float("-inf"))
+    for i, at in enumerate(where):
+        L[3 * i, at] = bad                                               # nothing else
+        L[3 * i + 1] = torch.randn(V, generator=torch.Generator().manual_seed(V + i))
+        L[3 * i + 1, at] = bad                                           # among finite entries
+        L[3 * i + 2, ::97] = 0.5
+        L[3 * i + 2, at] = bad                                           # among few unmasked entries
+    L[-1, 0] = 1.0                                                       # a good row beside them: H = 0
+    plan = cs.Plan(256, 1024, 64, 8, 4, 4, torch.float32, len(L), 1e-5)
+    m_t, H = cs.cs_uds_budget(plan, L.to(DEV), 16.0, 0.75, 8, 64)
+    assert torch.isnan(H[:-1]).all() and (m_t[:-1] == 64).all(), (H, m_t)
+    assert H[-1] == 0.0 and m_t[-1] == 16
+    plan.close()
+
+
 def test_uds_budget_selects_a_row_prefix_of_the_measurement_bank():
     """Sec. 8.1 (the sensing matrix varies in its row dimension): the first m_t rows of a bank
     S [m_max, d], Phi [m_max, G] are the operands of a plan created with m = m_t."""
