@@ -16,6 +16,12 @@
  *   - Calls only enqueue work on `stream` (a cudaStream_t passed as void*, NULL = default
  *     stream) and return without synchronising.  A plan must not be used from two streams at
  *     once: its scratch is shared by all calls.
+ *   - The arrays of a cs_layer (and S, Phi where a call takes them by themselves) are parameters: a
+ *     launch may read them while the launches ahead of it on the stream still run, as far as those
+ *     allow it (this library's do; so do kernels that trigger a programmatic launch themselves).
+ *     Updating them on the stream by copies or ordinary kernels ahead of a call is fine.  A
+ *     parameter that was written by a call of this library needs something in between that waits
+ *     for that call: an ordinary kernel or copy, a cs_uds_budget, an event or a synchronisation.
  *   - Matrices are dense row-major.  "f32" is IEEE binary32; "bf16" is bfloat16.
  *   - Errors are return codes.  Arguments are validated on the host before anything is
  *     launched; on any code other than CS_OK nothing was enqueued.  There is no CPU fallback:

@@ -85,9 +85,11 @@ uds_kernel(const float *__restrict__ logits, int V, int per, float m_base, float
     const int lo = s * per, hi = min(V, lo + per);
     const float *row = logits + (size_t)t * V;
     Moments acc{0.f, 0.f, 0.f};
-    pdl_launch_dependents();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // CTA 0 has started, see below
     pdl_wait();   // the logits may come from the kernel before
+    // Not earlier: the launch behind reads its parameters (S, Phi, weights) before its own wait, and what was enqueued ahead of this
+    // call may have written them.  From here on that has completed.
+    pdl_launch_dependents();
     int i = lo + (int)threadIdx.x;
     for (int end = lo + N * kUdsThreads; end < hi; end += N * kUdsThreads, i += N * kUdsThreads) {   // whole batches
         float v[N];

@@ -851,6 +851,43 @@ def test_uds_budget_nan_among_masked_logits(V, bad):
     plan.close()
 
 
+def test_parameters_written_ahead_of_a_budget_call_reach_the_step_behind_it():
+    """The launch behind a budget call starts once everything ahead of the call has completed.  S is the z output of a
+    recovery of some hundred microseconds that lets its successor start at once; the step reads S before its own wait."""
+    g = torch.Generator(device=DEV).manual_seed(5)
+    rn = lambda *s: torch.empty(s, device=DEV).normal_(0.0, 1.0, generator=g)
+    m, d = 8, 64
+    writer = cs.Plan(64, 128 * 64, 64, 32, d, 1000, torch.float32, m, 1e-5)   # 64 of 128 groups: z is [m, 64]
+    wPhi, wy = rn(32, 128) / 32 ** 0.5, rn(m, 32)
+    wmu = W.spectral_step(wPhi)
+    sup, resid = torch.empty((m, d), dtype=torch.int32, device=DEV), torch.empty((m,), device=DEV)
+    S = torch.zeros((m, d), device=DEV)
+    plan = cs.Plan(d, 1024, 64, m, 4, 10, torch.float32, 2, 1e-5)
+    Phi = rn(m, 16) / m ** 0.5
+    lay = cs.Layer(plan, S, Phi, rn(1024, d), rn(1024, d), rn(1024, d), W.spectral_step(Phi))
+    x, logits = rn(2, d), rn(2, 5000)
+
+    def write():
+        stream = torch.cuda.current_stream().cuda_stream
+        writer.check(writer.lib.cs_recover(writer.handle, wPhi.data_ptr(), wmu, wy.data_ptr(), m, sup.data_ptr(), S.data_ptr(),
+                                           resid.data_ptr(), stream), "cs_recover")
+
+    write()
+    torch.cuda.synchronize()
+    ref = [t.clone() for t in cs.cs_layer_step(plan, lay, x)]
+    assert ref[2].any()
+    for _ in range(10):
+        S.zero_()
+        torch.cuda.synchronize()
+        write()
+        cs.cs_uds_budget(plan, logits, 16.0, 0.75, 8, 64)
+        got = cs.cs_layer_step(plan, lay, x)
+        torch.cuda.synchronize()
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b)
+    plan.close(); writer.close()
+
+
 def test_uds_budget_selects_a_row_prefix_of_the_measurement_bank():
     """Sec. 8.1 (the sensing matrix varies in its row dimension): the first m_t rows of a bank
     S [m_max, d], Phi [m_max, G] are the operands of a plan created with m = m_t."""
