@@ -199,8 +199,8 @@ cs_status cs_sketch_srht(cs_plan *plan, const uint32_t *sign_bits, const int32_t
  * measurement bank the next cs_sketch / cs_recover use: S [m_max,d] and Phi [m_max,G] are row-major,
  * so their first m_t rows are the operands of a plan created with m = m_t (with the step mu of that
  * row prefix); the caller reads m_t back with the sampled token and picks the plan.
- * Uses the plan's scratch: order it on the stream of the plan's other calls.  1 <= m_min <= m_max,
- * m_base > 0, gamma >= 0, B <= max_tokens (else CS_ERR_SHAPE / CS_ERR_NONFINITE).
+ * Uses none of the plan's scratch.  1 <= m_min <= m_max, m_base > 0, gamma >= 0, B <= max_tokens
+ * (else CS_ERR_SHAPE / CS_ERR_NONFINITE).
  */
 cs_status cs_uds_budget(cs_plan *plan, const float *logits, int32_t B, int32_t V, float m_base, float gamma,
                         int32_t m_min, int32_t m_max, float *H, int32_t *m_t, void *stream);

@@ -74,14 +74,14 @@ __device__ __forceinline__ void warp_fold(Moments &s) {
     s.W = warp_sum(s.W);
 }
 
-// grid (CTAs of a row, B), the row's CTAs one cluster: CTA (s, t) takes elements [s * per, min(V, (s + 1) * per)) of row t, N of a
+// grid: B rows of `ctas` CTAs, which are one cluster: CTA s of row t takes elements [s * per, min(V, (s + 1) * per)), N of a
 // thread in flight.  The floor is taken in double precision from the f32 entropy; a NaN entropy (a NaN or +inf logit) asks for m_max.
 template <int N>
 __global__ void __launch_bounds__(kUdsThreads)
-uds_kernel(const float *__restrict__ logits, int V, int per, float m_base, float gamma, int m_min, int m_max, float *__restrict__ H_out,
+uds_kernel(const float *__restrict__ logits, int V, int ctas, int per, float m_base, float gamma, int m_min, int m_max, float *__restrict__ H_out,
            int32_t *__restrict__ m_out) {
     __shared__ Moments warp_s[kUdsWarps], cta_s[kUdsMaxCtas];
-    const int t = blockIdx.y, s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = blockIdx.x / ctas, s = blockIdx.x - t * ctas, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lo = s * per, hi = min(V, lo + per);
     const float *row = logits + (size_t)t * V;
     Moments acc{0.f, 0.f, 0.f};
@@ -125,7 +125,7 @@ uds_kernel(const float *__restrict__ logits, int V, int per, float m_base, float
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (s != 0 || warp != 0) return;
-    acc = lane < (int)gridDim.x ? cta_s[lane] : Moments{0.f, 0.f, 0.f};
+    acc = lane < ctas ? cta_s[lane] : Moments{0.f, 0.f, 0.f};
     warp_fold(acc);
     if (lane == 0) {
         float H = acc.Z > 0.f ? fmaxf(logf(acc.Z) - acc.W / acc.Z, 0.f) : (acc.Z == 0.f ? 0.f : acc.Z);
@@ -142,13 +142,12 @@ uds_kernel(const float *__restrict__ logits, int V, int per, float m_base, float
 
 cs_status launch_uds_budget(cs_plan *plan, const float *logits, int B, int V, float m_base, float gamma,
                             int m_min, int m_max, float *H, int32_t *m_t, cudaStream_t st) {
-    if ((size_t)B * sizeof(Moments) > (size_t)kGatherMaxTokens * plan->nx_max * plan->cfg.d * sizeof(float)) return CS_ERR_SHAPE;
     // about two CTAs per SM, each with 2048 elements at least
     int ctas = 1;
     while (ctas < kUdsMaxCtas && 2 * ctas * B <= 2 * plan->sm_count && V >= 2 * ctas * 2048) ctas *= 2;
     const int per = (V + ctas - 1) / ctas;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas, B); cfg.blockDim = dim3(kUdsThreads); cfg.stream = st;
+    cfg.gridDim = dim3(ctas * B); cfg.blockDim = dim3(kUdsThreads); cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -157,7 +156,7 @@ cs_status launch_uds_budget(cs_plan *plan, const float *logits, int B, int V, fl
     cfg.attrs = attr; cfg.numAttrs = 2;
     // 16 logits of a thread in flight where the CTAs are too few to keep the memory busy with 8
     const bool deep = per > 8 * kUdsThreads && ctas * B <= 2 * plan->sm_count;
-    cudaLaunchKernelEx(&cfg, deep ? uds_kernel<16> : uds_kernel<8>, logits, V, per, m_base, gamma, m_min, m_max, H, m_t);
+    cudaLaunchKernelEx(&cfg, deep ? uds_kernel<16> : uds_kernel<8>, logits, V, ctas, per, m_base, gamma, m_min, m_max, H, m_t);
     plan->launches++;
     CS_CUDA_TRY(plan, cudaGetLastError());
     return CS_OK;

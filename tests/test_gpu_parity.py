@@ -851,6 +851,19 @@ def test_uds_budget_nan_among_masked_logits(V, bad):
     plan.close()
 
 
+def test_uds_budget_takes_every_batch_of_the_plan():
+    """More tokens than a grid has rows (65535) or the gather's scratch of a narrow plan has moments."""
+    B, V = 70001, 5
+    rows = torch.randn((7, V), generator=torch.Generator().manual_seed(11)) * 2.0
+    plan = cs.Plan(64, 512, 64, 4, 2, 1, torch.float32, B, 1e-5)
+    m_t, H = cs.cs_uds_budget(plan, rows.to(DEV).repeat((B + 6) // 7, 1)[:B].contiguous(), 16.0, 0.75, 8, 64)
+    torch.cuda.synchronize()
+    for i in range(7):
+        assert (H[i::7] == H[i]).all() and (m_t[i::7] == m_t[i]).all()
+    _check_budget(m_t[:7], H[:7], oracle.uds_budget(rows, 16.0, 0.75, 8, 64), 16.0, 0.75)
+    plan.close()
+
+
 def test_parameters_written_ahead_of_a_budget_call_reach_the_step_behind_it():
     """The launch behind a budget call starts once everything ahead of the call has completed.  S is the z output of a
     recovery of some hundred microseconds that lets its successor start at once; the step reads S before its own wait."""
