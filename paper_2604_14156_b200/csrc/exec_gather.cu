@@ -75,9 +75,10 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 // FULL = every row is a whole number of units and of 512-chunk slices: no bounds checks inside.
 // check: the CTAs with blockIdx.x == 0 also validate their token's support row (ascending, distinct).
 // SPEC: `support` is the recovery's slot table, [tokens, kSlotTablePitch], still changing.
-// STEP: the supports of the recovery ahead: neither check nor warm, and no code for them, nor for changing segments where FULL rules
-// them out (the kernel begins with its code cold; 7B step of one token 23.35 and 22.85 us, three 38.7 and 38.1, 8B four 54.8 and 54.2;
-// rows that are not FULL, d = 5120 and 2048: equal).
+// STEP (FULL only): the supports of the recovery ahead: neither check nor warm, and no code for them (the kernel begins with its code
+// cold; 7B step of one token 23.35 and 22.85 us, three 38.7 and 38.1, 8B four 54.8 and 54.2).  Rows that are not FULL take the form
+// with both: one of their own gained nothing (27 of 108 groups of d = 5120, one token 37.1 us a step without it, 37.3 with it; 12 of 48
+// of d = 2048 16.9 either way).
 template <typename WT, int CPT, bool FULL, bool SPEC, bool STEP>
 __global__ void __launch_bounds__(SPEC ? kSpecThreads : kGatherThreads, 1)
 ffn_gather_kernel(const WT *__restrict__ Wg, const WT *__restrict__ Wu, const WT *__restrict__ Wdt,
@@ -477,7 +478,7 @@ static void launch_gather_kernel(dim3 grid, cudaStream_t st, int cpt, int chunks
     const bool full = chunks % kGatherThreads == 0 && (cpt == 1 || cpt == 2 || cpt == 4);
     const int lb = b == 64 ? 6 : 7;
 #define CS_GATHER_CASE(N, F)                                                                              \
-    launch_pdl(true, ffn_gather_kernel<WT, N, F, SPEC, STEP>, grid, dim3(SPEC ? kSpecThreads : kGatherThreads), kRingBytes, st, \
+    launch_pdl(true, ffn_gather_kernel<WT, N, F, SPEC, STEP && F>, grid, dim3(SPEC ? kSpecThreads : kGatherThreads), kRingBytes, st, \
                Wg, Wu, Wd, h, sup, d, lb, k, G, partial, status, check, warm)
     if (cpt <= 1) { if (full) CS_GATHER_CASE(1, true); else CS_GATHER_CASE(1, false); }
     else if (cpt <= 2) { if (full) CS_GATHER_CASE(2, true); else CS_GATHER_CASE(2, false); }
@@ -546,7 +547,8 @@ static cs_status gather_typed(cs_plan *plan, const cs_layer *L, const float *h, 
 template <typename WT, int N, bool SPEC, bool STEP>
 static cudaError_t gather_attr() {
     const cudaError_t e = cudaFuncSetAttribute(ffn_gather_kernel<WT, N, true, SPEC, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(ffn_gather_kernel<WT, N, false, SPEC, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if constexpr (STEP) return e;   // FULL only
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(ffn_gather_kernel<WT, N, false, SPEC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
 }
 template <typename WT, int N>
 static cudaError_t gather_attrs(bool fused_too) {
