@@ -127,7 +127,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     }
     __syncthreads();
     float phc[32];
-    if (PLAIN && rank == 0 && tid < GP) recover_init(rs, tid, m, a.k);
+    if (rank == 0 && tid < GP) recover_init<!PLAIN>(rs, tid, m, a.k);
     if (rank == 0 && m <= 32 && tid < GP) {
 #pragma unroll
         for (int row = 0; row < 32; ++row) phc[row] = row < m && tid < G ? phi_s[row * ppitch + tid] : 0.f;
@@ -264,7 +264,7 @@ sense_recover_kernel(const __grid_constant__ SenseArgs sa, const __grid_constant
     }
     if (rank != 0 || tid >= GP) return;
     const int g = tid;
-    recover_row<NW, KC, 1, PLAIN>(
+    recover_row<NW, KC, 1, PLAIN, true>(
         rs, a, SharedSource{M_s, phi_s, G, pitch},
         [&](auto &sm) {
             for (int i = g; i < m; i += GP) {
@@ -282,18 +282,15 @@ typedef void (*SenseFn)(SenseArgs, RecoverArgs);
 
 typedef void (*RecoverFn)(RecoverArgs);
 static int recover_kc(int k) { return k <= 64 ? (k + 7) / 8 : 0; }
+// k <= G <= 32 NW: the lists a width can meet, and from 65 groups on the dense form.
 template <int NW> static RecoverFn recover_fn_kc(int k) {
-    switch (recover_kc(k)) {
-        case 1: return recover_kernel<NW, 1, false>;
-        case 2: return recover_kernel<NW, 2, false>;
-        case 3: return recover_kernel<NW, 3, false>;
-        case 4: return recover_kernel<NW, 4, false>;
-        case 5: return recover_kernel<NW, 5, false>;
-        case 6: return recover_kernel<NW, 6, false>;
-        case 7: return recover_kernel<NW, 7, false>;
-        case 8: return recover_kernel<NW, 8, false>;
-        default: return recover_kernel<NW, 0, false>;
-    }
+    const int kc = recover_kc(k);
+#define CS_RECOVER(KC) if (kc == KC) return recover_kernel<NW, KC, false>
+    CS_RECOVER(1); CS_RECOVER(2); CS_RECOVER(3); CS_RECOVER(4);
+    if constexpr (NW > 1) { CS_RECOVER(5); CS_RECOVER(6); CS_RECOVER(7); CS_RECOVER(8); }
+#undef CS_RECOVER
+    if constexpr (NW > 2) return recover_kernel<NW, 0, false>;
+    return nullptr;
 }
 static RecoverFn recover_fn(int G, int k) {
     switch ((G + 31) / 32) {
@@ -325,12 +322,14 @@ RecoverArgs recover_args(const cs_plan *plan, const float *Phi, float mu, const 
 
 enum SenseKind { kSensePlain, kSensePlainNorm, kSenseOptions, kSenseStaged };
 // all: every row of S has its place in shared memory; a plain step whose rows do not takes the form for options.  The list goes in steps
-// of 8 slots in every form (in steps of 16, 24 of 128 groups of d = 4096, m = 64: 29.4 and 31.1 us a step, with a warm start 25.9 and 27.7).
+// of 8 slots in every form (in steps of 16, 24 of 128 groups of d = 4096, m = 64: 31.3 and 28.8 us a step, with a warm start 27.9 and 25.2).
+// One form for options whether the rows fit or not: a step with drift, 12 of 48 groups of d = 2048, four tokens 24.4 us, with two forms and
+// recover_init ahead of the wait 23.0; 10 of 40 of d = 1024, one token 15.7 and 15.3; 22 of 86 of d = 5120 29.4 and 28.5.
 template <int NW, int KC> static SenseFn sense_fn_form(SenseKind kind, bool all) {
     if (kind == kSenseStaged) return sense_recover_kernel<NW, KC, true, true, 0, false>;
     if (kind == kSensePlain && all) return sense_recover_kernel<NW, KC, false, true, 0, true>;
     if (kind == kSensePlainNorm && all) return sense_recover_kernel<NW, KC, false, true, 1, true>;
-    return sense_recover_kernel<NW, KC, false, false, 2, false>;
+    return all ? sense_recover_kernel<NW, KC, false, false, 2, true> : sense_recover_kernel<NW, KC, false, false, 2, false>;
 }
 // k <= G <= 32 NW: the lists a width can meet.  The dense form (65 groups at least) has the prompt's kind only.
 template <int NW> static SenseFn sense_fn_kc(int k, SenseKind kind, bool all) {
@@ -389,7 +388,8 @@ static int sense_tokens(const cs_plan *plan, int smem) {
 
 cs_status prepare_recover(cs_plan *plan) {
     for (SenseKind kind : {kSensePlain, kSensePlainNorm, kSenseOptions, kSenseStaged})
-        CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k, kind, true), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
+        for (bool all : {false, true})
+            CS_CUDA_TRY(plan, cudaFuncSetAttribute(sense_fn(plan->G, plan->cfg.k, kind, all), cudaFuncAttributeMaxDynamicSharedMemorySize, kSenseSmem));
     plan->sense_tokens = sense_tokens(plan, kSenseSmem);
     if (!decode_recovers(plan)) CS_CUDA_TRY(plan, prefer_shared(recover_decode_fn(plan->G)));
     return CS_OK;

@@ -194,14 +194,16 @@ __device__ __forceinline__ void recover_load_phi(const float *__restrict__ Phi, 
     for (int row = 0; row < 32; ++row) phc[row] = (valid && row < m) ? __ldg(Phi + row * G + g) : 0.f;
 }
 
-// What a PLAIN recovery starts from, by the same threads, with a barrier between this and recover_token: nothing of it depends on y.
+// What a recovery starts from, by the same threads, with a barrier between this and recover_token: nothing of it depends on y.
+// SLOTS: for a warm start too.
 // (In the sensing launch ahead of the wait for x, and a barrier less behind it: 7B step of one token 22.75 and 22.64 us, 2048-wide
 // layer 15.58 and 15.38, three tokens 21.2 and 20.9.)
-template <int NW, int KC>
+template <bool SLOTS, int NW, int KC>
 __device__ __forceinline__ void recover_init(RecoverSmem<NW, KC> &s, int g, int m, int k) {
     constexpr int GP = 32 * NW, NV = RecoverSmem<NW, KC>::NV;
     for (int i = m + g; i < kMaxM; i += GP) s.y[i] = 0.f;
     for (int i = g; i < NV; i += GP) { s.val[0][i] = 0.f; s.val[1][i] = 0.f; s.idx[i] = i < k ? i : 0; }
+    if constexpr (SLOTS) s.slot[g] = -1;
 }
 
 // Runs the recovery of one token.  g = this thread's entry (0 .. 32*NW-1); all 32*NW threads call it
@@ -213,9 +215,9 @@ __device__ __forceinline__ void recover_init(RecoverSmem<NW, KC> &s, int g, int 
 // start's own when T == 0 or the start is warm); from then on s.idx always holds k valid groups and changes only where the
 // support changes: slot_changed(slot, g) is called by the thread whose entry g has just taken `slot`.
 // table_final() is called once by every thread after the last iteration, before the outputs are
-// written.  mask (may be NULL): NW words of membership bits.  PLAIN: neither a warm start nor a temporal term, and no code for them
-// (recover_init has run).
-template <int NW, int KC, int BAR, bool PLAIN, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
+// written.  mask (may be NULL): NW words of membership bits.  PLAIN: neither a warm start nor a temporal term, and no code for them.
+// INIT: recover_init has run.
+template <int NW, int KC, int BAR, bool PLAIN, bool INIT, typename MSource, typename LoadY, typename TableReady, typename SlotChanged, typename TableFinal>
 __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int g, const float *__restrict__ Phi,
                                               const MSource M, float mu, LoadY load_y, int m, int G, int k, int T, int32_t *__restrict__ support,
                                               float *__restrict__ z_out, float *__restrict__ resid_out,
@@ -243,8 +245,7 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
     // started, the k-sparse iterate handed in (sup0 ascending and distinct, z0 its values).
     const bool warm = !PLAIN && sup0 != nullptr;
     const float tgamma = PLAIN ? 0.f : tgamma_;
-    if constexpr (!PLAIN) { recover_init(s, g, m, k); s.slot[g] = -1; }
-    bar_sync<BAR, GP>();
+    if constexpr (!INIT) { recover_init<!PLAIN>(s, g, m, k); bar_sync<BAR, GP>(); }
     if (warm) {
         for (int j = g; j < k; j += GP) {
             const int e = ld_dep(sup0 + j);
@@ -255,7 +256,7 @@ __device__ __forceinline__ void recover_token(RecoverSmem<NW, KC> &s, const int 
             else s.val[0][e] = zv;
         }
     }
-    if constexpr (!PLAIN) bar_sync<BAR, GP>();
+    bar_sync<BAR, GP>();
     bool kept = warm ? s.slot[g] >= 0 : g < k;
     int slot = warm ? max(s.slot[g], 0) : g;
     float v = 0.f;
@@ -542,8 +543,8 @@ __device__ __forceinline__ void y_from_parts(Smem &s, const SketchParts &p, int 
 
 // Token t of a batch, by the 32 * NW threads that meet on named barrier BAR: the check of the previous support, the
 // iteration, the outputs, the drift.  load_y as in recover_token; mask: [B, 4] membership bits, or NULL.
-// PLAIN: none of the options.
-template <int NW, int KC, int BAR, bool PLAIN = false, typename MSource, typename LoadY>
+// PLAIN: none of the options.  INIT: recover_init has run.
+template <int NW, int KC, int BAR, bool PLAIN = false, bool INIT = false, typename MSource, typename LoadY>
 __device__ __forceinline__ void recover_row(RecoverSmem<NW, KC> &s, const RecoverArgs &a, const MSource M, LoadY load_y,
                                             uint32_t *mask, int g, int t, const float (&phc)[32]) {
     const size_t row = (size_t)t * a.k;
@@ -552,7 +553,7 @@ __device__ __forceinline__ void recover_row(RecoverSmem<NW, KC> &s, const Recove
         const int e = ld_dep(p);
         if (e < 0 || e >= a.G || (g > 0 && ld_dep(p - 1) >= e)) atomicCAS(&a.status->code, 0, (int)CS_ERR_SUPPORT);
     }
-    recover_token<NW, KC, BAR, PLAIN>(
+    recover_token<NW, KC, BAR, PLAIN, INIT>(
         s, g, a.Phi, M, a.mu, load_y, a.m, a.G, a.k, a.T, a.support + row, a.z != nullptr ? a.z + row : nullptr,
         a.resid != nullptr ? a.resid + t : nullptr, a.sup0 != nullptr ? a.sup0 + row : nullptr,
         a.z0 != nullptr ? a.z0 + row : nullptr, a.tgamma, a.sup_prev != nullptr ? a.sup_prev + row : nullptr,

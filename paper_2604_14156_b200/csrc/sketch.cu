@@ -177,9 +177,9 @@ sketch_kernel(const float *__restrict__ S, const float *__restrict__ x, const fl
         }
         const int g = tid;
         const int k = ra.k;
-        recover_init(rs, g, m, k);
+        recover_init<false>(rs, g, m, k);
         bar_sync<1, 32 * kSketchRecNW>();
-        recover_token<kSketchRecNW, kSketchRecKC, 1, true>(
+        recover_token<kSketchRecNW, kSketchRecKC, 1, true, true>(
             rs, g, Phi, src, mu,
             [&](auto &sm) { for (int row = g; row < m; row += 32 * kSketchRecNW) sm.y[row] = ld_dep(y + (size_t)t * m + row); }, m, G, k, ra.T,
             ra.support != nullptr ? ra.support + (size_t)t * k : nullptr, ra.z != nullptr ? ra.z + (size_t)t * k : nullptr,
