@@ -13,7 +13,7 @@ LIB = os.path.join(PKG, "libcs_b200.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "-Xcompiler", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+    "-Xcompiler", "-fPIC", "-shared", "--threads", "0", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
 ]
 # No --use_fast_math: divisions and square roots stay IEEE; the kernels ask for the fast
 # exponential explicitly where they want it.
