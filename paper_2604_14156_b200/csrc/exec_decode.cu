@@ -379,6 +379,7 @@ decode_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int c0 = (int)(blockIdx.x >> 1) * 2 * R, t0 = (int)rank * half, nt = min(B - t0, half);   // the pair's channels, this CTA's tokens
+    const bool spare = c0 >= d_ff;   // the pair has no channels and recovers only
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int wbytes = 2 * R * BK * 2, stage_bytes = kPairTokenBytes + wbytes, stages = gateup_pair_stages(R), kblocks = d / BK;
     Barriers *bars = reinterpret_cast<Barriers *>(base + stages * stage_bytes);
@@ -389,7 +390,7 @@ decode_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid
         bars->aborted = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {   // the same warp of both CTAs allocates for the pair
+    if (warp == 1 && !spare) {   // the same warp of both CTAs allocates for the pair
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(&bars->tmem_base)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -399,7 +400,8 @@ decode_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid
     cluster_sync_all();        // the peer's barriers exist before anything signals them
     tc_fence_after();
 
-    if (warp == 0) {
+    if (spare && warp < kDecThreads / 32) {   // nothing to multiply
+    } else if (warp == 0) {
         if (lane == 0) {
             const uint32_t full0 = map_to_cta(smem_u32(&bars->full[0]), 0);   // the even CTA's full barriers
             const int tx = 2 * (wbytes + 2 * half * BK * 2);                   // both CTAs' bytes
@@ -526,7 +528,7 @@ decode_gateup_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
-    if (warp == 1) {
+    if (warp == 1 && !spare) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(bars->tmem_base), "r"(512) : "memory");
     }
@@ -801,7 +803,15 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
     const bool pair = recover != nullptr && mt == 2;
     const int unit = pair ? 16 : 8;   // the instructions take N = 2 R in units of 16, over a pair of CTAs of 32
     const int R = min(128, ((c.d_ff + plan->sm_count - 1) / plan->sm_count + unit - 1) & ~(unit - 1));
-    const int gateup_ctas = pair ? 2 * ((c.d_ff + 2 * R - 1) / (2 * R)) : (c.d_ff + R - 1) / R;
+    int gateup_ctas = pair ? 2 * ((c.d_ff + 2 * R - 1) / (2 * R)) : (c.d_ff + R - 1) / R;
+    // A pair's channels come in units of 32, so a narrow layer has few pairs, each with more tokens to recover in turn (8 groups of d = 256,
+    // 200 tokens: 64 CTAs and four rounds of 3 us, where units of 8 had given 128 CTAs).  Pairs without channels take over where
+    // that saves a round: that step 32.9 us, with the channels' pairs alone 46.6, on single CTAs 34.6; 24 groups of d = 1024, 256 tokens,
+    // 43.1, 49.9, 44.5; 40 of d = 1024, 129 tokens, 37.4, 43.0, 42.2.
+    if (pair) {
+        const int rounds = (B + plan->sm_count - 1) / plan->sm_count;
+        if (rounds < (B + gateup_ctas - 1) / gateup_ctas) gateup_ctas = max(gateup_ctas, ((B + rounds - 1) / rounds + 1) & ~1);
+    }
     const int half = ((B + 1) / 2 + 7) & ~7;   // pair: tokens of the even CTA
     __nv_bfloat16 *x_hi = static_cast<__nv_bfloat16 *>(plan->x_bf16), *x_lo = x_hi + (size_t)c.max_tokens * c.d;
     __nv_bfloat16 *act = static_cast<__nv_bfloat16 *>(plan->act), *act_lo = act + (size_t)c.max_tokens * c.d_ff;

@@ -56,6 +56,18 @@ def test_layer_step_on_pairs_of_ctas(d, G, m, k, B, norm):
     plan.close()
 
 
+# The same in layers so narrow that pairs without channels join in to recover: one and two tokens a CTA, the last CTA without any.
+@pytest.mark.parametrize("B", [129, 148, 149, 200, 255, 256])
+@pytest.mark.parametrize("d,G,m,k", [(256, 1, 2, 1), (256, 8, 6, 3), (1024, 24, 12, 6)])
+def test_layer_step_on_pairs_of_ctas_narrow_layers(d, G, m, k, B):
+    cfg = W.CONFIGS["l2_7b_b64"].with_(n_layers=1, d=d, d_ff=128 * G, m=m, k=k, T=6, B=B, index=360 + B)
+    L = W.make_layer(cfg, device="cuda:0")
+    plan = make_plan(cfg)
+    rep, _, _ = compare_layer_step(cfg, L, plan, W.make_tokens(cfg, L.A).h)   # output bound 1e-4 (parity_util)
+    assert rep.excused <= max(1, B // 16), rep
+    plan.close()
+
+
 # Gather path: few rows for many CTAs, and three or four tokens of 55 to 60 groups.
 @pytest.mark.parametrize("k,B", [(55, 4), (56, 4), (60, 3), (1, 3)])
 def test_gather_rows_per_cta_edges(k, B):
