@@ -782,16 +782,31 @@ def test_uds_budget_matches_oracle(B, V):
 
 
 # Rows over clusters of 1, 2, 4 and 8 CTAs (by tokens and by vocabulary), batches of 8 and 16 logits a thread, and rows that end
-# just before, on and behind a batch or a CTA's share.
+# just before, on and behind a batch or a CTA's share.  The probability lies on the first and last logit of every share and every batch
+# (16 to 118 of them, nearly equal), so H is about the logarithm of their number and one that is left out or counted twice moves it
+# by more than 0.005, against a bound of 1e-4.
 @pytest.mark.parametrize("B,V", [(1, 4095), (2, 4097), (2, 8191), (2, 8192), (37, 16385), (38, 4099), (74, 12289), (75, 8193), (149, 33),
                                  (3, 65537), (9, 32767), (20, 70001)])
 def test_uds_budget_splits_of_a_row(B, V):
+    edges = {0, V - 1}
+    for ctas in (1, 2, 4, 8):
+        per = -(-V // ctas)
+        for lo in range(0, V, per):
+            hi = min(V, lo + per)
+            starts = {lo} | {lo + i for i in range(4096, per, 4096)}
+            edges |= {e for s in starts for e in (s - 1, s) if 0 <= e < V} | {hi - 1}
+    edges = torch.tensor(sorted(edges))
     g = torch.Generator().manual_seed(300 + B + V)
-    logits = torch.randn((B, V), generator=g) * torch.logspace(-1, 1, B)[:, None]
-    logits[0, -1] = 30.0
+    logits = torch.randn((B, V), generator=g) - 30.0
+    logits[:, edges] = 0.1 * torch.randn((B, len(edges)), generator=g)
+    ref = oracle.uds_budget(logits, 16.0, 0.75, 8, 64)
+    fewer = logits[:1].clone()
+    for e in edges[:: max(1, len(edges) // 8)]:   # what the bound below would miss, by the oracle
+        fewer.copy_(logits[:1]); fewer[0, e] = float("-inf")
+        assert abs(oracle.uds_budget(fewer, 16.0, 0.75, 8, 64).H[0] - ref.H[0]) > 0.005
     plan = cs.Plan(256, 1024, 64, 8, 4, 4, torch.float32, B, 1e-5)
     m_t, H = cs.cs_uds_budget(plan, logits.to(DEV), 16.0, 0.75, 8, 64)
-    _check_budget(m_t, H, oracle.uds_budget(logits, 16.0, 0.75, 8, 64), 16.0, 0.75)
+    _check_budget(m_t, H, ref, 16.0, 0.75)
     plan.close()
 
 

@@ -6,7 +6,7 @@ import torch
 import oracle
 import paper_2604_14156_b200 as cs
 from gen import workloads as W
-from parity_util import compare_layer_step, device_layer, make_plan, recovery_matches
+from parity_util import compare_layer_step, device_layer, make_plan, recovery_matches, rel
 
 pytestmark = pytest.mark.gpu
 
@@ -27,11 +27,11 @@ def test_layer_step_sense_cluster_edges(d, G, m, k, B, norm):
     plan.close()
 
 
-# A plain step's form of the sensing launch (with or without the RMSNorm, every row of S in shared memory or not: 64 rows of 4096 beside
-# 128 groups are not) against the general one, which a request for the drift takes: the same bits.  List lengths around 8, 16 and 24.
+# A plain step's form of the sensing launch (with or without the RMSNorm; there is one only where every row of S fits in shared memory)
+# against the form for options, which a request for the drift takes: the same bits.  List lengths around 8, 16 and 24.
 @pytest.mark.parametrize("norm", [False, True])
-@pytest.mark.parametrize("d,G,m,k", [(256, 16, 8, 4), (320, 40, 20, 8), (1088, 70, 33, 9), (256, 100, 40, 16), (512, 128, 64, 17), (4096, 128, 64, 24),
-                                     (4096, 128, 64, 25), (256, 128, 30, 64)])
+@pytest.mark.parametrize("d,G,m,k", [(256, 16, 8, 4), (320, 40, 20, 8), (1088, 70, 33, 9), (256, 100, 40, 16), (512, 128, 64, 17), (2048, 128, 64, 24),
+                                     (2048, 128, 64, 25), (256, 128, 30, 64)])
 def test_sense_launch_plain_and_general_forms_agree(d, G, m, k, norm):
     cfg = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"].with_(n_layers=1, w_dtype="f32", d=d, d_ff=64 * G, group=64, m=m, k=k, T=7, B=3,
                                                                   index=470 + k)
@@ -43,6 +43,40 @@ def test_sense_launch_plain_and_general_forms_agree(d, G, m, k, norm):
     for a, b in zip(plain, cs.cs_layer_step_ex(plan, lay, x, opt)):
         assert torch.equal(a, b)
     assert not opt.delta.any() and plan.device_status() == 0
+    plan.close()
+
+
+# Steps with a warm start, the temporal term and the drift, and the plain steps before them, against the oracle: rows of S that do not fit in
+# shared memory (64 of 4096 beside 128 groups), where both kinds of step are one form, and rows that do.
+@pytest.mark.parametrize("norm", [False, True])
+@pytest.mark.parametrize("d,G,m,k", [(4096, 128, 64, 24), (4096, 128, 64, 25), (4096, 128, 64, 8), (320, 40, 20, 9), (192, 31, 12, 24), (512, 60, 33, 33)])
+def test_sense_launch_options_match_oracle(d, G, m, k, norm):
+    cfg = W.CONFIGS["l3_8b_stack" if norm else "l2_7b_b64"].with_(n_layers=1, w_dtype="f32", d=d, d_ff=64 * G, group=64, m=m, k=k, T=7, B=3,
+                                                                  index=490 + k)
+    L = W.make_layer(cfg, device="cuda:0")
+    Lc = L.to("cpu")
+    h, h2 = W.make_tokens(cfg, L.A).h, W.make_tokens(cfg, L.A, batch=1).h
+    plan = make_plan(cfg)
+    lay = device_layer(plan, L)
+    rep, _, _ = compare_layer_step(cfg, L, plan, h)
+    _, sup0, z0, _ = cs.cs_layer_step(plan, lay, h.to("cuda:0"))
+    x = 0.9 * h + 0.1 * h2
+    opt = cs.StepOptions(plan, 3, T=4, support_prev=sup0, z_prev=z0, warm_start=True, gamma=0.25, want_drift=True)
+    out, sup, z, resid = (t.cpu().numpy() for t in cs.cs_layer_step_ex(plan, lay, x.to("cuda:0"), opt))
+    assert plan.device_status() == 0
+    excused = rep.excused
+    for t in range(3):
+        n = oracle.rmsnorm(x[t], Lc.gamma, cfg.rms_eps) if norm else x[t].double().numpy()
+        y = oracle.sketch(Lc.S, n)
+        prev = np.zeros(G)
+        prev[sup0[t].cpu().numpy()] = z0[t].cpu().numpy()
+        ref = oracle.iht_temporal(Lc.Phi, y, k, 4, L.mu, 0.25, prev, prev)
+        excused += not recovery_matches(sup[t], z[t], float(resid[t]), ref, Lc.Phi.numpy(), y, (t,))
+        want = oracle.ffn(Lc.W_gate, Lc.W_up, Lc.Wd_t, cfg.group, n, sup[t])
+        want = want + x[t].double().numpy() if norm else want
+        assert rel(out[t], want) <= 1e-5, t   # f32 weights, on the support that was recovered
+    assert excused <= 1
+    assert opt.delta.cpu().numpy().tolist() == oracle.support_drift(sup0.cpu().numpy(), sup).tolist()
     plan.close()
 
 
