@@ -16,7 +16,7 @@
  *   - Calls only enqueue work on `stream` (a cudaStream_t passed as void*, NULL = default
  *     stream) and return without synchronising.  A plan must not be used from two streams at
  *     once: its scratch is shared by all calls.
- *   - The arrays of a cs_layer (and S, Phi where a call takes them by themselves) are parameters: a
+ *   - The arrays of a layer (and S, Phi where a call takes them by themselves) are parameters: a
  *     launch may read them while the launches ahead of it on the stream still run, as far as those
  *     allow it (this library's do; so do kernels that trigger a programmatic launch themselves).
  *     Updating them on the stream by copies or ordinary kernels ahead of a call is fine.  A
@@ -345,10 +345,11 @@ cs_status cs_layer_step_host(cs_plan *plan, const cs_layer *layer, const float *
  * Regime crossover (Sec. 7: which precompiled execution path a batch takes).  Decode batches of at
  * least `tokens` tokens (and at most 256) run on the tensor cores, smaller ones as the gather GEMV.
  * A plan starts at max(2, min(16, ceil(1.15 * G / k))), the point where streaming every group once
- * moves fewer bytes than streaming k groups per token; 1 <= tokens <= 129 (129: from 129 tokens on,
- * the largest value: no batch beyond 128 tokens takes the gather).  Only shapes the tensor-core path
- * supports (bf16 weights, 128-channel groups, d a multiple of 256) are affected.  cs_plan_crossover
- * returns the current value.
+ * moves fewer bytes than streaming k groups per token (the two paths are even within a batch of it at
+ * d = 2048, 4096 and 6144; at d = 5120 already at two thirds of it, where a smaller value saves up to a
+ * quarter of a step); 1 <= tokens <= 129 (129, the largest value: no batch beyond 128 tokens takes the
+ * gather).  Only shapes the tensor-core path supports (bf16 weights, 128-channel groups, d a multiple of
+ * 256) are affected.  cs_plan_crossover returns the current value.
  */
 cs_status cs_plan_set_crossover(cs_plan *plan, int32_t tokens);
 int32_t cs_plan_crossover(const cs_plan *plan);
