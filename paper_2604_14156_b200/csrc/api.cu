@@ -94,9 +94,10 @@ cs_status cs_plan_create(const cs_config *cfg, cs_plan **out) {
     p->mma_ok = cfg->w_dtype == CS_BF16 && cfg->group == 128 && cfg->d % 256 == 0;
     // The gather path streams B * k groups, the tensor-core path every group once: it takes over where the first exceeds
     // the second by 15 %.  One step, gather against tensor path, at the last batch on each side of the line: 22 of 86 groups of
-    // d = 4096, 4 tokens 44.0 and 48.2 us, 5 tokens 50.5 and 49.6; 9 of 86, 10 tokens 45.1 and 48.8, 11 tokens 46.7 and 47.7;
-    // 12 of 48 of d = 2048, 4 tokens 23.1 and 27.8, 5 tokens 26.5 and 28.7.  At d = 5120, whose rows are 1.25 of the gather's
-    // slices, the curves meet earlier than the rule has it (11 of 108 groups: 8 tokens 71.5 and 65.1, rule 12).
+    // d = 4096, 4 tokens 44.0 and 48.2 us, 5 tokens 50.5 and 49.6; 9 of 86, 10 tokens 45.1 and 48.8, 11 tokens 46.7 and 47.7, 12
+    // 50.7 and 49.5; 12 of 48 of d = 2048, 4 tokens 23.1 and 27.8, 5 tokens 26.5 and 28.7, 6 28.3 and 28.4: there the line is one batch
+    // early.  It knows nothing of the row width: at d = 5120, whose rows are 1.25 of the gather's slices, it is late (11 of 108 groups,
+    // 8 tokens 71.5 and 65.1, 11 tokens 85.3 and 67.7; 27 of 108, 3 tokens 64.8 both, 4 tokens 79.6 and 66.9); cs_plan_set_crossover moves it.
     p->mma_min_tokens = max(2, min(kMmaMinTokens, (int)ceilf(1.15f * (float)p->G / (float)cfg->k)));
     alloc((void **)&p->mask, nt * 4 * sizeof(uint32_t));
     alloc((void **)&p->mask_count, sizeof(unsigned));

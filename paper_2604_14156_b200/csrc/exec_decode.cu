@@ -17,8 +17,8 @@
 // f32 activations enter as two bf16 matrices, rounded value and remainder (16 mantissa bits together).  PACK
 // (at most 64 tokens): values are rows 0.. and remainders rows 64.. of ONE 128-row operand, their products are added in
 // the epilogue.  Otherwise values and remainders are two operands that accumulate into the same tensor-memory
-// columns; MT = 2 (more than 128 tokens) keeps two accumulators (a step's gate/up there runs on pairs of CTAs).  Rows no token
-// owns hold whatever shared memory held: rows of an MMA do not mix, and those results are never read.
+// columns; MT = 2 (more than 128 tokens) keeps two accumulators (gate/up of a step with at most 64 groups per token runs on pairs of
+// CTAs there).  Rows no token owns hold whatever shared memory held: rows of an MMA do not mix, and those results are never read.
 //
 // Balance: the channel tiles of gate/up are not tied to the 128-channel groups.  A CTA takes R channels, R the
 // multiple of 8 that gives every SM one CTA (80 at d_ff = 11008: 138 CTAs on 148 SMs; one CTA per group left 62 SMs
@@ -357,12 +357,13 @@ decode_gateup_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     teardown_cta(bars, warp, tcols);
 }
 
-// The same for a step of more than 128 tokens, on pairs of CTAs (a cluster of two).  With both accumulators in one CTA every weight tile
+// The same for a step of more than 128 tokens and at most 64 groups per token, on pairs of CTAs (a cluster of two).  (Beyond 64 groups the
+// recovery is a launch ahead and gate/up the kernel above with two accumulators, as with given supports.)  With both accumulators in one CTA every weight tile
 // is read from shared memory by four instructions and every k block moves 228 KB through that port for 20 KB of weights (1.03 us a k
 // block, 68 us at 7B and 200 tokens, the tensor pipe 51 % busy).  Here one instruction has M = 256: each CTA holds half of the tokens
 // (their values and their remainders, 128 rows each) and half of the pair's channels, R of 2 R, gate rows then up rows: 156 KB for the
 // same 20 KB of weights per CTA.  One step, 7B: 200 tokens 135.5 to 127.0 us, in short bursts 132 to 121, 256 tokens 139 to 127; d = 5120
-// with 27 of 108 groups, 200 tokens 189 to 181; 129 tokens 113.9 to 112.6, so every batch beyond 128 tokens takes it.
+// with 27 of 108 groups, 200 tokens 189 to 181; 129 tokens 113.9 to 112.6, so every such batch takes it.
 // Gate accumulates in tensor-memory columns 0 .. 2 R, up from 256 on.  The even CTA's MMA thread issues for both; no multicast load, each
 // CTA fetches its own tiles and signals the even CTA's barrier.
 constexpr int kPairTokenBytes = 2 * kABytes;   // value rows, then remainder rows
@@ -750,7 +751,7 @@ template <bool PACK, int MT> GateUpFn gateup_fn_kc(int kc) {
          : kc == 4 ? decode_gateup_kernel<PACK, MT, 4> : kc == 7 ? decode_gateup_kernel<PACK, MT, 7>
          : decode_gateup_kernel<PACK, MT, 8>;
 }
-GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators (2: supports known before; a step takes the pair kernel)
+GateUpFn gateup_fn(int form, int kc) {   // form: 0 packed, 1 / 2 accumulators (2: given supports, or the recovery a launch ahead)
     return form == 0 ? gateup_fn_kc<true, 1>(kc) : form == 1 ? gateup_fn_kc<false, 1>(kc) : decode_gateup_kernel<false, 2, 0>;
 }
 typedef void (*GateUpPairFn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, int, int, int, int, int, const float *, float, RecoverArgs,
@@ -838,12 +839,14 @@ cs_status launch_decode_ffn(cs_plan *plan, const cs_layer *L, int B, const Recov
                        1024 + (size_t)gateup_pair_stages(R) * (kPairTokenBytes + 2 * R * BK * 2) + sizeof(Barriers), st, tm_h, tm_h_lo, tm_g, tm_u, B, half,
                        R, c.d, c.d_ff, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr, c.rms_eps, *recover, act,
                        act_lo, plan->status);
-        } else
-        launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
-                   dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)), by_list ? 1024 + (size_t)kDecRing + sizeof(Barriers) : decode_smem(tt, 2 * R * BK * 2),
-                   st, tm_x, tm_x_lo, tm_g, tm_u, tm_gu, tm_uu, B, R, c.d, c.d_ff,
-                   by_list ? (const int32_t *)plan->mask : (const int32_t *)nullptr, norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr,
-                   c.rms_eps, recover != nullptr ? *recover : RecoverArgs{}, act, act_lo, plan->status);
+        } else {
+            launch_pdl(true, gateup_fn(form, recover != nullptr ? gateup_kc(plan) : 0), dim3(gateup_ctas),
+                       dim3(kDecThreads + (recover != nullptr ? kRecThreads : 0)),
+                       by_list ? 1024 + (size_t)kDecRing + sizeof(Barriers) : decode_smem(tt, 2 * R * BK * 2), st, tm_x, tm_x_lo, tm_g, tm_u, tm_gu,
+                       tm_uu, B, R, c.d, c.d_ff, by_list ? (const int32_t *)plan->mask : (const int32_t *)nullptr,
+                       norm ? (const float *)sketch_square_partials(plan, B) : (const float *)nullptr, c.rms_eps,
+                       recover != nullptr ? *recover : RecoverArgs{}, act, act_lo, plan->status);
+        }
         plan->launches++;
         CS_CUDA_TRY(plan, cudaGetLastError());
     }

@@ -8,8 +8,8 @@
 // thread, then plain sums in a fixed order (warp, CTA, cluster over distributed shared memory); CTA 0 ends with
 //     H = log Z - W / Z.
 // Small batches are a latency chain (at 11 tokens of 32000 logits one load round trip and the folds): as two launches, the row's
-// moments merged pairwise with two exponentials a merge and folded by the second launch, 1 x 32000 logits took 5.5 us and 11 x 32000 5.6,
-// now 2.5 and 3.1.  Large ones are bound by HBM and the arithmetic: 64 x 128256 16.7 and 10.8 us, 512 x 128256 66.6 and 54.0 (4.9 TB/s).
+// moments merged pairwise with two exponentials a merge and folded by the second launch, 1 x 32000 logits took 5.6 us and 11 x 32000 5.7,
+// now 2.6 and 2.8.  Large ones are bound by HBM and the arithmetic: 64 x 128256 16.6 and 10.9 us, 512 x 128256 66.6 and 52.9 (5.0 TB/s).
 #include "cs_internal.cuh"
 
 namespace cs {

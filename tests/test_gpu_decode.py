@@ -31,7 +31,7 @@ def test_layer_step_token_and_channel_tile_edges(B, d, G, m, k, norm):
 
 
 # Gather path: a step's form of the kernel against the one for given supports, the same bits.  Rows that are whole slices of 512 chunks
-# (one, two and four a thread) and rows that are not.
+# (one, two and four a thread); rows that are not have one form for both.
 @pytest.mark.parametrize("dtype,d", [("bf16", 4096), ("bf16", 8192), ("bf16", 5120), ("bf16", 320), ("f32", 2048), ("f32", 8192), ("f32", 2112), ("f32", 64)])
 def test_gather_step_and_given_supports_agree(dtype, d):
     cfg = W.CONFIGS["l2_7b_b64"].with_(n_layers=1, w_dtype=dtype, d=d, d_ff=64 * 20, group=64, m=12, k=5, T=6, B=2, index=350)
